@@ -1,24 +1,38 @@
 // sbr_gemm.cu -- BF16 tensor-core GEMM on the 5th-generation tensor cores
-// (tcgen05) for the learned surrogate: C = A B^T with A [M x K] and B [N x K]
-// both K-contiguous BF16, FP32 accumulation in tensor memory (TMEM).
+// (tcgen05) for the learned surrogate: C = A B^T with FP32 accumulation in
+// tensor memory (TMEM), for one problem or for a group of equal ones (the
+// ensemble's members, and for weight gradients every layer of every member).
 //
-// One CTA of 128 threads computes a 128 x BN tile (BN = 128, or 64 when the
-// 128-wide grid would leave SMs idle):
-//   - warp 0 (one lane) streams 128 x 64 tiles of A and BN x 64 tiles of B
-//     into shared memory with TMA (cp.async.bulk.tensor, 128-byte swizzle)
-//     through a 3-stage ring of mbarriers, refilling a stage once the MMAs
-//     that read it have completed;
+// A is [M x K] and B [N x K], each stored either K-contiguous or (for
+// gradients, whose contraction runs over the stored rows) with M or N
+// contiguous: the tensor core reads both forms from shared memory, so no
+// operand is transposed in memory.
+//
+// One persistent kernel: a CTA per SM loops over 128 x BN tiles
+// t = blockIdx.x, t + gridDim.x, ... (n-tile fastest, then m-tile, then group):
+//   - warp 0 (one lane) streams 64-deep slices of A and B of every k-step of
+//     every tile into a ring of shared-memory stages with TMA (128-byte
+//     swizzle), refilling a stage once the MMAs that read it have completed;
 //   - warp 1 (one lane) issues tcgen05.mma (M = 128, N = BN, K = 16 per
-//     instruction, 4 per stage) as soon as a stage lands and commits each
-//     stage back to the producer, so MMA issue never waits for a refill;
-//   - after the last K step all four warps read the accumulator out of TMEM
-//     with tcgen05.ld (warp w owns rows 32w .. 32w + 31), apply the fused
-//     epilogue (bias, GELU, GELU derivative) into the now idle pipeline
-//     buffers, and write the tile out row by row with coalesced 16-byte stores
-//     (the pre-activation read of the GELU-derivative epilogue is staged the
-//     same way).
-// Every wait is bounded: on a timeout the CTA records an error flag, skips the
-// remaining work, frees its TMEM and returns.
+//     instruction) for the CTA's tile j into TMEM accumulator j % 2 once the
+//     epilogue has drained it, and commits it;
+//   - the other 8 or 16 warps read the accumulator (warp w: TMEM lanes 32 (w % 4)
+//     .., a share of the columns), hand it back, and apply the fused epilogue 32
+//     columns at a time through staging rows of their own, so that a tile's
+//     read-out and stores overlap the next tile's MMAs.
+// Every wait is bounded and polls the CTA's failure flag: on a timeout the CTA
+// records an error flag, skips the remaining work, lets its loads and MMAs
+// finish, frees its TMEM and returns.
+//
+// What bounds it: the GELU epilogues cost ~36 instructions per output, twice
+// the MMAs' time at K = 512, and one epilogue warp per scheduler left them
+// latency-bound (issue 30 %). Four per scheduler where only BF16 is stored
+// (prediction: issue 72 %, 4 x 65536 x 512 x 512 in 188 us = 730 TFLOP/s, 111 us
+// per member alone before), two where FP32 staging rows take the shared memory.
+// Training's products are bound by their activations: 43 us per layer of 4
+// members x 8192 rows (134 MB moved, 3.1 TB/s) forward and 44 backward, 122 us
+// for all 24 weight gradients (51 GFLOP, 420 TFLOP/s, 2.3 tiles per SM), against
+// 23 us per member and layer and 46 us per weight gradient one by one.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -32,21 +46,30 @@ namespace sbr {
 
 namespace {
 
-constexpr int kBM = 128, kBK = 64, kStages = 3;  // 3 stages keep a CTA at ~103 KB: two per SM
+constexpr int kBM = 128, kBK = 64;
 constexpr int kTileA = kBM * kBK * 2;  // bytes
-constexpr unsigned kSpin = 1u << 24;  // try_wait rounds before a wait gives up
-template <int BN>
+constexpr unsigned kSpin = 1u << 24;   // try_wait rounds before a wait gives up
+// staging of one epilogue warp: 32 rows x 32 columns, FP32 (stride 36) and BF16 (stride 40)
+constexpr int kLdF = 36, kLdH = 40;
+constexpr int kWarpF = 32 * kLdF * 4, kWarpH = 32 * kLdH * 2;
+
+template <int BN, int kMode>
 struct Cfg {
-    static constexpr int kTileB = BN * kBK * 2;
-    static constexpr int kStageBytes = kTileA + kTileB;
+    static constexpr bool kF32 = kMode != kEpiGelu, kH16 = kMode != kEpiF32;  // staging an epilogue warp needs
+    static constexpr int kEpiWarps = kMode == kEpiGelu ? 16 : 8;
+    static constexpr int kThreads = 32 * (2 + kEpiWarps);
+    static constexpr int kWarpStage = (kF32 ? kWarpF : 0) + (kH16 ? kWarpH : 0);
+    static constexpr int kStages = BN == 256 ? 3 : (BN == 128 ? 5 : 6);
+    static constexpr int kStageBytes = kTileA + BN * kBK * 2;
     static constexpr int kPipe = kStages * kStageBytes;
-    // epilogue staging (reuses the pipeline buffers): FP32 [128][BN + 4] and BF16 [128][BN + 8]
-    static constexpr int kLdF = BN + 4, kLdH = BN + 8;
-    static constexpr int kStageF = kBM * kLdF * 4, kStageH = kBM * kLdH * 2;
-    static constexpr int kSmem = (kPipe > kStageF + kStageH ? kPipe : kStageF + kStageH) + 1024;
-    // instruction descriptor: D FP32, A and B BF16, both K-major, M = 128, N = BN
-    static constexpr uint32_t kIdesc =
-        (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
+    static constexpr int kSmem = kPipe + kEpiWarps * kWarpStage + 1024;
+    static_assert(kSmem <= 227 * 1024, "GEMM shared memory");
+    // instruction descriptor: D FP32, A and B BF16, M = 128, N = BN; bits 15 and 16: A, B with M, N contiguous
+    __host__ __device__ static constexpr uint32_t idesc(bool mn_a, bool mn_b)
+    {
+        return (1u << 4) | (1u << 7) | (1u << 10) | (mn_a ? 1u << 15 : 0u) | (mn_b ? 1u << 16 : 0u) |
+               ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
+    }
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -73,18 +96,25 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, unsigned parity)
     }
     return false;
 }
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* tm, int x, int y, uint64_t* bar)
+__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* tm, int x, int y, int z, uint64_t* bar)
 {
     asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-            smem_u32(dst)),
-        "l"((uint64_t)tm), "r"(x), "r"(y), "r"(smem_u32(bar))
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
+        "[%5];" ::"r"(smem_u32(dst)),
+        "l"((uint64_t)tm), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
         : "memory");
 }
-// shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 bytes apart
-__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr)
+// Shared-memory matrix descriptors of a 64-deep slice, 128-byte swizzle, for
+// the 16-deep step kk. K contiguous: rows of 128 bytes (64 k), 8-row groups
+// 1024 bytes apart, a step 32 bytes along the row. M or N contiguous: blocks of
+// 64 m by 64 k (a row of 128 bytes per k) 8192 bytes apart, 8-k groups 1024
+// bytes apart, a step two groups further.
+template <bool kMn>
+__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr, int kk)
 {
-    return (uint64_t)((saddr >> 4) & 0x3FFF) | (1ull << 16) | (64ull << 32) | (1ull << 46) | (2ull << 61);
+    const uint32_t a = kMn ? saddr + 2048u * kk : saddr + 32u * kk;
+    const uint64_t lead = kMn ? 512ull : 1ull;
+    return (uint64_t)((a >> 4) & 0x3FFF) | (lead << 16) | (64ull << 32) | (1ull << 46) | (2ull << 61);
 }
 __device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t acc)
 {
@@ -102,9 +132,9 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar)
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v)
+// 32 accumulator columns of the warp's rows; the registers hold them after tmem_wait
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r)
 {
-    uint32_t r[32];
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
         "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
@@ -113,189 +143,14 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v)
           "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
           "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
         : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
+__device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 __device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.f + erff(z * 0.70710678118654752f)); }
 __device__ __forceinline__ float gelu_grad(float z)
 {
     return 0.5f * (1.f + erff(z * 0.70710678118654752f)) + z * 0.3989422804014327f * expf(-0.5f * z * z);
 }
-
-template <int BN>
-__global__ void __launch_bounds__(128, 2) k_gemm_tn(const __grid_constant__ CUtensorMap tmA,
-                                                    const __grid_constant__ CUtensorMap tmB, const GemmEpi ep, int K,
-                                                    int* err)
-{
-    using C = Cfg<BN>;
-    extern __shared__ unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t full[kStages], empty[kStages], done;
-    __shared__ uint32_t tmem_base;
-    __shared__ int s_fail, s_issued, s_consumed;
-    unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.y * kBM, n0 = blockIdx.x * BN;
-    const int KT = K / kBK;
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
-                     "r"(BN)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    if (tid == 0) {
-        for (int st = 0; st < kStages; ++st) {
-            mbar_init(&full[st], 1);
-            mbar_init(&empty[st], 1);
-        }
-        mbar_init(&done, 1);
-        s_fail = 0;
-        s_issued = 0;
-        s_consumed = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = tmem_base;
-
-    if (tid == 0) {
-        // producer: stage kt % kStages is refilled once the MMAs of step kt - kStages have completed
-        for (int kt = 0; kt < KT; ++kt) {
-            const int st = kt % kStages;
-            if (kt >= kStages && !mbar_wait(&empty[st], (unsigned)(kt / kStages - 1) & 1u)) {
-                s_fail = 1;
-                break;
-            }
-            if (*(volatile int*)&s_fail) break;
-            unsigned char* sa = smem + st * C::kStageBytes;
-            mbar_expect_tx(&full[st], C::kStageBytes);
-            tma_load_2d(sa, &tmA, kt * kBK, m0, &full[st]);
-            tma_load_2d(sa + kTileA, &tmB, kt * kBK, n0, &full[st]);
-            *(volatile int*)&s_issued = kt + 1;
-        }
-    } else if (tid == 32) {
-        // MMA issuer
-        bool ok = true;
-        for (int kt = 0; kt < KT; ++kt) {
-            const int st = kt % kStages;
-            if (!mbar_wait(&full[st], (unsigned)(kt / kStages) & 1u)) {
-                ok = false;
-                break;
-            }
-            tc_fence_after();
-            const uint32_t sa = smem_u32(smem + st * C::kStageBytes);
-            const uint32_t sb = sa + kTileA;
-#pragma unroll
-            for (int kk = 0; kk < kBK / 16; ++kk)
-                mma_bf16(tmem, desc_sw128(sa + 32 * kk), desc_sw128(sb + 32 * kk), C::kIdesc, (kt | kk) != 0);
-            mma_commit(&empty[st]);
-            *(volatile int*)&s_consumed = kt + 1;
-        }
-        if (ok) mma_commit(&done);
-        else *(volatile int*)&s_fail = 1;
-    }
-    // wait for the accumulator (or for the issuer to give up)
-    bool ready = false;
-    for (int r = 0; r < 4 && !ready; ++r) {
-        ready = mbar_wait(&done, 0);
-        if (*(volatile int*)&s_fail) break;
-    }
-    tc_fence_after();
-    __syncthreads();  // all TMA writes and MMA reads of the pipeline buffers are over: reuse them
-    if (!ready || s_fail) {
-        if (tid == 0) {
-            atomicExch(err, 1);
-            // let the loads still in flight land before the CTA's shared memory goes away
-            for (int kt = s_consumed; kt < s_issued; ++kt) mbar_wait(&full[kt % kStages], (unsigned)(kt / kStages) & 1u);
-        }
-    } else {
-        float* sf = reinterpret_cast<float*>(smem);                          // FP32 [128][kLdF]
-        __nv_bfloat16* sh = reinterpret_cast<__nv_bfloat16*>(smem + C::kStageF);  // BF16 [128][kLdH]
-        const int r = warp * 32 + lane;  // tile row of this thread
-        if (ep.mode == kEpiGeluGrad) {
-            // stage the pre-activation tile with coalesced loads
-            for (int q = tid; q < kBM * (BN / 4); q += 128) {
-                const int rr = q / (BN / 4), cc = (q % (BN / 4)) * 4;
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (m0 + rr < ep.M) v = *reinterpret_cast<const float4*>(ep.z + (size_t)(m0 + rr) * ep.ldz + n0 + cc);
-                *reinterpret_cast<float4*>(sf + rr * C::kLdF + cc) = v;
-            }
-            __syncthreads();
-        }
-        for (int c0 = 0; c0 < BN; c0 += 32) {
-            float v[32];
-            tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
-            if (ep.mode == kEpiF32) {
-#pragma unroll
-                for (int i = 0; i < 32; i += 4)
-                    *reinterpret_cast<float4*>(sf + r * C::kLdF + c0 + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-            } else if (ep.mode == kEpiBiasGelu) {
-#pragma unroll
-                for (int i = 0; i < 32; i += 2) {
-                    const float z0 = v[i] + ep.bias[n0 + c0 + i], z1 = v[i + 1] + ep.bias[n0 + c0 + i + 1];
-                    *reinterpret_cast<float2*>(sf + r * C::kLdF + c0 + i) = make_float2(z0, z1);
-                    *reinterpret_cast<__nv_bfloat162*>(sh + r * C::kLdH + c0 + i) =
-                        __floats2bfloat162_rn(gelu(z0), gelu(z1));
-                }
-            } else {  // kEpiGeluGrad: dz = acc * gelu'(z)
-#pragma unroll
-                for (int i = 0; i < 32; i += 2) {
-                    const float2 z = *reinterpret_cast<const float2*>(sf + r * C::kLdF + c0 + i);
-                    *reinterpret_cast<__nv_bfloat162*>(sh + r * C::kLdH + c0 + i) =
-                        __floats2bfloat162_rn(v[i] * gelu_grad(z.x), v[i + 1] * gelu_grad(z.y));
-                }
-            }
-        }
-        __syncthreads();
-        // coalesced write-out: consecutive threads take consecutive 16-byte pieces of a row
-        if (ep.mode != kEpiGeluGrad && ep.c_f32) {
-            for (int q = tid; q < kBM * (BN / 4); q += 128) {
-                const int rr = q / (BN / 4), cc = (q % (BN / 4)) * 4;
-                if (m0 + rr < ep.M)
-                    *reinterpret_cast<float4*>(ep.c_f32 + (size_t)(m0 + rr) * ep.ldc + n0 + cc) =
-                        *reinterpret_cast<const float4*>(sf + rr * C::kLdF + cc);
-            }
-        }
-        if (ep.mode != kEpiF32) {
-            for (int q = tid; q < kBM * (BN / 8); q += 128) {
-                const int rr = q / (BN / 8), cc = (q % (BN / 8)) * 8;
-                if (m0 + rr < ep.M)
-                    *reinterpret_cast<uint4*>(ep.out_bf16 + (size_t)(m0 + rr) * ep.ldo + n0 + cc) =
-                        *reinterpret_cast<const uint4*>(sh + rr * C::kLdH + cc);
-            }
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN) : "memory");
-}
-
-// ---------------------------------------------------------------- persistent form
-// For grids of at least two 128 x 128 tiles per SM: one CTA per SM loops over
-// the tiles t = blockIdx.x, t + gridDim.x, ... (n-tile fastest) with six warps.
-// Warp 0 (one lane) streams the A and B tiles of every k-step of every tile
-// through the 3-stage ring; warp 1 (one lane) issues the MMAs of the CTA's
-// tile j into TMEM accumulator j % 2 (128 columns each) once the epilogue has
-// drained it and commits it; warps 2-5 read their 32 rows of the accumulator
-// (TMEM lanes 32 (w % 4) ..), release it, and apply the epilogue through
-// staging rows of their own, so that a tile's read-out, epilogue and stores
-// overlap the next tile's MMAs. The MMAs of a tile come in the same order and
-// the epilogue does the same arithmetic as in k_gemm_tn: the results are the
-// same bit for bit. Every wait is bounded and polls the CTA's failure flag.
-constexpr int kPpStages = 3;
-constexpr int kPpThreads = 192;
-struct PpCfg {
-    static constexpr int BN = 128;
-    static constexpr int kStageBytes = kTileA + BN * kBK * 2;  // 32 KB
-    static constexpr int kPipe = kPpStages * kStageBytes;
-    static constexpr int kLdF = BN + 4, kLdH = BN + 8;
-    static constexpr int kWarpF = 32 * kLdF * 4, kWarpH = 32 * kLdH * 2;  // staging of one epilogue warp
-    static constexpr int kSmem = kPipe + 4 * (kWarpF + kWarpH) + 1024;
-};
-static_assert(PpCfg::kSmem <= 227 * 1024, "persistent GEMM shared memory");
 
 // a bounded wait that also gives up once another role of the CTA has failed
 __device__ __forceinline__ bool pp_wait(uint64_t* b, unsigned parity, volatile int* fail)
@@ -314,33 +169,57 @@ __device__ __forceinline__ bool pp_wait(uint64_t* b, unsigned parity, volatile i
     return false;
 }
 
-__global__ void __launch_bounds__(kPpThreads, 1) k_gemm_pp(const __grid_constant__ CUtensorMap tmA,
-                                                           const __grid_constant__ CUtensorMap tmB, const GemmEpi ep,
-                                                           int K, int tiles_n, int n_tiles, int* err)
+// What a launch computes. Tile t < tiles0 belongs to the first segment: group
+// t / per[0] (operands at that index of the third map dimension, A from za[0]
+// on), tile rows and columns from the remainder; later tiles to the second one
+// (B from tmB1). Group g = layer * n_inner + member: its outputs start at
+// layer * (layer stride) + member * (member stride).
+struct GemmGrid {
+    int KT;                // 64-deep k-steps
+    int n_tiles, tiles0;
+    int tn[2], per[2];     // n-tiles per tile row, tiles per group
+    int za[2];
+    int n_inner;
+    GemmEpi ep[2];
+};
+
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b)
 {
-    using C = PpCfg;
+    __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<uint32_t*>(&p);
+}
+
+template <int BN, bool kMnA, bool kMnB, int kMode>
+__global__ void __launch_bounds__((Cfg<BN, kMode>::kThreads), 1) k_gemm(const __grid_constant__ CUtensorMap tmA,
+                                                          const __grid_constant__ CUtensorMap tmB0,
+                                                          const __grid_constant__ CUtensorMap tmB1,
+                                                          const __grid_constant__ GemmGrid G, int* err)
+{
+    using C = Cfg<BN, kMode>;
+    constexpr int kStages = C::kStages, kEpiWarps = C::kEpiWarps;
     extern __shared__ unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t full[kPpStages], empty[kPpStages], tfull[2], tempty[2], drained;
+    __shared__ __align__(8) uint64_t full[kStages], empty[kStages], tfull[2], tempty[2], drained;
     __shared__ uint32_t tmem_base;
     __shared__ int s_fail, s_issued, s_consumed;
     unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int KT = K / kBK;
-    const int my_tiles = (n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int KT = G.KT;
+    const int my_tiles = (G.n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
     volatile int* fail = &s_fail;
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(smem_u32(&tmem_base))
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
+                     "r"(2 * BN)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        for (int st = 0; st < kPpStages; ++st) {
+        for (int st = 0; st < kStages; ++st) {
             mbar_init(&full[st], 1);
             mbar_init(&empty[st], 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&tfull[b], 1);
-            mbar_init(&tempty[b], 4);  // one arrival per epilogue warp
+            mbar_init(&tempty[b], kEpiWarps);  // one arrival per epilogue warp
         }
         mbar_init(&drained, 1);
         s_fail = 0;
@@ -354,22 +233,36 @@ __global__ void __launch_bounds__(kPpThreads, 1) k_gemm_pp(const __grid_constant
     const uint32_t tmem = tmem_base;
 
     if (tid == 0) {
-        // producer: global k-step g of the CTA refills stage g % kPpStages once the MMAs of step g - kPpStages
-        // have completed
+        // producer: global k-step g of the CTA refills stage g % kStages once the MMAs of step g - kStages have
+        // completed
         int g = 0;
         for (int j = 0; j < my_tiles && !*fail; ++j) {
             const int t = (int)blockIdx.x + j * (int)gridDim.x;
-            const int m0 = (t / tiles_n) * kBM, n0 = (t % tiles_n) * C::BN;
+            const int sg = t >= G.tiles0, tt = sg ? t - G.tiles0 : t;
+            const int z = tt / G.per[sg], r = tt - z * G.per[sg];
+            const int m0 = (r / G.tn[sg]) * kBM, n0 = (r % G.tn[sg]) * BN, zA = G.za[sg] + z;
+            const CUtensorMap* tmB = sg ? &tmB1 : &tmB0;
             for (int kt = 0; kt < KT; ++kt, ++g) {
-                const int st = g % kPpStages;
-                if (g >= kPpStages && !pp_wait(&empty[st], (unsigned)(g / kPpStages - 1) & 1u, fail)) {
+                const int st = g % kStages;
+                if (g >= kStages && !pp_wait(&empty[st], (unsigned)(g / kStages - 1) & 1u, fail)) {
                     *fail = 1;
                     break;
                 }
-                unsigned char* sa = smem + st * C::kStageBytes;
+                unsigned char *sa = smem + st * C::kStageBytes, *sb = sa + kTileA;
                 mbar_expect_tx(&full[st], C::kStageBytes);
-                tma_load_2d(sa, &tmA, kt * kBK, m0, &full[st]);
-                tma_load_2d(sa + kTileA, &tmB, kt * kBK, n0, &full[st]);
+                if (kMnA) {
+                    tma_load_3d(sa, &tmA, m0, kt * kBK, zA, &full[st]);
+                    tma_load_3d(sa + 8192, &tmA, m0 + 64, kt * kBK, zA, &full[st]);
+                } else {
+                    tma_load_3d(sa, &tmA, kt * kBK, m0, zA, &full[st]);
+                }
+                if (kMnB) {
+#pragma unroll
+                    for (int b = 0; b < BN / 64; ++b)
+                        tma_load_3d(sb + 8192 * b, tmB, n0 + 64 * b, kt * kBK, z, &full[st]);
+                } else {
+                    tma_load_3d(sb, tmB, kt * kBK, n0, z, &full[st]);
+                }
                 *(volatile int*)&s_issued = g + 1;
             }
         }
@@ -384,10 +277,10 @@ __global__ void __launch_bounds__(kPpThreads, 1) k_gemm_pp(const __grid_constant
                 break;
             }
             tc_fence_after();
-            const uint32_t acc = tmem + (uint32_t)(b * C::BN);
+            const uint32_t acc = tmem + (uint32_t)(b * BN);
             for (int kt = 0; kt < KT; ++kt, ++g) {
-                const int st = g % kPpStages;
-                if (!pp_wait(&full[st], (unsigned)(g / kPpStages) & 1u, fail)) {
+                const int st = g % kStages;
+                if (!pp_wait(&full[st], (unsigned)(g / kStages) & 1u, fail)) {
                     ok = false;
                     break;
                 }
@@ -396,7 +289,7 @@ __global__ void __launch_bounds__(kPpThreads, 1) k_gemm_pp(const __grid_constant
                 const uint32_t sb = sa + kTileA;
 #pragma unroll
                 for (int kk = 0; kk < kBK / 16; ++kk)
-                    mma_bf16(acc, desc_sw128(sa + 32 * kk), desc_sw128(sb + 32 * kk), Cfg<128>::kIdesc,
+                    mma_bf16(acc, desc_sw128<kMnA>(sa, kk), desc_sw128<kMnB>(sb, kk), C::idesc(kMnA, kMnB),
                              (kt | kk) != 0);
                 mma_commit(&empty[st]);
                 *(volatile int*)&s_consumed = g + 1;
@@ -408,71 +301,115 @@ __global__ void __launch_bounds__(kPpThreads, 1) k_gemm_pp(const __grid_constant
         mma_commit(&drained);
         mbar_wait(&drained, 0);
     } else if (warp >= 2) {
-        // epilogue: warp w owns tile rows (TMEM lanes) 32 (w % 4) .. 32 (w % 4) + 31
-        const int q = warp & 3;
-        float* sf = reinterpret_cast<float*>(smem + C::kPipe + (warp - 2) * (C::kWarpF + C::kWarpH));
-        __nv_bfloat16* sh = reinterpret_cast<__nv_bfloat16*>(reinterpret_cast<unsigned char*>(sf) + C::kWarpF);
+        // epilogue: warp w owns tile rows (TMEM lanes) 32 (w % 4) .. 32 (w % 4) + 31 and a share of the columns
+        constexpr int kCols = BN / (kEpiWarps / 4) < 32 ? 32 : BN / (kEpiWarps / 4);
+        constexpr int kShares = BN / kCols;  // warps beyond them (64 columns, 16 warps) only hand back
+        const int q = warp & 3, share = (warp - 2) >> 2, c_off = share * kCols;
+        unsigned char* stage = smem + C::kPipe + (warp - 2) * C::kWarpStage;
+        float* sf = reinterpret_cast<float*>(stage);
+        __nv_bfloat16* sh = reinterpret_cast<__nv_bfloat16*>(stage + (C::kF32 ? kWarpF : 0));
+        const int fr = lane >> 3, fc = 4 * (lane & 7);  // FP32 staging: 16-byte piece of rows fr, fr + 4, ...
+        const int hr = lane >> 2, hc = 8 * (lane & 3);  // BF16 staging: 16-byte piece of rows hr, hr + 8, ...
         for (int j = 0; j < my_tiles; ++j) {
             const int b = j & 1;
             const int t = (int)blockIdx.x + j * (int)gridDim.x;
-            const int m0 = (t / tiles_n) * kBM + 32 * q, n0 = (t % tiles_n) * C::BN;
+            const int sg = t >= G.tiles0, tt = sg ? t - G.tiles0 : t;
+            const int z = tt / G.per[sg], r = tt - z * G.per[sg];
+            const int m0 = (r / G.tn[sg]) * kBM + 32 * q, n0 = (r % G.tn[sg]) * BN + c_off;
+            const GemmEpi& ep = G.ep[sg];
+            const int layer = z / G.n_inner, member = z - layer * G.n_inner;
+            const long long gc = layer * ep.sl_c + member * ep.sg_c;
+            float4 zr[8];  // GELU derivative: the chunk's pre-activations, coalesced, loaded ahead
+            const float* zp = nullptr;
+            if (kMode == kEpiGeluGrad) {
+                zp = ep.z + member * ep.sg_z + (size_t)(m0 + fr) * ep.ldz + n0 + fc;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) zr[i] = *reinterpret_cast<const float4*>(zp + (size_t)(4 * i) * ep.ldz);
+            }
             // warp-uniform decision: the TMEM loads below are warp-collective
             if (!__all_sync(0xffffffffu, pp_wait(&tfull[b], (unsigned)(j >> 1) & 1u, fail))) {
                 *fail = 1;
                 break;
             }
             tc_fence_after();
-            if (ep.mode == kEpiGeluGrad) {
-                // the warp's 32 rows of the pre-activation, coalesced (lane l: columns 4 l .. 4 l + 3)
-                for (int rr = 0; rr < 32; ++rr) {
-                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (m0 + rr < ep.M) v = *reinterpret_cast<const float4*>(ep.z + (size_t)(m0 + rr) * ep.ldz + n0 + 4 * lane);
-                    *reinterpret_cast<float4*>(sf + rr * C::kLdF + 4 * lane) = v;
-                }
-                __syncwarp();
-            }
-            for (int c0 = 0; c0 < C::BN; c0 += 32) {
+            const uint32_t acc = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * BN + c_off);
+            uint32_t vn[32];
+            if (share < kShares) tmem_ld32(acc, vn);
+#pragma unroll 1
+            for (int c0 = 0; c0 < kCols; c0 += 32) {
                 float v[32];
-                tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * C::BN + c0), v);
-                if (ep.mode == kEpiF32) {
+                tmem_wait();
+#pragma unroll
+                for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(vn[i]);
+                if (c0 + 32 < kCols) {
+                    tmem_ld32(acc + c0 + 32, vn);  // the next chunk's columns arrive during this one's epilogue
+                } else {
+                    // the accumulator is in registers: hand it back to the MMA issuer
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0)
+                        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tempty[b])) : "memory");
+                    if (share >= kShares) break;
+                }
+                if (kMode == kEpiF32) {
 #pragma unroll
                     for (int i = 0; i < 32; i += 4)
-                        *reinterpret_cast<float4*>(sf + lane * C::kLdF + c0 + i) =
-                            make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-                } else if (ep.mode == kEpiBiasGelu) {
+                        *reinterpret_cast<float4*>(sf + lane * kLdF + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+                } else if (kMode == kEpiBiasGelu || kMode == kEpiGelu) {
+                    const float4* bias = reinterpret_cast<const float4*>(ep.bias + member * ep.sg_bias + n0 + c0);
 #pragma unroll
-                    for (int i = 0; i < 32; i += 2) {
-                        const float z0 = v[i] + ep.bias[n0 + c0 + i], z1 = v[i + 1] + ep.bias[n0 + c0 + i + 1];
-                        *reinterpret_cast<float2*>(sf + lane * C::kLdF + c0 + i) = make_float2(z0, z1);
-                        *reinterpret_cast<__nv_bfloat162*>(sh + lane * C::kLdH + c0 + i) =
-                            __floats2bfloat162_rn(gelu(z0), gelu(z1));
+                    for (int i = 0; i < 32; i += 8) {
+                        uint32_t o[4];
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) {
+                            const float4 bb = bias[i / 4 + u];
+                            const float* w = v + i + 4 * u;
+                            const float z0 = w[0] + bb.x, z1 = w[1] + bb.y, z2 = w[2] + bb.z, z3 = w[3] + bb.w;
+                            if (C::kF32) *reinterpret_cast<float4*>(sf + lane * kLdF + i + 4 * u) = make_float4(z0, z1, z2, z3);
+                            o[2 * u] = pack_bf16(gelu(z0), gelu(z1));
+                            o[2 * u + 1] = pack_bf16(gelu(z2), gelu(z3));
+                        }
+                        *reinterpret_cast<uint4*>(sh + lane * kLdH + i) = make_uint4(o[0], o[1], o[2], o[3]);
                     }
                 } else {  // kEpiGeluGrad: dz = acc * gelu'(z)
 #pragma unroll
-                    for (int i = 0; i < 32; i += 2) {
-                        const float2 z = *reinterpret_cast<const float2*>(sf + lane * C::kLdF + c0 + i);
-                        *reinterpret_cast<__nv_bfloat162*>(sh + lane * C::kLdH + c0 + i) =
-                            __floats2bfloat162_rn(v[i] * gelu_grad(z.x), v[i + 1] * gelu_grad(z.y));
+                    for (int i = 0; i < 8; ++i) *reinterpret_cast<float4*>(sf + (fr + 4 * i) * kLdF + fc) = zr[i];
+                    if (c0 + 32 < kCols) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            zr[i] = *reinterpret_cast<const float4*>(zp + (size_t)(4 * i) * ep.ldz + c0 + 32);
+                    }
+                    __syncwarp();
+#pragma unroll
+                    for (int i = 0; i < 32; i += 8) {
+                        uint32_t o[4];
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) {
+                            const float4 zz = *reinterpret_cast<const float4*>(sf + lane * kLdF + i + 4 * u);
+                            const float* w = v + i + 4 * u;
+                            o[2 * u] = pack_bf16(w[0] * gelu_grad(zz.x), w[1] * gelu_grad(zz.y));
+                            o[2 * u + 1] = pack_bf16(w[2] * gelu_grad(zz.z), w[3] * gelu_grad(zz.w));
+                        }
+                        *reinterpret_cast<uint4*>(sh + lane * kLdH + i) = make_uint4(o[0], o[1], o[2], o[3]);
                     }
                 }
-            }
-            // the accumulator is in registers and staging: hand it back to the MMA issuer
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tempty[b])) : "memory");
-            if (ep.mode != kEpiGeluGrad && ep.c_f32)
-                for (int rr = 0; rr < 32; ++rr)
-                    if (m0 + rr < ep.M)
-                        *reinterpret_cast<float4*>(ep.c_f32 + (size_t)(m0 + rr) * ep.ldc + n0 + 4 * lane) =
-                            *reinterpret_cast<const float4*>(sf + rr * C::kLdF + 4 * lane);
-            if (ep.mode != kEpiF32)
-                for (int rr = 0; rr < 32; rr += 2) {
-                    const int row = rr + (lane >> 4), col = 8 * (lane & 15);
-                    if (m0 + row < ep.M)
-                        *reinterpret_cast<uint4*>(ep.out_bf16 + (size_t)(m0 + row) * ep.ldo + n0 + col) =
-                            *reinterpret_cast<const uint4*>(sh + row * C::kLdH + col);
+                __syncwarp();
+                if (kMode == kEpiF32 || kMode == kEpiBiasGelu) {
+                    float* o = ep.c_f32 + gc + (size_t)(m0 + fr) * ep.ldc + n0 + c0 + fc;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        *reinterpret_cast<float4*>(o + (size_t)(4 * i) * ep.ldc) =
+                            *reinterpret_cast<const float4*>(sf + (fr + 4 * i) * kLdF + fc);
                 }
-            __syncwarp();  // the staging rows are rewritten by the next tile
+                if (kMode != kEpiF32) {
+                    __nv_bfloat16* o = ep.out_bf16 + member * ep.sg_o + (size_t)(m0 + hr) * ep.ldo + n0 + c0 + hc;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        *reinterpret_cast<uint4*>(o + (size_t)(8 * i) * ep.ldo) =
+                            *reinterpret_cast<const uint4*>(sh + (hr + 8 * i) * kLdH + hc);
+                }
+                __syncwarp();  // the staging rows are rewritten by the next chunk
+            }
         }
     }
     tc_fence_before();
@@ -480,10 +417,11 @@ __global__ void __launch_bounds__(kPpThreads, 1) k_gemm_pp(const __grid_constant
     if (*fail && tid == 0) {
         atomicExch(err, 1);
         // let the loads still in flight land before the CTA's shared memory goes away
-        for (int g = s_consumed; g < s_issued; ++g) mbar_wait(&full[g % kPpStages], (unsigned)(g / kPpStages) & 1u);
+        for (int g = s_consumed; g < s_issued; ++g) mbar_wait(&full[g % kStages], (unsigned)(g / kStages) & 1u);
     }
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem) : "memory");
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * BN) : "memory");
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
@@ -499,20 +437,83 @@ cudaError_t get_encode()
     return cudaSuccess;
 }
 
-// 2-D BF16 tensor map over a row-major [rows x cols] matrix (row stride ld
-// elements), box of 64 columns x box_rows rows, 128-byte swizzle
-cudaError_t make_map(CUtensorMap* m, const void* base, int rows, int cols, int ld, int box_rows)
+// BF16 tensor map (inner, rows, groups) over a matrix with contiguous rows of
+// `inner` elements (row stride ld, group stride sg elements), box of 64 inner
+// elements x box_rows rows, 128-byte swizzle
+cudaError_t make_map(CUtensorMap* m, const GemmOperand& p, int inner, int rows, int box_rows)
 {
     cudaError_t e = get_encode();
     if (e != cudaSuccess) return e;
-    cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-    cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)box_rows};
-    cuuint32_t estr[2] = {1, 1};
-    CUresult r = g_encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
+    const long long sg = p.groups > 1 ? p.sg : (long long)p.ld * rows;
+    cuuint64_t dims[3] = {(cuuint64_t)inner, (cuuint64_t)rows, (cuuint64_t)p.groups};
+    cuuint64_t strides[2] = {(cuuint64_t)p.ld * 2, (cuuint64_t)sg * 2};
+    cuuint32_t box[3] = {(cuuint32_t)kBK, (cuuint32_t)box_rows, 1};
+    cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = g_encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(p.p), dims, strides, box, estr,
                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+bool operand_ok(const GemmOperand& p)
+{
+    return p.p && p.groups > 0 && p.ld % 8 == 0 && ((uintptr_t)p.p & 15) == 0 && (p.groups == 1 || p.sg % 8 == 0);
+}
+
+template <int BN, bool kMnA, bool kMnB, int kMode>
+cudaError_t launch_gemm(const GemmProblem& P, int sms, int dev, int* err, cudaStream_t st)
+{
+    static bool attr[64] = {false};  // per device
+    if (!attr[dev]) {
+        cudaError_t e = cudaFuncSetAttribute(k_gemm<BN, kMnA, kMnB, kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (Cfg<BN, kMode>::kSmem));
+        if (e != cudaSuccess) return e;
+        attr[dev] = true;
+    }
+    CUtensorMap ta, tb[2];
+    cudaError_t e = kMnA ? make_map(&ta, P.A, P.M, P.K, kBK) : make_map(&ta, P.A, P.K, P.M, kBM);
+    for (int s = 0; s < 2 && e == cudaSuccess; ++s) {
+        if (s == 1 && !P.n2) {
+            tb[1] = tb[0];
+            break;
+        }
+        const GemmOperand& B = s ? P.B2 : P.B;
+        const int N = s ? P.n2 : P.N;
+        e = kMnB ? make_map(&tb[s], B, N, P.K, kBK) : make_map(&tb[s], B, P.K, N, BN);
+    }
+    if (e != cudaSuccess) return e;
+    GemmGrid g;
+    g.KT = P.K / kBK;
+    g.n_inner = P.n_inner;
+    for (int s = 0; s < 2; ++s) {
+        const int N = s && P.n2 ? P.n2 : P.N;
+        g.tn[s] = N / BN;
+        g.per[s] = (P.M / kBM) * (N / BN);
+        g.za[s] = s ? P.za2 : P.za;
+        g.ep[s] = s ? P.ep2 : P.ep;
+    }
+    g.tiles0 = P.groups * g.per[0];
+    g.n_tiles = g.tiles0 + (P.n2 ? P.groups2 * g.per[1] : 0);
+    k_gemm<BN, kMnA, kMnB, kMode><<<g.n_tiles < sms ? g.n_tiles : sms, Cfg<BN, kMode>::kThreads, (Cfg<BN, kMode>::kSmem), st>>>(ta, tb[0], tb[1],
+                                                                                                      g, err);
+    return cudaGetLastError();
+}
+
+template <bool kMnA, bool kMnB, int kMode>
+cudaError_t launch_gemm_bn(const GemmProblem& P, int sms, int dev, int* err, cudaStream_t st)
+{
+    // 128 x 128 tiles of the whole launch
+    const long long tiles = (long long)(P.M / kBM) * ((long long)P.groups * (P.N / 128) + (long long)P.groups2 * (P.n2 / 128));
+    if (tiles >= (1ll << 30)) return cudaErrorInvalidValue;
+    // 256 columns (three quarters of the operand reads per output) where half the tiles still make an even last
+    // wave and the epilogue stores BF16 only: 300k x 4 members' prediction 6.85 against 8.3 ms with 128 columns. With
+    // FP32 pre-activations stored or read the epilogue's memory traffic sets the time and smaller tiles balance
+    // better: 43 against 48 us per forward layer of 4 x 8192 rows. 64 columns where 128 would leave SMs idle.
+    if constexpr (kMode == kEpiGelu)
+        if (P.N % 256 == 0 && P.n2 % 256 == 0 && tiles >= 4ll * sms)
+            return launch_gemm<256, kMnA, kMnB, kMode>(P, sms, dev, err, st);
+    if (tiles >= sms) return launch_gemm<128, kMnA, kMnB, kMode>(P, sms, dev, err, st);
+    return launch_gemm<64, kMnA, kMnB, kMode>(P, sms, dev, err, st);
 }
 
 }  // namespace
@@ -522,66 +523,37 @@ bool gemm_shape_ok(int M, int N, int K)
     return M > 0 && N > 0 && K > 0 && M % kBM == 0 && N % 128 == 0 && K % kBK == 0;
 }
 
-namespace {
-
-template <int BN>
-cudaError_t launch_gemm(const void* A, int lda, const void* B, int ldb, int M, int N, int K, const GemmEpi& ep,
-                        int* err, cudaStream_t st)
+cudaError_t gemm_bf16(const GemmProblem& P, int* err, cudaStream_t st)
 {
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_gemm_tn<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN>::kSmem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
-    CUtensorMap ta, tb;
-    cudaError_t e = make_map(&ta, A, M, K, lda, kBM);
-    if (e == cudaSuccess) e = make_map(&tb, B, N, K, ldb, BN);
-    if (e != cudaSuccess) return e;
-    dim3 grid(N / BN, M / kBM);
-    k_gemm_tn<BN><<<grid, 128, Cfg<BN>::kSmem, st>>>(ta, tb, ep, K, err);
-    return cudaGetLastError();
-}
-
-int g_sms = 0;
-
-}  // namespace
-
-// C = A B^T; A [M x K] (row stride lda), B [N x K] (row stride ldb), BF16, K-contiguous.
-// 128 x 64 tiles when 128 x 128 tiles would cover fewer CTAs than SMs.
-cudaError_t gemm_bf16_tn(const void* A, int lda, const void* B, int ldb, int M, int N, int K, const GemmEpi& ep,
-                         int* err, cudaStream_t st)
-{
-    if (!gemm_shape_ok(M, N, K) || lda % 8 || ldb % 8 || ((uintptr_t)A & 15) || ((uintptr_t)B & 15))
+    if (!gemm_shape_ok(P.M, P.N, P.K) || !operand_ok(P.A) || !operand_ok(P.B) || P.groups < 1 || P.n_inner < 1)
         return cudaErrorInvalidValue;
-    if (ep.mode != kEpiGeluGrad && (ep.ldc % 4 || ((uintptr_t)ep.c_f32 & 15))) return cudaErrorInvalidValue;
-    if (ep.mode == kEpiF32 && !ep.c_f32) return cudaErrorInvalidValue;
-    if (ep.mode != kEpiF32 && (ep.ldo % 8 || ((uintptr_t)ep.out_bf16 & 15))) return cudaErrorInvalidValue;
-    if (ep.mode == kEpiGeluGrad && (ep.ldz % 4 || ((uintptr_t)ep.z & 15))) return cudaErrorInvalidValue;
-    if (!g_sms) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev);
-        if (g_sms <= 0) g_sms = 1;
+    if (P.n2 && (!gemm_shape_ok(P.M, P.n2, P.K) || !operand_ok(P.B2) || P.groups2 < 1 || P.ep2.mode != P.ep.mode))
+        return cudaErrorInvalidValue;
+    for (int s = 0; s < (P.n2 ? 2 : 1); ++s) {
+        const GemmEpi& ep = s ? P.ep2 : P.ep;
+        if ((ep.mode == kEpiF32 || ep.mode == kEpiBiasGelu) && (!ep.c_f32 || ep.ldc % 4 || ((uintptr_t)ep.c_f32 & 15) || ep.sg_c % 4 || ep.sl_c % 4))
+            return cudaErrorInvalidValue;
+        if (ep.mode != kEpiF32 && (!ep.out_bf16 || ep.ldo % 8 || ((uintptr_t)ep.out_bf16 & 15) || ep.sg_o % 8))
+            return cudaErrorInvalidValue;
+        if ((ep.mode == kEpiBiasGelu || ep.mode == kEpiGelu) && (!ep.bias || ((uintptr_t)ep.bias & 15) || ep.sg_bias % 4))
+            return cudaErrorInvalidValue;
+        if (ep.mode == kEpiGeluGrad && (!ep.z || ep.ldz % 4 || ((uintptr_t)ep.z & 15) || ep.sg_z % 4))
+            return cudaErrorInvalidValue;
     }
-    const long long tiles = (long long)(M / kBM) * (N / 128);
-    if (tiles < g_sms) return launch_gemm<64>(A, lda, B, ldb, M, N, K, ep, err, st);
-    if (tiles >= 2ll * g_sms && tiles < (1ll << 31)) {
-        // persistent: one CTA per SM, accumulators double-buffered in TMEM
-        static bool attr = false;
-        if (!attr) {
-            cudaError_t e = cudaFuncSetAttribute(k_gemm_pp, cudaFuncAttributeMaxDynamicSharedMemorySize, PpCfg::kSmem);
-            if (e != cudaSuccess) return e;
-            attr = true;
-        }
-        CUtensorMap ta, tb;
-        cudaError_t e = make_map(&ta, A, M, K, lda, kBM);
-        if (e == cudaSuccess) e = make_map(&tb, B, N, K, ldb, 128);
-        if (e != cudaSuccess) return e;
-        k_gemm_pp<<<g_sms, kPpThreads, PpCfg::kSmem, st>>>(ta, tb, ep, K, N / 128, (int)tiles, err);
-        return cudaGetLastError();
-    }
-    return launch_gemm<128>(A, lda, B, ldb, M, N, K, ep, err, st);
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64 || sms < 1) return cudaErrorInvalidDevice;
+    if (P.ep.mode == kEpiBiasGelu && !P.A.mn && !P.B.mn)
+        return launch_gemm_bn<false, false, kEpiBiasGelu>(P, sms, dev, err, st);
+    if (P.ep.mode == kEpiGelu && !P.A.mn && !P.B.mn)
+        return launch_gemm_bn<false, false, kEpiGelu>(P, sms, dev, err, st);
+    if (P.ep.mode == kEpiGeluGrad && !P.A.mn && P.B.mn)
+        return launch_gemm_bn<false, true, kEpiGeluGrad>(P, sms, dev, err, st);
+    if (P.ep.mode == kEpiF32 && P.A.mn && P.B.mn) return launch_gemm_bn<true, true, kEpiF32>(P, sms, dev, err, st);
+    if (P.ep.mode == kEpiF32 && !P.A.mn && !P.B.mn) return launch_gemm_bn<false, false, kEpiF32>(P, sms, dev, err, st);
+    return cudaErrorInvalidValue;  // no other combination is used
 }
 
 }  // namespace sbr

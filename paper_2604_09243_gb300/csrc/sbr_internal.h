@@ -286,23 +286,41 @@ cudaError_t launch_po_final(const double* partial, const PoItem* items, const Po
                             const double* kfreq, int n_pol, double* E, double* rcs, cudaStream_t st);
 
 // ---------------------------------------------------------------- tensor-core GEMM (surrogate)
-// C = A B^T, A [M x K] and B [N x K] BF16 with K contiguous; M, N multiples of
-// 128 and K a multiple of 64. The epilogue is fused:
-enum { kEpiF32 = 0, kEpiBiasGelu = 1, kEpiGeluGrad = 2 };
+// C = A B^T, A [M x K] and B [N x K] BF16, for `groups` equal problems; M, N
+// multiples of 128 and K a multiple of 64. The epilogue is fused. Group g =
+// layer * n_inner + member: its member offsets (sg_*, elements) and, for c_f32,
+// its layer offset (sl_c) are added to the pointers.
+enum { kEpiF32 = 0, kEpiBiasGelu = 1, kEpiGeluGrad = 2, kEpiGelu = 3 };
 struct GemmEpi {
     int mode;                 // kEpi*
-    int M;                    // rows of C
-    float* c_f32;             // kEpiF32: C; kEpiBiasGelu: z = acc + bias, or null where no backward pass reads it
-                              // (row stride ldc)
+    float* c_f32;             // kEpiF32: C; kEpiBiasGelu: z = acc + bias (row stride ldc)
     int ldc;
-    __nv_bfloat16* out_bf16;  // kEpiBiasGelu: gelu(z); kEpiGeluGrad: acc * gelu'(z)  (row stride ldo)
+    __nv_bfloat16* out_bf16;  // kEpiBiasGelu, kEpiGelu: gelu(acc + bias); kEpiGeluGrad: acc * gelu'(z)  (row stride ldo)
     int ldo;
-    const float* bias;        // kEpiBiasGelu: [N]
+    const float* bias;        // kEpiBiasGelu, kEpiGelu: [N], 16-byte aligned
     const float* z;           // kEpiGeluGrad: pre-activation [M x N] (row stride ldz)
     int ldz;
+    long long sg_c, sl_c, sg_o, sg_bias, sg_z;
+};
+struct GemmOperand {
+    const void* p;
+    int ld;        // row stride of the stored matrix (elements, a multiple of 8)
+    bool mn;       // stored [K x M] or [K x N] (M or N contiguous) instead of [M x K], [N x K]
+    int groups;    // matrices at p, sg elements apart
+    long long sg;
+};
+struct GemmProblem {
+    GemmOperand A, B;
+    int M, N, K;
+    int groups, n_inner;  // group g: A matrix za + g, B matrix g
+    int za;
+    GemmEpi ep;
+    // optional second set of groups in the same launch (n2 = 0: none): B matrices B2 [n2 x K], A matrices from za2 on
+    GemmOperand B2;
+    int n2, groups2, za2;
+    GemmEpi ep2;
 };
 bool gemm_shape_ok(int M, int N, int K);
-cudaError_t gemm_bf16_tn(const void* A, int lda, const void* B, int ldb, int M, int N, int K, const GemmEpi& ep,
-                         int* err, cudaStream_t st);
+cudaError_t gemm_bf16(const GemmProblem& P, int* err, cudaStream_t st);
 
 }  // namespace sbr

@@ -14,9 +14,10 @@
 //            y = h_D W_h^T + b_h                                        (head kernel)
 //   loss     mean squared error over the 4 outputs
 //   backward dz_{D-1} = (dy W_h) * GELU'(z_{D-1});
-//            dW_l = dz_l^T h_l (GEMM on transposed operands), db_l = sum_m dz_l
-//            dz_{l-1} = (dz_l W_l) * GELU'(z_{l-1})                     (GEMM with W_l^T, fused epilogue)
-//   Adam on all FP32 parameters, then BF16 copies of W_l and W_l^T refreshed.
+//            dz_{l-1} = (dz_l W_l) * GELU'(z_{l-1})                     (GEMM, fused epilogue)
+//            dW_l = dz_l^T h_l (one GEMM launch for all layers), db_l = sum_m dz_l
+//   Adam on all FP32 parameters, the BF16 copies of W_l written with them.
+// The members of the ensemble take each step together (grouped launches).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -26,6 +27,7 @@
 #include <mutex>
 #include <random>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "sbr.h"
@@ -37,6 +39,7 @@ namespace {
 
 constexpr double kPi = 3.14159265358979323846;
 constexpr int kMaxDepth = 16;
+constexpr int kMaxMembers = 16;
 constexpr int kOut = 4;
 constexpr int kIn = 4;
 
@@ -44,6 +47,11 @@ std::mutex g_gemm_mu;
 int* g_gemm_err[64] = {nullptr};
 
 // ---------------------------------------------------------------- small kernels
+// Every kernel below works on a group of members at once (a grid dimension is
+// the member, its arrays a fixed stride apart): one member's arrays are too
+// small to fill the GPU, and a launch costs as much as its work. Each sum keeps
+// its order whatever the group, so the members' results do not depend on it.
+
 // raw (az deg, el deg, f Hz) -> the 4 network inputs
 __global__ void k_encode(const double* raw, int n, float* x4)
 {
@@ -56,31 +64,40 @@ __global__ void k_encode(const double* raw, int n, float* x4)
     x4[4 * i + 3] = (float)(2.0 * (log(f / 1e9) / log(12.0)) - 1.0);
 }
 
-__global__ void k_gather(const float* x4, const float* y4, const int* idx, int n, float* xb, float* yb)
+// member blockIdx.y's batch: rows idx[member * n_idx + i], i < n
+__global__ void k_gather(const float4* x4, const float4* y4, const int* idx, long long n_idx, int n, float4* xb,
+                         float4* yb)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const int j = idx[i];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        xb[4 * i + c] = x4[4 * (size_t)j + c];
-        if (yb) yb[4 * i + c] = y4[4 * (size_t)j + c];
-    }
+    const int j = idx[blockIdx.y * n_idx + i];
+    const size_t o = (size_t)blockIdx.y * n + i;
+    xb[o] = x4[j];
+    yb[o] = y4[j];
 }
 
-// Fourier features: h0[m][j] = sin(2 pi B_j . x_m) (j < nf/2), cos(...) (j >= nf/2)
-__global__ void k_fourier(const float* x4, const float* B, int M, int nh, __nv_bfloat16* h0)
+// Fourier features: h0[m][j] = sin(2 pi B_j . x_m) (j < nf/2), cos(...) (j >= nf/2); two frequencies per thread.
+// sx: rows between the members' inputs (0: all members read the same)
+__global__ void k_fourier(const float4* x4, long long sx, const float4* B, int M, int nh, __nv_bfloat16* h0)
 {
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= (long long)M * nh) return;
-    const int m = (int)(i / nh), j = (int)(i % nh);
-    const float* b = B + 4 * j;
-    const float* x = x4 + 4 * m;
-    const float arg = b[0] * x[0] + b[1] * x[1] + b[2] * x[2] + b[3] * x[3];
-    float s, c;
-    sincospif(2.f * arg, &s, &c);
-    h0[(size_t)m * (2 * nh) + j] = __float2bfloat16_rn(s);
-    h0[(size_t)m * (2 * nh) + nh + j] = __float2bfloat16_rn(c);
+    const int half = nh / 2;
+    if (i >= (long long)M * half) return;
+    const int m = (int)(i / half), j = 2 * (int)(i % half);
+    const float4 x = x4[blockIdx.y * sx + m];
+    __nv_bfloat162 sv, cv;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const float4 b = B[(size_t)blockIdx.y * nh + j + u];
+        const float arg = b.x * x.x + b.y * x.y + b.z * x.z + b.w * x.w;
+        float s, c;
+        sincospif(2.f * arg, &s, &c);
+        (u ? sv.y : sv.x) = __float2bfloat16_rn(s);
+        (u ? cv.y : cv.x) = __float2bfloat16_rn(c);
+    }
+    __nv_bfloat16* o = h0 + ((size_t)blockIdx.y * M + m) * (2 * nh) + j;
+    *reinterpret_cast<__nv_bfloat162*>(o) = sv;
+    *reinterpret_cast<__nv_bfloat162*>(o + nh) = cv;
 }
 
 __device__ __forceinline__ float gelu_grad_f(float z)
@@ -88,14 +105,18 @@ __device__ __forceinline__ float gelu_grad_f(float z)
     return 0.5f * (1.f + erff(z * 0.70710678118654752f)) + z * 0.3989422804014327f * expf(-0.5f * z * z);
 }
 
-// head: y[m][o] = sum_k h[m][k] W[o][k] + b[o]; one warp per row
-__global__ void k_head_fwd(const __nv_bfloat16* h, int M, int K, const float* W, const float* b, float* y)
+// head: y[m][o] = sum_k h[m][k] W[o][k] + b[o]; one warp per row, lane l the terms k = l, l + 32, ...
+__global__ void k_head_fwd(const __nv_bfloat16* h, int M, int K, const float* P, long long sp, long long ow,
+                           long long ob, float* y)
 {
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (warp >= M) return;
+    const float* W = P + blockIdx.y * sp + ow;
+    const float* b = P + blockIdx.y * sp + ob;
+    const __nv_bfloat16* row = h + ((size_t)blockIdx.y * M + warp) * K;
     float acc[kOut] = {0.f, 0.f, 0.f, 0.f};
     for (int k = lane; k < K; k += 32) {
-        const float v = __bfloat162float(h[(size_t)warp * K + k]);
+        const float v = __bfloat162float(row[k]);
 #pragma unroll
         for (int o = 0; o < kOut; ++o) acc[o] = fmaf(v, W[o * K + k], acc[o]);
     }
@@ -104,18 +125,59 @@ __global__ void k_head_fwd(const __nv_bfloat16* h, int M, int K, const float* W,
         for (int s = 16; s > 0; s >>= 1) acc[o] += __shfl_xor_sync(0xffffffffu, acc[o], s);
     if (lane == 0)
 #pragma unroll
-        for (int o = 0; o < kOut; ++o) y[(size_t)warp * kOut + o] = acc[o] + b[o];
+        for (int o = 0; o < kOut; ++o) y[((size_t)blockIdx.y * M + warp) * kOut + o] = acc[o] + b[o];
 }
 
-// dy = 2 (y - t) / (M * 4); loss sum in FP64
-__global__ void k_loss(const float* y, const float* t, int n, float* dy, double* loss)
+// The same for widths up to 512 (kT terms per lane): the weights stay in registers while a warp walks its rows
+// (reading them again for every row was four loads per activation), and the four sums are reduced together, each
+// lane keeping the half it will finish (6 exchanges instead of 20, every sum in the order of the plain butterfly).
+// Bound by loads in flight: 17 us for 4 x 8192 rows, 25 us before.
+template <int kT>
+__global__ void __launch_bounds__(256) k_head_fwd_reg(const __nv_bfloat16* __restrict__ h, int M,
+                                                      const float* __restrict__ P, long long sp, long long ow,
+                                                      long long ob, float* __restrict__ y)
+{
+    constexpr int K = 32 * kT;
+    const int lane = threadIdx.x & 31, nw = (gridDim.x * blockDim.x) >> 5;
+    const float* W = P + blockIdx.y * sp + ow;
+    float w[kOut][kT];
+#pragma unroll
+    for (int o = 0; o < kOut; ++o)
+#pragma unroll
+        for (int i = 0; i < kT; ++i) w[o][i] = W[o * K + 32 * i + lane];
+    const bool b16 = lane & 16, b8 = lane & 8;
+    const int out = (b16 ? 2 : 0) + (b8 ? 1 : 0);
+    const float bias = P[blockIdx.y * sp + ob + out];
+    for (int m = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; m < M; m += nw) {
+        const __nv_bfloat16* row = h + ((size_t)blockIdx.y * M + m) * K + lane;
+        float v[kT];
+#pragma unroll
+        for (int i = 0; i < kT; ++i) v[i] = __bfloat162float(row[32 * i]);
+        float acc[kOut] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int i = 0; i < kT; ++i)
+#pragma unroll
+            for (int o = 0; o < kOut; ++o) acc[o] = fmaf(v[i], w[o][i], acc[o]);
+        const float r0 = __shfl_xor_sync(0xffffffffu, b16 ? acc[0] : acc[2], 16);
+        const float r1 = __shfl_xor_sync(0xffffffffu, b16 ? acc[1] : acc[3], 16);
+        const float a0 = (b16 ? acc[2] : acc[0]) + r0, a1 = (b16 ? acc[3] : acc[1]) + r1;
+        float a = (b8 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, b8 ? a0 : a1, 8);
+#pragma unroll
+        for (int s = 4; s > 0; s >>= 1) a += __shfl_xor_sync(0xffffffffu, a, s);
+        if ((lane & 7) == 0) y[((size_t)blockIdx.y * M + m) * kOut + out] = a + bias;
+    }
+}
+
+// dy = 2 (y - t) / (M * 4); loss sum in FP64 (loss[member * sl])
+__global__ void k_loss(const float* y, const float* t, int n, float* dy, double* loss, int sl)
 {
     __shared__ double s_red[8];
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const size_t g = (size_t)blockIdx.y * n;
     double l = 0.0;
     if (i < n) {
-        const float d = y[i] - t[i];
-        dy[i] = 2.f * d / (float)n;
+        const float d = y[g + i] - t[g + i];
+        dy[g + i] = 2.f * d / (float)n;
         l = (double)d * d;
     }
     for (int s = 16; s > 0; s >>= 1) l += __shfl_xor_sync(0xffffffffu, l, s);
@@ -124,20 +186,35 @@ __global__ void k_loss(const float* y, const float* t, int n, float* dy, double*
     if (threadIdx.x == 0) {
         double t2 = 0.0;
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t2 += s_red[w];
-        atomicAdd(loss, t2);
+        atomicAdd(loss + (size_t)blockIdx.y * sl, t2);
     }
 }
 
-// dz[m][k] = (sum_o dy[m][o] W[o][k]) * gelu'(z[m][k])
-__global__ void k_head_bwd_dz(const float* dy, const float* W, const float* z, int M, int K, __nv_bfloat16* dz)
+// dz[m][k] = (sum_o dy[m][o] W[o][k]) * gelu'(z[m][k]), four k per thread
+__global__ void k_head_bwd_dz(const float4* dy, const float* P, long long sp, long long ow, const float4* z, int M,
+                              int K, uint2* dz)
 {
+    const int k4 = K / 4;
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= (long long)M * K) return;
-    const int m = (int)(i / K), k = (int)(i % K);
-    float s = 0.f;
+    if (i >= (long long)M * k4) return;
+    const int m = (int)(i / k4), k = 4 * (int)(i % k4);
+    const float* W = P + blockIdx.y * sp + ow;
+    const float4 d4 = dy[(size_t)blockIdx.y * M + m];
+    const float d[kOut] = {d4.x, d4.y, d4.z, d4.w};
+    const size_t at = (size_t)blockIdx.y * M * k4 + i;
+    const float4 zz = z[at];
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int o = 0; o < kOut; ++o) s = fmaf(dy[m * kOut + o], W[o * K + k], s);
-    dz[i] = __float2bfloat16_rn(s * gelu_grad_f(z[i]));
+    for (int o = 0; o < kOut; ++o) {
+        const float4 w = *reinterpret_cast<const float4*>(W + (size_t)o * K + k);
+        s[0] = fmaf(d[o], w.x, s[0]);
+        s[1] = fmaf(d[o], w.y, s[1]);
+        s[2] = fmaf(d[o], w.z, s[2]);
+        s[3] = fmaf(d[o], w.w, s[3]);
+    }
+    __nv_bfloat162 a = __floats2bfloat162_rn(s[0] * gelu_grad_f(zz.x), s[1] * gelu_grad_f(zz.y));
+    __nv_bfloat162 b = __floats2bfloat162_rn(s[2] * gelu_grad_f(zz.z), s[3] * gelu_grad_f(zz.w));
+    dz[at] = make_uint2(*reinterpret_cast<unsigned*>(&a), *reinterpret_cast<unsigned*>(&b));
 }
 
 // Column sums over the batch in two fixed-order stages (deterministic): stage 1
@@ -146,11 +223,14 @@ __global__ void k_head_bwd_dz(const float* dy, const float* W, const float* z, i
 constexpr int kRedRows = 256;
 
 // head gradient, stage 1: part[p][o][k] = sum over rows m of chunk p of dy[m][o] h[m][k]
-// (k < K) and of dy[m][o] (k = K, the bias)
+// (k < K) and of dy[m][o] (k = K, the bias); member blockIdx.z
 __global__ void k_head_dw_part(const float* dy, const __nv_bfloat16* h, int M, int K, float* part)
 {
     __shared__ float sh[8][kOut][33];
     const int k = blockIdx.x * 32 + threadIdx.x, p = blockIdx.y;
+    dy += (size_t)blockIdx.z * M * kOut;
+    h += (size_t)blockIdx.z * M * K;
+    part += (size_t)blockIdx.z * gridDim.y * kOut * (K + 1);
     float acc[kOut] = {0.f, 0.f, 0.f, 0.f};
     if (k <= K) {
         const int r1 = min(M, (p + 1) * kRedRows);
@@ -172,75 +252,112 @@ __global__ void k_head_dw_part(const float* dy, const __nv_bfloat16* h, int M, i
     }
 }
 
-// head gradient, stage 2: dW[o][k], db[o] = sum over the P partials
-__global__ void k_head_dw_fin(const float* part, int P, int K, float* dW, float* db)
+// head gradient, stage 2: dW[o][k], db[o] = sum over the n_part partials; member blockIdx.y
+__global__ void k_head_dw_fin(const float* part, int n_part, int K, float* G, long long sp, long long ow, long long ob)
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= kOut * (K + 1)) return;
+    part += (size_t)blockIdx.y * n_part * kOut * (K + 1);
     const int o = j / (K + 1), k = j % (K + 1);
     float t = 0.f;
-    for (int q = 0; q < P; ++q) t += part[((size_t)q * kOut + o) * (K + 1) + k];
-    if (k < K) dW[o * K + k] = t;
-    else db[o] = t;
+    for (int q = 0; q < n_part; ++q) t += part[((size_t)q * kOut + o) * (K + 1) + k];
+    if (k < K) G[blockIdx.y * sp + ow + o * K + k] = t;
+    else G[blockIdx.y * sp + ob + o] = t;
 }
 
-// bias gradient, stage 1: part[p][n] = sum over rows m of chunk p of dz[m][n]
-__global__ void k_colsum_part(const __nv_bfloat16* dz, int M, int N, float* part)
+// bias gradient, stage 1: part[p][n] = sum over rows m of chunk p of dz[m][n]; (layer, member) blockIdx.z; four
+// columns per thread (8-byte loads; N is a multiple of 128)
+__global__ void __launch_bounds__(256) k_colsum_part(const __nv_bfloat16* dz, int M, int N, float* part)
 {
-    __shared__ float sh[8][33];
-    const int n = blockIdx.x * 32 + threadIdx.x, p = blockIdx.y;
-    float acc = 0.f;
-    if (n < N) {
-        const int r1 = min(M, (p + 1) * kRedRows);
-#pragma unroll 4
-        for (int m = p * kRedRows + threadIdx.y; m < r1; m += 8) acc += __bfloat162float(dz[(size_t)m * N + n]);
+    __shared__ float4 sh[8][32];
+    const int n = blockIdx.x * 128 + 4 * threadIdx.x, p = blockIdx.y;
+    dz += (size_t)blockIdx.z * M * N + n;
+    part += (size_t)blockIdx.z * gridDim.y * N;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int r1 = min(M, (p + 1) * kRedRows);
+#pragma unroll 8
+    for (int m = p * kRedRows + threadIdx.y; m < r1; m += 8) {
+        const uint2 u = *reinterpret_cast<const uint2*>(dz + (size_t)m * N);
+        const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x)),
+                     b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
+        acc.x += a.x;
+        acc.y += a.y;
+        acc.z += b.x;
+        acc.w += b.y;
     }
     sh[threadIdx.y][threadIdx.x] = acc;
     __syncthreads();
-    if (threadIdx.y == 0 && n < N) {
-        float t = 0.f;
-        for (int y = 0; y < 8; ++y) t += sh[y][threadIdx.x];
-        part[(size_t)p * N + n] = t;
+    if (threadIdx.y == 0) {
+        float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int y = 0; y < 8; ++y) {
+            const float4 v = sh[y][threadIdx.x];
+            t.x += v.x;
+            t.y += v.y;
+            t.z += v.z;
+            t.w += v.w;
+        }
+        *reinterpret_cast<float4*>(part + (size_t)p * N + n) = t;
     }
 }
 
-// bias gradient, stage 2
-__global__ void k_colsum_fin(const float* part, int P, int N, float* db)
+// offsets of the layers' weights and biases in a member's parameters, and of the BF16 weights (layer depth = head)
+struct Layout {
+    int depth;
+    long long offW[kMaxDepth + 1], offb[kMaxDepth + 1], offWbf[kMaxDepth + 1];
+};
+
+// bias gradient, stage 2; blockIdx.y = layer * members + member
+__global__ void k_colsum_fin(const float* part, int n_part, int N, int members, float* G, long long sp, const Layout L)
 {
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= N) return;
+    const int layer = blockIdx.y / members, e = blockIdx.y - layer * members;
+    part += (size_t)blockIdx.y * n_part * N;
     float t = 0.f;
-    for (int q = 0; q < P; ++q) t += part[(size_t)q * N + n];
-    db[n] = t;
+    for (int q = 0; q < n_part; ++q) t += part[(size_t)q * N + n];
+    G[e * sp + L.offb[layer] + n] = t;
 }
 
-// out[c][r] = in[r][c] for a [R x Cc] BF16 matrix, 32 x 32 tiles through shared memory
-__global__ void k_transpose(const __nv_bfloat16* in, int R, int Cc, __nv_bfloat16* out)
+struct AdamBias {
+    float c1[kMaxMembers], c2[kMaxMembers];  // bias corrections of each member of the group
+};
+
+__device__ __forceinline__ void adam1(float& p, float& m, float& v, float gi, float lr, float b1, float b2, float c1,
+                                      float c2, float eps)
 {
-    __shared__ __nv_bfloat16 t[32][33];
-    const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-    for (int y = threadIdx.y; y < 32; y += blockDim.y) {
-        const int r = r0 + y, c = c0 + threadIdx.x;
-        if (r < R && c < Cc) t[y][threadIdx.x] = in[(size_t)r * Cc + c];
-    }
-    __syncthreads();
-    for (int y = threadIdx.y; y < 32; y += blockDim.y) {
-        const int c = c0 + y, r = r0 + threadIdx.x;
-        if (r < R && c < Cc) out[(size_t)c * R + r] = t[threadIdx.x][y];
-    }
+    // one rounding per product and sum as written, so that training gives the same bits however it is compiled
+    const float mi = __fmaf_rn(1.f - b1, gi, __fmul_rn(b1, m));
+    const float vi = __fmaf_rn(__fmul_rn(1.f - b2, gi), gi, __fmul_rn(b2, v));
+    m = mi;
+    v = vi;
+    p -= lr * (mi * c1) / (sqrtf(vi * c2) + eps);
 }
 
-__global__ void k_adam(float* p, float* m, float* v, const float* g, long long n, float lr, float b1, float b2,
-                       float c1, float c2, float eps)
+// Adam on four parameters per thread, the BF16 copies of the hidden weights written with them
+__global__ void k_adam(float* p, float* m, float* v, const float* g, long long n, __nv_bfloat16* wbf, long long n_bf,
+                       const Layout L, float lr, float b1, float b2, const AdamBias A, float eps)
 {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const long long i = 4 * (blockIdx.x * (long long)blockDim.x + threadIdx.x);
     if (i >= n) return;
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    p[i] -= lr * (mi * c1) / (sqrtf(vi * c2) + eps);
+    const int e = blockIdx.y;
+    const size_t at = (size_t)e * n + i;
+    float4 pp = *reinterpret_cast<float4*>(p + at), mm = *reinterpret_cast<float4*>(m + at),
+           vv = *reinterpret_cast<float4*>(v + at);
+    const float4 gg = *reinterpret_cast<const float4*>(g + at);
+    const float c1 = A.c1[e], c2 = A.c2[e];
+    adam1(pp.x, mm.x, vv.x, gg.x, lr, b1, b2, c1, c2, eps);
+    adam1(pp.y, mm.y, vv.y, gg.y, lr, b1, b2, c1, c2, eps);
+    adam1(pp.z, mm.z, vv.z, gg.z, lr, b1, b2, c1, c2, eps);
+    adam1(pp.w, mm.w, vv.w, gg.w, lr, b1, b2, c1, c2, eps);
+    *reinterpret_cast<float4*>(p + at) = pp;
+    *reinterpret_cast<float4*>(m + at) = mm;
+    *reinterpret_cast<float4*>(v + at) = vv;
+    for (int l = 0; l < L.depth; ++l)
+        if (i >= L.offW[l] && i < L.offb[l]) {
+            __nv_bfloat162 a = __floats2bfloat162_rn(pp.x, pp.y), b = __floats2bfloat162_rn(pp.z, pp.w);
+            *reinterpret_cast<uint2*>(wbf + (size_t)e * n_bf + L.offWbf[l] + (i - L.offW[l])) =
+                make_uint2(*reinterpret_cast<unsigned*>(&a), *reinterpret_cast<unsigned*>(&b));
+        }
 }
 
 __global__ void k_to_bf16(const float* in, long long n, __nv_bfloat16* out)
@@ -277,6 +394,28 @@ __global__ void k_ens_stats(const float* y, int n_members, long long stride, int
 
 inline unsigned blocks(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 
+struct Buf {
+    void* p = nullptr;
+    size_t cap = 0;
+    cudaError_t ensure(size_t bytes)
+    {
+        if (bytes <= cap) return cudaSuccess;
+        release();
+        const cudaError_t e = cudaMalloc(&p, bytes);
+        if (e == cudaSuccess) cap = bytes;
+        else p = nullptr;
+        return e;
+    }
+    void release()
+    {
+        if (p) cudaFree(p);
+        p = nullptr;
+        cap = 0;
+    }
+    template <class T>
+    T* as() const { return (T*)p; }
+};
+
 }  // namespace
 
 // ------------------------------------------------------------------ surrogate state
@@ -287,27 +426,17 @@ struct sbr_surrogate {
     sbr_surrogate_opts opt;
     std::string err;
     int nh = 0;  // Fourier frequencies (features = 2 nh)
-    std::vector<int> K, N;  // hidden layer l: N[l] x K[l]
-    std::vector<long long> offW, offb;  // offsets in the flat parameter vector (layer depth = head)
-    long long n_params = 0;
-    long long offWbf_total = 0;
-    std::vector<long long> offWbf;  // offsets of the BF16 copies
-    // per member, device
-    std::vector<float*> P, Pm, Pv, Bf;  // parameters, Adam moments, Fourier matrices
-    std::vector<__nv_bfloat16*> Wbf, WTbf;
+    std::vector<int> K;  // inputs of hidden layer l (each has width outputs)
+    Layout L;
+    long long n_params = 0;  // per member (a multiple of 4)
+    long long n_bf = 0;      // BF16 hidden weights per member
+    // all members, n_params / n_bf / 4 nh apart: parameters, Adam moments, gradients, Fourier matrices, BF16 weights
+    Buf P, Pm, Pv, G, Bf, Wbf;
     std::vector<long long> steps;
-    float* G = nullptr;  // gradient (shared by members)
-    // activations for batches of up to cap rows
-    int cap = 0;
-    std::vector<__nv_bfloat16*> h;   // h[0..depth] BF16 [cap x width_l]
-    std::vector<float*> z;           // z[0..depth-1] FP32 [cap x N_l]
-    std::vector<__nv_bfloat16*> dz;  // dz[l] BF16 [cap x N_l]
-    __nv_bfloat16 *dzT = nullptr, *hT = nullptr;
-    float *y = nullptr, *dy = nullptr, *xb = nullptr, *yb = nullptr;
-    float* red = nullptr;  // partial column sums [cap / 256 x 4 (width + 1)]
-    double* loss = nullptr;
-    int* gerr = nullptr;
-    int* idx = nullptr;
+    // Workspace of a group of g members on a batch of M rows, member-major: h0 [g][M][nf], h [layer][g][M][width]
+    // (h_{l+1} at l), z and dz [layer][g][M][width], outputs and targets [g][M][4]. Kept and grown as needed.
+    Buf h0, h, z, dz, y, dy, xb, yb, red;
+    Buf loss, gerr;
     float target_scale = 1.f;
     bool trained = false;
 };
@@ -330,131 +459,184 @@ int sfail(sbr_surrogate* s, int code, const char* msg)
         }                                                                                 \
     } while (0)
 
-int ensure_cap(sbr_surrogate* s, int M)
+// the workspace of g members on M rows: `layers` activations kept (all of them for a backward pass, two to
+// alternate between for prediction), pre-activations and deltas with `train`
+cudaError_t ensure_ws(sbr_surrogate* s, int M, int g, bool train)
 {
-    if (M <= s->cap) return SBR_OK;
-    const int D = s->opt.depth;
-    auto fr = [](void* p) {
-        if (p) cudaFree(p);
-    };
-    for (auto p : s->h) fr(p);
-    for (auto p : s->z) fr(p);
-    for (auto p : s->dz) fr(p);
-    fr(s->dzT);
-    fr(s->hT);
-    fr(s->y);
-    fr(s->dy);
-    fr(s->xb);
-    fr(s->yb);
-    fr(s->idx);
-    fr(s->red);
-    s->h.assign(D + 1, nullptr);
-    s->z.assign(D, nullptr);
-    s->dz.assign(D, nullptr);
-    const int wmax = std::max(s->opt.width, s->opt.n_fourier);
-    for (int l = 0; l <= D; ++l) SCK(cudaMalloc(&s->h[l], sizeof(__nv_bfloat16) * (size_t)M * (l == 0 ? s->opt.n_fourier : s->opt.width)), "alloc h");
-    for (int l = 0; l < D; ++l) {
-        SCK(cudaMalloc(&s->z[l], sizeof(float) * (size_t)M * s->opt.width), "alloc z");
-        SCK(cudaMalloc(&s->dz[l], sizeof(__nv_bfloat16) * (size_t)M * s->opt.width), "alloc dz");
+    const size_t D = (size_t)s->opt.depth, W = (size_t)s->opt.width, R = (size_t)M * g;
+    const size_t layers = train ? D : std::min<size_t>(D, 2);
+    cudaError_t e = s->h0.ensure(sizeof(__nv_bfloat16) * R * s->opt.n_fourier);
+    if (e == cudaSuccess) e = s->h.ensure(sizeof(__nv_bfloat16) * R * W * layers);
+    if (e == cudaSuccess) e = s->y.ensure(sizeof(float) * R * kOut);
+    if (e == cudaSuccess) e = s->xb.ensure(sizeof(float) * R * kIn);
+    if (!train || e != cudaSuccess) return e;
+    e = s->z.ensure(sizeof(float) * R * W * D);
+    if (e == cudaSuccess) e = s->dz.ensure(sizeof(__nv_bfloat16) * R * W * D);
+    if (e == cudaSuccess) e = s->dy.ensure(sizeof(float) * R * kOut);
+    if (e == cudaSuccess) e = s->yb.ensure(sizeof(float) * R * kOut);
+    const size_t parts = (size_t)((M + kRedRows - 1) / kRedRows) * g;
+    if (e == cudaSuccess) e = s->red.ensure(sizeof(float) * parts * std::max<size_t>(kOut * (W + 1), D * W));
+    return e;
+}
+
+// Members worked on at once: all of them while their workspace (200 MB per
+// member at 8192 rows of the default network) stays within kGroupBytes and can
+// be had, else fewer, down to one. A step of four members of 8192 rows takes
+// 0.75 ms of device time together, 3.1 ms one member at a time.
+constexpr size_t kGroupBytes = (size_t)8 << 30;
+int choose_group(sbr_surrogate* s, int M, int* g_out)
+{
+    const size_t row = (size_t)s->opt.depth * s->opt.width * 8 + (size_t)s->opt.n_fourier * 2 + 128;
+    int g = (int)std::min<size_t>((size_t)s->opt.n_members, std::max<size_t>(1, kGroupBytes / (row * (size_t)M)));
+    cudaError_t e = ensure_ws(s, M, g, true);
+    while (e == cudaErrorMemoryAllocation && g > 1) {
+        cudaGetLastError();
+        g = (g + 1) / 2;
+        for (Buf* b : {&s->h0, &s->h, &s->z, &s->dz, &s->y, &s->dy, &s->xb, &s->yb, &s->red}) b->release();
+        e = ensure_ws(s, M, g, true);
     }
-    SCK(cudaMalloc(&s->dzT, sizeof(__nv_bfloat16) * (size_t)M * s->opt.width), "alloc dzT");
-    SCK(cudaMalloc(&s->hT, sizeof(__nv_bfloat16) * (size_t)M * wmax), "alloc hT");
-    SCK(cudaMalloc(&s->y, sizeof(float) * (size_t)M * kOut * std::max(1, s->opt.n_members)), "alloc y");
-    SCK(cudaMalloc(&s->dy, sizeof(float) * (size_t)M * kOut), "alloc dy");
-    SCK(cudaMalloc(&s->xb, sizeof(float) * (size_t)M * kIn), "alloc xb");
-    SCK(cudaMalloc(&s->yb, sizeof(float) * (size_t)M * kOut), "alloc yb");
-    SCK(cudaMalloc(&s->idx, sizeof(int) * (size_t)M), "alloc idx");
-    SCK(cudaMalloc(&s->red, sizeof(float) * (size_t)((M + kRedRows - 1) / kRedRows) * kOut * (wmax + 1)),
-        "alloc partial sums");
-    s->cap = M;
+    SCK(e, "alloc training workspace");
+    *g_out = g;
     return SBR_OK;
 }
 
-// refresh the BF16 copies of W_l and W_l^T of member e
+// refresh the BF16 copies of the hidden weights of member e
 int refresh_bf16(sbr_surrogate* s, int e)
 {
     for (int l = 0; l < s->opt.depth; ++l) {
-        const long long n = (long long)s->N[l] * s->K[l];
-        __nv_bfloat16* w = s->Wbf[e] + s->offWbf[l];
-        k_to_bf16<<<blocks(n, 256), 256, 0, s->stream>>>(s->P[e] + s->offW[l], n, w);
-        dim3 g((s->K[l] + 31) / 32, (s->N[l] + 31) / 32);
-        k_transpose<<<g, dim3(32, 8), 0, s->stream>>>(w, s->N[l], s->K[l], s->WTbf[e] + s->offWbf[l]);
+        const long long n = (long long)s->opt.width * s->K[l];
+        k_to_bf16<<<blocks(n, 256), 256, 0, s->stream>>>(s->P.as<float>() + e * s->n_params + s->L.offW[l], n,
+                                                         s->Wbf.as<__nv_bfloat16>() + e * s->n_bf + s->L.offWbf[l]);
     }
     SCK(cudaGetLastError(), "refresh weights");
     return SBR_OK;
 }
 
-// forward pass of member e on xb[0..M): fills h, z and y (at y + yoff)
-// keep_z: store the FP32 pre-activations for a backward pass (prediction writes only the BF16 activations)
-int forward(sbr_surrogate* s, int e, int M, float* yout, bool keep_z = true)
+// forward pass of members e0 .. e0 + g - 1 on M rows each: fills h0, h and y. sx: rows between the members' inputs
+// at xb (0: shared). keep_z: store the FP32 pre-activations and every layer's activations for a backward pass
+// (prediction writes only BF16 activations, into two buffers in turn).
+int forward(sbr_surrogate* s, int e0, int g, int M, const float* xb, long long sx, float* yout, bool keep_z)
 {
-    const int D = s->opt.depth;
-    k_fourier<<<blocks((long long)M * s->nh, 256), 256, 0, s->stream>>>(s->xb, s->Bf[e], M, s->nh, s->h[0]);
+    const int D = s->opt.depth, W = s->opt.width, nf = s->opt.n_fourier;
+    const long long S = (long long)M * W;
+    const float* P = s->P.as<float>() + e0 * s->n_params;
+    __nv_bfloat16* h = s->h.as<__nv_bfloat16>();
+    auto hl = [&](int l) { return h + (size_t)(keep_z ? l : l & 1) * g * S; };  // h_{l+1}
+    k_fourier<<<dim3(blocks((long long)M * (s->nh / 2), 256), g), 256, 0, s->stream>>>(
+        (const float4*)xb, sx, s->Bf.as<float4>() + (size_t)e0 * s->nh, M, s->nh, s->h0.as<__nv_bfloat16>());
     for (int l = 0; l < D; ++l) {
-        GemmEpi ep;
-        memset(&ep, 0, sizeof(ep));
-        ep.mode = kEpiBiasGelu;
-        ep.M = M;
-        ep.c_f32 = keep_z ? s->z[l] : nullptr;
-        ep.ldc = s->N[l];
-        ep.out_bf16 = s->h[l + 1];
-        ep.ldo = s->N[l];
-        ep.bias = s->P[e] + s->offb[l];
-        SCK(gemm_bf16_tn(s->h[l], s->K[l], s->Wbf[e] + s->offWbf[l], s->K[l], M, s->N[l], s->K[l], ep, s->gerr,
-                         s->stream),
-            "forward gemm");
+        GemmProblem p;
+        memset(&p, 0, sizeof(p));
+        if (l == 0) p.A = GemmOperand{s->h0.p, nf, false, g, (long long)M * nf};
+        else p.A = GemmOperand{hl(l - 1), W, false, g, S};
+        p.B = GemmOperand{s->Wbf.as<__nv_bfloat16>() + e0 * s->n_bf + s->L.offWbf[l], s->K[l], false, g, s->n_bf};
+        p.M = M;
+        p.N = W;
+        p.K = s->K[l];
+        p.groups = p.n_inner = g;
+        p.ep.mode = keep_z ? kEpiBiasGelu : kEpiGelu;
+        p.ep.c_f32 = keep_z ? s->z.as<float>() + (size_t)l * g * S : nullptr;
+        p.ep.ldc = W;
+        p.ep.sg_c = S;
+        p.ep.out_bf16 = hl(l);
+        p.ep.ldo = W;
+        p.ep.sg_o = S;
+        p.ep.bias = P + s->L.offb[l];
+        p.ep.sg_bias = s->n_params;
+        SCK(gemm_bf16(p, s->gerr.as<int>(), s->stream), "forward gemm");
     }
-    k_head_fwd<<<blocks((long long)M * 32, 256), 256, 0, s->stream>>>(s->h[D], M, s->opt.width, s->P[e] + s->offW[D],
-                                                                       s->P[e] + s->offb[D], yout);
+    {
+        const __nv_bfloat16* hD = hl(D - 1);
+        const long long np = s->n_params, ow = s->L.offW[D], ob = s->L.offb[D];
+        // about eight rows per warp pay for the weight loads; no more blocks than stay resident
+        const dim3 grid(std::min<unsigned>(blocks(M, 64), 1216u / (unsigned)g + 1u), g);
+        if (W == 512) k_head_fwd_reg<16><<<grid, 256, 0, s->stream>>>(hD, M, P, np, ow, ob, yout);
+        else if (W == 384) k_head_fwd_reg<12><<<grid, 256, 0, s->stream>>>(hD, M, P, np, ow, ob, yout);
+        else if (W == 256) k_head_fwd_reg<8><<<grid, 256, 0, s->stream>>>(hD, M, P, np, ow, ob, yout);
+        else if (W == 128) k_head_fwd_reg<4><<<grid, 256, 0, s->stream>>>(hD, M, P, np, ow, ob, yout);
+        else
+            k_head_fwd<<<dim3(blocks((long long)M * 32, 256), g), 256, 0, s->stream>>>(hD, M, W, P, np, ow, ob, yout);
+    }
     SCK(cudaGetLastError(), "head");
     return SBR_OK;
 }
 
-// backward pass of member e (after forward on the same batch; targets in yb): gradient in G
-// The sum of squared errors is added to *lacc (zeroed first when lacc is null: s->loss).
-int backward(sbr_surrogate* s, int e, int M, double* lacc = nullptr)
+// backward pass of the group after forward with keep_z on the same batch (targets in yb): gradients in G (the
+// group's first member at G). The sums of squared errors are added to lacc[member * sl].
+int backward(sbr_surrogate* s, int e0, int g, int M, double* lacc, int sl)
 {
-    const int D = s->opt.depth, W = s->opt.width;
-    if (!lacc) {
-        lacc = s->loss;
-        cudaMemsetAsync(lacc, 0, sizeof(double), s->stream);
+    const int D = s->opt.depth, W = s->opt.width, nf = s->opt.n_fourier;
+    const long long S = (long long)M * W, np = s->n_params;
+    const float* P = s->P.as<float>() + e0 * np;
+    float* G = s->G.as<float>();
+    __nv_bfloat16 *h = s->h.as<__nv_bfloat16>(), *dz = s->dz.as<__nv_bfloat16>();
+    float* z = s->z.as<float>();
+    k_loss<<<dim3(blocks((long long)M * kOut, 256), g), 256, 0, s->stream>>>(s->y.as<float>(), s->yb.as<float>(),
+                                                                             M * kOut, s->dy.as<float>(), lacc, sl);
+    const int parts = (M + kRedRows - 1) / kRedRows;
+    k_head_dw_part<<<dim3((W + 1 + 31) / 32, parts, g), dim3(32, 8), 0, s->stream>>>(
+        s->dy.as<float>(), h + (size_t)(D - 1) * g * S, M, W, s->red.as<float>());
+    k_head_dw_fin<<<dim3(blocks(kOut * (W + 1), 256), g), 256, 0, s->stream>>>(s->red.as<float>(), parts, W, G, np,
+                                                                               s->L.offW[D], s->L.offb[D]);
+    k_head_bwd_dz<<<dim3(blocks((long long)M * (W / 4), 256), g), 256, 0, s->stream>>>(
+        s->dy.as<float4>(), P, np, s->L.offW[D], (const float4*)(z + (size_t)(D - 1) * g * S), M, W,
+        (uint2*)(dz + (size_t)(D - 1) * g * S));
+    for (int l = D - 1; l > 0; --l) {
+        // dz_{l-1} = (dz_l W_l) * gelu'(z_{l-1}): W_l as stored, its inputs contiguous
+        GemmProblem p;
+        memset(&p, 0, sizeof(p));
+        p.A = GemmOperand{dz + (size_t)l * g * S, W, false, g, S};
+        p.B = GemmOperand{s->Wbf.as<__nv_bfloat16>() + e0 * s->n_bf + s->L.offWbf[l], W, true, g, s->n_bf};
+        p.M = M;
+        p.N = W;
+        p.K = W;
+        p.groups = p.n_inner = g;
+        p.ep.mode = kEpiGeluGrad;
+        p.ep.out_bf16 = dz + (size_t)(l - 1) * g * S;
+        p.ep.ldo = W;
+        p.ep.sg_o = S;
+        p.ep.z = z + (size_t)(l - 1) * g * S;
+        p.ep.ldz = W;
+        p.ep.sg_z = S;
+        SCK(gemm_bf16(p, s->gerr.as<int>(), s->stream), "input-gradient gemm");
     }
-    k_loss<<<blocks((long long)M * kOut, 256), 256, 0, s->stream>>>(s->y, s->yb, M * kOut, s->dy, lacc);
-    const int P = (M + kRedRows - 1) / kRedRows;
-    k_head_dw_part<<<dim3((W + 1 + 31) / 32, P), dim3(32, 8), 0, s->stream>>>(s->dy, s->h[D], M, W, s->red);
-    k_head_dw_fin<<<blocks(kOut * (W + 1), 256), 256, 0, s->stream>>>(s->red, P, W, s->G + s->offW[D],
-                                                                        s->G + s->offb[D]);
-    k_head_bwd_dz<<<blocks((long long)M * W, 256), 256, 0, s->stream>>>(s->dy, s->P[e] + s->offW[D], s->z[D - 1], M, W,
-                                                                         s->dz[D - 1]);
-    for (int l = D - 1; l >= 0; --l) {
-        // dW_l = dz_l^T h_l : A = dz_l^T [N x M], B = h_l^T [K x M]
-        dim3 g1((s->N[l] + 31) / 32, (M + 31) / 32), g2((s->K[l] + 31) / 32, (M + 31) / 32);
-        k_transpose<<<g1, dim3(32, 8), 0, s->stream>>>(s->dz[l], M, s->N[l], s->dzT);
-        k_transpose<<<g2, dim3(32, 8), 0, s->stream>>>(s->h[l], M, s->K[l], s->hT);
-        GemmEpi ep;
-        memset(&ep, 0, sizeof(ep));
-        ep.mode = kEpiF32;
-        ep.M = s->N[l];
-        ep.c_f32 = s->G + s->offW[l];
-        ep.ldc = s->K[l];
-        SCK(gemm_bf16_tn(s->dzT, M, s->hT, M, s->N[l], s->K[l], M, ep, s->gerr, s->stream), "weight-gradient gemm");
-        k_colsum_part<<<dim3((s->N[l] + 31) / 32, P), dim3(32, 8), 0, s->stream>>>(s->dz[l], M, s->N[l], s->red);
-        k_colsum_fin<<<blocks(s->N[l], 256), 256, 0, s->stream>>>(s->red, P, s->N[l], s->G + s->offb[l]);
-        if (l > 0) {
-            // dz_{l-1} = (dz_l W_l) * gelu'(z_{l-1}) : A = dz_l [M x N], B = W_l^T [K x N]
-            GemmEpi eg;
-            memset(&eg, 0, sizeof(eg));
-            eg.mode = kEpiGeluGrad;
-            eg.M = M;
-            eg.out_bf16 = s->dz[l - 1];
-            eg.ldo = s->K[l];
-            eg.z = s->z[l - 1];
-            eg.ldz = s->K[l];
-            SCK(gemm_bf16_tn(s->dz[l], s->N[l], s->WTbf[e] + s->offWbf[l], s->N[l], M, s->K[l], s->N[l], eg, s->gerr,
-                             s->stream),
-                "input-gradient gemm");
+    // dW_l = dz_l^T h_l, every layer of every member in one launch: the batch is the contraction, both operands
+    // as stored; the hidden-to-hidden layers first, then layer 0 on the Fourier features
+    {
+        GemmProblem p;
+        memset(&p, 0, sizeof(p));
+        p.A = GemmOperand{dz, W, true, D * g, S};
+        p.M = W;
+        p.K = M;
+        p.n_inner = g;
+        p.ep.mode = kEpiF32;
+        p.ep.sg_c = np;
+        GemmEpi e0p = p.ep;  // layer 0
+        e0p.c_f32 = G + s->L.offW[0];
+        e0p.ldc = nf;
+        const GemmOperand b0{s->h0.p, nf, true, g, (long long)M * nf};
+        if (D > 1) {
+            p.B = GemmOperand{h, W, true, (D - 1) * g, S};
+            p.N = W;
+            p.groups = (D - 1) * g;
+            p.za = g;
+            p.ep.c_f32 = G + s->L.offW[1];
+            p.ep.ldc = W;
+            p.ep.sl_c = (long long)W * W + W;
+            p.B2 = b0;
+            p.n2 = nf;
+            p.groups2 = g;
+            p.ep2 = e0p;
+        } else {
+            p.B = b0;
+            p.N = nf;
+            p.groups = g;
+            p.ep = e0p;
         }
+        SCK(gemm_bf16(p, s->gerr.as<int>(), s->stream), "weight-gradient gemm");
     }
+    k_colsum_part<<<dim3(W / 128, parts, D * g), dim3(32, 8), 0, s->stream>>>(dz, M, W, s->red.as<float>());
+    k_colsum_fin<<<dim3(blocks(W, 256), D * g), 256, 0, s->stream>>>(s->red.as<float>(), parts, W, g, G, np, s->L);
     SCK(cudaGetLastError(), "backward");
     return SBR_OK;
 }
@@ -462,7 +644,7 @@ int backward(sbr_surrogate* s, int e, int M, double* lacc = nullptr)
 int check_gemm_err(sbr_surrogate* s)
 {
     int herr = 0;
-    SCK(cudaMemcpyAsync(&herr, s->gerr, sizeof(int), cudaMemcpyDeviceToHost, s->stream), "copy error flag");
+    SCK(cudaMemcpyAsync(&herr, s->gerr.p, sizeof(int), cudaMemcpyDeviceToHost, s->stream), "copy error flag");
     SCK(cudaStreamSynchronize(s->stream), "sync");
     if (herr) return sfail(s, SBR_ERR_TIMEOUT, "tensor-core GEMM: a bounded wait gave up");
     return SBR_OK;
@@ -486,6 +668,24 @@ int upload_inputs(sbr_surrogate* s, const double* x, int64_t n, float** x4)
 }  // namespace
 
 // ------------------------------------------------------------------ C ABI
+namespace {
+GemmProblem plain_gemm(const void* A, int lda, const void* B, int ldb, int M, int N, int K, float* C, int ldc)
+{
+    GemmProblem p;
+    memset(&p, 0, sizeof(p));
+    p.A = GemmOperand{A, lda, false, 1, 0};
+    p.B = GemmOperand{B, ldb, false, 1, 0};
+    p.M = M;
+    p.N = N;
+    p.K = K;
+    p.groups = p.n_inner = 1;
+    p.ep.mode = kEpiF32;
+    p.ep.c_f32 = C;
+    p.ep.ldc = ldc;
+    return p;
+}
+}  // namespace
+
 extern "C" {
 
 int sbr_gemm_bf16_tn(const void* A, int lda, const void* B, int ldb, int M, int N, int K, float* C, int ldc,
@@ -502,13 +702,7 @@ int sbr_gemm_bf16_tn(const void* A, int lda, const void* B, int ldb, int M, int 
     }
     cudaStream_t st = (cudaStream_t)cuda_stream;
     if (cudaMemsetAsync(g_gemm_err[dev], 0, sizeof(int), st) != cudaSuccess) return SBR_ERR_CUDA;
-    GemmEpi ep;
-    memset(&ep, 0, sizeof(ep));
-    ep.mode = kEpiF32;
-    ep.M = M;
-    ep.c_f32 = C;
-    ep.ldc = ldc;
-    if (gemm_bf16_tn(A, lda, B, ldb, M, N, K, ep, g_gemm_err[dev], st) != cudaSuccess) return SBR_ERR_CUDA;
+    if (gemm_bf16(plain_gemm(A, lda, B, ldb, M, N, K, C, ldc), g_gemm_err[dev], st) != cudaSuccess) return SBR_ERR_CUDA;
     int herr = 0;
     if (cudaMemcpyAsync(&herr, g_gemm_err[dev], sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
@@ -522,14 +716,9 @@ int sbr_gemm_bf16_tn_async(const void* A, int lda, const void* B, int ldb, int M
     if (!A || !B || !C || !err_dev) return SBR_ERR_ARG;
     if (!gemm_shape_ok(M, N, K) || lda < K || ldb < K || ldc < N || lda % 8 || ldb % 8 || ldc % 4)
         return SBR_ERR_ARG;
-    GemmEpi ep;
-    memset(&ep, 0, sizeof(ep));
-    ep.mode = kEpiF32;
-    ep.M = M;
-    ep.c_f32 = C;
-    ep.ldc = ldc;
-    return gemm_bf16_tn(A, lda, B, ldb, M, N, K, ep, err_dev, (cudaStream_t)cuda_stream) == cudaSuccess ? SBR_OK
-                                                                                                      : SBR_ERR_CUDA;
+    return gemm_bf16(plain_gemm(A, lda, B, ldb, M, N, K, C, ldc), err_dev, (cudaStream_t)cuda_stream) == cudaSuccess
+               ? SBR_OK
+               : SBR_ERR_CUDA;
 }
 
 const char* sbr_surrogate_last_error(const sbr_surrogate* s) { return s ? s->err.c_str() : ""; }
@@ -546,7 +735,7 @@ int sbr_surrogate_create(sbr_surrogate** out, int device, void* cuda_stream, con
     o.fourier_sigma = 4.f;
     o.seed = 1;
     if (opt) o = *opt;
-    if (o.n_members < 1 || o.n_members > 16 || o.width < 128 || o.width % 128 || o.depth < 1 || o.depth > kMaxDepth ||
+    if (o.n_members < 1 || o.n_members > kMaxMembers || o.width < 128 || o.width % 128 || o.depth < 1 || o.depth > kMaxDepth ||
         o.n_fourier < 128 || o.n_fourier % 128 || !(o.fourier_sigma > 0.f))
         return SBR_ERR_ARG;
     int nd = 0;
@@ -570,67 +759,52 @@ int sbr_surrogate_create(sbr_surrogate** out, int device, void* cuda_stream, con
     }
     const int D = o.depth;
     s->K.resize(D);
-    s->N.resize(D);
-    for (int l = 0; l < D; ++l) {
-        s->K[l] = l == 0 ? o.n_fourier : o.width;
-        s->N[l] = o.width;
-    }
+    memset(&s->L, 0, sizeof(s->L));
+    s->L.depth = D;
     long long off = 0, offbf = 0;
     for (int l = 0; l <= D; ++l) {
-        const int Kl = l < D ? s->K[l] : o.width, Nl = l < D ? s->N[l] : kOut;
-        s->offW.push_back(off);
+        if (l < D) s->K[l] = l == 0 ? o.n_fourier : o.width;
+        const int Kl = l < D ? s->K[l] : o.width, Nl = l < D ? o.width : kOut;
+        s->L.offW[l] = off;
         off += (long long)Nl * Kl;
-        s->offb.push_back(off);
+        s->L.offb[l] = off;
         off += Nl;
         if (l < D) {
-            s->offWbf.push_back(offbf);
+            s->L.offWbf[l] = offbf;
             offbf += (long long)Nl * Kl;
         }
     }
     s->n_params = off;
-    s->offWbf_total = offbf;
+    s->n_bf = offbf;
+    const size_t ne = (size_t)o.n_members;
+    int rc = SBR_OK;
+    if (s->P.ensure(sizeof(float) * off * ne) != cudaSuccess || s->Pm.ensure(sizeof(float) * off * ne) != cudaSuccess ||
+        s->Pv.ensure(sizeof(float) * off * ne) != cudaSuccess || s->G.ensure(sizeof(float) * off * ne) != cudaSuccess ||
+        s->Bf.ensure(sizeof(float) * 4 * s->nh * ne) != cudaSuccess ||
+        s->Wbf.ensure(sizeof(__nv_bfloat16) * offbf * ne) != cudaSuccess ||
+        s->loss.ensure(sizeof(double)) != cudaSuccess || s->gerr.ensure(sizeof(int)) != cudaSuccess)
+        rc = SBR_ERR_OOM;
     // parameters: He-normal hidden layers, small head, zero biases; Fourier matrix N(0, sigma^2)
     std::mt19937_64 rng(o.seed);
     std::normal_distribution<float> nd01(0.f, 1.f);
     std::vector<float> hp((size_t)off), hb((size_t)4 * s->nh);
-    int rc = SBR_OK;
     for (int e = 0; e < o.n_members && rc == SBR_OK; ++e) {
         std::fill(hp.begin(), hp.end(), 0.f);
         for (int l = 0; l <= D; ++l) {
-            const int Kl = l < D ? s->K[l] : o.width, Nl = l < D ? s->N[l] : kOut;
+            const int Kl = l < D ? s->K[l] : o.width, Nl = l < D ? o.width : kOut;
             const float sd = l < D ? sqrtf(2.f / (float)Kl) : sqrtf(1.f / (float)Kl);
-            for (long long i = 0; i < (long long)Nl * Kl; ++i) hp[(size_t)(s->offW[l] + i)] = sd * nd01(rng);
+            for (long long i = 0; i < (long long)Nl * Kl; ++i) hp[(size_t)(s->L.offW[l] + i)] = sd * nd01(rng);
         }
         for (auto& v : hb) v = o.fourier_sigma * nd01(rng);
-        float *P, *Pm, *Pv, *Bf;
-        __nv_bfloat16 *Wb, *WTb;
-        if (cudaMalloc(&P, sizeof(float) * off) != cudaSuccess || cudaMalloc(&Pm, sizeof(float) * off) != cudaSuccess ||
-            cudaMalloc(&Pv, sizeof(float) * off) != cudaSuccess ||
-            cudaMalloc(&Bf, sizeof(float) * hb.size()) != cudaSuccess ||
-            cudaMalloc(&Wb, sizeof(__nv_bfloat16) * offbf) != cudaSuccess ||
-            cudaMalloc(&WTb, sizeof(__nv_bfloat16) * offbf) != cudaSuccess) {
-            rc = SBR_ERR_OOM;
-            break;
-        }
-        s->P.push_back(P);
-        s->Pm.push_back(Pm);
-        s->Pv.push_back(Pv);
-        s->Bf.push_back(Bf);
-        s->Wbf.push_back(Wb);
-        s->WTbf.push_back(WTb);
         s->steps.push_back(0);
-        cudaMemcpy(P, hp.data(), sizeof(float) * off, cudaMemcpyHostToDevice);
-        cudaMemcpy(Bf, hb.data(), sizeof(float) * hb.size(), cudaMemcpyHostToDevice);
-        cudaMemset(Pm, 0, sizeof(float) * off);
-        cudaMemset(Pv, 0, sizeof(float) * off);
+        cudaMemcpy(s->P.as<float>() + e * off, hp.data(), sizeof(float) * off, cudaMemcpyHostToDevice);
+        cudaMemcpy(s->Bf.as<float>() + (size_t)e * 4 * s->nh, hb.data(), sizeof(float) * hb.size(), cudaMemcpyHostToDevice);
         rc = refresh_bf16(s, e);
     }
-    if (rc == SBR_OK && (cudaMalloc(&s->G, sizeof(float) * off) != cudaSuccess ||
-                         cudaMalloc(&s->loss, sizeof(double)) != cudaSuccess ||
-                         cudaMalloc(&s->gerr, sizeof(int)) != cudaSuccess))
-        rc = SBR_ERR_OOM;
-    if (rc == SBR_OK && cudaMemsetAsync(s->gerr, 0, sizeof(int), s->stream) != cudaSuccess) rc = SBR_ERR_CUDA;
-    if (rc == SBR_OK && cudaStreamSynchronize(s->stream) != cudaSuccess) rc = SBR_ERR_CUDA;
+    if (rc == SBR_OK && (cudaMemset(s->Pm.p, 0, s->Pm.cap) != cudaSuccess || cudaMemset(s->Pv.p, 0, s->Pv.cap) != cudaSuccess ||
+                         cudaMemsetAsync(s->gerr.p, 0, sizeof(int), s->stream) != cudaSuccess ||
+                         cudaStreamSynchronize(s->stream) != cudaSuccess))
+        rc = SBR_ERR_CUDA;
     if (rc != SBR_OK) {
         sbr_surrogate_destroy(s);
         return rc;
@@ -644,29 +818,9 @@ void sbr_surrogate_destroy(sbr_surrogate* s)
     if (!s) return;
     cudaSetDevice(s->device);
     cudaStreamSynchronize(s->stream);
-    auto fr = [](void* p) {
-        if (p) cudaFree(p);
-    };
-    for (auto p : s->P) fr(p);
-    for (auto p : s->Pm) fr(p);
-    for (auto p : s->Pv) fr(p);
-    for (auto p : s->Bf) fr(p);
-    for (auto p : s->Wbf) fr(p);
-    for (auto p : s->WTbf) fr(p);
-    for (auto p : s->h) fr(p);
-    for (auto p : s->z) fr(p);
-    for (auto p : s->dz) fr(p);
-    fr(s->G);
-    fr(s->dzT);
-    fr(s->hT);
-    fr(s->y);
-    fr(s->dy);
-    fr(s->xb);
-    fr(s->yb);
-    fr(s->loss);
-    fr(s->gerr);
-    fr(s->idx);
-    fr(s->red);
+    for (Buf* b : {&s->P, &s->Pm, &s->Pv, &s->G, &s->Bf, &s->Wbf, &s->h0, &s->h, &s->z, &s->dz, &s->y, &s->dy, &s->xb,
+                   &s->yb, &s->red, &s->loss, &s->gerr})
+        b->release();
     if (s->own_stream) cudaStreamDestroy(s->stream);
     delete s;
 }
@@ -678,12 +832,13 @@ int sbr_surrogate_params(sbr_surrogate* s, int member, float* get, const float* 
     if (!s || member < 0 || member >= s->opt.n_members) return SBR_ERR_ARG;
     SCK(cudaSetDevice(s->device), "cudaSetDevice");
     const size_t b = sizeof(float) * (size_t)s->n_params;
+    float* p = s->P.as<float>() + member * s->n_params;
     if (set) {
-        SCK(cudaMemcpyAsync(s->P[member], set, b, cudaMemcpyHostToDevice, s->stream), "set params");
+        SCK(cudaMemcpyAsync(p, set, b, cudaMemcpyHostToDevice, s->stream), "set params");
         int rc = refresh_bf16(s, member);
         if (rc != SBR_OK) return rc;
     }
-    if (get) SCK(cudaMemcpyAsync(get, s->P[member], b, cudaMemcpyDeviceToHost, s->stream), "get params");
+    if (get) SCK(cudaMemcpyAsync(get, p, b, cudaMemcpyDeviceToHost, s->stream), "get params");
     SCK(cudaStreamSynchronize(s->stream), "sync");
     return SBR_OK;
 }
@@ -692,7 +847,7 @@ int sbr_surrogate_fourier(sbr_surrogate* s, int member, float* B)
 {
     if (!s || !B || member < 0 || member >= s->opt.n_members) return SBR_ERR_ARG;
     SCK(cudaSetDevice(s->device), "cudaSetDevice");
-    SCK(cudaMemcpy(B, s->Bf[member], sizeof(float) * 4 * s->nh, cudaMemcpyDeviceToHost), "get Fourier matrix");
+    SCK(cudaMemcpy(B, s->Bf.as<float>() + (size_t)member * 4 * s->nh, sizeof(float) * 4 * s->nh, cudaMemcpyDeviceToHost), "get Fourier matrix");
     return SBR_OK;
 }
 
@@ -701,25 +856,24 @@ int sbr_surrogate_grads(sbr_surrogate* s, int member, const double* x, const dou
 {
     if (!s || !x || !y || n < 128 || n % 128 || member < 0 || member >= s->opt.n_members) return SBR_ERR_ARG;
     SCK(cudaSetDevice(s->device), "cudaSetDevice");
-    int rc = ensure_cap(s, (int)n);
-    if (rc != SBR_OK) return rc;
+    SCK(ensure_ws(s, (int)n, 1, true), "alloc training workspace");
     float* x4 = nullptr;
-    rc = upload_inputs(s, x, n, &x4);
+    int rc = upload_inputs(s, x, n, &x4);
     if (rc != SBR_OK) return rc;
     std::vector<float> yt((size_t)n * kOut);
     for (size_t i = 0; i < yt.size(); ++i) yt[i] = (float)(y[i] / s->target_scale);
-    cudaMemcpyAsync(s->xb, x4, sizeof(float) * kIn * (size_t)n, cudaMemcpyDeviceToDevice, s->stream);
-    cudaMemcpyAsync(s->yb, yt.data(), sizeof(float) * yt.size(), cudaMemcpyHostToDevice, s->stream);
-    cudaMemsetAsync(s->gerr, 0, sizeof(int), s->stream);
-    rc = forward(s, member, (int)n, s->y);
-    if (rc == SBR_OK) rc = backward(s, member, (int)n);
+    cudaMemcpyAsync(s->yb.p, yt.data(), sizeof(float) * yt.size(), cudaMemcpyHostToDevice, s->stream);
+    cudaMemsetAsync(s->gerr.p, 0, sizeof(int), s->stream);
+    cudaMemsetAsync(s->loss.p, 0, sizeof(double), s->stream);
+    rc = forward(s, member, 1, (int)n, x4, 0, s->y.as<float>(), true);
+    if (rc == SBR_OK) rc = backward(s, member, 1, (int)n, s->loss.as<double>(), 0);
     if (rc == SBR_OK) rc = check_gemm_err(s);
     cudaFree(x4);
     if (rc != SBR_OK) return rc;
     double hl = 0.0;
-    SCK(cudaMemcpy(&hl, s->loss, sizeof(double), cudaMemcpyDeviceToHost), "copy loss");
+    SCK(cudaMemcpy(&hl, s->loss.p, sizeof(double), cudaMemcpyDeviceToHost), "copy loss");
     if (loss) *loss = hl / (double)(n * kOut);
-    if (grads) SCK(cudaMemcpy(grads, s->G, sizeof(float) * (size_t)s->n_params, cudaMemcpyDeviceToHost), "copy grads");
+    if (grads) SCK(cudaMemcpy(grads, s->G.p, sizeof(float) * (size_t)s->n_params, cudaMemcpyDeviceToHost), "copy grads");
     return SBR_OK;
 }
 
@@ -730,7 +884,8 @@ int sbr_surrogate_train(sbr_surrogate* s, const double* x, const double* y, int6
     if (n > (1ll << 31) - 1) return SBR_ERR_ARG;
     SCK(cudaSetDevice(s->device), "cudaSetDevice");
     const int M = (int)std::min<long long>(batch, (n / 128) * 128);
-    int rc = ensure_cap(s, M);
+    int group = 1;
+    int rc = choose_group(s, M, &group);
     if (rc != SBR_OK) return rc;
     // target scale: RMS of the targets
     double ss = 0.0;
@@ -748,59 +903,84 @@ int sbr_surrogate_train(sbr_surrogate* s, const double* x, const double* y, int6
         SCK(ce, "upload targets");
     }
     const long long steps_per_epoch = n / M;
-    // one permutation per epoch on the device; per-epoch squared-error sums on the device
+    // per member of the group one permutation per epoch and the per-epoch squared-error sums, on the device
     int* dperm = nullptr;
     double* dloss = nullptr;
-    ce = cudaMalloc(&dperm, sizeof(int) * (size_t)n);
-    if (ce == cudaSuccess) ce = cudaMalloc(&dloss, sizeof(double) * (size_t)epochs);
+    ce = cudaMalloc(&dperm, sizeof(int) * (size_t)n * group);
+    if (ce == cudaSuccess) ce = cudaMalloc(&dloss, sizeof(double) * (size_t)epochs * group);
     if (ce != cudaSuccess) {
         cudaFree(x4);
         cudaFree(y4);
         cudaFree(dperm);
         SCK(ce, "alloc permutation");
     }
-    std::vector<int> perm((size_t)n);
-    std::vector<double> hloss((size_t)epochs);
-    cudaMemsetAsync(s->gerr, 0, sizeof(int), s->stream);
+    std::vector<int> perm((size_t)n * group);
+    std::vector<double> hloss((size_t)epochs * group);
+    cudaMemsetAsync(s->gerr.p, 0, sizeof(int), s->stream);
     const double total_steps = (double)epochs * (double)steps_per_epoch;
-    for (int e = 0; e < s->opt.n_members && rc == SBR_OK; ++e) {
-        std::mt19937_64 rng(s->opt.seed * 7919 + (uint64_t)e);
-        cudaMemsetAsync(dloss, 0, sizeof(double) * (size_t)epochs, s->stream);
+    // the members of a group take each step together: they share no data, and one member's batch leaves most of
+    // the GPU idle
+    for (int e0 = 0; e0 < s->opt.n_members && rc == SBR_OK; e0 += group) {
+        const int g = std::min(group, s->opt.n_members - e0);
+        std::vector<std::mt19937_64> rng;
+        for (int e = 0; e < g; ++e) rng.emplace_back(s->opt.seed * 7919 + (uint64_t)(e0 + e));
+        cudaMemsetAsync(dloss, 0, sizeof(double) * (size_t)epochs * g, s->stream);
         long long call_step = 0;
         for (int ep = 0; ep < epochs && rc == SBR_OK; ++ep) {
-            for (int64_t i = 0; i < n; ++i) perm[(size_t)i] = (int)i;
-            std::shuffle(perm.begin(), perm.end(), rng);
+            auto shuffle = [&](int e) {
+                int* pe = perm.data() + (size_t)e * n;
+                for (int64_t i = 0; i < n; ++i) pe[i] = (int)i;
+                std::shuffle(pe, pe + n, rng[(size_t)e]);
+            };
+            // each member's permutation on a thread of its own (the GPU waits for the first epoch's)
+            std::vector<std::thread> th;
+            int started = 0;
+            try {
+                if (n >= 8192)
+                    for (; started < g - 1; ++started) th.emplace_back(shuffle, started);
+            } catch (const std::exception&) {  // no thread to be had: the rest here
+            }
+            for (int e = started; e < g; ++e) shuffle(e);
+            for (auto& t : th) t.join();
             // pageable source: the call returns once the host buffer has been consumed
-            if (cudaMemcpyAsync(dperm, perm.data(), sizeof(int) * (size_t)n, cudaMemcpyHostToDevice, s->stream) !=
+            if (cudaMemcpyAsync(dperm, perm.data(), sizeof(int) * (size_t)n * g, cudaMemcpyHostToDevice, s->stream) !=
                 cudaSuccess) {
                 rc = sfail(s, SBR_ERR_CUDA, "upload permutation");
                 break;
             }
             for (long long st = 0; st < steps_per_epoch && rc == SBR_OK; ++st) {
-                k_gather<<<blocks(M, 256), 256, 0, s->stream>>>(x4, y4, dperm + st * M, M, s->xb, s->yb);
-                rc = forward(s, e, M, s->y);
-                if (rc == SBR_OK) rc = backward(s, e, M, dloss + ep);
+                k_gather<<<dim3(blocks(M, 256), g), 256, 0, s->stream>>>((const float4*)x4, (const float4*)y4,
+                                                                         dperm + st * M, n, M, s->xb.as<float4>(),
+                                                                         s->yb.as<float4>());
+                rc = forward(s, e0, g, M, s->xb.as<float>(), M, s->y.as<float>(), true);
+                if (rc == SBR_OK) rc = backward(s, e0, g, M, dloss + ep, epochs);
                 if (rc != SBR_OK) break;
-                const long long t = ++s->steps[(size_t)e];
                 const float b1 = 0.9f, b2 = 0.999f;
-                const float c1 = 1.f / (1.f - powf(b1, (float)t)), c2 = 1.f / (1.f - powf(b2, (float)t));
+                AdamBias ab;
+                for (int e = 0; e < g; ++e) {
+                    const long long t = ++s->steps[(size_t)(e0 + e)];
+                    ab.c1[e] = 1.f / (1.f - powf(b1, (float)t));
+                    ab.c2[e] = 1.f / (1.f - powf(b2, (float)t));
+                }
                 // cosine schedule lr -> lr / 100 over this call
                 const double ph = (double)(call_step++) / std::max(1.0, total_steps - 1.0);
                 const float lr_t = (float)(lr * (0.01 + 0.99 * 0.5 * (1.0 + cos(kPi * ph))));
-                k_adam<<<blocks(s->n_params, 256), 256, 0, s->stream>>>(s->P[e], s->Pm[e], s->Pv[e], s->G,
-                                                                         s->n_params, lr_t, b1, b2, c1, c2, 1e-8f);
-                rc = refresh_bf16(s, e);
+                const size_t at = (size_t)e0 * s->n_params;
+                k_adam<<<dim3(blocks(s->n_params / 4, 256), g), 256, 0, s->stream>>>(
+                    s->P.as<float>() + at, s->Pm.as<float>() + at, s->Pv.as<float>() + at, s->G.as<float>(), s->n_params,
+                    s->Wbf.as<__nv_bfloat16>() + (size_t)e0 * s->n_bf, s->n_bf, s->L, lr_t, b1, b2, ab, 1e-8f);
             }
         }
         if (rc == SBR_OK &&
-            (cudaMemcpyAsync(hloss.data(), dloss, sizeof(double) * (size_t)epochs, cudaMemcpyDeviceToHost,
+            (cudaMemcpyAsync(hloss.data(), dloss, sizeof(double) * (size_t)epochs * g, cudaMemcpyDeviceToHost,
                              s->stream) != cudaSuccess ||
              cudaStreamSynchronize(s->stream) != cudaSuccess))
             rc = sfail(s, SBR_ERR_CUDA, "copy losses");
         if (rc == SBR_OK && loss_per_epoch)
-            for (int ep = 0; ep < epochs; ++ep)
-                loss_per_epoch[(size_t)e * epochs + ep] =
-                    (float)(hloss[(size_t)ep] / ((double)M * kOut * (double)steps_per_epoch));
+            for (int e = 0; e < g; ++e)
+                for (int ep = 0; ep < epochs; ++ep)
+                    loss_per_epoch[(size_t)(e0 + e) * epochs + ep] =
+                        (float)(hloss[(size_t)e * epochs + ep] / ((double)M * kOut * (double)steps_per_epoch));
     }
     cudaFree(dperm);
     cudaFree(dloss);
@@ -816,10 +996,14 @@ int sbr_surrogate_predict(sbr_surrogate* s, const double* x, int64_t n, double* 
     if (!s || !x || n < 1 || (!y_mean && !spread_db)) return SBR_ERR_ARG;
     if (n > (1ll << 31) - 1) return SBR_ERR_ARG;
     SCK(cudaSetDevice(s->device), "cudaSetDevice");
-    // prediction batches of 65536 rows: the GEMMs fill the GPU with two or more tiles per SM
-    const int M = (int)std::min<int64_t>(65536, ((n + 127) / 128) * 128);
-    int rc = ensure_cap(s, M);
-    if (rc != SBR_OK) return rc;
+    // all members at once, batches of about 512 MB of activations: 65536 rows of the default ensemble. Smaller ones
+    // would stay in L2 but pay a pipeline fill and a last wave per launch (64 MB: 12.2, 256 MB: 8.9, 512 MB: 8.1,
+    // 1 GB: 7.9 ms for 300k points)
+    const int g = s->opt.n_members;
+    const long long fit = (512ll << 20) / (4ll * s->opt.width * g) / 128 * 128;
+    const int M = (int)std::min<int64_t>(std::max<long long>(1024, fit), ((n + 127) / 128) * 128);
+    SCK(ensure_ws(s, M, g, false), "alloc prediction workspace");
+    int rc = SBR_OK;
     float* x4 = nullptr;
     rc = upload_inputs(s, x, n, &x4);
     if (rc != SBR_OK) return rc;
@@ -832,16 +1016,19 @@ int sbr_surrogate_predict(sbr_surrogate* s, const double* x, int64_t n, double* 
         cudaFree(dmean);
         SCK(ce, "alloc outputs");
     }
-    cudaMemsetAsync(s->gerr, 0, sizeof(int), s->stream);
+    cudaMemsetAsync(s->gerr.p, 0, sizeof(int), s->stream);
     for (int64_t b0 = 0; b0 < n && rc == SBR_OK; b0 += M) {
         const int cnt = (int)std::min<int64_t>(M, n - b0);
         const int Mp = ((cnt + 127) / 128) * 128;  // padded rows are computed and ignored
-        cudaMemsetAsync(s->xb, 0, sizeof(float) * kIn * (size_t)Mp, s->stream);
-        cudaMemcpyAsync(s->xb, x4 + kIn * b0, sizeof(float) * kIn * (size_t)cnt, cudaMemcpyDeviceToDevice, s->stream);
-        for (int e = 0; e < s->opt.n_members && rc == SBR_OK; ++e)
-            rc = forward(s, e, Mp, s->y + (size_t)e * M * kOut, false);
+        const float* xb = x4 + kIn * b0;
+        if (Mp > cnt) {
+            cudaMemsetAsync(s->xb.p, 0, sizeof(float) * kIn * (size_t)Mp, s->stream);
+            cudaMemcpyAsync(s->xb.p, xb, sizeof(float) * kIn * (size_t)cnt, cudaMemcpyDeviceToDevice, s->stream);
+            xb = s->xb.as<float>();
+        }
+        rc = forward(s, 0, g, Mp, xb, 0, s->y.as<float>(), false);
         if (rc == SBR_OK)
-            k_ens_stats<<<blocks(cnt, 256), 256, 0, s->stream>>>(s->y, s->opt.n_members, (long long)M * kOut, cnt,
+            k_ens_stats<<<blocks(cnt, 256), 256, 0, s->stream>>>(s->y.as<float>(), g, (long long)Mp * kOut, cnt,
                                                                  s->target_scale, dmean + kOut * b0, dspread + b0);
     }
     if (rc == SBR_OK) rc = check_gemm_err(s);

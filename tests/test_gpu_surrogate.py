@@ -146,6 +146,36 @@ def test_prediction_batches_agree_bit_for_bit(G):
     assert np.array_equal(sp_all, np.concatenate([p[1] for p in parts]))
 
 
+# widths on both sides of the register-weight head (up to 512), 64- and 128-column tiles, a single hidden layer
+@pytest.mark.parametrize("width,depth,nf,members,n", [(128, 1, 128, 3, 128), (384, 2, 256, 2, 640), (512, 6, 256, 4, 2048),
+                                                      (640, 2, 128, 3, 256)])
+def test_grouped_training_step_is_adam_on_each_members_gradient(G, width, depth, nf, members, n):
+    """One Adam step of all members together (one batch, so the rows only change order) against the update computed
+    from each member's own gradient. Adam's first step is lr g / (|g| + eps'): for entries of at least 1e-2 of the
+    largest and 1e-5 in size, the FP32 sums' order changes g by far less than |g|, and eps = 1e-8 the quotient by
+    at most 1e-3, so the parameters agree within 2e-3 lr plus two roundings of the parameter."""
+    rng, x = _samples(n, 8)
+    y = rng.normal(0, 1, (n, 4))
+    y /= np.sqrt(np.mean(y ** 2))
+    s = G.Surrogate(0, n_members=members, width=width, depth=depth, n_fourier=nf, fourier_sigma=2.0, seed=5)
+    p0 = [s.params(e).astype(np.float64) for e in range(members)]
+    lg = [s.grads(x, y, e) for e in range(members)]
+    lr = 1e-3
+    loss = s.train(x, y, epochs=1, batch=n, lr=lr)
+    p1 = [s.params(e).astype(np.float64) for e in range(members)]
+    s.close()
+    lay, _ = mlp.layout(width, depth, nf)
+    for e in range(members):
+        assert abs(loss[e, 0] - lg[e][0]) <= 1e-5 * lg[e][0]
+        g = lg[e][1].astype(np.float64)
+        for o, shp, ob, nb in lay:
+            for a, b in ((o, o + shp[0] * shp[1]), (ob, ob + nb)):
+                ok = np.abs(g[a:b]) >= max(1e-2 * np.abs(g[a:b]).max(), 1e-5)
+                assert ok.any()
+                d = p1[e][a:b] - p0[e][a:b] + lr * np.sign(g[a:b])
+                assert np.all(np.abs(d[ok]) <= 2e-3 * lr + 2.0 ** -23 * np.abs(p0[e][a:b][ok]))
+
+
 def test_training_reduces_loss_and_ensemble_spread(G):
     rng, x = _samples(8192, 5)
     az, el = np.radians(x[:, 0]), np.radians(x[:, 1])
