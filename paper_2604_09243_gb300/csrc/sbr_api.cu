@@ -956,6 +956,7 @@ int po_run(sbr_ctx* c, PoArgs pa, int64_t a0, int64_t a1, const std::vector<int>
     PoAngle* pang = (PoAngle*)hs;
     long long* off = (long long*)(hs + b_ang);
     long long part = 0, n_items = 0;
+    int max_nf = 0;
     for (int i = 0; i < na; ++i) {
         const AngleHost& h = c->ang[(size_t)(a0 + i)];
         if (i > 0 && h.rec_begin != off[i])
@@ -968,6 +969,7 @@ int po_run(sbr_ctx* c, PoArgs pa, int64_t a0, int64_t a1, const std::vector<int>
         A.item_end = (int)(n_items + ni);
         A.f0 = f0[(size_t)(a0 + i)];
         A.nf = nf[(size_t)(a0 + i)];
+        max_nf = std::max(max_nf, A.nf);
         A.out_row = out_row[(size_t)(a0 + i)];
         A.part = part;
         n_items += ni;
@@ -994,7 +996,7 @@ int po_run(sbr_ctx* c, PoArgs pa, int64_t a0, int64_t a1, const std::vector<int>
     pa.item_records = c->tune.po_item;
     pa.err = c->err_dev.as<int>() + 3;  // bounded waits of the staged single-frequency sum (callers clear it)
     CK(launch_po(pa, c->stream), "po reduce");
-    CK(launch_po_final(pa.partial, pa.items, c->itemoff.as<PoAngle>(), na, pa.kfreq, pa.n_pol, dE, dR, c->stream),
+    CK(launch_po_final(pa.partial, pa.items, c->itemoff.as<PoAngle>(), na, max_nf, pa.kfreq, pa.n_pol, dE, dR, c->stream),
        "po final");
     if (n_launch) *n_launch += (n_items > 0 ? 2 : 0) + 1;
     return SBR_OK;
@@ -1021,6 +1023,7 @@ struct BatchPlan {
     long long launched = 0;
     int64_t n_launch = 0, n_pass = 0;
     bool count = false;
+    int max_nf = 0;        // most frequencies of a request
     unsigned big_cap = 0;  // entries of rbig
     PoArgs pa;
     // device buffers
@@ -1157,7 +1160,7 @@ cudaError_t enqueue_plan(const sbr_ctx* c, BatchPlan& P, cudaStream_t st)
             e = launch_po(pa, st, (int)std::min<long long>(P.items_bound[k], (long long)c->n_sms * 8));
         }
         if (e == cudaSuccess)
-            e = launch_po_final(P.partial.as<double>(), P.items.as<PoItem>(), pang, na, P.kfreq.as<double>(),
+            e = launch_po_final(P.partial.as<double>(), P.items.as<PoItem>(), pang, na, P.max_nf, P.kfreq.as<double>(),
                                 P.pa.n_pol, P.E, P.R, st);
     }
     return e;
@@ -1264,6 +1267,7 @@ int build_plan(sbr_ctx* c, BatchPlan& P)
         memset(&A, 0, sizeof(A));
         A.f0 = (int)P.req[(size_t)a].freq_offset;
         A.nf = P.req[(size_t)a].n_freq;
+        P.max_nf = std::max(P.max_nf, A.nf);
         A.out_row = row;
         row += A.nf;
     }

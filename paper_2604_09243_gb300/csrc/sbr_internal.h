@@ -281,9 +281,10 @@ cudaError_t launch_po_items(const unsigned* recoff, PoAngle* angles, int n_angle
 // whose item ranges and partial offsets are set
 cudaError_t launch_po_items_fill(const long long* recoff, const PoAngle* angles, int n_angles, int n_pol,
                                  int item_records, PoItem* items, cudaStream_t st);
-// E[row][n_pol][2] and rcs[row][n_pol] for every aspect's rows (fixed-order FP64 sums of the partials)
+// E[row][n_pol][2] and rcs[row][n_pol] for every aspect's rows (fixed-order FP64 sums of the partials). An
+// aspect's items, and their partials, are consecutive; max_freq: the largest PoAngle.nf.
 cudaError_t launch_po_final(const double* partial, const PoItem* items, const PoAngle* angles, int n_angles,
-                            const double* kfreq, int n_pol, double* E, double* rcs, cudaStream_t st);
+                            int max_freq, const double* kfreq, int n_pol, double* E, double* rcs, cudaStream_t st);
 
 // ---------------------------------------------------------------- tensor-core GEMM (surrogate)
 // C = A B^T, A [M x K] and B [N x K] BF16, for `groups` equal problems; M, N

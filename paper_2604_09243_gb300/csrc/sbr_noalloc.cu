@@ -175,7 +175,7 @@ extern "C" int sbr_po_integrate_noalloc(const void* records, const int64_t* rec_
     pa.partial = (double*)(base + kOffPartial);  // every entry read below is written by this call first
     e = launch_po(pa, st);
     if (e == cudaSuccess)
-        e = launch_po_final(pa.partial, pa.items, (const PoAngle*)(base + kOffOff), (int)n_angles, pa.kfreq, pa.n_pol,
+        e = launch_po_final(pa.partial, pa.items, (const PoAngle*)(base + kOffOff), (int)n_angles, (int)n_freq, pa.kfreq, pa.n_pol,
                             E_re_im, rcs_dbsm, st);
     if (e != cudaSuccess) return reject(SBR_ERR_CUDA, "sbr_po_integrate_noalloc: kernel launch failed");
     return SBR_OK;

@@ -27,10 +27,12 @@ namespace {
 constexpr int kPoThreads = 256;
 constexpr int kWarps = kPoThreads / 32;
 
+// kComp: the compensated phase alone (the default), without the other modes' branches and slow paths
+template <bool kComp>
 __device__ __forceinline__ void phase_cs(const PoArgs& a, float4 fq, double kd, float lh, float ll, float& c,
                                          float& s)
 {
-    if (a.phase_mode == 0) {
+    if (kComp || a.phase_mode == 0) {
         const float p = __fmul_rn(fq.x, lh);
         float e = __fmaf_rn(fq.x, lh, -p);
         e = __fadd_rn(e, __fadd_rn(__fmul_rn(fq.x, ll), __fmul_rn(fq.y, lh)));
@@ -47,18 +49,57 @@ __device__ __forceinline__ void phase_cs(const PoArgs& a, float4 fq, double kd, 
     }
 }
 
-// kPoPer records per thread: items of kPoPer * kPoThreads records
+// Sums of kN values over a warp, every sum in the order of the plain butterfly
+// (lane distance 16, 8, 4, 2, 1). As long as a lane holds several values it
+// keeps one half of them and sends its partner the other, so that kN values
+// take about kN exchanges instead of 5 kN; afterwards lane l holds value
+// warp_sum_index<kN>(l).
+template <int kN>
+__device__ __forceinline__ float warp_sums(float* v)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int n = kN, o = 16; o > 0; o >>= 1) {
+        if (n > 1) {
+            n >>= 1;
+            const bool up = lane & o;
+#pragma unroll
+            for (int j = 0; j < kN / 2; ++j) {
+                if (j >= n) break;
+                const float r = __shfl_xor_sync(0xffffffffu, up ? v[j] : v[j + n], o);
+                v[j] = (up ? v[j + n] : v[j]) + r;
+            }
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+        }
+    }
+    return v[0];
+}
+template <int kN>
+__device__ __forceinline__ int warp_sum_index(int lane)
+{
+    return lane / (32 / kN);
+}
+
 // kPoPer records per thread (items of kPoPer * kPoThreads records) and room for
-// kPol polarisations (2 or 4). Every block reduction carries 8 sums: two
-// frequencies at a time when kPol = 2, one when kPol = 4. Each sum is formed
-// in the same order whatever kPol, so the results do not depend on it.
-template <int kPoPer, int kPol>
+// kPol polarisations (2 or 4). A block reduction carries kSums sums: four
+// frequencies at a time when kPol = 2, two when kPol = 4, one barrier each
+// (the partial sums of consecutive reductions alternate between two buffers).
+// Each sum is formed in the same order whatever kPol, so the results do not
+// depend on it. Bound by instruction issue (~45 per tube and frequency in the
+// phase and its products): 9 aspects of 175k tubes, 201 frequencies, 4
+// polarisations in 472 us, 670 G tube-frequencies/s; 635 us with every sum
+// exchanged at every step of the butterfly and the other phase modes' code in
+// the loop.
+constexpr int kSums = 16;
+template <int kPoPer, int kPol, bool kComp>
 __global__ void __launch_bounds__(kPoThreads) k_po(const PoArgs a)
 {
-    constexpr int kF = 4 / kPol;  // frequencies per block reduction
-    __shared__ float s_red[kWarps][8];
+    constexpr int kF = kSums / (2 * kPol);  // frequencies per block reduction
+    __shared__ float s_red[2][kWarps][kSums];
     const int n_items = a.n_items_dev ? *a.n_items_dev : a.n_items;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    int buf = 0;
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
         const PoItem I = a.items[item];
         float cf[kPoPer][kPol];
@@ -87,20 +128,20 @@ __global__ void __launch_bounds__(kPoThreads) k_po(const PoArgs a)
                 ll[k] = 0.f;
             }
         }
-        for (int f0 = 0; f0 < I.nf; f0 += kF) {
-            float acc[8];
+        for (int f0 = 0; f0 < I.nf; f0 += kF, buf ^= 1) {
+            float acc[kSums];
 #pragma unroll
-            for (int v = 0; v < 8; ++v) acc[v] = 0.f;
+            for (int v = 0; v < kSums; ++v) acc[v] = 0.f;
 #pragma unroll
             for (int fj = 0; fj < kF; ++fj) {
                 if (f0 + fj >= I.nf) break;
                 const float4 fq = a.freq[I.f0 + f0 + fj];
-                const double kd = a.kfreq[I.f0 + f0 + fj];
+                const double kd = kComp ? 0.0 : a.kfreq[I.f0 + f0 + fj];
 #pragma unroll
                 for (int k = 0; k < kPoPer; ++k) {
                     if (k * kPoThreads + tid >= I.count) break;
                     float c, s;
-                    phase_cs(a, fq, kd, lh[k], ll[k], c, s);
+                    phase_cs<kComp>(a, fq, kd, lh[k], ll[k], c, s);
 #pragma unroll
                     for (int q = 0; q < kPol; ++q) {
                         acc[(fj * kPol + q) * 2] = fmaf(cf[k][q], c, acc[(fj * kPol + q) * 2]);
@@ -108,24 +149,18 @@ __global__ void __launch_bounds__(kPoThreads) k_po(const PoArgs a)
                     }
                 }
             }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                for (int v = 0; v < 8; ++v) acc[v] += __shfl_xor_sync(0xffffffffu, acc[v], o);
-            if (lane == 0)
-#pragma unroll
-                for (int v = 0; v < 8; ++v) s_red[w][v] = acc[v];
+            const float sum = warp_sums<kSums>(acc);
+            if ((lane & 1) == 0) s_red[buf][w][warp_sum_index<kSums>(lane)] = sum;
             __syncthreads();
-            if (tid < 8) {
+            if (tid < kSums) {
                 const int fj = tid / (2 * kPol), r = tid - fj * (2 * kPol);  // r = 2 q + (0 re, 1 im)
                 if (f0 + fj < I.nf && r < 2 * a.n_pol) {
                     float v = 0.f;
 #pragma unroll
-                    for (int k = 0; k < kWarps; ++k) v += s_red[k][tid];
+                    for (int k = 0; k < kWarps; ++k) v += s_red[buf][k][tid];
                     a.partial[I.part + (size_t)(f0 + fj) * (2 * a.n_pol) + r] = (double)v;
                 }
             }
-            __syncthreads();
         }
     }
 }
@@ -140,7 +175,8 @@ static_assert(kPoItemRecords == 4 * kPoThreads, "PO item size");
 // mbarrier each, issued ahead across item boundaries, so the loads of the next
 // stages overlap the phases, sums and reductions of the current one. Thread t
 // takes record k * kPoThreads + t of an item in stage k, in order, so every
-// term and every addition is that of k_po: the sums are bit-identical.
+// term and every addition is that of k_po: the sums are bit-identical. 4 GB of
+// records in 632 us, 6.3 TB/s (840 us with the other phase modes' code inside).
 constexpr int kBulkStages = 4;
 constexpr unsigned kPoSpin = 1u << 22;  // try_wait rounds before a wait gives up
 
@@ -161,7 +197,7 @@ __device__ __forceinline__ bool po_wait(uint64_t* bar, unsigned parity)
     return false;
 }
 
-template <int kPol>
+template <int kPol, bool kComp>
 __global__ void __launch_bounds__(kPoThreads) k_po_bulk(const PoArgs a)
 {
     constexpr int kF = 4 / kPol;
@@ -246,9 +282,9 @@ __global__ void __launch_bounds__(kPoThreads) k_po_bulk(const PoArgs a)
             for (int fj = 0; fj < kF; ++fj) {
                 if (fj >= I.nf) break;
                 const float4 fq = a.freq[I.f0 + fj];
-                const double kd = a.kfreq[I.f0 + fj];
+                const double kd = kComp ? 0.0 : a.kfreq[I.f0 + fj];
                 float c, sn;
-                phase_cs(a, fq, kd, y.y, y.z, c, sn);
+                phase_cs<kComp>(a, fq, kd, y.y, y.z, c, sn);
 #pragma unroll
                 for (int q = 0; q < kPol; ++q) {
                     acc[(fj * kPol + q) * 2] = fmaf(cf[q], c, acc[(fj * kPol + q) * 2]);
@@ -256,13 +292,8 @@ __global__ void __launch_bounds__(kPoThreads) k_po_bulk(const PoArgs a)
                 }
             }
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int v = 0; v < 8; ++v) acc[v] += __shfl_xor_sync(0xffffffffu, acc[v], o);
-        if (lane == 0)
-#pragma unroll
-            for (int v = 0; v < 8; ++v) s_red[w][v] = acc[v];
+        const float sum = warp_sums<8>(acc);
+        if ((lane & 3) == 0) s_red[w][warp_sum_index<8>(lane)] = sum;
         __syncthreads();
         if (tid < 8) {
             const int fj = tid / (2 * kPol), r = tid - fj * (2 * kPol);
@@ -333,73 +364,96 @@ __global__ void k_po_items_scan(const unsigned* recoff, PoAngle* angles, int na,
     }
 }
 
-// Work list, stage 2: one warp per aspect writes its items. recoff: the record
-// offsets of the aspects (32-bit within a chunk, or 64-bit over a whole trace).
+// Work list, stage 2: the warps of row blockIdx.y's grid share the aspect's
+// items. recoff: the record offsets of the aspects (32-bit within a chunk, or
+// 64-bit over a whole trace).
 template <typename Off>
-__global__ void k_po_items_fill(const Off* recoff, const PoAngle* angles, int na, int n_pol, int item_records,
-                                PoItem* items)
+__global__ void k_po_items_fill(const Off* recoff, const PoAngle* angles, int n_pol, int item_records, PoItem* items)
 {
-    const int lane = threadIdx.x & 31;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    for (int a = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; a < na; a += nwarps) {
-        const PoAngle A = angles[a];
-        const long long r0 = (long long)recoff[a], rc = (long long)recoff[a + 1] - r0;
-        for (int r = lane; r < A.item_end - A.item_begin; r += 32) {
-            PoItem it;
-            it.angle = a;
-            it.count = (int)min((long long)item_records, rc - (long long)r * item_records);
-            it.first = r0 + (long long)r * item_records;
-            it.f0 = A.f0;
-            it.nf = A.nf;
-            it.part = A.part + (long long)r * A.nf * 2 * n_pol;
-            items[A.item_begin + r] = it;
-        }
+    const int a = blockIdx.x;
+    const PoAngle A = angles[a];
+    const long long r0 = (long long)recoff[a], rc = (long long)recoff[a + 1] - r0;
+    for (int r = blockIdx.y * blockDim.x + threadIdx.x; r < A.item_end - A.item_begin; r += gridDim.y * blockDim.x) {
+        PoItem it;
+        it.angle = a;
+        it.count = (int)min((long long)item_records, rc - (long long)r * item_records);
+        it.first = r0 + (long long)r * item_records;
+        it.f0 = A.f0;
+        it.nf = A.nf;
+        it.part = A.part + (long long)r * A.nf * 2 * n_pol;
+        items[A.item_begin + r] = it;
     }
 }
 
-// one block per aspect; its threads stride over (frequency, polarisation) outputs
-__global__ void k_po_final(const double* partial, const PoItem* items, const PoAngle* angles, const double* kfreq,
-                           int n_pol, double* E, double* rcs)
+// Blocks of 8 outputs (frequency, polarisation; re and im each) x kSlices item
+// slices per aspect: slice s adds the partials of items s, s + kSlices, ... in
+// item order, then the slices are added in a fixed tree, so a sum's order
+// depends on its aspect's item count alone. One thread adding an aspect's items
+// one after another was a chain of up to thousands of dependent FP64 additions
+// (3,300 items per aspect of the aircraft at 10 GHz, 37 aspects: 967 us, now 68).
+constexpr int kSlices = 32, kOutB = 8;
+__global__ void __launch_bounds__(kSlices* kOutB) k_po_final(const double* partial, const PoItem* items,
+                                                            const PoAngle* angles, const double* kfreq, int n_pol,
+                                                            double* E, double* rcs)
 {
+    __shared__ double2 s_sum[kSlices][kOutB];
     const PoAngle A = angles[blockIdx.x];
-    for (int o = threadIdx.x; o < A.nf * n_pol; o += blockDim.x) {
-        const int q = o / n_pol, p = o - q * n_pol;
-        // item order, as written; the loads of 8 items are issued before their additions
+    const int n_out = A.nf * n_pol, oi = threadIdx.x % kOutB, slice = threadIdx.x / kOutB;
+    const int n = A.item_end - A.item_begin;
+    // an aspect's items are consecutive and so are their partials, nf x n_pol x (re, im) each
+    const double2* p0 = n > 0 ? reinterpret_cast<const double2*>(partial + items[A.item_begin].part) : nullptr;
+    for (int o0 = blockIdx.y * kOutB; o0 < n_out; o0 += gridDim.y * kOutB) {
+        const int o = o0 + oi;
         double sr = 0.0, si = 0.0;
-        for (int it0 = A.item_begin; it0 < A.item_end; it0 += 8) {
-            double vr[8], vi[8];
+        if (o < n_out) {
+            // the loads of 8 items are issued before their additions
+            for (int it = slice; it < n; it += 8 * kSlices) {
+                double2 v[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                vr[u] = 0.0;
-                vi[u] = 0.0;
-                if (it0 + u < A.item_end) {
-                    const double* v = partial + items[it0 + u].part + (size_t)q * (2 * n_pol) + 2 * p;
-                    vr[u] = v[0];
-                    vi[u] = v[1];
+                for (int u = 0; u < 8; ++u) {
+                    const int k = it + u * kSlices;
+                    v[u] = k < n ? __ldg(p0 + (size_t)k * n_out + o) : make_double2(0.0, 0.0);
                 }
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (it + u * kSlices < n) {
+                        sr += v[u].x;
+                        si += v[u].y;
+                    }
             }
+        }
+        s_sum[slice][oi] = make_double2(sr, si);
 #pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if (it0 + u < A.item_end) {
-                    sr += vr[u];
-                    si += vi[u];
-                }
+        for (int h = kSlices / 2; h > 0; h >>= 1) {
+            __syncthreads();
+            if (slice < h) {
+                sr += s_sum[slice + h][oi].x;
+                si += s_sum[slice + h][oi].y;
+                s_sum[slice][oi] = make_double2(sr, si);
+            }
         }
-        // E = (-j k / 4 pi) (sr + j si)
-        const double pre = kfreq[A.f0 + q] / (4.0 * 3.14159265358979323846);
-        const double er = pre * si, ei = -pre * sr;
-        const long long i = (A.out_row + q) * n_pol + p;
-        if (E) {
-            E[2 * i] = er;
-            E[2 * i + 1] = ei;
+        if (slice == 0 && o < n_out) {
+            // E = (-j k / 4 pi) (sr + j si)
+            const int q = o / n_pol, p = o - q * n_pol;
+            const double pre = kfreq[A.f0 + q] / (4.0 * 3.14159265358979323846);
+            const double er = pre * si, ei = -pre * sr;
+            const long long i = (A.out_row + q) * n_pol + p;
+            if (E) {
+                E[2 * i] = er;
+                E[2 * i + 1] = ei;
+            }
+            if (rcs) rcs[i] = 10.0 * log10(4.0 * 3.14159265358979323846 * (er * er + ei * ei));
         }
-        if (rcs) rcs[i] = 10.0 * log10(4.0 * 3.14159265358979323846 * (er * er + ei * ei));
+        __syncthreads();  // the next outputs' sums reuse the shared rows
     }
 }
 
 }  // namespace
 
-cudaError_t launch_po(const PoArgs& a, cudaStream_t st, int n_blocks)
+namespace {
+
+template <bool kComp>
+cudaError_t launch_po_mode(const PoArgs& a, cudaStream_t st, int n_blocks)
 {
     const int grid = n_blocks > 0 ? n_blocks : a.n_items;
     if (grid <= 0) return cudaSuccess;
@@ -411,36 +465,47 @@ cudaError_t launch_po(const PoArgs& a, cudaStream_t st, int n_blocks)
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e == cudaSuccess)
-            e = two ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_po_bulk<2>, kPoThreads, 0)
-                    : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_po_bulk<4>, kPoThreads, 0);
+            e = two ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_po_bulk<2, kComp>, kPoThreads, 0)
+                    : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_po_bulk<4, kComp>, kPoThreads, 0);
         if (e != cudaSuccess) return e;
         const int g = (int)std::min<long long>(a.n_items, (long long)sms * std::max(occ, 1));
-        if (two) k_po_bulk<2><<<g, kPoThreads, 0, st>>>(a);
-        else k_po_bulk<4><<<g, kPoThreads, 0, st>>>(a);
+        if (two) k_po_bulk<2, kComp><<<g, kPoThreads, 0, st>>>(a);
+        else k_po_bulk<4, kComp><<<g, kPoThreads, 0, st>>>(a);
         return cudaGetLastError();
     }
     if (per == 2) {
-        if (two) k_po<2, 2><<<grid, kPoThreads, 0, st>>>(a);
-        else k_po<2, 4><<<grid, kPoThreads, 0, st>>>(a);
+        if (two) k_po<2, 2, kComp><<<grid, kPoThreads, 0, st>>>(a);
+        else k_po<2, 4, kComp><<<grid, kPoThreads, 0, st>>>(a);
     } else if (per == 8) {
-        if (two) k_po<8, 2><<<grid, kPoThreads, 0, st>>>(a);
-        else k_po<8, 4><<<grid, kPoThreads, 0, st>>>(a);
+        if (two) k_po<8, 2, kComp><<<grid, kPoThreads, 0, st>>>(a);
+        else k_po<8, 4, kComp><<<grid, kPoThreads, 0, st>>>(a);
     } else if (per == 4) {
-        if (two) k_po<4, 2><<<grid, kPoThreads, 0, st>>>(a);
-        else k_po<4, 4><<<grid, kPoThreads, 0, st>>>(a);
+        if (two) k_po<4, 2, kComp><<<grid, kPoThreads, 0, st>>>(a);
+        else k_po<4, 4, kComp><<<grid, kPoThreads, 0, st>>>(a);
     } else {
         return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
 }
 
+}  // namespace
+
+cudaError_t launch_po(const PoArgs& a, cudaStream_t st, int n_blocks)
+{
+    return a.phase_mode == 0 ? launch_po_mode<true>(a, st, n_blocks) : launch_po_mode<false>(a, st, n_blocks);
+}
+
+namespace {
+// a block row per aspect, more of them where few aspects hold many items
+dim3 fill_grid(int n_angles) { return dim3((unsigned)n_angles, (unsigned)std::max(1, std::min(16, 1024 / n_angles))); }
+}  // namespace
+
 cudaError_t launch_po_items(const unsigned* recoff, PoAngle* angles, int n_angles, int n_pol, int item_records,
                             PoItem* items, int* n_items, long long* valid, cudaStream_t st)
 {
     if (n_angles <= 0 || item_records <= 0) return cudaErrorInvalidValue;
     k_po_items_scan<<<1, 1024, 0, st>>>(recoff, angles, n_angles, n_pol, item_records, n_items, valid);
-    const int blocks = (int)std::min<long long>(((long long)n_angles * 32 + 255) / 256, 4096);
-    k_po_items_fill<unsigned><<<blocks, 256, 0, st>>>(recoff, angles, n_angles, n_pol, item_records, items);
+    k_po_items_fill<unsigned><<<fill_grid(n_angles), 128, 0, st>>>(recoff, angles, n_pol, item_records, items);
     return cudaGetLastError();
 }
 
@@ -448,16 +513,17 @@ cudaError_t launch_po_items_fill(const long long* recoff, const PoAngle* angles,
                                  int item_records, PoItem* items, cudaStream_t st)
 {
     if (n_angles <= 0 || item_records <= 0) return cudaErrorInvalidValue;
-    const int blocks = (int)std::min<long long>(((long long)n_angles * 32 + 255) / 256, 4096);
-    k_po_items_fill<long long><<<blocks, 256, 0, st>>>(recoff, angles, n_angles, n_pol, item_records, items);
+    k_po_items_fill<long long><<<fill_grid(n_angles), 128, 0, st>>>(recoff, angles, n_pol, item_records, items);
     return cudaGetLastError();
 }
 
 cudaError_t launch_po_final(const double* partial, const PoItem* items, const PoAngle* angles, int n_angles,
-                            const double* kfreq, int n_pol, double* E, double* rcs, cudaStream_t st)
+                            int max_freq, const double* kfreq, int n_pol, double* E, double* rcs, cudaStream_t st)
 {
     if (n_angles <= 0) return cudaSuccess;
-    k_po_final<<<n_angles, 128, 0, st>>>(partial, items, angles, kfreq, n_pol, E, rcs);
+    const long long blocks = ((long long)max_freq * n_pol + kOutB - 1) / kOutB;
+    k_po_final<<<dim3((unsigned)n_angles, (unsigned)std::max(1ll, std::min(blocks, 1024ll))), kSlices * kOutB, 0, st>>>(
+        partial, items, angles, kfreq, n_pol, E, rcs);
     return cudaGetLastError();
 }
 
