@@ -758,6 +758,7 @@ int trace_chunk(sbr_ctx* c, TraceRun& R, int64_t a0, int64_t a1, long long rec_b
     for (int i = 0; i < na; ++i) ta.bistatic |= c->ang[(size_t)(a0 + i)].bistatic ? 1 : 0;
     if (ta.octant) CK(ensure_octant_nodes(c, c->stream), "octant nodes");
     ta.nodes = ta.wide ? c->nodes4.as<float4>() : (ta.octant ? c->nodes_oct.as<float4>() : c->nodes.as<float4>());
+    ta.nodes2 = c->nodes.as<float4>();
     ta.tris = c->tris.as<float4>();
     ta.tri_nrm = ta.tris + 3 * (size_t)c->n_tri;
     ta.tri_v12 = ta.tris + 4 * (size_t)c->n_tri;
@@ -786,9 +787,9 @@ int trace_chunk(sbr_ctx* c, TraceRun& R, int64_t a0, int64_t a1, long long rec_b
         ta.tri_pos = c->tripos.as<int>();
         ta.list_count = total_dev + 4;
         // a bounce pass follows: list the hits and let it rebuild their states (not for B = 1, whose
-        // records are written from the stored states, nor for bistatic chunks; binary traversals only,
-        // where the rebuilding fits the bounce kernel's registers)
-        if (!ta.bistatic && !ta.wide && !ta.packet && (R.max_bounces >= 2 || R.escape))
+        // records are written from the stored states; binary per-lane traversals only, where the rebuilding
+        // fits the bounce kernel's registers)
+        if (!ta.wide && (!ta.packet || ta.bistatic) && (R.max_bounces >= 2 || R.escape))
             ta.hit_list = c->hitlist.as<uint2>();
     } else if (c->tune.silhouette) {
         CK(cudaMemsetAsync(c->cover.p, 0, sizeof(unsigned) * (size_t)(chunk_rays / 32 + na), c->stream), "memset cover");
@@ -1084,7 +1085,8 @@ cudaError_t enqueue_plan(const sbr_ctx* c, BatchPlan& P, cudaStream_t st)
         ta.octant = P.tune.octant;
         ta.n_nodes = c->n_nodes;
         ta.nodes = ta.wide ? c->nodes4.as<float4>() : (ta.octant ? c->nodes_oct.as<float4>() : c->nodes.as<float4>());
-        ta.tris = c->tris.as<float4>();
+        ta.nodes2 = c->nodes.as<float4>();
+    ta.tris = c->tris.as<float4>();
         ta.tri_nrm = ta.tris + 3 * (size_t)c->n_tri;
         ta.tri_v12 = ta.tris + 4 * (size_t)c->n_tri;
         ta.angles = P.angles.as<AngleDev>() + a0;
@@ -1356,6 +1358,7 @@ int flush_pool(sbr_ctx* c, TraceRun& R, PoolRun& P, RayState* partner)
     for (int64_t a = 0; a < P.n_angles; ++a) ta.bistatic |= c->ang[(size_t)a].bistatic ? 1 : 0;
     if (ta.octant) CK(ensure_octant_nodes(c, c->stream), "octant nodes");
     ta.nodes = ta.wide ? c->nodes4.as<float4>() : (ta.octant ? c->nodes_oct.as<float4>() : c->nodes.as<float4>());
+    ta.nodes2 = c->nodes.as<float4>();
     ta.tris = c->tris.as<float4>();
     ta.tri_nrm = ta.tris + 3 * (size_t)c->n_tri;
     ta.tri_v12 = ta.tris + 4 * (size_t)c->n_tri;

@@ -138,6 +138,7 @@ cudaError_t bvh_build(const BvhBuild& b, cudaStream_t st);
 
 struct TraceArgs {
     const float4* nodes;          // binary nodes, or 4-wide nodes when wide = 1
+    const float4* nodes2;         // binary nodes (visibility queries, whatever the traversal)
     int wide;
     int packet;                   // 1: warp-cooperative traversal of the binary tree
     int bistatic;                 // 1: some aspect of the chunk has a bistatic receiver (visibility tests)

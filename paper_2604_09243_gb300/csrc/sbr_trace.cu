@@ -908,6 +908,62 @@ __device__ __forceinline__ void tile_ij(const AngleDev& A, int p, int& i, int& j
     j = bv * (32 >> tw) + (l >> tw);
 }
 
+// Whether a query meets any triangle: binary traversal, near child first, that
+// ends at the first certain hit (whether one exists depends on no order). Out of
+// line, so that its registers do not burden the bounce kernel, which asks it at
+// one place (33 bistatic aspects of a 250k-triangle aircraft at 3 GHz: with the
+// first hits listed instead of stored, 6.82 -> 6.51 ms per trace and PO sum).
+__device__ __noinline__ bool any_hit(const TraceArgs& a, float3 o, float3 d, int skip, bool& overflow)
+{
+    constexpr int kStack = 64;
+    int stack[kStack];
+    const float3 inv = make_float3(safe_rcp(d.x), safe_rcp(d.y), safe_rcp(d.z));
+    const float3 oi = make_float3(o.x * inv.x, o.y * inv.y, o.z * inv.z);
+    const float2 ix = make_float2(inv.x, inv.x), iy = make_float2(inv.y, inv.y), iz = make_float2(inv.z, inv.z);
+    const float2 mx = make_float2(-oi.x, -oi.x), my = make_float2(-oi.y, -oi.y), mz = make_float2(-oi.z, -oi.z);
+    int sp = 0, ref = 0;
+    for (int it = 0;; ++it) {
+        if (it >= a.visit_limit) {
+            overflow = true;
+            return true;
+        }
+        if (ref >= 0) {
+            const float4* nd = a.nodes2 + 4 * (size_t)ref;
+            const float4 n0 = __ldg(nd), n1 = __ldg(nd + 1), n2 = __ldg(nd + 2), n3 = __ldg(nd + 3);
+            const float2 ax = fma2(make_float2(n0.x, n0.y), ix, mx), ay = fma2(make_float2(n0.z, n0.w), iy, my);
+            const float2 az = fma2(make_float2(n2.x, n2.y), iz, mz), bx = fma2(make_float2(n1.x, n1.y), ix, mx);
+            const float2 by = fma2(make_float2(n1.z, n1.w), iy, my), bz = fma2(make_float2(n2.z, n2.w), iz, mz);
+            const float an = fmaxf(fmaxf(fminf(ax.x, ax.y), fminf(ay.x, ay.y)), fmaxf(fminf(az.x, az.y), 0.f));
+            const float af = fminf(fminf(fmaxf(ax.x, ax.y), fmaxf(ay.x, ay.y)), fmaxf(az.x, az.y));
+            const float bn = fmaxf(fmaxf(fminf(bx.x, bx.y), fminf(by.x, by.y)), fmaxf(fminf(bz.x, bz.y), 0.f));
+            const float bf = fminf(fminf(fmaxf(bx.x, bx.y), fmaxf(by.x, by.y)), fmaxf(bz.x, bz.y));
+            const int lref = __float_as_int(n3.x), rref = __float_as_int(n3.y);
+            const bool hl = an <= af * kBoxGrow;
+            const bool hr = (bn <= bf * kBoxGrow) && (rref != kEmptyRef);
+            if (hl && hr) {
+                const bool lnear = an <= bn;
+                if (sp < kStack) stack[sp++] = lnear ? rref : lref;
+                else overflow = true;
+                ref = lnear ? lref : rref;
+                continue;
+            }
+            if (hl) { ref = lref; continue; }
+            if (hr) { ref = rref; continue; }
+        } else {
+            const int first = leaf_first(ref), cnt = leaf_count(ref);
+            for (int k = first; k < first + cnt; ++k) {
+                if (k == skip) continue;
+                const float4* tp = a.tris + 3 * (size_t)k;
+                float tc, et;
+                const int f = tri_filter(__ldg(tp), __ldg(tp + 1), __ldg(tp + 2), o, d, tc, et);
+                if (f == 1 || (f >= 2 && (tri_refine(a.tris, a.tri_v12, k, o, d, f + 2, tc) & 1))) return true;
+            }
+        }
+        if (sp == 0) return false;
+        ref = stack[--sp];
+    }
+}
+
 // Bistatic: the last hit contributes only if the receiver lies on the side of
 // its oriented FP32 normal (the sign of the exact dot product) and a query from
 // the offset origin toward the receiver meets no triangle (the one just hit is
@@ -921,14 +977,11 @@ __device__ __forceinline__ bool rx_visible(const TraceArgs& a, const AngleDev& A
     float sh, sl;
     tf_dot3(n, rx, sh, sl);  // the sign of the exact dot product
     if (!(sh > 0.f)) return false;
-    Hit h;
-    unsigned nv = 0, nt = 0;
-    if (a.wide) closest_hit4<false, 64>(a.nodes, tri_refs(a), r.o, rx, r.last, a.visit_limit, h, nv, nt, ovf);
-    else if (a.octant)
-        closest_hit_oct<false, 64>(a.nodes, a.n_nodes, tri_refs(a), r.o, rx, r.last, a.visit_limit, h, nv, nt, ovf);
-    else closest_hit<false, 64>(a.nodes, tri_refs(a), r.o, rx, r.last, a.visit_limit, h, nv, nt, ovf);
     ++nq;
-    return h.k < 0;
+    bool over = false;
+    const bool hit = any_hit(a, r.o, rx, r.last, over);
+    ovf = ovf || over;
+    return !hit;
 }
 
 __device__ __forceinline__ void emit(const TraceArgs& a, const Ray& r, bool zero)
@@ -1851,17 +1904,21 @@ __global__ void __launch_bounds__(kTraceThreads, 4) k_bounce(const TraceArgs a)
             else load_payload(a.q_in, src, r);
             const AngleDev& A = a.angles[r.angle];
             ++nq;
+            bool done = true, zero = false;
             if (h.k < 0) {
                 // escaped: its last hit radiates
-                emit(a, r, kBi && A.bistatic && !rx_visible(a, A, r, nq, ovf));
             } else if (escape_pass) {
-                emit(a, r, true);                      // still trapped after B_max: invalid
+                zero = true;  // still trapped after B_max: invalid
             } else {
                 if (kCount) ++nhit;
                 apply_hit(A, a.tri_nrm, h, a.flags, r);
                 record_hit(a, r, h);
-                if (r.nb < a.max_bounces || (a.flags & kFlagEscape)) again = true;
-                else emit(a, r, kBi && A.bistatic && !rx_visible(a, A, r, nq, ovf));
+                again = r.nb < a.max_bounces || (a.flags & kFlagEscape);
+                done = !again;
+            }
+            if (done) {
+                if (kBi && !zero && A.bistatic) zero = !rx_visible(a, A, r, nq, ovf);
+                emit(a, r, zero);
             }
         }
         push(a, again, r);
@@ -2025,6 +2082,18 @@ void launch_trace_m(const TraceArgs& a, int n_blocks, bool count_visits, int sta
     launch_trace_s<64, kMode>(a, n_blocks, count_visits, st);
 }
 
+template <int kMode>
+void launch_bistatic(const TraceArgs& a, int n_blocks, bool count_visits, cudaStream_t st)
+{
+    if (a.bounce == 1 && a.hit_list) {
+        if (count_visits) k_bounce<true, 64, kMode, true, true><<<n_blocks, kTraceThreads, 0, st>>>(a);
+        else k_bounce<false, 64, kMode, true, true><<<n_blocks, kTraceThreads, 0, st>>>(a);
+    } else {
+        if (count_visits) k_bounce<true, 64, kMode, true><<<n_blocks, kTraceThreads, 0, st>>>(a);
+        else k_bounce<false, 64, kMode, true><<<n_blocks, kTraceThreads, 0, st>>>(a);
+    }
+}
+
 cudaError_t launch_trace(const TraceArgs& a, int n_blocks, bool count_visits, int stack_depth, cudaStream_t st)
 {
     if (a.bistatic && a.bounce > 0) {
@@ -2033,11 +2102,9 @@ cudaError_t launch_trace(const TraceArgs& a, int n_blocks, bool count_visits, in
             if (count_visits) k_bounce<true, 64, 1, true><<<n_blocks, kTraceThreads, 0, st>>>(a);
             else k_bounce<false, 64, 1, true><<<n_blocks, kTraceThreads, 0, st>>>(a);
         } else if (a.octant) {
-            if (count_visits) k_bounce<true, 64, 3, true><<<n_blocks, kTraceThreads, 0, st>>>(a);
-            else k_bounce<false, 64, 3, true><<<n_blocks, kTraceThreads, 0, st>>>(a);
+            launch_bistatic<3>(a, n_blocks, count_visits, st);
         } else {
-            if (count_visits) k_bounce<true, 64, 0, true><<<n_blocks, kTraceThreads, 0, st>>>(a);
-            else k_bounce<false, 64, 0, true><<<n_blocks, kTraceThreads, 0, st>>>(a);
+            launch_bistatic<0>(a, n_blocks, count_visits, st);
         }
         return cudaGetLastError();
     }
