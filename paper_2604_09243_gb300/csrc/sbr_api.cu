@@ -288,6 +288,14 @@ AngleDev to_dev(const sbr_ray_grid& g, long long ray_off, int tw, const double* 
         d.bistatic = 0;
     }
     d.ray_off = ray_off;
+    for (int k = 0; k < 3; ++k) {
+        d.r_p0[k] = d.p0[k];
+        d.r_hs[k] = d.hhat[k] * d.ids;
+        d.r_vs[k] = d.vhat[k] * d.ids;
+    }
+    d.r_nu = d.nu;
+    d.r_nv = d.nv;
+    d.r_ids = d.ids;
     return d;
 }
 

@@ -40,7 +40,7 @@ __host__ __device__ inline int leaf_count(int ref) { return (int)((unsigned)ref 
 // leaves a decision open and it is taken again in FP64.
 
 // ---------------------------------------------------------------- per-aspect data
-struct AngleDev {            // 192 bytes
+struct __align__(16) AngleDev {  // 256 bytes
     float p0[3], du[3], dv[3], dir[3];  // FP32 ray grid: o(i, j) = (p0 + i du) + j dv
     float rhat[3], vhat[3], hhat[3];    // radar direction, V (theta_hat), H (phi_hat)
     float dA, eps;                      // tube area ds^2, origin offset after a hit
@@ -54,8 +54,16 @@ struct AngleDev {            // 192 bytes
     float rxdir[3];                     // -rxr in FP32 (= dir monostatic): the path term of the receiver
     float ids;                          // 1 / sqrt(dA) in FP32: grid cells per metre (rasterisation)
     float pad2[3];
+    // what the projection of a triangle onto a sparse grid reads, in three 16-byte words
+    float r_p0[3];
+    int r_nu;
+    float r_hs[3];                      // hhat ids
+    int r_nv;
+    float r_vs[3];                      // vhat ids
+    float r_ids;
+    float pad3[4];
 };
-static_assert(sizeof(AngleDev) == 192, "AngleDev layout");
+static_assert(sizeof(AngleDev) == 256, "AngleDev layout");
 
 // live ray between bounces (96 bytes, three 32-byte sectors)
 struct __align__(16) RayState {
@@ -181,7 +189,7 @@ struct TraceArgs {
                                   // [n_angles]: 1 if any aspect does
     const int* tri_pos;           // with vis: [n_tri] position in tris of each original triangle index
     unsigned* list_count;         // with vis: device count of the rasterised primary hits
-    int4* big;                    // with vis: triangles of more than 32 cells, (triangle, aspect, i0 | j0 << 16,
+    int4* big;                    // with vis: triangles of more than 512 (sparse grids: 16) cells, (triangle, aspect, i0 | j0 << 16,
                                   // (i1 - i0) | (j1 - j0) << 16), tested by warps after the per-thread pass
     unsigned* big_ctr;            // with vis: [2] entries appended, (unused)
     unsigned big_cap;             // with vis: capacity of big (an aspect whose entry does not fit traverses)
