@@ -681,6 +681,17 @@ cudaError_t ensure_octant_nodes(sbr_ctx* c, cudaStream_t st)
     return e;
 }
 
+// The rays that k_tail may take from bounce pass b on (0: it is not launched):
+// it looks at passes 2, 3, 4, 6, 8, 12, 16, ... (4 us for a look that finds too
+// many or none), and only under the default stack depth and the per-lane binary
+// traversals, whose stack it has.
+unsigned tail_rays(const sbr_tuning& t, int b, int n_blocks)
+{
+    if (t.stack_depth != 64 || t.bvh_width != 2 || t.packet) return 0u;
+    while (b > 4 && (b & 1) == 0) b >>= 1;
+    return b >= 2 && b <= 4 ? trace_tail_rays(n_blocks) : 0u;
+}
+
 // Enqueue the trace of the aspects [a0, a1) (one chunk): primary pass, popcount
 // scan of the hit masks, bounce passes, and the copy of the per-aspect record
 // offsets to *hro_out (pinned). Nothing waits for the GPU: the record buffer is
@@ -842,6 +853,8 @@ int trace_chunk(sbr_ctx* c, TraceRun& R, int64_t a0, int64_t a1, long long rec_b
                 ta.pool_cap = R.pool_cap;
                 ta.angle_shift = (int)a0;
             }
+            ta.tail_rays = ta.pool ? 0u : tail_rays(c->tune, b, R.n_blocks);
+            if (ta.tail_rays) ++R.n_launch;
             CK(pass(ta), "trace bounce");
             ta.hit_list = nullptr;  // only bounce pass 1 reads the list
         }
@@ -1149,6 +1162,7 @@ cudaError_t enqueue_plan(const sbr_ctx* c, BatchPlan& P, cudaStream_t st)
                 ta.q_in_count = q_count + b;
                 ta.q_out = qs[b & 1];
                 ta.q_out_count = q_count + b + 1;
+                ta.tail_rays = tail_rays(P.tune, b, n_blocks);
                 e = launch_trace(ta, n_blocks, P.count, P.tune.stack_depth, st);
                 ta.hit_list = nullptr;  // only bounce pass 1 reads the list
             }
@@ -1307,6 +1321,8 @@ int build_plan(sbr_ctx* c, BatchPlan& P)
     const int passes = (P.max_bounces == 1 && !escape) ? 1 : 1 + (escape ? P.max_bounces : P.max_bounces - 1);
     P.n_pass = (int64_t)nc * passes;
     P.n_launch = 0;
+    for (int b = 1; b < passes; ++b)
+        if (tail_rays(P.tune, b, c->n_sms * P.tune.blocks_per_sm)) P.n_launch += (int64_t)nc;
     for (size_t k = 0; k < nc; ++k)
         P.n_launch += passes + ((P.max_bounces == 1 && !escape) ? 1 : 0) + 3 + 1 + 2 + (P.items_bound[k] > 0 ? 1 : 0) + 1 +
                       (P.tune.raster ? 6 : (P.tune.silhouette ? 1 : 0));
@@ -1402,6 +1418,8 @@ int flush_pool(sbr_ctx* c, TraceRun& R, PoolRun& P, RayState* partner)
            "group rays");
         R.n_launch += 5;
         ta.q_order = P.order;
+        ta.tail_rays = tail_rays(c->tune, b, R.n_blocks);
+        if (ta.tail_rays) ++R.n_launch;
         CK(run_pass(c, R, ta), "trace pooled pass");
     }
     CK(cudaMemsetAsync(ctr, 0, sizeof(unsigned) * 2, c->stream), "memset pool count");

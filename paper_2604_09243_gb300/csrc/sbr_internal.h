@@ -147,6 +147,8 @@ cudaError_t bvh_build(const BvhBuild& b, cudaStream_t st);
 struct TraceArgs {
     const float4* nodes;          // binary nodes, or 4-wide nodes when wide = 1
     const float4* nodes2;         // binary nodes (visibility queries, whatever the traversal)
+    unsigned tail_rays;           // bounce pass: when at most this many rays are left, k_tail follows them to their
+                                  // end (0: never); the pass kernel then returns
     int wide;
     int packet;                   // 1: warp-cooperative traversal of the binary tree
     int bistatic;                 // 1: some aspect of the chunk has a bistatic receiver (visibility tests)
@@ -198,6 +200,8 @@ struct TraceArgs {
                                   // its state, and bounce pass 1 rebuilds the state from the list
 };
 int trace_blocks_per_sm();
+// rays that k_tail can take in a launch of n_blocks blocks
+unsigned trace_tail_rays(int n_blocks);
 // stack_depth: 32, 64 or 128 entries of the traversal stack (other values: 64;
 // the warp-cooperative traversal uses at most 64)
 cudaError_t launch_trace(const TraceArgs& a, int n_blocks, bool count_visits, int stack_depth, cudaStream_t st);
