@@ -235,7 +235,7 @@ cudaError_t launch_silhouette(const TraceArgs& a, int n_tri, unsigned* cover, cu
 // their exclusive scan and *a.q_out_count to their number: the primary pass
 // stores those rays at fixed queue slots and appends the traversing ones after
 // them.
-constexpr long long kRasterMaxCells = 1 << 14;
+constexpr long long kRasterMaxCells = 1 << 24;
 cudaError_t launch_raster(const TraceArgs& a, int n_tri, unsigned long long* vis, unsigned* full, bool count,
                           int n_blocks, void* scan_scratch, cudaStream_t st);
 

@@ -1277,7 +1277,8 @@ __device__ __forceinline__ float3 primary_origin(const AngleDev& A, int i, int j
 // (t bits << 32 | original index) by a 64-bit atomic minimum. t > 0, so the
 // key order is (t, index): the closest hit and the tie rule of the traversal,
 // whose t is <= FLT_MAX. A triangle spanning more than kRasterMaxCells cells
-// flags its aspect instead, whose primary rays then traverse the tree.
+// (or of an aperture row or column of more than 65,535 rays) flags its aspect
+// instead, whose primary rays then traverse the tree.
 
 // An aspect's ray grid held in registers for the cell loops: the loops' atomics
 // could alias the aspect table as far as the compiler knows, so fields read
@@ -1397,6 +1398,48 @@ constexpr int kRasterWarps = 8;    // warps of a k_raster block
 constexpr int kRasterFlat = 512;   // cells of a triangle the warps flatten; larger ones go to k_raster_big
 constexpr size_t kRasterSmem = sizeof(RasterItem) * 32 * kRasterWarps;
 
+// Appends the large triangles of the warp's lanes (want; cell ranges i0..i1,
+// j0..j1 of aspect ang) to the list of k_raster_big, cut into bands of rows of
+// about kRasterBand cells: a warp of k_raster_big takes a band at a time, so a
+// plate of millions of cells is shared by all of them (an aspect with a triangle
+// above 2^14 cells used to traverse all its rays: 4.0 of 41 ms for 23 aircraft
+// aspects at 7 to 12 GHz). The aspects of entries that find the list full
+// traverse. Every lane of the warp calls it.
+constexpr int kRasterBand = 4096;
+__device__ __forceinline__ void append_big(const TraceArgs& a, unsigned* full, bool want, int t, int ang, int i0, int i1,
+                                           int j0, int j1)
+{
+    if (!__any_sync(kFull, want)) return;
+    const int lane = threadIdx.x & 31;
+    const int rows = want ? max(1, kRasterBand / (i1 - i0 + 1)) : 1;
+    const unsigned n = want ? (unsigned)((j1 - j0 + rows) / rows) : 0u;  // bands
+    unsigned incl = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += y;
+    }
+    unsigned base = 0xFFFFFFFFu;
+    // (a full list is left alone, so that its counter cannot wrap)
+    if (lane == 31 && __ldcg(a.big_ctr) < a.big_cap) base = atomicAdd(a.big_ctr, incl);
+    base = __shfl_sync(kFull, base, 31);
+    if (!want) return;
+    bool fit = base != 0xFFFFFFFFu;
+    if (fit) {
+        const unsigned slot = base + incl - n;
+        for (unsigned k = 0; k < n; ++k) {
+            const int jb = j0 + (int)k * rows;
+            if (slot + k < a.big_cap)
+                a.big[slot + k] = make_int4(t, ang, i0 | (jb << 16), (i1 - i0) | ((min(j1, jb + rows - 1) - jb) << 16));
+            else fit = false;
+        }
+    }
+    if (!fit) {
+        atomicOr(full + ang, 1u);
+        atomicOr(full + a.n_angles, 1u);  // some aspect of the chunk traverses
+    }
+}
+
 // Items q = aspect * n_tri + triangle, one per lane in grid-stride order
 // (aspect-major: neighbouring lanes take neighbouring triangles of one
 // aspect). Each lane projects its triangle and, for a range of at most
@@ -1438,7 +1481,7 @@ __global__ void __launch_bounds__(256, 4) k_raster(const TraceArgs a, int n_tri,
                     atomicOr(full + a.n_angles, 1u);  // some aspect of the chunk traverses
                 } else if (ncell > kRasterFlat) {
                     want_big = true;
-                    rng = make_int4(t, ang, i0 | (j0 << 16), (i1 - i0) | ((j1 - j0) << 16));
+                    rng = make_int4(i0, i1, j0, j1);
                 } else {
                     // each group of constants goes to shared memory as soon as it is formed
                     RasterItem& it = my[lane];
@@ -1486,20 +1529,7 @@ __global__ void __launch_bounds__(256, 4) k_raster(const TraceArgs a, int n_tri,
                 }
             }
         }
-        const unsigned m = __ballot_sync(kFull, want_big);
-        if (m) {
-            unsigned slot = 0;
-            if (lane == __ffs(m) - 1) slot = atomicAdd(a.big_ctr, (unsigned)__popc(m));
-            slot = __shfl_sync(kFull, slot, __ffs(m) - 1) + __popc(m & ((1u << lane) - 1u));
-            if (want_big) {
-                if (slot < a.big_cap) {
-                    a.big[slot] = rng;
-                } else {  // no room: this aspect's primary rays traverse
-                    atomicOr(full + rng.y, 1u);
-                    atomicOr(full + a.n_angles, 1u);
-                }
-            }
-        }
+        append_big(a, full, want_big, t, ang, rng.x, rng.y, rng.z, rng.w);
         // inclusive scan of the cell counts: off[k] = first pair of lane k's triangle
         int incl = nc;
 #pragma unroll
@@ -1752,20 +1782,7 @@ __global__ void __launch_bounds__(256, 3) k_raster_sparse(const TraceArgs a, int
                     }
                 }
             }
-            const unsigned m = __ballot_sync(kFull, want_big);
-            if (m) {
-                unsigned slot = 0;
-                if (lane == __ffs(m) - 1) slot = atomicAdd(a.big_ctr, (unsigned)__popc(m));
-                slot = __shfl_sync(kFull, slot, __ffs(m) - 1) + __popc(m & ((1u << lane) - 1u));
-                if (want_big) {
-                    if (slot < a.big_cap) {
-                        a.big[slot] = make_int4(t, ang, i0 | (j0 << 16), (i1 - i0) | ((j1 - j0) << 16));
-                    } else {  // no room: this aspect's primary rays traverse
-                        atomicOr(full + ang, 1u);
-                        atomicOr(full + a.n_angles, 1u);
-                    }
-                }
-            }
+            append_big(a, full, want_big, t, ang, i0, i1, j0, j1);
             // the triangle's cells row by row, one of each lane's at a time
             int ci = i0, cj = j0;
             for (unsigned mc = __ballot_sync(kFull, n_cell > 0); mc; mc = __ballot_sync(kFull, n_cell > 0)) {
