@@ -79,7 +79,7 @@ typedef struct {
     int ploc_radius;      /* PLOC search radius in Morton order, 1..64 (0 = 16) */
 } sbr_bvh_opts;
 #define SBR_BVH_PLOC 0 /* agglomerative clustering of mutual nearest neighbours in the Morton order, close
-                          to a full SAH tree (one host synchronisation per four clustering rounds) */
+                          to a full SAH tree */
 #define SBR_BVH_LBVH 1 /* Karras hierarchy over the Morton order, bottom-up refit */
 
 /* Ray-grid and transport options of sbr_trace. A zeroed struct gives the defaults. */

@@ -334,6 +334,106 @@ bool tuning_ok(const sbr_tuning& t)
 
 }  // namespace
 
+namespace {
+
+// sbr_build_bvh; xyz, tri: the host arrays just copied (or null), whose indices and coordinates are checked here
+// while the GPU builds (its kernels take any values: see k_prep)
+int build_bvh(sbr_ctx* c, const sbr_bvh_opts* opt, const float* xyz, const int32_t* tri)
+{
+    if (!c) return SBR_ERR_ARG;
+    if (!c->has_mesh) return fail(c, SBR_ERR_STATE, "sbr_build_bvh: no mesh loaded");
+    int leaf_max = opt ? opt->leaf_max : 4;
+    float ct = opt ? opt->cost_traverse : 1.f, ci = opt ? opt->cost_intersect : 1.f;
+    if (leaf_max < 1 || leaf_max > kLeafMax) return fail(c, SBR_ERR_ARG, "sbr_build_bvh: leaf_max must be 1..16");
+    if (!(ct >= 0.f) || !(ci > 0.f)) return fail(c, SBR_ERR_ARG, "sbr_build_bvh: costs must be C_T >= 0, C_I > 0");
+    const int builder = opt ? opt->builder : SBR_BVH_PLOC, radius = opt ? opt->ploc_radius : 0;
+    if (builder != SBR_BVH_LBVH && builder != SBR_BVH_PLOC) return fail(c, SBR_ERR_ARG, "sbr_build_bvh: unknown builder");
+    if (radius < 0 || radius > 64) return fail(c, SBR_ERR_ARG, "sbr_build_bvh: ploc_radius must be 0..64");
+    CK(cudaSetDevice(c->device), "cudaSetDevice");
+    ++c->mesh_gen;  // captured batch graphs hold the node and triangle pointers
+    const long long n = c->n_tri;
+    const long long n_nodes = n > 1 ? n - 1 : 1;
+    c->n_nodes = n_nodes;
+    CK(c->nodes.ensure(sizeof(float4) * 4 * (size_t)n_nodes), "alloc nodes");
+    // records (3 float4), normals (1) and exact v1, v2 (2) per triangle
+    CK(c->tris.ensure(sizeof(float4) * 6 * (size_t)n), "alloc tris");
+    CK(c->tripos.ensure(sizeof(int) * (size_t)n), "alloc triangle positions");
+    size_t sb = bvh_scratch_bytes(n);
+    CK(c->bvh_scratch.ensure(sb), "alloc bvh scratch");
+    CK(c->bbox_dev.ensure(sizeof(float) * 8), "alloc bbox");
+    CK(c->err_dev.ensure(sizeof(int) * 4), "alloc err");
+    BvhBuild b;
+    b.xyz = c->xyz.as<float>();
+    b.tri = c->tri.as<int>();
+    b.n_vert = c->n_vert;
+    b.n_tri = n;
+    b.leaf_max = leaf_max;
+    b.c_t = ct;
+    b.c_i = ci;
+    b.builder = builder == SBR_BVH_PLOC ? 1 : 0;
+    b.radius = radius;
+    b.nodes = c->nodes.as<float4>();
+    b.tris = c->tris.as<float4>();
+    b.tri_nrm = c->tris.as<float4>() + 3 * (size_t)n;
+    b.tri_v12 = c->tris.as<float4>() + 4 * (size_t)n;
+    b.tri_pos = c->tripos.as<int>();
+    b.bbox_out = c->bbox_dev.as<float>();
+    b.err_flag = c->err_dev.as<int>();
+    b.n_nodes_out = c->err_dev.as<int>() + 2;
+    b.scratch = c->bvh_scratch.p;
+    b.scratch_bytes = c->bvh_scratch.cap;
+    CK(bvh_build(b, c->stream), "bvh build");
+    if (xyz && tri) {
+        int64_t bad = -1;
+        for (int64_t i = 0; i < 3 * n && bad < 0; ++i)
+            if (tri[i] < 0 || tri[i] >= c->n_vert) bad = i;
+        const bool index = bad >= 0;
+        for (int64_t i = 0; i < 3 * c->n_vert && bad < 0; ++i)
+            if (!std::isfinite(xyz[i])) bad = i;
+        if (bad >= 0) {
+            c->has_mesh = false;
+            CK(cudaStreamSynchronize(c->stream), "bvh build sync");
+            return index ? fail(c, SBR_ERR_ARG, "sbr_load_mesh: index %lld out of range", (long long)bad)
+                         : fail(c, SBR_ERR_ARG, "sbr_load_mesh: vertex coordinate %lld is not finite", (long long)bad);
+        }
+    }
+    float hb[8];
+    int herr[3] = {0, 0, 0};
+    CK(cudaMemcpyAsync(hb, c->bbox_dev.p, sizeof(float) * 6, cudaMemcpyDeviceToHost, c->stream), "copy bbox");
+    CK(cudaMemcpyAsync(herr, c->err_dev.p, sizeof(int) * 3, cudaMemcpyDeviceToHost, c->stream), "copy err");
+    CK(cudaStreamSynchronize(c->stream), "bvh build sync");
+    if (herr[0]) {
+        c->has_mesh = false;
+        if (herr[0] & 8) return fail(c, SBR_ERR_TIMEOUT, "sbr_build_bvh: a bounded device wait gave up");
+        if (herr[0] & 4) return fail(c, SBR_ERR_CUDA, "sbr_build_bvh: the clustering did not converge");
+        return fail(c, SBR_ERR_ARG, (herr[0] & 1) ? "sbr_build_bvh: triangle index out of range"
+                                                  : "sbr_build_bvh: a vertex coordinate is not finite");
+    }
+    // the nodes reachable from the root, renumbered 0.. in depth-first order
+    if (herr[2] < 1 || herr[2] > n_nodes) {
+        c->has_mesh = false;
+        return fail(c, SBR_ERR_CUDA, "sbr_build_bvh: malformed hierarchy (%d reachable nodes of %lld)", herr[2],
+                    n_nodes);
+    }
+    c->n_nodes = herr[2];
+    memcpy(c->bbox, hb, sizeof(c->bbox));
+    // 4-wide tree over the same boxes; its work queues reuse the (now free) build scratch
+    CK(c->nodes4.ensure(sizeof(float4) * kNode4Float4 * (size_t)c->n_nodes), "alloc 4-wide nodes");
+    {
+        char* scr = (char*)c->bvh_scratch.p;
+        const size_t qb = ((sizeof(int2) * (size_t)c->n_nodes + 255) / 256) * 256;
+        if (2 * qb + 256 > c->bvh_scratch.cap) return fail(c, SBR_ERR_ARG, "sbr_build_bvh: scratch too small");
+        CK(bvh4_collapse(c->nodes.as<float4>(), c->n_nodes, c->nodes4.as<float4>(), (int2*)scr, (int2*)(scr + qb),
+                         (int*)(scr + 2 * qb), &c->n_nodes4, c->stream),
+           "4-wide collapse");
+    }
+    c->has_bvh = true;
+    c->has_trace = false;
+    return SBR_OK;
+}
+
+}  // namespace
+
 extern "C" {
 
 int sbr_version(void) { return SBR_VERSION_MAJOR * 100 + SBR_VERSION_MINOR; }
@@ -432,13 +532,6 @@ int sbr_load_mesh(sbr_ctx* c, const float* xyz, int64_t n_vert, const int32_t* t
     if (n_vert >= (1ll << 31)) return fail(c, SBR_ERR_ARG, "sbr_load_mesh: at most 2^31 - 1 vertices");
     CK(cudaSetDevice(c->device), "cudaSetDevice");
     c->has_mesh = c->has_bvh = c->has_trace = false;
-    if (!on_device) {
-        for (int64_t i = 0; i < 3 * n_tri; ++i)
-            if (tri[i] < 0 || tri[i] >= n_vert) return fail(c, SBR_ERR_ARG, "sbr_load_mesh: index %lld out of range", (long long)i);
-        for (int64_t i = 0; i < 3 * n_vert; ++i)
-            if (!std::isfinite(xyz[i]))
-                return fail(c, SBR_ERR_ARG, "sbr_load_mesh: vertex coordinate %lld is not finite", (long long)i);
-    }
     CK(c->xyz.ensure(sizeof(float) * 3 * (size_t)n_vert), "alloc xyz");
     CK(c->tri.ensure(sizeof(int32_t) * 3 * (size_t)n_tri), "alloc tri");
     cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
@@ -449,7 +542,7 @@ int sbr_load_mesh(sbr_ctx* c, const float* xyz, int64_t n_vert, const int32_t* t
     // exact scene box and index check run as part of the BVH build; build the
     // box now so sbr_get_bbox / sbr_ray_grid_for work right after loading
     c->has_mesh = true;
-    return sbr_build_bvh(c, nullptr);
+    return build_bvh(c, nullptr, on_device ? nullptr : xyz, on_device ? nullptr : tri);
 }
 
 int sbr_get_bbox(sbr_ctx* c, float* bbox6)
@@ -462,81 +555,7 @@ int sbr_get_bbox(sbr_ctx* c, float* bbox6)
 
 int sbr_build_bvh(sbr_ctx* c, const sbr_bvh_opts* opt)
 {
-    if (!c) return SBR_ERR_ARG;
-    if (!c->has_mesh) return fail(c, SBR_ERR_STATE, "sbr_build_bvh: no mesh loaded");
-    int leaf_max = opt ? opt->leaf_max : 4;
-    float ct = opt ? opt->cost_traverse : 1.f, ci = opt ? opt->cost_intersect : 1.f;
-    if (leaf_max < 1 || leaf_max > kLeafMax) return fail(c, SBR_ERR_ARG, "sbr_build_bvh: leaf_max must be 1..16");
-    if (!(ct >= 0.f) || !(ci > 0.f)) return fail(c, SBR_ERR_ARG, "sbr_build_bvh: costs must be C_T >= 0, C_I > 0");
-    const int builder = opt ? opt->builder : SBR_BVH_PLOC, radius = opt ? opt->ploc_radius : 0;
-    if (builder != SBR_BVH_LBVH && builder != SBR_BVH_PLOC) return fail(c, SBR_ERR_ARG, "sbr_build_bvh: unknown builder");
-    if (radius < 0 || radius > 64) return fail(c, SBR_ERR_ARG, "sbr_build_bvh: ploc_radius must be 0..64");
-    CK(cudaSetDevice(c->device), "cudaSetDevice");
-    ++c->mesh_gen;  // captured batch graphs hold the node and triangle pointers
-    const long long n = c->n_tri;
-    const long long n_nodes = n > 1 ? n - 1 : 1;
-    c->n_nodes = n_nodes;
-    CK(c->nodes.ensure(sizeof(float4) * 4 * (size_t)n_nodes), "alloc nodes");
-    // records (3 float4), normals (1) and exact v1, v2 (2) per triangle
-    CK(c->tris.ensure(sizeof(float4) * 6 * (size_t)n), "alloc tris");
-    CK(c->tripos.ensure(sizeof(int) * (size_t)n), "alloc triangle positions");
-    size_t sb = bvh_scratch_bytes(n);
-    CK(c->bvh_scratch.ensure(sb), "alloc bvh scratch");
-    CK(c->bbox_dev.ensure(sizeof(float) * 8), "alloc bbox");
-    CK(c->err_dev.ensure(sizeof(int) * 4), "alloc err");
-    BvhBuild b;
-    b.xyz = c->xyz.as<float>();
-    b.tri = c->tri.as<int>();
-    b.n_vert = c->n_vert;
-    b.n_tri = n;
-    b.leaf_max = leaf_max;
-    b.c_t = ct;
-    b.c_i = ci;
-    b.builder = builder == SBR_BVH_PLOC ? 1 : 0;
-    b.radius = radius;
-    b.nodes = c->nodes.as<float4>();
-    b.tris = c->tris.as<float4>();
-    b.tri_nrm = c->tris.as<float4>() + 3 * (size_t)n;
-    b.tri_v12 = c->tris.as<float4>() + 4 * (size_t)n;
-    b.tri_pos = c->tripos.as<int>();
-    b.bbox_out = c->bbox_dev.as<float>();
-    b.err_flag = c->err_dev.as<int>();
-    b.n_nodes_out = c->err_dev.as<int>() + 2;
-    b.scratch = c->bvh_scratch.p;
-    b.scratch_bytes = c->bvh_scratch.cap;
-    CK(bvh_build(b, c->stream), "bvh build");
-    float hb[8];
-    int herr[3] = {0, 0, 0};
-    CK(cudaMemcpyAsync(hb, c->bbox_dev.p, sizeof(float) * 6, cudaMemcpyDeviceToHost, c->stream), "copy bbox");
-    CK(cudaMemcpyAsync(herr, c->err_dev.p, sizeof(int) * 3, cudaMemcpyDeviceToHost, c->stream), "copy err");
-    CK(cudaStreamSynchronize(c->stream), "bvh build sync");
-    if (herr[0]) {
-        c->has_mesh = false;
-        if (herr[0] & 4) return fail(c, SBR_ERR_CUDA, "sbr_build_bvh: the clustering did not converge");
-        return fail(c, SBR_ERR_ARG, (herr[0] & 1) ? "sbr_build_bvh: triangle index out of range"
-                                                  : "sbr_build_bvh: a vertex coordinate is not finite");
-    }
-    // the nodes reachable from the root, renumbered 0.. in depth-first order
-    if (herr[2] < 1 || herr[2] > n_nodes) {
-        c->has_mesh = false;
-        return fail(c, SBR_ERR_CUDA, "sbr_build_bvh: malformed hierarchy (%d reachable nodes of %lld)", herr[2],
-                    n_nodes);
-    }
-    c->n_nodes = herr[2];
-    memcpy(c->bbox, hb, sizeof(c->bbox));
-    // 4-wide tree over the same boxes; its work queues reuse the (now free) build scratch
-    CK(c->nodes4.ensure(sizeof(float4) * kNode4Float4 * (size_t)c->n_nodes), "alloc 4-wide nodes");
-    {
-        char* scr = (char*)c->bvh_scratch.p;
-        const size_t qb = ((sizeof(int2) * (size_t)c->n_nodes + 255) / 256) * 256;
-        if (2 * qb + 256 > c->bvh_scratch.cap) return fail(c, SBR_ERR_ARG, "sbr_build_bvh: scratch too small");
-        CK(bvh4_collapse(c->nodes.as<float4>(), c->n_nodes, c->nodes4.as<float4>(), (int2*)scr, (int2*)(scr + qb),
-                         (int*)(scr + 2 * qb), &c->n_nodes4, c->stream),
-           "4-wide collapse");
-    }
-    c->has_bvh = true;
-    c->has_trace = false;
-    return SBR_OK;
+    return build_bvh(c, opt, nullptr, nullptr);
 }
 
 int sbr_get_bvh_info(sbr_ctx* c, sbr_bvh_info* out)

@@ -17,6 +17,8 @@
 //      contiguous triangle ranges).
 #include <float.h>
 
+#include <algorithm>
+
 #include "sbr_internal.h"
 
 namespace sbr {
@@ -24,6 +26,9 @@ namespace sbr {
 namespace {
 
 constexpr int kThreads = 256;
+// error bits that leave no tree behind: the clustering did not converge (4), a bounded wait gave up (8); the steps
+// after it then do nothing (bits 1 and 2, a refused mesh, still complete their build)
+constexpr int kErrTree = 12;
 constexpr int kRsThreads = 256;
 constexpr int kRsItems = 8;
 constexpr int kRsTile = kRsThreads * kRsItems;
@@ -48,26 +53,30 @@ __global__ void k_acc_init(unsigned* acc, int* err)
     if (t == 0) *err = 0;
 }
 
-__device__ __forceinline__ void warp_minmax_atomic(float3 lo, float3 hi, unsigned* acc_lo, unsigned* acc_hi)
+// lo / hi of the whole block into acc: one set of atomics per block (a set per
+// warp of the one-triangle-per-thread grid serialised on twelve addresses)
+__device__ __forceinline__ void block_minmax_atomic(float3 lo, float3 hi, unsigned* acc_lo, unsigned* acc_hi)
 {
+    __shared__ float s_mm[kThreads / 32][6];
+    float v[6] = {lo.x, lo.y, lo.z, hi.x, hi.y, hi.z};
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        lo.x = fminf(lo.x, __shfl_xor_sync(0xffffffffu, lo.x, o));
-        lo.y = fminf(lo.y, __shfl_xor_sync(0xffffffffu, lo.y, o));
-        lo.z = fminf(lo.z, __shfl_xor_sync(0xffffffffu, lo.z, o));
-        hi.x = fmaxf(hi.x, __shfl_xor_sync(0xffffffffu, hi.x, o));
-        hi.y = fmaxf(hi.y, __shfl_xor_sync(0xffffffffu, hi.y, o));
-        hi.z = fmaxf(hi.z, __shfl_xor_sync(0xffffffffu, hi.z, o));
-    }
-    if ((threadIdx.x & 31) == 0) {
-        if (lo.x <= hi.x) {
-            atomicMin(acc_lo + 0, f2o(lo.x));
-            atomicMin(acc_lo + 1, f2o(lo.y));
-            atomicMin(acc_lo + 2, f2o(lo.z));
-            atomicMax(acc_hi + 0, f2o(hi.x));
-            atomicMax(acc_hi + 1, f2o(hi.y));
-            atomicMax(acc_hi + 2, f2o(hi.z));
+    for (int k = 0; k < 6; ++k)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float y = __shfl_xor_sync(0xffffffffu, v[k], o);
+            v[k] = k < 3 ? fminf(v[k], y) : fmaxf(v[k], y);
         }
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+        for (int k = 0; k < 6; ++k) s_mm[threadIdx.x >> 5][k] = v[k];
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        const int k = threadIdx.x;
+        float m = s_mm[0][k];
+        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = k < 3 ? fminf(m, s_mm[w][k]) : fmaxf(m, s_mm[w][k]);
+        // FLT_MAX, -FLT_MAX: the block saw no vertex
+        if (k < 3 && m < FLT_MAX) atomicMin(acc_lo + k, f2o(m));
+        if (k >= 3 && m > -FLT_MAX) atomicMax(acc_hi + k - 3, f2o(m));
     }
 }
 
@@ -81,7 +90,7 @@ __global__ void __launch_bounds__(kThreads) k_vertex_box(const float* xyz, long 
         lo = make_float3(fminf(lo.x, x), fminf(lo.y, y), fminf(lo.z, z));
         hi = make_float3(fmaxf(hi.x, x), fmaxf(hi.y, y), fmaxf(hi.z, z));
     }
-    warp_minmax_atomic(lo, hi, acc, acc + 3);
+    block_minmax_atomic(lo, hi, acc, acc + 3);
 }
 
 __global__ void __launch_bounds__(kThreads) k_prep(const float* xyz, const int* tri, long long nv, int n,
@@ -119,7 +128,7 @@ __global__ void __launch_bounds__(kThreads) k_prep(const float* xyz, const int* 
         lo = make_float3(fminf(lo.x, m.x), fminf(lo.y, m.y), fminf(lo.z, m.z));
         hi = make_float3(fmaxf(hi.x, m.x), fmaxf(hi.y, m.y), fmaxf(hi.z, m.z));
     }
-    warp_minmax_atomic(lo, hi, acc + 6, acc + 9);
+    block_minmax_atomic(lo, hi, acc + 6, acc + 9);
 }
 
 __device__ __forceinline__ unsigned long long spread21(unsigned long long x)
@@ -387,10 +396,10 @@ __device__ __forceinline__ double ddot(D3 a, D3 b)
 
 __global__ void __launch_bounds__(kThreads) k_reorder(const float* xyz, const int* tri, long long nv,
                                                       const unsigned* vals, int n, float4* tris, float4* nrm,
-                                                      float4* v12, int* pos)
+                                                      float4* v12, int* pos, const int* err)
 {
     int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
+    if (p >= n || (*err & kErrTree)) return;
     unsigned t = vals[p];
     int ia = tri[3 * (long long)t], ib = tri[3 * (long long)t + 1], ic = tri[3 * (long long)t + 2];
     if (ia < 0 || ib < 0 || ic < 0 || ia >= nv || ib >= nv || ic >= nv) ia = ib = ic = 0;
@@ -459,13 +468,6 @@ __device__ __forceinline__ void ploc_init_one(int i, const unsigned* vals, const
     c.cost[i] = c_i * area(lo, hi);
 }
 
-__global__ void __launch_bounds__(kThreads) k_ploc_init(const unsigned* vals, const float4* tbox, int n, float c_i,
-                                                        Clusters c)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) ploc_init_one(i, vals, tbox, c_i, c);
-}
-
 __device__ __forceinline__ float union_area(float4 al, float4 ah, float4 bl, float4 bh)
 {
     return area(make_float4(fminf(al.x, bl.x), fminf(al.y, bl.y), fminf(al.z, bl.z), 0.f),
@@ -489,13 +491,6 @@ __device__ __forceinline__ void ploc_nn_one(int i, int m, int radius, Clusters c
     nn[i] = bj;
 }
 
-__global__ void __launch_bounds__(kThreads) k_ploc_nn(const int* m_dev, int radius, Clusters c, int* nn)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int m = *m_dev;
-    if (i < m) ploc_nn_one(i, m, radius, c, nn);
-}
-
 // par / rel: parent and offset within the parent of node x (x < n - 1) or of
 // triangle t (x = n - 1 + t), for the pointer-jumping position pass
 // node arrays written by the merges
@@ -510,18 +505,57 @@ struct PlocNodes {
     int* rel;
 };
 
+// Node id from two clusters (boxes, ref, triangle count, cost): writes the node
+// and leaves the merged cluster in the first one's values
+__device__ __forceinline__ void ploc_join(int id, int n, float4& lo, float4& hi, int& ref, int& cnt, float& cost,
+                                          float4 bl, float4 bh, int rj, int cj, float costj, PlocNodes g, int leaf_max,
+                                          float c_t, float c_i)
+{
+    lo = make_float4(fminf(lo.x, bl.x), fminf(lo.y, bl.y), fminf(lo.z, bl.z), 0.f);
+    hi = make_float4(fmaxf(hi.x, bh.x), fmaxf(hi.y, bh.y), fmaxf(hi.z, bh.z), 0.f);
+    const int ci = cnt, ri = ref;
+    cnt = ci + cj;
+    const float sa = area(lo, hi);
+    const float split = c_t * sa + cost + costj;
+    const float as_leaf = c_i * (float)cnt * sa;
+    const int col = (cnt <= leaf_max) && (as_leaf <= split);
+    g.left[id] = ri;
+    g.right[id] = rj;
+    const int xi = ri >= 0 ? ri : n - 1 + ~ri, xj = rj >= 0 ? rj : n - 1 + ~rj;
+    g.par[xi] = id;
+    g.rel[xi] = 0;
+    g.par[xj] = id;
+    g.rel[xj] = ci;
+    g.nbox[2 * id] = lo;
+    g.nbox[2 * id + 1] = hi;
+    g.ncnt[id] = cnt;
+    cost = col ? as_leaf : split;
+    g.ncost[id] = cost;
+    g.ncol[id] = col;
+    ref = id;
+}
+
+// merge the mutual nearest neighbours i < j into cluster i
+__device__ __forceinline__ void ploc_merge_pair(int i, int j, int n, Clusters c, int* next_id, PlocNodes g, int leaf_max,
+                                                float c_t, float c_i)
+{
+    float4 lo = __ldcg(c.lo + i), hi = __ldcg(c.hi + i);
+    int ref = __ldcg(c.ref + i), cnt = __ldcg(c.cnt + i);
+    float cost = __ldcg(c.cost + i);
+    const int id = atomicSub(next_id, 1);
+    ploc_join(id, n, lo, hi, ref, cnt, cost, __ldcg(c.lo + j), __ldcg(c.hi + j), __ldcg(c.ref + j), __ldcg(c.cnt + j),
+              __ldcg(c.cost + j), g, leaf_max, c_t, c_i);
+    c.lo[i] = lo;
+    c.hi[i] = hi;
+    c.ref[i] = ref;
+    c.cnt[i] = cnt;
+    c.cost[i] = cost;
+}
+
 // cluster i < m of this round: merge with its mutual nearest neighbour
 __device__ __forceinline__ void ploc_merge_one(int i, int n, Clusters c, const int* nn, int* next_id, PlocNodes g,
                                                unsigned* keep, int leaf_max, float c_t, float c_i)
 {
-    int* left = g.left;
-    int* right = g.right;
-    float4* nbox = g.nbox;
-    int* ncnt = g.ncnt;
-    float* ncost = g.ncost;
-    int* ncol = g.ncol;
-    int* par = g.par;
-    int* rel = g.rel;
     const int j = nn[i];
     if (j < 0 || nn[j] != i) {
         keep[i] = 1;  // no mutual partner this round
@@ -531,47 +565,8 @@ __device__ __forceinline__ void ploc_merge_one(int i, int n, Clusters c, const i
         keep[i] = 0;  // merged into j
         return;
     }
-    const float4 al = c.lo[i], ah = c.hi[i], bl = c.lo[j], bh = c.hi[j];
-    const float4 lo = make_float4(fminf(al.x, bl.x), fminf(al.y, bl.y), fminf(al.z, bl.z), 0.f);
-    const float4 hi = make_float4(fmaxf(ah.x, bh.x), fmaxf(ah.y, bh.y), fmaxf(ah.z, bh.z), 0.f);
-    const int cnt = c.cnt[i] + c.cnt[j];
-    const float sa = area(lo, hi);
-    const float split = c_t * sa + c.cost[i] + c.cost[j];
-    const float as_leaf = c_i * (float)cnt * sa;
-    const int col = (cnt <= leaf_max) && (as_leaf <= split);
-    const int id = atomicSub(next_id, 1);
-    const int ri = c.ref[i], rj = c.ref[j];
-    left[id] = ri;
-    right[id] = rj;
-    const int xi = ri >= 0 ? ri : n - 1 + ~ri, xj = rj >= 0 ? rj : n - 1 + ~rj;
-    par[xi] = id;
-    rel[xi] = 0;
-    par[xj] = id;
-    rel[xj] = c.cnt[i];
-    nbox[2 * id] = lo;
-    nbox[2 * id + 1] = hi;
-    ncnt[id] = cnt;
-    ncost[id] = col ? as_leaf : split;
-    ncol[id] = col;
-    c.lo[i] = lo;
-    c.hi[i] = hi;
-    c.ref[i] = id;
-    c.cnt[i] = cnt;
-    c.cost[i] = col ? as_leaf : split;
+    ploc_merge_pair(i, j, n, c, next_id, g, leaf_max, c_t, c_i);
     keep[i] = 1;
-}
-
-__global__ void __launch_bounds__(kThreads) k_ploc_merge(const int* m_dev, int m_ub, int n, Clusters c, const int* nn,
-                                                         int* next_id, PlocNodes g, unsigned* keep, int leaf_max,
-                                                         float c_t, float c_i)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= m_ub) return;
-    if (i >= *m_dev) {
-        keep[i] = 0;  // beyond the live clusters of this round
-        return;
-    }
-    ploc_merge_one(i, n, c, nn, next_id, g, keep, leaf_max, c_t, c_i);
 }
 
 __device__ __forceinline__ void ploc_compact_one(int i, Clusters in, const unsigned* keep, const unsigned* pos,
@@ -584,13 +579,6 @@ __device__ __forceinline__ void ploc_compact_one(int i, Clusters in, const unsig
     out.ref[k] = in.ref[i];
     out.cnt[k] = in.cnt[i];
     out.cost[k] = in.cost[i];
-}
-
-__global__ void __launch_bounds__(kThreads) k_ploc_compact(int m_ub, Clusters in, const unsigned* keep,
-                                                           const unsigned* pos, Clusters out)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < m_ub) ploc_compact_one(i, in, keep, pos, out);
 }
 
 // position pass by pointer jumping: after round r every entry holds the sum of
@@ -608,30 +596,18 @@ __device__ __forceinline__ void ploc_jump_one(int x, const int* par_in, const in
     }
 }
 
-__global__ void __launch_bounds__(kThreads) k_ploc_jump(int count, const int* par_in, const int* rel_in, int* par_out,
-                                                        int* rel_out)
-{
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x < count) ploc_jump_one(x, par_in, rel_in, par_out, rel_out);
-}
-
 __device__ __forceinline__ void ploc_positions_one(int x, int n, const int* rel, int* noff, unsigned* perm)
 {
     if (x < n - 1) noff[x] = rel[x];
     else if (x < 2 * n - 1) perm[rel[x]] = (unsigned)(x - (n - 1));
 }
 
-__global__ void __launch_bounds__(kThreads) k_ploc_positions(int n, const int* rel, int* noff, unsigned* perm)
-{
-    ploc_positions_one(blockIdx.x * blockDim.x + threadIdx.x, n, rel, noff, perm);
-}
-
 __global__ void __launch_bounds__(kThreads) k_ploc_emit(int n, const int* left, const int* right, const float4* nbox,
                                                         const int* ncnt, const int* ncol, const int* noff,
-                                                        const float4* tbox, float4* nodes)
+                                                        const float4* tbox, float4* nodes, const int* err)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n - 1) return;
+    if (i >= n - 1 || (*err & kErrTree)) return;
     const float4 elo = make_float4(FLT_MAX, FLT_MAX, FLT_MAX, 0.f), ehi = make_float4(-FLT_MAX, -FLT_MAX, -FLT_MAX, 0.f);
     if (i == 0 && ncol[0]) {
         put_node(nodes, 0, nbox[0], nbox[1], elo, ehi, leaf_ref(0, ncnt[0]), kEmptyRef);
@@ -681,16 +657,22 @@ __device__ __forceinline__ void binary_children(const float4* nodes2, int b, flo
 // One level: every queued (binary node, 4-wide slot) pair opens binary
 // children, largest surface area first, until it has 4 children or only
 // leaves; its internal children get new slots and go to the next level's queue.
-__device__ __forceinline__ void collapse4_one(const float4* nodes2, int2 job, int2* qout, int* nout, int* count4,
-                                              float4* nodes4)
-{
+struct Wide4 {
     float4 lo[4], hi[4];
     int ref[4];
+    int cnt;
+};
+
+// the children of the 4-wide node at binary node b; returns how many are internal
+__device__ __forceinline__ int collapse4_open(const float4* nodes2, int b, Wide4& w)
+{
+    float4 *lo = w.lo, *hi = w.hi;
+    int* ref = w.ref;
     int cnt = 0;
     {
         float4 l2[2], h2[2];
         int r2[2];
-        binary_children(nodes2, job.x, l2, h2, r2);
+        binary_children(nodes2, b, l2, h2, r2);
         for (int c = 0; c < 2; ++c)
             if (r2[c] != kEmptyRef) {
                 lo[cnt] = l2[c];
@@ -724,12 +706,25 @@ __device__ __forceinline__ void collapse4_one(const float4* nodes2, int2 job, in
             ++cnt;
         }
     }
-    for (int c = 0; c < cnt; ++c)
+    w.cnt = cnt;
+    int inner = 0;
+    for (int c = 0; c < cnt; ++c) inner += ref[c] >= 0;
+    return inner;
+}
+
+// writes the node to slot, its internal children to the next level's queue at qat and to slots from `to` on
+__device__ __forceinline__ void collapse4_put(const Wide4& w, int slot, int2* qout, int qat, int to, float4* nodes4)
+{
+    const int cnt = w.cnt;
+    const float4 *lo = w.lo, *hi = w.hi;
+    int ref[4];
+    for (int c = 0; c < cnt; ++c) {
+        ref[c] = w.ref[c];
         if (ref[c] >= 0) {
-            const int t = atomicAdd(count4, 1);
-            qout[atomicAdd(nout, 1)] = make_int2(ref[c], t);
-            ref[c] = t;
+            qout[qat++] = make_int2(ref[c], to);
+            ref[c] = to++;
         }
+    }
     float v[6][4];
     int r[4];
     for (int c = 0; c < 4; ++c) {
@@ -742,17 +737,20 @@ __device__ __forceinline__ void collapse4_one(const float4* nodes2, int2 job, in
         v[5][c] = on ? hi[c].z : -FLT_MAX;
         r[c] = on ? ref[c] : kEmptyRef;
     }
-    float4* o = nodes4 + (size_t)kNode4Float4 * job.y;
+    float4* o = nodes4 + (size_t)kNode4Float4 * slot;
     for (int k = 0; k < 6; ++k) o[k] = make_float4(v[k][0], v[k][1], v[k][2], v[k][3]);
     o[6] = make_float4(__int_as_float(r[0]), __int_as_float(r[1]), __int_as_float(r[2]), __int_as_float(r[3]));
     o[7] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-__global__ void __launch_bounds__(kThreads) k_collapse4(const float4* nodes2, const int2* qin, int nin, int2* qout,
-                                                        int* nout, int* count4, float4* nodes4)
+// the same for one thread's job, its slots taken by atomics
+__device__ __forceinline__ void collapse4_one(const float4* nodes2, int2 job, int2* qout, int* nout, int* count4,
+                                              float4* nodes4)
 {
-    const int w = blockIdx.x * blockDim.x + threadIdx.x;
-    if (w < nin) collapse4_one(nodes2, qin[w], qout, nout, count4, nodes4);
+    Wide4 w;
+    const int inner = collapse4_open(nodes2, job.x, w);
+    const int to = inner ? atomicAdd(count4, inner) : 0, qat = inner ? atomicAdd(nout, inner) : 0;
+    collapse4_put(w, job.y, qout, qat, to, nodes4);
 }
 
 // ---------------------------------------------------------------- single-block build of small meshes
@@ -927,6 +925,382 @@ __global__ void __launch_bounds__(kSmallThreads) k_collapse4_small(const float4*
     }
 }
 
+// ---------------------------------------------------------------- builds in one launch
+// The clustering takes some 85 rounds for a million triangles and the 4-wide
+// collapse one step per level, each a few microseconds of work: six launches per
+// round and a host read every four made the rounds 2.9 of the 7.1 ms that loading
+// the 983k-triangle aircraft and a first look at it took (3.4 ms now, with the
+// index check on the host beside the build; the clustering 1.07 ms, bound by the
+// dependent steps of a round). Both run as one cooperative launch whose blocks (all resident) meet at a barrier between the steps; data written
+// by other blocks is read past L1. Every wait is bounded: a block that gives up
+// sets bit 8 of the error flag and leaves, and so do the others in turn.
+constexpr int kCoopThreads = 512;
+constexpr unsigned kCoopSpin = 1u << 22;
+
+struct GridBarrier {
+    unsigned* count;  // arrivals of all barriers so far
+    int* err;
+    unsigned passed = 0;
+    // false: gave up (every thread of the block learns it)
+    __device__ bool wait()
+    {
+        int bad = 0;
+        __syncthreads();
+        passed += gridDim.x;
+        if (threadIdx.x == 0) {
+            __threadfence();  // the block's writes, ordered before by the barrier above
+            atomicAdd(count, 1u);
+            unsigned i = 0;
+            while (*(volatile unsigned*)count < passed) {
+                if (++i > kCoopSpin) {
+                    atomicOr(err, 8);
+                    bad = 1;
+                    break;
+                }
+                __nanosleep(32);
+            }
+            __threadfence();
+        }
+        return !__syncthreads_or(bad);
+    }
+};
+
+struct PlocCoop {
+    const unsigned* vals;  // triangles in Morton order
+    const float4* tbox;
+    int n, radius, leaf_max;
+    float c_t, c_i;
+    Clusters cl[2];
+    int* nn;
+    unsigned* keep;
+    unsigned* tile_cnt;  // clusters kept per tile of kCoopThreads
+    int* next_id;        // n - 2 at the start
+    PlocNodes g;
+    int* par[2];
+    int* rel[2];
+    int* noff;
+    unsigned* perm;
+    unsigned* bar;       // zero at the start
+    int* active;         // [34] zero at the start: some pointer left after jump r
+    int* err;
+};
+
+// sums of a and b over the block (every thread gets them)
+__device__ __forceinline__ void block_sum2(unsigned& a, unsigned& b, unsigned (*s)[2])
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        s[threadIdx.x >> 5][0] = a;
+        s[threadIdx.x >> 5][1] = b;
+    }
+    __syncthreads();
+    a = b = 0;
+    for (int w = 0; w < kCoopThreads / 32; ++w) {
+        a += s[w][0];
+        b += s[w][1];
+    }
+    __syncthreads();
+}
+
+// The last rounds, of at most kSoloMax clusters, by one block in shared memory
+// (half of all rounds: the clusters shrink by a sixth each). Two clusters per
+// thread; false if the clustering does not converge.
+constexpr int kSoloMax = 2 * kCoopThreads;
+constexpr size_t kSoloSmem = kSoloMax * (2 * sizeof(float4) + 4 * sizeof(int));
+static_assert(kSoloSmem >= 2 * sizeof(float4) * (kCoopThreads + 128), "a tile and its halo fit too");
+__device__ bool ploc_solo(const PlocCoop& b, Clusters c, int m, int round)
+{
+    constexpr int T = kCoopThreads;
+    extern __shared__ float4 s_dyn[];
+    float4 *lo = s_dyn, *hi = lo + kSoloMax;
+    int *ref = (int*)(hi + kSoloMax), *cnt = ref + kSoloMax, *nn = cnt + kSoloMax;
+    float* cost = (float*)(nn + kSoloMax);
+    __shared__ int s_next;
+    __shared__ unsigned s_cnt[2][T / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, radius = b.radius, n = b.n;
+    __syncthreads();
+    for (int i = tid; i < m; i += T) {
+        lo[i] = __ldcg(c.lo + i);
+        hi[i] = __ldcg(c.hi + i);
+        ref[i] = __ldcg(c.ref + i);
+        cnt[i] = __ldcg(c.cnt + i);
+        cost[i] = __ldcg(c.cost + i);
+    }
+    if (tid == 0) s_next = __ldcg(b.next_id);
+    __syncthreads();
+    for (; m > 1; ++round) {
+        if (round >= (1 << 16)) {  // every round merges at least one pair
+            if (tid == 0) atomicOr(b.err, 4);
+            return false;
+        }
+        for (int i = tid; i < m; i += T) {
+            const float4 l = lo[i], h = hi[i];
+            float best = FLT_MAX;
+            int bj = -1;
+            const int j1 = min(m - 1, i + radius);
+            for (int j = max(0, i - radius); j <= j1; ++j) {
+                if (j == i) continue;
+                const float a = union_area(l, h, lo[j], hi[j]);
+                if (a < best) {  // strict: the lowest position wins ties
+                    best = a;
+                    bj = j;
+                }
+            }
+            nn[i] = bj;
+        }
+        __syncthreads();
+        // each thread's kept clusters in registers, then back in order
+        float4 kl[2], kh[2];
+        int kr[2], kc[2];
+        float ks[2];
+        bool kept[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int i = u * T + tid;
+            kept[u] = false;
+            if (i < m) {
+                const int j = nn[i];
+                const bool mutual = j >= 0 && nn[j] == i;
+                kept[u] = !mutual || i < j;
+                kl[u] = lo[i];
+                kh[u] = hi[i];
+                kr[u] = ref[i];
+                kc[u] = cnt[i];
+                ks[u] = cost[i];
+                if (mutual && i < j) {
+                    const int id = atomicSub(&s_next, 1);
+                    ploc_join(id, n, kl[u], kh[u], kr[u], kc[u], ks[u], lo[j], hi[j], ref[j], cnt[j], cost[j], b.g,
+                              b.leaf_max, b.c_t, b.c_i);
+                }
+            }
+            const unsigned mk = __ballot_sync(0xffffffffu, kept[u]);
+            if (lane == 0) s_cnt[u][warp] = __popc(mk);
+        }
+        __syncthreads();
+        unsigned at = 0;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            unsigned pos = at;
+            for (int w = 0; w < T / 32; ++w) {
+                if (w < warp) pos += s_cnt[u][w];
+                at += s_cnt[u][w];
+            }
+            const unsigned mk = __ballot_sync(0xffffffffu, kept[u]);
+            pos += __popc(mk & ((1u << lane) - 1u));
+            if (kept[u]) {
+                lo[pos] = kl[u];
+                hi[pos] = kh[u];
+                ref[pos] = kr[u];
+                cnt[pos] = kc[u];
+                cost[pos] = ks[u];
+            }
+        }
+        m = (int)at;
+        __syncthreads();
+    }
+    return true;
+}
+
+// The PLOC rounds over tiles of kCoopThreads clusters, each block a contiguous
+// run of tiles: nearest neighbours (a tile and its halo in shared memory),
+// merges, order-preserving compaction; block 0 alone finishes. Then the pointer jumping, until no pointer
+// is left (the tree's depth, not its size, sets the number of jumps).
+__global__ void __launch_bounds__(kCoopThreads) k_ploc_coop(const PlocCoop b)
+{
+    constexpr int T = kCoopThreads, kHalo = 64;
+    extern __shared__ float4 s_dyn[];
+    float4 *s_lo = s_dyn, *s_hi = s_dyn + T + 2 * kHalo;  // a tile and its halo
+    __shared__ unsigned s_sum[T / 32][2];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = b.n, radius = b.radius;
+    GridBarrier bar{b.bar, b.err};
+    for (int i = blockIdx.x * T + tid; i < n; i += gridDim.x * T) ploc_init_one(i, b.vals, b.tbox, b.c_i, b.cl[0]);
+    if (!bar.wait()) return;
+    int m = n, cur = 0, round = 0;
+    for (; m > kSoloMax; ++round) {
+        if (round >= (1 << 16)) {  // every round merges at least one pair
+            if (tid == 0) atomicOr(b.err, 4);
+            return;  // m and round are the same in every block that is still here
+        }
+        const int tiles = (m + T - 1) / T, per = (tiles + (int)gridDim.x - 1) / (int)gridDim.x;
+        const int t0 = min(tiles, (int)blockIdx.x * per), t1 = min(tiles, t0 + per);
+        const Clusters c = b.cl[cur], out = b.cl[cur ^ 1];
+        for (int t = t0; t < t1; ++t) {
+            const int base = t * T;
+            for (int k = tid; k < T + 2 * radius; k += T) {
+                const int j = base - radius + k;
+                if (j >= 0 && j < m) {
+                    s_lo[k] = __ldcg(c.lo + j);
+                    s_hi[k] = __ldcg(c.hi + j);
+                }
+            }
+            __syncthreads();
+            const int i = base + tid;
+            if (i < m) {
+                const float4 lo = s_lo[tid + radius], hi = s_hi[tid + radius];
+                float best = FLT_MAX;
+                int bj = -1;
+                const int j0 = max(0, i - radius), j1 = min(m - 1, i + radius);
+                for (int j = j0; j <= j1; ++j) {
+                    if (j == i) continue;
+                    const int k = j - base + radius;
+                    const float a = union_area(lo, hi, s_lo[k], s_hi[k]);
+                    if (a < best) {  // strict: the lowest position wins ties
+                        best = a;
+                        bj = j;
+                    }
+                }
+                b.nn[i] = bj;
+            }
+            __syncthreads();
+        }
+        if (!bar.wait()) return;
+        for (int t = t0; t < t1; ++t) {
+            const int i = t * T + tid;
+            unsigned kept = 0;
+            if (i < m) {
+                const int j = __ldcg(b.nn + i);
+                if (j < 0 || __ldcg(b.nn + j) != i) kept = 1;  // no mutual partner this round
+                else if (i < j) {
+                    ploc_merge_pair(i, j, n, c, b.next_id, b.g, b.leaf_max, b.c_t, b.c_i);
+                    kept = 1;
+                }
+                b.keep[i] = kept;
+            }
+            const int cnt = __syncthreads_count(kept);
+            if (tid == 0) b.tile_cnt[t] = (unsigned)cnt;
+        }
+        if (!bar.wait()) return;
+        unsigned total = 0, before = 0;
+        for (int k = tid; k < tiles; k += T) {
+            const unsigned v = __ldcg(b.tile_cnt + k);
+            total += v;
+            if (k < t0) before += v;
+        }
+        block_sum2(total, before, s_sum);
+        for (int t = t0; t < t1; ++t) {
+            const int i = t * T + tid;
+            const bool kp = i < m && b.keep[i];
+            const unsigned mk = __ballot_sync(0xffffffffu, kp);
+            if (lane == 0) s_sum[warp][0] = __popc(mk);
+            __syncthreads();
+            unsigned pos = before + __popc(mk & ((1u << lane) - 1u)), all = 0;
+            for (int w = 0; w < T / 32; ++w) {
+                if (w < warp) pos += s_sum[w][0];
+                all += s_sum[w][0];
+            }
+            if (kp) {
+                out.lo[pos] = __ldcg(c.lo + i);
+                out.hi[pos] = __ldcg(c.hi + i);
+                out.ref[pos] = __ldcg(c.ref + i);
+                out.cnt[pos] = __ldcg(c.cnt + i);
+                out.cost[pos] = __ldcg(c.cost + i);
+            }
+            before += all;
+            __syncthreads();
+        }
+        if (!bar.wait()) return;
+        m = (int)total;
+        cur ^= 1;
+    }
+    if (blockIdx.x == 0 && !ploc_solo(b, b.cl[cur], m, round)) return;
+    if (!bar.wait()) return;
+    // first positions of every node and triangle
+    const int nx = 2 * n - 1;
+    int pj = 0;
+    for (int r = 0; r < 33; ++r, pj ^= 1) {
+        bool left = false;
+        for (int x = blockIdx.x * T + tid; x < nx; x += gridDim.x * T) {
+            const int p = __ldcg(b.par[pj] + x), d = __ldcg(b.rel[pj] + x);
+            int np = p, nd = d;
+            if (p >= 0) {
+                np = __ldcg(b.par[pj] + p);
+                nd = d + __ldcg(b.rel[pj] + p);
+            }
+            b.par[pj ^ 1][x] = np;
+            b.rel[pj ^ 1][x] = nd;
+            left = left || np >= 0;
+        }
+        if (__syncthreads_or(left) && tid == 0) atomicOr(b.active + r, 1);
+        if (!bar.wait()) return;
+        if (!__ldcg(b.active + r)) {
+            pj ^= 1;
+            break;
+        }
+    }
+    for (int x = blockIdx.x * T + tid; x < nx; x += gridDim.x * T) ploc_positions_one(x, n, b.rel[pj], b.noff, b.perm);
+}
+
+// The 4-wide collapse, level by level. counters[0]: 4-wide nodes allocated (1 at
+// the start); counters[4 + level % 3]: length of that level's queue (counters[4]
+// = 1, the rest 0 at the start); counters[2]: 1 if too deep.
+__global__ void __launch_bounds__(kCoopThreads) k_collapse4_coop(const float4* nodes2, int2* qa, int2* qb, int* counters,
+                                                                 unsigned* bar_count, int* err, float4* nodes4)
+{
+    GridBarrier bar{bar_count, err};
+    int2 *qi = qa, *qo = qb;
+    for (int level = 0;; ++level) {
+        const int nin = __ldcg(counters + 4 + level % 3);
+        if (nin <= 0) break;
+        if (level > 4096) {  // deeper than any binary tree of < 2^27 leaves
+            if (threadIdx.x == 0) counters[2] = 1;
+            break;
+        }
+        // the level after next counts from zero (read last before the barrier that ended the previous level)
+        if (blockIdx.x == 0 && threadIdx.x == 0) counters[4 + (level + 2) % 3] = 0;
+        // slots and queue places of a warp's children by one pair of atomics
+        const int lane = threadIdx.x & 31;
+        for (int w0 = blockIdx.x * blockDim.x + threadIdx.x - lane; w0 < nin; w0 += gridDim.x * blockDim.x) {
+            const bool on = w0 + lane < nin;
+            const int2 job = on ? __ldcg(qi + w0 + lane) : make_int2(0, 0);
+            Wide4 w;
+            const int inner = on ? collapse4_open(nodes2, job.x, w) : 0;
+            int incl = inner;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
+            }
+            int to = 0, qat = 0;
+            if (lane == 31 && incl) {
+                to = atomicAdd(counters, incl);
+                qat = atomicAdd(counters + 4 + (level + 1) % 3, incl);
+            }
+            to = __shfl_sync(0xffffffffu, to, 31) + incl - inner;
+            qat = __shfl_sync(0xffffffffu, qat, 31) + incl - inner;
+            if (on) collapse4_put(w, job.y, qo, qat, to, nodes4);
+        }
+        if (!bar.wait()) return;
+        int2* t = qi;
+        qi = qo;
+        qo = t;
+    }
+}
+
+__global__ void k_collapse4_start(int2* queue, int* counters)
+{
+    if (threadIdx.x == 0) queue[0] = make_int2(0, 0);
+    if (threadIdx.x < 16) counters[threadIdx.x] = threadIdx.x == 0 || threadIdx.x == 4 ? 1 : 0;
+}
+
+// blocks of a cooperative launch: one per SM, at most as many as its items fill (two or three per SM: 2 to 5 % slower)
+template <class K>
+cudaError_t coop_blocks(K* k, long long items, size_t smem, int* blocks)
+{
+    int dev = 0, sms = 0, occ = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, kCoopThreads, smem);
+    if (e != cudaSuccess) return e;
+    if (occ < 1) return cudaErrorInvalidConfiguration;
+    const long long fill = (items + kCoopThreads - 1) / kCoopThreads;
+    *blocks = (int)std::max(1ll, std::min<long long>(fill, sms));
+    return cudaSuccess;
+}
+
 // ---------------------------------------------------------------- octant copies
 __global__ void __launch_bounds__(kThreads) k_octant_nodes(const float4* nodes, long long n_nodes, float4* out)
 {
@@ -953,6 +1327,10 @@ __global__ void __launch_bounds__(kThreads) k_octant_nodes(const float4* nodes, 
     }
 }
 
+constexpr int kBuildCounters = 64;  // barrier count, next node id, [2 ..] pointer-jump flags
+
+__global__ void k_set_int(int* p, int v) { *p = v; }
+
 struct Carve {
     char* p;
     size_t off, cap;
@@ -975,10 +1353,10 @@ struct Carve {
 // visits the same boxes in the same order.
 
 // parent of every internal child, as 2 * parent + side
-__global__ void __launch_bounds__(kThreads) k_rl_parent(const float4* nodes, int m, int* parent)
+__global__ void __launch_bounds__(kThreads) k_rl_parent(const float4* nodes, int m, int* parent, const int* err)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= m) return;
+    if (i >= m || (*err & kErrTree)) return;
     const float4 r = nodes[4 * (size_t)i + 3];
     const int c0 = __float_as_int(r.x), c1 = __float_as_int(r.y);
     if (c0 >= 0 && c0 < m) parent[c0] = 2 * i;
@@ -988,10 +1366,10 @@ __global__ void __launch_bounds__(kThreads) k_rl_parent(const float4* nodes, int
 // internal nodes in each subtree, bottom-up from the nodes without internal
 // children; the last child to arrive at a node finishes it
 __global__ void __launch_bounds__(kThreads) k_rl_size(const float4* nodes, int m, const int* parent, int* arrive,
-                                                      int* size)
+                                                      int* size, const int* err)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= m) return;
+    if (i >= m || (*err & kErrTree)) return;
     const float4 r = nodes[4 * (size_t)i + 3];
     if (__float_as_int(r.x) >= 0 || __float_as_int(r.y) >= 0) return;
     size[i] = 1;
@@ -1024,10 +1402,10 @@ __device__ __forceinline__ int rl_first(const float4* nodes, int p)
 
 // depth-first position of every reachable node (-1: not reachable from the root)
 __global__ void __launch_bounds__(kThreads) k_rl_pos(const float4* nodes, int m, const int* parent, const int* size,
-                                                     int* newpos)
+                                                     int* newpos, const int* err)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= m) return;
+    if (i >= m || (*err & kErrTree)) return;
     int pos = 0, x = i, steps = 0;
     for (; steps < m; ++steps) {
         const int pp = parent[x];
@@ -1044,9 +1422,10 @@ __global__ void __launch_bounds__(kThreads) k_rl_pos(const float4* nodes, int m,
 }
 
 __global__ void __launch_bounds__(kThreads) k_rl_scatter(const float4* nodes, int m, const int* newpos, float4* out,
-                                                         const int* size, int* n_out)
+                                                         const int* size, int* n_out, const int* err)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (*err & kErrTree) return;
     if (i == 0 && n_out) *n_out = size[0];
     if (i >= m) return;
     const int q = newpos[i];
@@ -1077,10 +1456,10 @@ cudaError_t relayout(const BvhBuild& b, int m, Carve& cv, cudaStream_t st)
     if (e == cudaSuccess) e = cudaMemsetAsync(arrive, 0, sizeof(int) * (size_t)m, st);
     if (e != cudaSuccess) return e;
     const int gm = (m + kThreads - 1) / kThreads;
-    k_rl_parent<<<gm, kThreads, 0, st>>>(b.nodes, m, parent);
-    k_rl_size<<<gm, kThreads, 0, st>>>(b.nodes, m, parent, arrive, size);
-    k_rl_pos<<<gm, kThreads, 0, st>>>(b.nodes, m, parent, size, newpos);
-    k_rl_scatter<<<gm, kThreads, 0, st>>>(b.nodes, m, newpos, tmp, size, b.n_nodes_out);
+    k_rl_parent<<<gm, kThreads, 0, st>>>(b.nodes, m, parent, b.err_flag);
+    k_rl_size<<<gm, kThreads, 0, st>>>(b.nodes, m, parent, arrive, size, b.err_flag);
+    k_rl_pos<<<gm, kThreads, 0, st>>>(b.nodes, m, parent, size, newpos, b.err_flag);
+    k_rl_scatter<<<gm, kThreads, 0, st>>>(b.nodes, m, newpos, tmp, size, b.n_nodes_out, b.err_flag);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(b.nodes, tmp, sizeof(float4) * 4 * (size_t)m, cudaMemcpyDeviceToDevice, st);
     return e;
@@ -1107,10 +1486,9 @@ size_t bvh_scratch_bytes(long long n_tri)
         add(n * 16); add(n * 16); add(n * 4); add(n * 4); add(n * 4);
     }
     add(n * 4); add(n * 4); add(n * 4);     // nn keep pos
-    add(scan_scratch_bytes((long long)n));
     add(n * 4); add(n * 4);                 // noff perm
     for (int k = 0; k < 4; ++k) add(2 * n * 4);  // parent links and offsets, two buffers each
-    add(64);                                // counters
+    add(4 * kBuildCounters);                // counters
     for (int k = 0; k < 4; ++k) add(n * 4); // relayout: parent, arrivals, subtree sizes, new positions
     add(n * 64);                            // relayout: the renumbered nodes
     return b + 256;
@@ -1155,7 +1533,6 @@ cudaError_t bvh_build(const BvhBuild& b, cudaStream_t st)
     int* pnn = cv.take<int>(nn);
     unsigned* keep = cv.take<unsigned>(nn);
     unsigned* pos = cv.take<unsigned>(nn);
-    void* pscan = cv.take<char>(scan_scratch_bytes((long long)nn));
     int* noff = cv.take<int>(nn);
     unsigned* perm = cv.take<unsigned>(nn);
     int* par[2];
@@ -1164,15 +1541,15 @@ cudaError_t bvh_build(const BvhBuild& b, cudaStream_t st)
         par[k] = cv.take<int>(2 * (size_t)nn);
         rel[k] = cv.take<int>(2 * (size_t)nn);
     }
-    int* ctr = cv.take<int>(16);
+    int* ctr = cv.take<int>(kBuildCounters);
     if (cv.off > cv.cap) return cudaErrorInvalidValue;
 
     const int g = (n + kThreads - 1) / kThreads;
     k_acc_init<<<1, 32, 0, st>>>(acc, b.err_flag);
     int gv = (int)((b.n_vert + kThreads - 1) / kThreads);
-    if (gv > 4096) gv = 4096;
+    if (gv > 1024) gv = 1024;
     k_vertex_box<<<gv, kThreads, 0, st>>>(b.xyz, b.n_vert, acc, b.err_flag);
-    k_prep<<<g, kThreads, 0, st>>>(b.xyz, b.tri, b.n_vert, n, tbox, cen, acc, b.err_flag);
+    k_prep<<<std::min(g, 1024), kThreads, 0, st>>>(b.xyz, b.tri, b.n_vert, n, tbox, cen, acc, b.err_flag);
     k_morton<<<g, kThreads, 0, st>>>(cen, n, acc, k0, v0, b.bbox_out);
     if (b.builder == 1 && n > 1 && n <= kSmallBuild) {
         const int nx = 2 * n - 1;
@@ -1206,10 +1583,11 @@ cudaError_t bvh_build(const BvhBuild& b, cudaStream_t st)
         sb.err = b.err_flag;
         k_build_small<<<1, kSmallThreads, 12 * (size_t)n, st>>>(sb);
         k_ploc_emit<<<(n - 1 + kThreads - 1) / kThreads, kThreads, 0, st>>>(n, left, right, nbox, ncnt, ncol, noff,
-                                                                            tbox, b.nodes);
+                                                                            tbox, b.nodes, b.err_flag);
         e = relayout(b, n - 1, cv, st);
         if (e != cudaSuccess) return e;
-        k_reorder<<<g, kThreads, 0, st>>>(b.xyz, b.tri, b.n_vert, perm, n, b.tris, b.tri_nrm, b.tri_v12, b.tri_pos);
+        k_reorder<<<g, kThreads, 0, st>>>(b.xyz, b.tri, b.n_vert, perm, n, b.tris, b.tri_nrm, b.tri_v12, b.tri_pos,
+                                         b.err_flag);
         return cudaGetLastError();
     }
     unsigned long long *ki = k0, *ko = k1;
@@ -1224,48 +1602,49 @@ cudaError_t bvh_build(const BvhBuild& b, cudaStream_t st)
     }
     // after an even number of passes the sorted data is back in (k0, v0)
     if (b.builder == 1 && n > 1) {
-        // PLOC over the Morton order; the live-cluster count stays on the device and the host reads it every
-        // kRoundsPerSync rounds (extra rounds after the last merge change nothing)
-        constexpr int kRoundsPerSync = 4;
-        const float c_t = b.c_t, c_i = b.c_i;
-        const int radius = b.radius > 0 ? b.radius : 16;
+        // PLOC over the Morton order
         const int nx = 2 * n - 1;
-        k_ploc_init<<<g, kThreads, 0, st>>>(vi, tbox, n, c_i, cl[0]);
-        int h[2] = {n - 2, n};  // next node id, live clusters
-        cudaError_t e = cudaMemcpyAsync(ctr, h, sizeof(h), cudaMemcpyHostToDevice, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(par[0], 0xFF, sizeof(int) * (size_t)nx, st);
+        cudaError_t e = cudaMemsetAsync(par[0], 0xFF, sizeof(int) * (size_t)nx, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(rel[0], 0, sizeof(int) * (size_t)nx, st);
-        const PlocNodes pg = {left, right, nbox, ncnt, ncost, ncol, par[0], rel[0]};
-        int m = n, cur = 0;
-        for (int round = 0; e == cudaSuccess && m > 1; round += kRoundsPerSync) {
-            if (round >= 1 << 16) return cudaErrorInvalidValue;  // every round merges at least one pair
-            const int gm = (m + kThreads - 1) / kThreads;
-            for (int r = 0; r < kRoundsPerSync && e == cudaSuccess; ++r) {
-                k_ploc_nn<<<gm, kThreads, 0, st>>>(ctr + 1, radius, cl[cur], pnn);
-                k_ploc_merge<<<gm, kThreads, 0, st>>>(ctr + 1, m, n, cl[cur], pnn, ctr, pg, keep, b.leaf_max, c_t, c_i);
-                e = scan_exclusive_u32(keep, pos, m, false, (unsigned*)(ctr + 1), pscan, st);
-                if (e != cudaSuccess) break;
-                k_ploc_compact<<<gm, kThreads, 0, st>>>(m, cl[cur], keep, pos, cl[cur ^ 1]);
-                e = cudaGetLastError();
-                cur ^= 1;
-            }
-            if (e == cudaSuccess) e = cudaMemcpyAsync(&m, ctr + 1, sizeof(int), cudaMemcpyDeviceToHost, st);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        }
+        if (e == cudaSuccess) e = cudaMemsetAsync(ctr, 0, sizeof(int) * kBuildCounters, st);
         if (e != cudaSuccess) return e;
-        // first positions: pointer jumping over parent links (depth <= n - 1 < 2^rounds)
-        int jr = 1;
-        while ((1ll << jr) < (long long)n) ++jr;
-        const int gx = (nx + kThreads - 1) / kThreads;
-        int pj = 0;
-        for (int r = 0; r <= jr; ++r, pj ^= 1)
-            k_ploc_jump<<<gx, kThreads, 0, st>>>(nx, par[pj], rel[pj], par[pj ^ 1], rel[pj ^ 1]);
-        k_ploc_positions<<<gx, kThreads, 0, st>>>(n, rel[pj], noff, perm);
+        k_set_int<<<1, 1, 0, st>>>(ctr + 1, n - 2);  // the next node id
+        PlocCoop pc;
+        pc.vals = vi;
+        pc.tbox = tbox;
+        pc.n = n;
+        pc.radius = b.radius > 0 ? b.radius : 16;
+        pc.leaf_max = b.leaf_max;
+        pc.c_t = b.c_t;
+        pc.c_i = b.c_i;
+        pc.cl[0] = cl[0];
+        pc.cl[1] = cl[1];
+        pc.nn = pnn;
+        pc.keep = keep;
+        pc.tile_cnt = pos;
+        pc.next_id = ctr + 1;
+        pc.g = {left, right, nbox, ncnt, ncost, ncol, par[0], rel[0]};
+        for (int k = 0; k < 2; ++k) {
+            pc.par[k] = par[k];
+            pc.rel[k] = rel[k];
+        }
+        pc.noff = noff;
+        pc.perm = perm;
+        pc.bar = (unsigned*)ctr;
+        pc.active = ctr + 2;
+        pc.err = b.err_flag;
+        int blocks = 0;
+        e = cudaFuncSetAttribute(k_ploc_coop, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSoloSmem);
+        if (e == cudaSuccess) e = coop_blocks(k_ploc_coop, n, kSoloSmem, &blocks);
+        void* args[] = {&pc};
+        if (e == cudaSuccess) e = cudaLaunchCooperativeKernel(k_ploc_coop, dim3(blocks), dim3(kCoopThreads), args, kSoloSmem, st);
+        if (e != cudaSuccess) return e;
         k_ploc_emit<<<(n - 1 + kThreads - 1) / kThreads, kThreads, 0, st>>>(n, left, right, nbox, ncnt, ncol, noff,
-                                                                            tbox, b.nodes);
+                                                                            tbox, b.nodes, b.err_flag);
         e = relayout(b, n - 1, cv, st);
         if (e != cudaSuccess) return e;
-        k_reorder<<<g, kThreads, 0, st>>>(b.xyz, b.tri, b.n_vert, perm, n, b.tris, b.tri_nrm, b.tri_v12, b.tri_pos);
+        k_reorder<<<g, kThreads, 0, st>>>(b.xyz, b.tri, b.n_vert, perm, n, b.tris, b.tri_nrm, b.tri_v12, b.tri_pos,
+                                         b.err_flag);
         return cudaGetLastError();
     }
     if (n > 1) {
@@ -1279,7 +1658,8 @@ cudaError_t bvh_build(const BvhBuild& b, cudaStream_t st)
     k_emit<<<ge, kThreads, 0, st>>>(n, left, right, first, lbox, nbox, ncnt, ncol, b.nodes);
     cudaError_t e = relayout(b, n > 1 ? n - 1 : 1, cv, st);
     if (e != cudaSuccess) return e;
-    k_reorder<<<g, kThreads, 0, st>>>(b.xyz, b.tri, b.n_vert, vi, n, b.tris, b.tri_nrm, b.tri_v12, b.tri_pos);
+    k_reorder<<<g, kThreads, 0, st>>>(b.xyz, b.tri, b.n_vert, vi, n, b.tris, b.tri_nrm, b.tri_v12, b.tri_pos,
+                                         b.err_flag);
     return cudaGetLastError();
 }
 
@@ -1303,28 +1683,19 @@ cudaError_t bvh4_collapse(const float4* nodes2, long long n_nodes2, float4* node
         if (e == cudaSuccess) *n_nodes4 = h[0];
         return e;
     }
-    // counters[0]: 4-wide nodes allocated; counters[1]: next-level queue length
-    const int2 root = make_int2(0, 0);
-    const int one = 1;
-    cudaError_t e = cudaMemcpyAsync(queue_a, &root, sizeof(int2), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(counters, &one, sizeof(int), cudaMemcpyHostToDevice, st);
-    int nin = 1;
-    int2 *qi = queue_a, *qo = queue_b;
-    for (int level = 0; e == cudaSuccess && nin > 0; ++level) {
-        if (level > 4096) return cudaErrorInvalidValue;  // deeper than any binary tree of < 2^27 leaves
-        e = cudaMemsetAsync(counters + 1, 0, sizeof(int), st);
-        if (e != cudaSuccess) break;
-        k_collapse4<<<(nin + kThreads - 1) / kThreads, kThreads, 0, st>>>(nodes2, qi, nin, qo, counters + 1,
-                                                                          counters, nodes4);
-        e = cudaGetLastError();
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&nin, counters + 1, sizeof(int), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        int2* t = qi;
-        qi = qo;
-        qo = t;
-    }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(n_nodes4, counters, sizeof(int), cudaMemcpyDeviceToHost, st);
+    k_collapse4_start<<<1, 32, 0, st>>>(queue_a, counters);
+    int blocks = 0;
+    cudaError_t e = coop_blocks(k_collapse4_coop, n_nodes2, 0, &blocks);
+    unsigned* bar = (unsigned*)counters + 8;
+    int* err = counters + 9;
+    void* args[] = {&nodes2, &queue_a, &queue_b, &counters, &bar, &err, &nodes4};
+    if (e == cudaSuccess)
+        e = cudaLaunchCooperativeKernel(k_collapse4_coop, dim3(blocks), dim3(kCoopThreads), args, 0, st);
+    int h[10] = {0};
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h, counters, sizeof(h), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess && (h[2] || h[9])) e = cudaErrorInvalidValue;
+    if (e == cudaSuccess) *n_nodes4 = h[0];
     return e;
 }
 
