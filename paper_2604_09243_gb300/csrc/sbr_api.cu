@@ -97,6 +97,8 @@ struct sbr_ctx {
     DevBuf hit_tri, hit_t, hit_nb;
     DevBuf tripos, vis, visfull;  // position of each original triangle; raster keys and per-aspect flags
     DevBuf rbig, rbigctr;         // large triangles of a rasterised chunk and their two counters
+    DevBuf slotscr;               // scratch of the primary pass's masks and slots
+    unsigned long long* stats_host = nullptr;  // pinned copy of stats
     long long rbig_cap = 0;
     DevBuf hitlist;               // (ray, aspect) of the rasterised primary hits, read by bounce pass 1
     // pooled late passes of sbr_trace: the live rays the chunks leave for pass kPoolPass, the trace's aspect
@@ -109,7 +111,7 @@ struct sbr_ctx {
     bool has_trace = false;
     std::vector<AngleHost> ang;
     // PO
-    DevBuf items, itemoff, recbeg, freq, kfreq, partial, E, rcs;
+    DevBuf items, potab, po, partial;  // work list; aspect table and record offsets; results, flag and frequencies
     // pinned staging
     void* host_stage = nullptr;
     size_t host_stage_cap = 0;
@@ -513,10 +515,11 @@ void sbr_destroy(sbr_ctx* c)
                      &c->angles, &c->rayoff, &c->mask, &c->tilebase, &c->scan_scr, &c->recoff, &c->q0, &c->q1, &c->cover,
                      &c->nodes_oct, &c->tripos, &c->pool, &c->angall, &c->rayoffall, &c->recofall, &c->poolctr,
                      &c->poolwork, &c->poolgroup, &c->vis, &c->visfull, &c->hitlist, &c->rbig, &c->rbigctr, &c->ctr64, &c->ctr32, &c->stats, &c->rec, &c->hit_tri, &c->hit_t, &c->hit_nb, &c->items,
-                     &c->itemoff, &c->recbeg, &c->freq, &c->kfreq, &c->partial, &c->E, &c->rcs};
+                     &c->potab, &c->po, &c->partial, &c->slotscr};
     for (DevBuf* b : all) b->release();
     if (c->host_stage) cudaFreeHost(c->host_stage);
     if (c->pool_host) cudaFreeHost(c->pool_host);
+    if (c->stats_host) cudaFreeHost(c->stats_host);
     if (c->stage_ev) cudaEventDestroy(c->stage_ev);
     for (cudaEvent_t e : c->evpool) cudaEventDestroy(e);
     free_plan(c->plan);
@@ -656,6 +659,7 @@ int plan_chunks(sbr_ctx* c, TraceRun& R, std::vector<int64_t>& cut, long long* t
         c->rbig_cap = raster_big_cap(max_chunk);
         CK(c->rbig.ensure(sizeof(int4) * (size_t)c->rbig_cap), "alloc raster triangle list");
         CK(c->rbigctr.ensure(sizeof(unsigned) * 2), "alloc raster triangle counters");
+        CK(c->slotscr.ensure(sizeof(unsigned) * kSlotWords), "alloc slot scratch");
     }
     CK(c->tilebase.ensure(sizeof(unsigned) * (size_t)all_tiles), "alloc tile base");
     CK(c->scan_scr.ensure(scan_scratch_bytes(max_tiles)), "alloc scan scratch");
@@ -664,7 +668,6 @@ int plan_chunks(sbr_ctx* c, TraceRun& R, std::vector<int64_t>& cut, long long* t
     CK(c->ctr64.ensure(sizeof(unsigned long long) * 2 * (kMaxBounces + 2)), "alloc counters");
     CK(c->ctr32.ensure(sizeof(unsigned) * 2 * (kMaxBounces + 2) + 64), "alloc counters");
     CK(c->stats.ensure(sizeof(unsigned long long) * kStatCount), "alloc stats");
-    CK(cudaMemsetAsync(c->stats.p, 0, sizeof(unsigned long long) * kStatCount, c->stream), "memset stats");
     if (R.hits) {
         const size_t B = (size_t)R.max_bounces;
         CK(c->hit_tri.ensure(sizeof(int) * (size_t)total * B), "alloc hit ids");
@@ -732,14 +735,37 @@ cudaError_t run_pass(sbr_ctx* c, TraceRun& R, const TraceArgs& t)
     cudaError_t e = cudaSuccess;
     if (t.vis && t.bounce == 0) {
         e = launch_raster(t, (int)c->n_tri, c->vis.as<unsigned long long>(), c->visfull.as<unsigned>(), R.count,
-                          c->n_sms * 16, c->scan_scr.p, c->stream);
-        R.n_launch += 6;  // rasterisation, masks, 3-kernel scan, primary pass of the rasterised rays
+                          c->n_sms * 16, c->stream);
+        R.n_launch += t.hit_list ? 4 : 5;  // rasterisation (2), masks, slots, states or records of the hits
     }
     if (e == cudaSuccess) e = launch_trace(t, R.n_blocks, R.count, c->tune.stack_depth, c->stream);
     if (R.timed) cudaEventRecord(e1, c->stream);
     ++R.n_launch;
     ++R.n_pass;
     return e;
+}
+
+// k_trace_begin's ranges for a chunk of na aspects and `rays` rays (stats: cleared with the first chunk)
+TraceInit trace_init(unsigned long long* stats, const DevBuf& ctr64, const DevBuf& ctr32, int raster, const DevBuf& vis,
+                     long long rays, const DevBuf& visfull, int na, const DevBuf& rbigctr)
+{
+    TraceInit b;
+    memset(&b, 0, sizeof(b));
+    int k = 0;
+    auto zero = [&](void* p, size_t bytes) {
+        b.zero[k] = (unsigned*)p;
+        b.n_zero[k++] = (long long)(bytes / sizeof(unsigned));
+    };
+    zero(ctr64.p, sizeof(unsigned long long) * 2 * (kMaxBounces + 2));
+    zero(ctr32.p, sizeof(unsigned) * 2 * (kMaxBounces + 2) + 64);
+    if (stats) zero(stats, sizeof(unsigned long long) * kStatCount);
+    if (raster) {
+        zero(visfull.p, sizeof(unsigned) * (size_t)(na + 1));
+        zero(rbigctr.p, sizeof(unsigned) * 2);
+        b.vis16 = vis.as<uint4>();
+        b.n_vis16 = rays / 2;
+    }
+    return b;
 }
 
 int trace_chunk(sbr_ctx* c, TraceRun& R, int64_t a0, int64_t a1, long long rec_base, unsigned** hro_out)
@@ -783,10 +809,18 @@ int trace_chunk(sbr_ctx* c, TraceRun& R, int64_t a0, int64_t a1, long long rec_b
         ha[i] = to_dev(h.grid, ho[i], h.tw, h.bistatic ? rx : nullptr);
     }
     ho[na] = chunk_rays;
-    CK(cudaMemcpyAsync(c->angles.p, ha, bytes_a, cudaMemcpyHostToDevice, c->stream), "copy angles");
-    CK(cudaMemcpyAsync(c->rayoff.p, ho, bytes_o, cudaMemcpyHostToDevice, c->stream), "copy ray offsets");
-    CK(cudaMemsetAsync(c->ctr64.p, 0, c->ctr64.cap, c->stream), "memset counters");
-    CK(cudaMemsetAsync(c->ctr32.p, 0, c->ctr32.cap, c->stream), "memset counters");
+    unsigned* hro = (unsigned*)(hs + bytes_a + bytes_o);
+    TraceInit init = trace_init(a0 == 0 ? c->stats.as<unsigned long long>() : nullptr, c->ctr64, c->ctr32,
+                                c->tune.raster, c->vis, chunk_rays, c->visfull, na, c->rbigctr);
+    static_assert(sizeof(AngleDev) % sizeof(uint4) == 0, "the aspect table is copied in 16-byte words");
+    init.table_host = (const uint4*)ha;
+    init.table = c->angles.as<uint4>();
+    init.n_table = (long long)(bytes_a / sizeof(uint4));
+    init.off_host = ho;
+    init.off = c->rayoff.as<long long>();
+    init.n_off = na + 1;
+    CK(launch_trace_begin(init, c->n_sms, c->stream), "trace begin");
+    ++R.n_launch;
     TraceArgs ta;
     memset(&ta, 0, sizeof(ta));
     ta.wide = c->tune.bvh_width == 4;
@@ -823,7 +857,10 @@ int trace_chunk(sbr_ctx* c, TraceRun& R, int64_t a0, int64_t a1, long long rec_b
         ta.big_ctr = c->rbigctr.as<unsigned>();
         ta.big_cap = (unsigned)c->rbig_cap;
         ta.tri_pos = c->tripos.as<int>();
-        ta.list_count = total_dev + 4;
+        ta.slot_scr = c->slotscr.as<unsigned>();
+        ta.rec_off = c->recoff.as<unsigned>();
+        ta.rec_off_host = hro;
+        ta.emit_primary = R.max_bounces == 1 && !R.escape && !ta.bistatic;
         // a bounce pass follows: list the hits and let it rebuild their states (not for B = 1, whose
         // records are written from the stored states; binary per-lane traversals only, where the rebuilding
         // fits the bounce kernel's registers)
@@ -839,19 +876,19 @@ int trace_chunk(sbr_ctx* c, TraceRun& R, int64_t a0, int64_t a1, long long rec_b
     ta.work = c->ctr64.as<unsigned long long>();
     ta.q_out = qs[0];
     ta.q_out_count = q_count + 1;
+    ta.rec = c->rec.as<Record>() + rec_base;
     CK(pass(ta), "trace primary");
-    CK(scan_popc(ta.mask, tilebase, chunk_rays / 32, total_dev, c->scan_scr.p, c->stream), "scan");
-    R.n_launch += 3;
-    CK(launch_angle_offsets(ta.ray_off, tilebase, total_dev, na, c->recoff.as<unsigned>(), c->stream),
-       "angle offsets");
-    ++R.n_launch;
-    unsigned* hro = (unsigned*)(hs + bytes_a + bytes_o);
-    CK(cudaMemcpyAsync(hro, c->recoff.p, sizeof(unsigned) * (size_t)(na + 1), cudaMemcpyDeviceToHost, c->stream),
-       "copy record offsets");
+    if (!ta.vis) {  // (the primary pass of keyed rays has done both)
+        CK(scan_popc(ta.mask, tilebase, chunk_rays / 32, total_dev, c->scan_scr.p, c->stream), "scan");
+        CK(launch_angle_offsets(ta.ray_off, tilebase, total_dev, na, c->recoff.as<unsigned>(), hro, c->stream),
+           "angle offsets");
+        R.n_launch += 4;
+    }
     CK(cudaEventRecord(c->stage_ev, c->stream), "record staging event");
     *hro_out = hro;
-    ta.rec = c->rec.as<Record>() + rec_base;
-    if (R.max_bounces == 1 && !R.escape) {
+    if (ta.emit_primary) {
+        // the records are written
+    } else if (R.max_bounces == 1 && !R.escape) {
         ta.q_in = qs[0];
         ta.q_in_count = q_count + 1;
         CK(launch_emit_all(ta, R.n_blocks, c->stream), "emit");
@@ -898,10 +935,14 @@ long long chunk_records(sbr_ctx* c, int64_t a0, int64_t a1, long long rec_base, 
 // wait for the stream and read the device counters
 int read_counters(sbr_ctx* c, unsigned long long* hs_stats)
 {
-    CK(cudaMemcpyAsync(hs_stats, c->stats.p, sizeof(unsigned long long) * kStatCount, cudaMemcpyDeviceToHost,
-                       c->stream),
-       "copy stats");
+    const size_t bytes = sizeof(unsigned long long) * kStatCount;
+    if (!c->stats_host && cudaMallocHost((void**)&c->stats_host, bytes) != cudaSuccess) {
+        c->stats_host = nullptr;
+        return fail(c, SBR_ERR_OOM, "pinned allocation failed");
+    }
+    CK(cudaMemcpyAsync(c->stats_host, c->stats.p, bytes, cudaMemcpyDeviceToHost, c->stream), "copy stats");
     CK(cudaStreamSynchronize(c->stream), "trace end sync");
+    memcpy(hs_stats, c->stats_host, bytes);
     return SBR_OK;
 }
 
@@ -956,18 +997,23 @@ int check_po_mode(sbr_ctx* c, int pol_mask, int po_mode, PoArgs& pa)
     return SBR_OK;
 }
 
-// upload the frequency table: (kappa_hi, kappa_lo, k) per frequency, kappa = f / c0
-int upload_freqs(sbr_ctx* c, const double* freq_hz, int64_t n_freq)
+// One device buffer holds a PO call's results for the host, the flag of its bounded waits and its frequency
+// table, (kappa_hi, kappa_lo, k) and k per frequency, kappa = f / c0:
+//   [E 2 n_out doubles][rcs n_out doubles][flag, 16 bytes][float4 n_freq][double n_freq]
+// so that one copy takes flag (cleared) and frequencies there and one brings the results and the flag back.
+// n_out: values per output array for the host (0: the caller's device arrays). Sets pa's pointers.
+int upload_freqs(sbr_ctx* c, const double* freq_hz, int64_t n_freq, size_t n_out, PoArgs& pa)
 {
     for (int64_t f = 0; f < n_freq; ++f)
         if (!(freq_hz[f] > 0.0)) return fail(c, SBR_ERR_ARG, "frequencies must be > 0");
+    const size_t b_out = (sizeof(double) * 3 * n_out + 15) / 16 * 16;
     const size_t b_freq = sizeof(float4) * (size_t)n_freq, b_kf = sizeof(double) * (size_t)n_freq;
-    CK(c->freq.ensure(b_freq), "alloc freq");
-    CK(c->kfreq.ensure(b_kf), "alloc freq");
-    char* hs = (char*)stage(c, b_freq + b_kf + 64);
+    CK(c->po.ensure(b_out + 16 + b_freq + b_kf), "alloc po results");
+    char* hs = (char*)stage(c, 16 + b_freq + b_kf);
     if (!hs) return fail(c, SBR_ERR_OOM, "pinned staging allocation failed");
-    float4* hf = (float4*)hs;
-    double* hk = (double*)(hs + b_freq);
+    memset(hs, 0, 16);
+    float4* hf = (float4*)(hs + 16);
+    double* hk = (double*)(hs + 16 + b_freq);
     for (int64_t f = 0; f < n_freq; ++f) {
         const double kappa = freq_hz[f] / kC0;  // cycles per metre
         const float kh = (float)kappa;
@@ -975,9 +1021,39 @@ int upload_freqs(sbr_ctx* c, const double* freq_hz, int64_t n_freq)
         hf[f] = make_float4(kh, (float)(kappa - (double)kh), (float)k, 0.f);
         hk[f] = k;
     }
-    CK(cudaMemcpyAsync(c->freq.p, hf, b_freq, cudaMemcpyHostToDevice, c->stream), "copy freq");
-    CK(cudaMemcpyAsync(c->kfreq.p, hk, b_kf, cudaMemcpyHostToDevice, c->stream), "copy freq");
+    char* d = (char*)c->po.p + b_out;
+    CK(cudaMemcpyAsync(d, hs, 16 + b_freq + b_kf, cudaMemcpyHostToDevice, c->stream), "copy freq");
     CK(cudaEventRecord(c->stage_ev, c->stream), "record staging event");
+    pa.err = (int*)d;  // bounded waits of the staged single-frequency sum
+    pa.freq = (float4*)(d + 16);
+    pa.kfreq = (double*)(d + 16 + b_freq);
+    return SBR_OK;
+}
+
+// Bring the n_out results (c->po) to the host arrays and read the flag: through pinned memory in one copy up
+// to kStagedResults, directly above.
+constexpr size_t kStagedResults = 1 << 20;
+int fetch_results(sbr_ctx* c, const PoArgs& pa, size_t n_out, double* E_out, double* rcs_out, int* flag)
+{
+    const char* base = (const char*)c->po.p;
+    const size_t b_e = sizeof(double) * 2 * n_out, b_r = sizeof(double) * n_out, b_all = (size_t)((const char*)pa.err - base) + 16;
+    const bool staged = b_all <= kStagedResults;
+    char* hs = (char*)stage(c, staged ? b_all : 16);
+    if (!hs) return fail(c, SBR_ERR_OOM, "pinned staging allocation failed");
+    if (staged) {
+        CK(cudaMemcpyAsync(hs, base, b_all, cudaMemcpyDeviceToHost, c->stream), "copy results");
+    } else {
+        if (E_out) CK(cudaMemcpyAsync(E_out, base, b_e, cudaMemcpyDeviceToHost, c->stream), "copy E");
+        if (rcs_out) CK(cudaMemcpyAsync(rcs_out, base + b_e, b_r, cudaMemcpyDeviceToHost, c->stream), "copy rcs");
+        CK(cudaMemcpyAsync(hs, pa.err, 16, cudaMemcpyDeviceToHost, c->stream), "copy po flag");
+    }
+    CK(cudaStreamSynchronize(c->stream), "po sync");
+    if (staged) {
+        if (E_out) memcpy(E_out, hs, b_e);
+        if (rcs_out) memcpy(rcs_out, hs + b_e, b_r);
+        hs += b_all - 16;
+    }
+    memcpy(flag, hs, sizeof(int));
     return SBR_OK;
 }
 
@@ -1018,26 +1094,22 @@ int po_run(sbr_ctx* c, PoArgs pa, int64_t a0, int64_t a1, const std::vector<int>
     }
     if (n_items >= (1ll << 31)) return fail(c, SBR_ERR_ARG, "too many PO work items");
     CK(c->items.ensure(std::max(sizeof(PoItem) * (size_t)n_items, (size_t)32)), "alloc items");
-    CK(c->itemoff.ensure(b_ang), "alloc aspect table");
-    CK(c->recbeg.ensure(b_off), "alloc record offsets");
+    CK(c->potab.ensure(b_ang + b_off), "alloc aspect table");
     CK(c->partial.ensure(sizeof(double) * (size_t)std::max(part, 1ll)), "alloc partials");
-    CK(cudaMemcpyAsync(c->itemoff.p, pang, b_ang, cudaMemcpyHostToDevice, c->stream), "copy aspect table");
-    CK(cudaMemcpyAsync(c->recbeg.p, off, b_off, cudaMemcpyHostToDevice, c->stream), "copy record offsets");
+    const PoAngle* d_ang = c->potab.as<PoAngle>();
+    CK(cudaMemcpyAsync(c->potab.p, hs, b_ang + b_off, cudaMemcpyHostToDevice, c->stream), "copy aspect table");
     CK(cudaEventRecord(c->stage_ev, c->stream), "record staging event");
     if (n_items > 0)
-        CK(launch_po_items_fill(c->recbeg.as<long long>(), c->itemoff.as<PoAngle>(), na, pa.n_pol, per,
+        CK(launch_po_items_fill((const long long*)(c->potab.as<char>() + b_ang), d_ang, na, pa.n_pol, per,
                                 c->items.as<PoItem>(), c->stream),
            "po work list");
     pa.rec = c->rec.as<Record>();
     pa.items = c->items.as<PoItem>();
     pa.n_items = (int)n_items;
-    pa.freq = c->freq.as<float4>();
-    pa.kfreq = c->kfreq.as<double>();
     pa.partial = c->partial.as<double>();
     pa.item_records = c->tune.po_item;
-    pa.err = c->err_dev.as<int>() + 3;  // bounded waits of the staged single-frequency sum (callers clear it)
     CK(launch_po(pa, c->stream), "po reduce");
-    CK(launch_po_final(pa.partial, pa.items, c->itemoff.as<PoAngle>(), na, max_nf, pa.kfreq, pa.n_pol, dE, dR, c->stream),
+    CK(launch_po_final(pa.partial, pa.items, d_ang, na, max_nf, pa.kfreq, pa.n_pol, dE, dR, c->stream),
        "po final");
     if (n_launch) *n_launch += (n_items > 0 ? 2 : 0) + 1;
     return SBR_OK;
@@ -1069,7 +1141,7 @@ struct BatchPlan {
     PoArgs pa;
     // device buffers
     DevBuf angles, rayoff, pang, recoff, mask, tilebase, scan_scr, q0, q1, ctr64, ctr32, stats, rec, items, nitems,
-        valid, freq_t, kfreq, partial, cover, vis, visfull, hitlist, rbig, rbigctr;
+        valid, freq_t, kfreq, partial, cover, vis, visfull, hitlist, rbig, rbigctr, slotscr;
     cudaStream_t cap = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -1084,7 +1156,7 @@ void free_plan(BatchPlan* p)
     DevBuf* all[] = {&p->angles, &p->rayoff, &p->pang,   &p->recoff, &p->mask,   &p->tilebase, &p->scan_scr,
                      &p->q0,     &p->q1,     &p->ctr64,  &p->ctr32,  &p->stats,  &p->rec,      &p->items,
                      &p->nitems, &p->valid,  &p->freq_t, &p->kfreq,  &p->partial, &p->cover,
-                     &p->vis,    &p->visfull, &p->hitlist, &p->rbig, &p->rbigctr};
+                     &p->vis,    &p->visfull, &p->hitlist, &p->rbig, &p->rbigctr, &p->slotscr};
     for (DevBuf* b : all) b->release();
     delete p;
 }
@@ -1105,7 +1177,7 @@ bool same_submission(const BatchPlan& P, const sbr_ctx* c, const sbr_request* re
 // record scan, the device-built PO work list, the PO sums and the final sums.
 cudaError_t enqueue_plan(const sbr_ctx* c, BatchPlan& P, cudaStream_t st)
 {
-    cudaError_t e = cudaMemsetAsync(P.stats.p, 0, sizeof(unsigned long long) * kStatCount, st);
+    cudaError_t e = cudaSuccess;
     unsigned* q_count = P.ctr32.as<unsigned>();
     unsigned* total_dev = q_count + 2 * (kMaxBounces + 2);
     RayState* qs[2] = {P.q0.as<RayState>(), P.q1.as<RayState>()};
@@ -1115,8 +1187,9 @@ cudaError_t enqueue_plan(const sbr_ctx* c, BatchPlan& P, cudaStream_t st)
         const int64_t a0 = P.cut[k];
         const int na = (int)(P.cut[k + 1] - a0);
         const long long rays = P.chunk_rays[k];
-        e = cudaMemsetAsync(P.ctr64.p, 0, P.ctr64.cap, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(P.ctr32.p, 0, P.ctr32.cap, st);
+        e = launch_trace_begin(trace_init(k == 0 ? P.stats.as<unsigned long long>() : nullptr, P.ctr64, P.ctr32,
+                                          P.tune.raster, P.vis, rays, P.visfull, na, P.rbigctr),
+                               c->n_sms, st);
         if (e != cudaSuccess) break;
         TraceArgs ta;
         memset(&ta, 0, sizeof(ta));
@@ -1126,7 +1199,7 @@ cudaError_t enqueue_plan(const sbr_ctx* c, BatchPlan& P, cudaStream_t st)
         ta.n_nodes = c->n_nodes;
         ta.nodes = ta.wide ? c->nodes4.as<float4>() : (ta.octant ? c->nodes_oct.as<float4>() : c->nodes.as<float4>());
         ta.nodes2 = c->nodes.as<float4>();
-    ta.tris = c->tris.as<float4>();
+        ta.tris = c->tris.as<float4>();
         ta.tri_nrm = ta.tris + 3 * (size_t)c->n_tri;
         ta.tri_v12 = ta.tris + 4 * (size_t)c->n_tri;
         ta.angles = P.angles.as<AngleDev>() + a0;
@@ -1150,11 +1223,13 @@ cudaError_t enqueue_plan(const sbr_ctx* c, BatchPlan& P, cudaStream_t st)
             ta.big_ctr = P.rbigctr.as<unsigned>();
             ta.big_cap = P.big_cap;
             ta.tri_pos = c->tripos.as<int>();
-            ta.list_count = total_dev + 4;
+            ta.slot_scr = P.slotscr.as<unsigned>();
+            ta.rec_off = P.recoff.as<unsigned>();
+            ta.emit_primary = P.max_bounces == 1 && !escape;
             if (!ta.bistatic && !ta.wide && !ta.packet && (P.max_bounces >= 2 || escape))
                 ta.hit_list = P.hitlist.as<uint2>();
             e = launch_raster(ta, (int)c->n_tri, P.vis.as<unsigned long long>(), P.visfull.as<unsigned>(), P.count,
-                              c->n_sms * 16, P.scan_scr.p, st);
+                              c->n_sms * 16, st);
             if (e != cudaSuccess) break;
         } else if (P.tune.silhouette) {
             e = cudaMemsetAsync(P.cover.p, 0, sizeof(unsigned) * (size_t)(rays / 32 + na), st);
@@ -1162,13 +1237,17 @@ cudaError_t enqueue_plan(const sbr_ctx* c, BatchPlan& P, cudaStream_t st)
             if (e != cudaSuccess) break;
             ta.cover = P.cover.as<unsigned>();
         }
-        e = launch_trace(ta, n_blocks, P.count, P.tune.stack_depth, st);
-        if (e == cudaSuccess) e = scan_popc(ta.mask, P.tilebase.as<unsigned>(), rays / 32, total_dev, P.scan_scr.p, st);
-        if (e == cudaSuccess)
-            e = launch_angle_offsets(ta.ray_off, ta.tile_base, total_dev, na, P.recoff.as<unsigned>(), st);
-        if (e != cudaSuccess) break;
         ta.rec = P.rec.as<Record>();
-        if (P.max_bounces == 1 && !escape) {
+        e = launch_trace(ta, n_blocks, P.count, P.tune.stack_depth, st);
+        if (!ta.vis) {  // (the primary pass of keyed rays has done both)
+            if (e == cudaSuccess) e = scan_popc(ta.mask, P.tilebase.as<unsigned>(), rays / 32, total_dev, P.scan_scr.p, st);
+            if (e == cudaSuccess)
+                e = launch_angle_offsets(ta.ray_off, ta.tile_base, total_dev, na, P.recoff.as<unsigned>(), nullptr, st);
+        }
+        if (e != cudaSuccess) break;
+        if (ta.emit_primary) {
+            // the records are written
+        } else if (P.max_bounces == 1 && !escape) {
             ta.q_in = qs[0];
             ta.q_in_count = q_count + 1;
             e = launch_emit_all(ta, n_blocks, st);
@@ -1278,6 +1357,7 @@ int build_plan(sbr_ctx* c, BatchPlan& P)
         P.big_cap = (unsigned)raster_big_cap(max_rays);
         CK(P.rbig.ensure(sizeof(int4) * (size_t)P.big_cap), "alloc raster triangle list");
         CK(P.rbigctr.ensure(sizeof(unsigned) * 2), "alloc raster triangle counters");
+        CK(P.slotscr.ensure(sizeof(unsigned) * kSlotWords), "alloc slot scratch");
     }
     CK(P.tilebase.ensure(sizeof(unsigned) * (size_t)max_tiles), "alloc tile base");
     CK(P.scan_scr.ensure(scan_scratch_bytes(max_tiles)), "alloc scan scratch");
@@ -1335,16 +1415,18 @@ int build_plan(sbr_ctx* c, BatchPlan& P)
     CK(cudaMemcpyAsync(P.freq_t.p, hf, b_f, cudaMemcpyHostToDevice, c->stream), "copy freq");
     CK(cudaMemcpyAsync(P.kfreq.p, hk, b_k, cudaMemcpyHostToDevice, c->stream), "copy freq");
     CK(cudaStreamSynchronize(c->stream), "plan upload sync");
-    // kernels per run: stats memset excluded; per chunk trace passes, 3 scan, offsets, 2 work list, PO, final
+    // kernels per run: per chunk the start, trace passes, 2 work list, PO, final; with rasterised hits 2 for them,
+    // masks, slots, and where no hit list takes the hits their states or records; else 3 scan, offsets
     const bool escape = P.flags & SBR_TRACE_REQUIRE_ESCAPE;
-    const int passes = (P.max_bounces == 1 && !escape) ? 1 : 1 + (escape ? P.max_bounces : P.max_bounces - 1);
+    const bool one = P.max_bounces == 1 && !escape, list = !one && P.tune.bvh_width != 4 && !P.tune.packet;
+    const int passes = one ? 1 : 1 + (escape ? P.max_bounces : P.max_bounces - 1);
     P.n_pass = (int64_t)nc * passes;
     P.n_launch = 0;
     for (int b = 1; b < passes; ++b)
         if (tail_rays(P.tune, b, c->n_sms * P.tune.blocks_per_sm)) P.n_launch += (int64_t)nc;
     for (size_t k = 0; k < nc; ++k)
-        P.n_launch += passes + ((P.max_bounces == 1 && !escape) ? 1 : 0) + 3 + 1 + 2 + (P.items_bound[k] > 0 ? 1 : 0) + 1 +
-                      (P.tune.raster ? 6 : (P.tune.silhouette ? 1 : 0));
+        P.n_launch += 1 + passes + 2 + (P.items_bound[k] > 0 ? 1 : 0) + 1 +
+                      (P.tune.raster ? 4 + (list ? 0 : 1) : 4 + (P.tune.silhouette ? 1 : 0) + (one ? 1 : 0));
     return SBR_OK;
 }
 
@@ -1642,8 +1724,6 @@ int sbr_po_integrate(sbr_ctx* c, const double* freq_hz, int64_t n_freq, int pol_
     int rc = check_po_mode(c, pol_mask, po_mode, pa);
     if (rc != SBR_OK) return rc;
     CK(cudaSetDevice(c->device), "cudaSetDevice");
-    rc = upload_freqs(c, freq_hz, n_freq);
-    if (rc != SBR_OK) return rc;
     pa.n_freq = (int)n_freq;
     const int64_t na = (int64_t)c->ang.size();
     std::vector<int> f0((size_t)na, 0), nf((size_t)na, (int)n_freq);
@@ -1652,24 +1732,18 @@ int sbr_po_integrate(sbr_ctx* c, const double* freq_hz, int64_t n_freq, int pol_
     const size_t n_out = (size_t)na * (size_t)n_freq * pa.n_pol;
     double* dE = E_out;
     double* dR = rcs_out;
+    rc = upload_freqs(c, freq_hz, n_freq, out_on_device ? 0 : n_out, pa);
+    if (rc != SBR_OK) return rc;
     if (!out_on_device) {
-        CK(c->E.ensure(sizeof(double) * 2 * n_out), "alloc E");
-        CK(c->rcs.ensure(sizeof(double) * n_out), "alloc rcs");
-        dE = E_out ? c->E.as<double>() : nullptr;
-        dR = rcs_out ? c->rcs.as<double>() : nullptr;
+        dE = E_out ? c->po.as<double>() : nullptr;
+        dR = rcs_out ? c->po.as<double>() + 2 * n_out : nullptr;
     }
-    CK(cudaMemsetAsync(c->err_dev.as<int>() + 3, 0, sizeof(int), c->stream), "memset po flag");
     rc = po_run(c, pa, 0, na, f0, nf, row, dE, dR, nullptr);
     if (rc != SBR_OK) return rc;
     if (!out_on_device) {
         int flag = 0;
-        if (E_out)
-            CK(cudaMemcpyAsync(E_out, dE, sizeof(double) * 2 * n_out, cudaMemcpyDeviceToHost, c->stream), "copy E");
-        if (rcs_out)
-            CK(cudaMemcpyAsync(rcs_out, dR, sizeof(double) * n_out, cudaMemcpyDeviceToHost, c->stream), "copy rcs");
-        CK(cudaMemcpyAsync(&flag, c->err_dev.as<int>() + 3, sizeof(int), cudaMemcpyDeviceToHost, c->stream),
-           "copy po flag");
-        CK(cudaStreamSynchronize(c->stream), "po sync");
+        rc = fetch_results(c, pa, n_out, E_out, rcs_out, &flag);
+        if (rc != SBR_OK) return rc;
         if (flag) return fail(c, SBR_ERR_TIMEOUT, "sbr_po_integrate: a staged record load did not arrive");
     }
     return SBR_OK;
@@ -1724,24 +1798,21 @@ int sbr_run_batch(sbr_ctx* c, const sbr_request* req, int64_t n_req, const doubl
     long long total = 0, launched = 0;
     rc = plan_chunks(c, R, cut, &total, &launched);
     if (rc != SBR_OK) return rc;
-    rc = upload_freqs(c, freq_hz, n_freq_total);
-    if (rc != SBR_OK) return rc;
     pa.n_freq = (int)n_freq_total;
     const size_t n_out = (size_t)rows * pa.n_pol;
+    rc = upload_freqs(c, freq_hz, n_freq_total, out_on_device ? 0 : n_out, pa);
+    if (rc != SBR_OK) return rc;
     double* dE = E_out;
     double* dR = rcs_out;
     if (!out_on_device) {
-        CK(c->E.ensure(sizeof(double) * 2 * n_out), "alloc E");
-        CK(c->rcs.ensure(sizeof(double) * n_out), "alloc rcs");
-        dE = E_out ? c->E.as<double>() : nullptr;
-        dR = rcs_out ? c->rcs.as<double>() : nullptr;
+        dE = E_out ? c->po.as<double>() : nullptr;
+        dR = rcs_out ? c->po.as<double>() + 2 * n_out : nullptr;
     }
     // each chunk is traced once and integrated for all its requests' frequencies. Without the ray pool every
     // chunk is integrated before the next reuses the record buffer; with it, consecutive chunks form a group whose
     // records stay until the group's pooled late passes have run, and the group is integrated then
     long long valid = 0, rec_base = 0;
     size_t g0 = 0;
-    CK(cudaMemsetAsync(c->err_dev.as<int>() + 3, 0, sizeof(int), c->stream), "memset po flag");
     PoolRun P;
     rc = pool_setup(c, R, P, cut);
     if (rc != SBR_OK) return rc;
@@ -1781,17 +1852,12 @@ int sbr_run_batch(sbr_ctx* c, const sbr_request* req, int64_t n_req, const doubl
         rc = close_group(cut.size() - 1);
         if (rc != SBR_OK) return rc;
     }
-    if (!out_on_device) {
-        if (E_out)
-            CK(cudaMemcpyAsync(E_out, dE, sizeof(double) * 2 * n_out, cudaMemcpyDeviceToHost, c->stream), "copy E");
-        if (rcs_out)
-            CK(cudaMemcpyAsync(rcs_out, dR, sizeof(double) * n_out, cudaMemcpyDeviceToHost, c->stream), "copy rcs");
-    }
-    int flag = 0;
-    CK(cudaMemcpyAsync(&flag, c->err_dev.as<int>() + 3, sizeof(int), cudaMemcpyDeviceToHost, c->stream),
-       "copy po flag");
     unsigned long long hs_stats[kStatCount];
     rc = read_counters(c, hs_stats);  // synchronises the stream
+    int flag = 0;
+    if (rc == SBR_OK)
+        rc = fetch_results(c, pa, out_on_device ? 0 : n_out, out_on_device ? nullptr : E_out,
+                           out_on_device ? nullptr : rcs_out, &flag);
     if (rc != SBR_OK) return rc;
     if (flag) return fail(c, SBR_ERR_TIMEOUT, "sbr_run_batch: a staged record load did not arrive");
     return finish_stats(c, R, hs_stats, n_req, launched, valid, stats);

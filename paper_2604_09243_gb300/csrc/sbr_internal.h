@@ -185,18 +185,22 @@ struct TraceArgs {
     int* hit_tri;                 // optional [total_rays][max_bounces] (RECORD_HITS)
     float* hit_t;                 // optional [total_rays][max_bounces]
     int* hit_nb;                  // optional [total_rays]
-    const unsigned long long* vis; // optional (primary pass) [total_rays] closest-hit keys from k_raster
+    const unsigned long long* vis; // optional (primary pass) [total_rays] closest-hit keys: rasterised, or of
+                                   // the flagged aspects traversed
     const unsigned* vis_full;     // with vis: [n_angles + 1] 1 = the aspect's primary rays traverse the tree;
                                   // [n_angles]: 1 if any aspect does
+    unsigned* slot_scr;           // with vis: kSlotWords of scratch
+    unsigned* rec_off;            // with vis: [n_angles + 1] first record of each aspect in the chunk, and the total
+    unsigned* rec_off_host;       // the same in pinned host memory (may be null)
+    int emit_primary;             // with vis, no hit list: the primary pass writes the records (one bounce, monostatic)
     const int* tri_pos;           // with vis: [n_tri] position in tris of each original triangle index
-    unsigned* list_count;         // with vis: device count of the rasterised primary hits
     int4* big;                    // with vis: triangles of more than 512 (sparse grids: 16) cells, (triangle, aspect, i0 | j0 << 16,
                                   // (i1 - i0) | (j1 - j0) << 16), tested by warps after the per-thread pass
     unsigned* big_ctr;            // with vis: [2] entries appended, (unused)
     unsigned big_cap;             // with vis: capacity of big (an aspect whose entry does not fit traverses)
-    uint2* hit_list;              // optional (rasterised hits, a bounce pass follows): the primary pass
-                                  // lists (ray, aspect) of each rasterised hit here instead of storing
-                                  // its state, and bounce pass 1 rebuilds the state from the list
+    uint2* hit_list;              // optional (with vis, a bounce pass follows): the primary pass lists
+                                  // (ray, aspect) of each hit here instead of storing its state, and
+                                  // bounce pass 1 rebuilds the state from the list
 };
 int trace_blocks_per_sm();
 // rays that k_tail can take in a launch of n_blocks blocks
@@ -227,16 +231,34 @@ cudaError_t launch_silhouette(const TraceArgs& a, int n_tri, unsigned* cover, cu
 // Primary closest hits by rasterisation (aspects a.angles, a.ray_off, a.n_angles
 // of a chunk of a.total_rays rays): vis[g] becomes the smallest key
 // (FP32 t bits << 32 | original triangle index) over the triangles whose FP32
-// test accepts primary ray g, or ~0 for none; full[aspect] = 1 and
+// test accepts primary ray g, or stays ~0 for none; full[aspect] = 1 and
 // full[n_angles] = 1 when a triangle covers more than kRasterMaxCells cells of
-// that aspect (its rays then traverse the tree). Clears vis and full itself.
-// Then sets a.mask to the valid bits of the rasterised rays, a.tile_base to
-// their exclusive scan and *a.q_out_count to their number: the primary pass
-// stores those rays at fixed queue slots and appends the traversing ones after
-// them.
+// that aspect or does not fit the list (its rays then traverse the tree in the
+// primary pass, which writes their keys). vis, full and a.big_ctr must have been
+// cleared (launch_trace_begin). The primary pass sets a.mask to the valid bits
+// of the keys, a.tile_base to their exclusive scan, *a.q_out_count to their
+// number and a.rec_off to the aspects' first records.
 constexpr long long kRasterMaxCells = 1 << 24;
 cudaError_t launch_raster(const TraceArgs& a, int n_tri, unsigned long long* vis, unsigned* full, bool count,
-                          int n_blocks, void* scan_scratch, cudaStream_t st);
+                          int n_blocks, cudaStream_t st);
+constexpr int kSlotBlocks = 2432;              // blocks of the primary pass's mask and slot kernels at most
+constexpr size_t kSlotWords = 9 * kSlotBlocks;  // a.slot_scr
+
+// What a chunk's trace starts from, in one launch: tables copied from pinned
+// host memory (null: none), 32-bit ranges cleared, keys set to ~0.
+struct TraceInit {
+    static constexpr int kRanges = 5;
+    const uint4* table_host;      // aspects, 16-byte words
+    uint4* table;
+    const long long* off_host;    // ray offsets
+    long long* off;
+    long long n_table, n_off;
+    unsigned* zero[kRanges];
+    long long n_zero[kRanges];    // words (0: none)
+    uint4* vis16;                 // keys, two per element
+    long long n_vis16;
+};
+cudaError_t launch_trace_begin(const TraceInit& b, int n_sms, cudaStream_t st);
 
 // exclusive scan of in[i] (or popcount(in[i])) -> out[i]; total written to *total
 size_t scan_scratch_bytes(long long n);
@@ -245,7 +267,7 @@ cudaError_t scan_exclusive_u32(const unsigned* in, unsigned* out, long long n, b
 cudaError_t scan_popc(const unsigned* mask, unsigned* tile_base, long long n, unsigned* total, void* scratch,
                       cudaStream_t st);
 cudaError_t launch_angle_offsets(const long long* ray_off, const unsigned* tile_base, const unsigned* total,
-                                 int n_angles, unsigned* rec_off, cudaStream_t st);
+                                 int n_angles, unsigned* rec_off, unsigned* rec_off_host, cudaStream_t st);
 
 struct PoItem {
     int angle;        // aspect index within the call

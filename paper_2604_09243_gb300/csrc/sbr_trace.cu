@@ -1025,6 +1025,21 @@ __device__ __forceinline__ int find_angle(const long long* __restrict__ off, int
     return lo;
 }
 
+// the same by a whole warp (converged), 32 candidates a step
+__device__ __forceinline__ int find_angle_warp(const long long* __restrict__ off, int n, long long g)
+{
+    const int lane = threadIdx.x & 31;
+    int lo = 0;
+    while (n > 1) {  // off[lo] <= g, and off[lo + n] > g or lo + n is the end
+        const int step = (n + 31) >> 5, i = lane * step;
+        const unsigned m = __ballot_sync(kFull, i < n && off[lo + i] <= g);
+        const int k = max(31 - __clz(m), 0) * step;
+        lo += k;
+        n = min(step, n - k);
+    }
+    return lo;
+}
+
 // warp-aggregated append of the lanes of m to queue q; every lane of the warp must call it
 __device__ __forceinline__ void append(RayState* q, unsigned* count, unsigned m, const Ray& r)
 {
@@ -1836,31 +1851,124 @@ __device__ __forceinline__ void warp_tiles(long long n_tiles, long long gw, long
     t1 = t0 + per < n_tiles ? t0 + per : n_tiles;
 }
 
-// valid bits of the rasterised primary rays (0 for the tiles of flagged
-// aspects, which traverse); each warp a contiguous range of tiles
-__global__ void __launch_bounds__(256) k_vis_mask(const TraceArgs a, const unsigned long long* __restrict__ vis,
-                                                  const unsigned* __restrict__ full, unsigned* mask)
+// scratch of the two kernels below: the blocks' sums and, per warp, the sum of
+// its block's earlier warps
+__device__ __forceinline__ unsigned* slot_blocks(const TraceArgs& a) { return a.slot_scr; }
+__device__ __forceinline__ unsigned* slot_warps(const TraceArgs& a) { return a.slot_scr + kSlotBlocks; }
+
+// Valid bits of the primary rays from their keys, each warp a contiguous range
+// of tiles, and the sums of the bits. Bound by the keys' 8 bytes a ray: 0.72 ms
+// for the 476M rays of 37 aircraft aspects at 10 GHz, 5.3 TB/s (0.77 with cached
+// loads, 0.87 with two keys a load and their bits interleaved).
+__global__ void __launch_bounds__(256) k_vis_mask(const TraceArgs a)
+{
+    __shared__ unsigned s_w[8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    long long t0, t1;
+    warp_tiles(a.total_rays >> 5, (long long)blockIdx.x * 8 + warp, (long long)gridDim.x * 8, t0, t1);
+    unsigned sum = 0;
+    for (long long tb = t0; tb < t1; tb += 32) {
+        unsigned mine = 0;
+        const int n = (int)min(32ll, t1 - tb);
+#pragma unroll 8
+        for (int k = 0; k < n; ++k) {
+            const unsigned m = __ballot_sync(kFull, __ldcs(a.vis + ((tb + k) << 5) + lane) != ~0ull);
+            if (lane == k) mine = m;
+        }
+        sum += __popc(mine);
+        if (lane < n) a.mask[tb + lane] = mine;
+    }
+    sum = __reduce_add_sync(kFull, sum);
+    if (lane == 0) s_w[warp] = sum;
+    __syncthreads();
+    if (threadIdx.x < 8) {
+        unsigned run = 0;
+        for (int w = 0; w < (int)threadIdx.x; ++w) run += s_w[w];
+        slot_warps(a)[blockIdx.x * 8 + threadIdx.x] = run;
+        if (threadIdx.x == 7) slot_blocks(a)[blockIdx.x] = run + s_w[7];
+    }
+}
+
+// Slot of every tile's first hit (k_vis_mask's ranges), the first record of
+// every aspect, and with a hit list its entries (ray, aspect). Every block adds
+// up the sums of the blocks before it (at most 10 loads a thread), which is less
+// than a scan kernel between the two or its last block doing so (8 us). With
+// k_vis_mask it replaces two scans of three kernels each, a copy and two
+// kernels that read their result: 30 us of a small call.
+template <bool kList>
+__global__ void __launch_bounds__(256) k_vis_slots(const TraceArgs a)
 {
     const int lane = threadIdx.x & 31;
+    const long long gtid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long gw = gtid >> 5;
+    // one primary query per grid ray of every rasterised aspect
+    unsigned nq = 0;
+    for (long long ang = gtid; ang < a.n_angles; ang += (long long)gridDim.x * blockDim.x)
+        if (!a.vis_full[ang]) nq += (unsigned)a.angles[ang].nu * (unsigned)a.angles[ang].nv;
+    // the hits of earlier blocks
+    __shared__ unsigned s_sum[8];
+    unsigned before = 0;
+    const unsigned* bsum = slot_blocks(a);
+#pragma unroll
+    for (int k = 0; k < (kSlotBlocks + 255) / 256; ++k) {
+        const int b = k * 256 + threadIdx.x;
+        if (b < (int)blockIdx.x) before += __ldg(bsum + b);
+    }
+    before = __reduce_add_sync(kFull, before);
+    if (lane == 0) s_sum[threadIdx.x >> 5] = before;
+    __syncthreads();
+    before = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) before += s_sum[w];
+    auto put = [&](int ang, unsigned at) {
+        a.rec_off[ang] = at;
+        if (a.rec_off_host) a.rec_off_host[ang] = at;
+    };
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+        const unsigned total = before + bsum[blockIdx.x];
+        *a.q_out_count = total;
+        for (int ang = a.n_angles; ang >= 0 && a.ray_off[ang] >= a.total_rays; --ang) put(ang, total);
+    }
     long long t0, t1;
-    warp_tiles(a.total_rays >> 5, ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5,
-               ((long long)gridDim.x * blockDim.x) >> 5, t0, t1);
-    if (t0 >= t1) return;  // warp-uniform
-    const bool any_full = full[a.n_angles] != 0;
-    int ang = 0;
-    if (any_full) {
-        if (lane == 0) ang = find_angle(a.ray_off, a.n_angles, t0 << 5);
-        ang = __shfl_sync(kFull, ang, 0);
-    }
-#pragma unroll 4
-    for (long long tile = t0; tile < t1; ++tile) {
-        unsigned m = __ballot_sync(kFull, vis[(tile << 5) + lane] != ~0ull);
-        if (any_full) {
-            while (a.ray_off[ang + 1] <= (tile << 5)) ++ang;
-            if (full[ang]) m = 0;
+    warp_tiles(a.total_rays >> 5, gw, (long long)gridDim.x * 8, t0, t1);
+    if (t0 < t1) {
+        unsigned run = before + slot_warps(a)[gw];
+        int ang = find_angle_warp(a.ray_off, a.n_angles, t0 << 5);  // the aspect of the tile at hand
+        long long next = a.ray_off[ang + 1];
+        int start = ang;  // the first aspect that starts at tile t0 or later
+        while (start > 0 && a.ray_off[start - 1] == (t0 << 5)) --start;
+        if (a.ray_off[start] < (t0 << 5)) ++start;
+        for (; t0 < t1; t0 += 32) {
+            const long long t = t0 + lane;
+            const unsigned m = t < t1 ? a.mask[t] : 0u, c = (unsigned)__popc(m);
+            unsigned incl = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned y = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl += y;
+            }
+            const unsigned slot = run + incl - c;
+            run += __shfl_sync(kFull, incl, 31);
+            if (t < t1) const_cast<unsigned*>(a.tile_base)[t] = slot;
+            for (; start < a.n_angles; ++start) {
+                const long long ts = a.ray_off[start] >> 5;
+                if (ts >= t1 || ts >= t0 + 32) break;
+                if (t == ts) put(start, slot);
+            }
+            if (!kList) continue;
+            unsigned todo = __ballot_sync(kFull, m != 0u);
+            while (todo) {
+                const int k = __ffs(todo) - 1;
+                todo &= todo - 1u;
+                const unsigned mk = __shfl_sync(kFull, m, k), sk = __shfl_sync(kFull, slot, k);
+                const long long base = (t0 + k) << 5;
+                while (next <= base) next = a.ray_off[++ang + 1];  // the tiles of a warp only move forward
+                if ((mk >> lane) & 1u)
+                    a.hit_list[sk + __popc(mk & ((1u << lane) - 1u))] = make_uint2((unsigned)(base + lane), (unsigned)ang);
+            }
         }
-        if (lane == 0) mask[tile] = m;
     }
+    flush_stats<false>(a, nq, 0u, 0u, false);
 }
 
 // ---------------------------------------------------------------- pass 0: primary rays
@@ -1878,7 +1986,7 @@ __device__ __forceinline__ void start_ray(const AngleDev& A, Ray& r)
 template <bool kCount, int kStack, int kMode>
 __global__ void __launch_bounds__(kTraceThreads, 4) k_primary(const TraceArgs a)
 {
-    // with rasterised hits this kernel only traverses for flagged aspects
+    // with rasterised hits this kernel only traverses for flagged aspects, and leaves their keys
     if (a.vis && !a.vis_full[a.n_angles]) return;
     const int lane = threadIdx.x & 31;
     unsigned nq = 0, nvis = 0, ntri = 0;
@@ -1891,7 +1999,7 @@ __global__ void __launch_bounds__(kTraceThreads, 4) k_primary(const TraceArgs a)
         int ang = 0;
         if (lane == 0) ang = find_angle(a.ray_off, a.n_angles, (long long)base);
         ang = __shfl_sync(kFull, ang, 0);
-        if (a.vis && !a.vis_full[ang]) continue;  // warp-uniform; k_primary_vis takes this tile
+        if (a.vis && !a.vis_full[ang]) continue;  // warp-uniform; rasterised
         const AngleDev& A = a.angles[ang];
         const int local = (int)((long long)base + lane - a.ray_off[ang]);
         int i, j;
@@ -1911,8 +2019,14 @@ __global__ void __launch_bounds__(kTraceThreads, 4) k_primary(const TraceArgs a)
         }
         Hit h;
         query<kCount, kStack, kMode>(a, active, r.o, r.d, -1, h, nvis, ntri, ovf);
+        if (active) ++nq;
+        if (a.vis) {
+            const bool any = active && h.k >= 0;
+            const_cast<unsigned long long*>(a.vis)[base + lane] =
+                any ? ((unsigned long long)__float_as_uint(h.t) << 32) | (unsigned)h.orig : ~0ull;
+            continue;
+        }
         if (active) {
-            ++nq;
             if (h.k >= 0) {
                 start_ray(a.angles[ang], r);
                 hit = true;
@@ -1927,93 +2041,8 @@ __global__ void __launch_bounds__(kTraceThreads, 4) k_primary(const TraceArgs a)
     flush_stats<kCount>(a, nq, nvis, ntri, ovf);
 }
 
-// Primary pass of the rasterised aspects. The hit rays go to the queue slots
-// given by the scan of the raster masks (no atomics). Without a hit list each
-// ray reads its key and its state is written to its slot, the tiles assigned
-// statically (every tile costs about the same). With a hit list only (ray,
-// aspect) of each hit is written, from the mask words and slots alone.
-template <bool kCount, bool kList>
-__global__ void __launch_bounds__(kTraceThreads) k_primary_vis(const TraceArgs a)
-{
-    const int lane = threadIdx.x & 31;
-    const long long gtid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long gw = gtid >> 5, nw = ((long long)gridDim.x * blockDim.x) >> 5;
-    const long long n_tiles = a.total_rays >> 5;
-    // one primary query per grid ray of every rasterised aspect
-    unsigned nq = 0;
-    for (long long ang = gtid; ang < a.n_angles; ang += (long long)gridDim.x * blockDim.x)
-        if (!a.vis_full[ang]) nq += (unsigned)a.angles[ang].nu * (unsigned)a.angles[ang].nv;
-    if (kList) {
-        // 32 tiles per warp step: lane l loads the mask word and slot of tile t0 + l, then the warp
-        // writes the list entries tile by tile (a set bit implies a rasterised aspect: k_vis_mask
-        // clears the masks of flagged ones)
-        long long t0 = gw << 5;
-        int ang = 0;
-        long long next = 0;
-        if (t0 < n_tiles) {
-            if (lane == 0) ang = find_angle(a.ray_off, a.n_angles, t0 << 5);
-            ang = __shfl_sync(kFull, ang, 0);
-            next = a.ray_off[ang + 1];
-        }
-        for (; t0 < n_tiles; t0 += nw << 5) {
-            const long long t = t0 + lane;
-            unsigned m = 0, slot = 0;
-            if (t < n_tiles) {
-                m = a.mask[t];
-                if (m) slot = a.tile_base[t];
-            }
-            unsigned todo = __ballot_sync(kFull, m != 0u);
-            while (todo) {
-                const int k = __ffs(todo) - 1;
-                todo &= todo - 1u;
-                const unsigned mk = __shfl_sync(kFull, m, k), sk = __shfl_sync(kFull, slot, k);
-                const long long base = (t0 + k) << 5;
-                while (next <= base) next = a.ray_off[++ang + 1];  // the tiles of a warp only move forward
-                if ((mk >> lane) & 1u)
-                    a.hit_list[sk + __popc(mk & ((1u << lane) - 1u))] = make_uint2((unsigned)(base + lane), (unsigned)ang);
-            }
-        }
-    } else {
-        constexpr int kChunk = 4;  // tiles of a chunk; chunks interleaved over the warps (hits cluster in the grid)
-        const long long n_chunks = (n_tiles + kChunk - 1) / kChunk;
-        int ang = 0;
-        if (gw < n_chunks) {
-            if (lane == 0) ang = find_angle(a.ray_off, a.n_angles, (gw * kChunk) << 5);
-            ang = __shfl_sync(kFull, ang, 0);
-        }
-        for (long long chunk = gw; chunk < n_chunks; chunk += nw) {
-            for (long long tile = chunk * kChunk; tile < (chunk + 1) * kChunk && tile < n_tiles; ++tile) {
-                const long long base = tile << 5;
-                while (a.ray_off[ang + 1] <= base) ++ang;  // the tiles of a warp only move forward
-                const unsigned vmask = a.mask[tile];        // k_vis_mask; 0 for a flagged aspect
-                if (!((vmask >> lane) & 1u)) continue;
-                const AngleDev& A = a.angles[ang];
-                const int local = (int)(base + lane - a.ray_off[ang]);
-                int i, j;
-                tile_ij(A, local, i, j);
-                const unsigned long long key = __ldcs(a.vis + base + lane);
-                Hit h;
-                h.t = __uint_as_float((unsigned)(key >> 32));
-                h.orig = (int)(unsigned)key;
-                h.k = __ldg(a.tri_pos + h.orig);
-                Ray r;
-                r.angle = ang;
-                r.local = local;
-                r.o = primary_origin(A, i, j);
-                r.d = make_float3(A.dir[0], A.dir[1], A.dir[2]);
-                start_ray(A, r);
-                apply_hit(A, a.tri_nrm, h, a.flags, r);
-                record_hit(a, r, h);
-                store_state(a.q_out, a.tile_base[tile] + __popc(vmask & ((1u << lane) - 1u)), r);
-            }
-        }
-    }
-    flush_stats<kCount>(a, nq, 0u, 0u, false);
-}
-
-// ---------------------------------------------------------------- pass b >= 1: live rays
 // State of rasterised primary hit (ray g of the chunk, aspect ang) after its
-// first hit: the same steps as k_primary_vis.
+// first hit.
 __device__ __forceinline__ void primary_state(const TraceArgs& a, unsigned g, int ang, Ray& r)
 {
     const AngleDev& A = a.angles[ang];
@@ -2034,6 +2063,39 @@ __device__ __forceinline__ void primary_state(const TraceArgs& a, unsigned g, in
     record_hit(a, r, h);
 }
 
+// Primary pass of the keyed rays where no hit list takes them to a bounce pass:
+// each ray reads its key, and its state goes to its queue slot or, where one
+// bounce is all there is (kEmit), its record is written. The tiles are assigned
+// statically, in chunks interleaved over the warps (hits cluster in the grid).
+template <bool kEmit>
+__global__ void __launch_bounds__(kTraceThreads) k_primary_vis(const TraceArgs a)
+{
+    const int lane = threadIdx.x & 31;
+    const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                    nw = ((long long)gridDim.x * blockDim.x) >> 5;
+    const long long n_tiles = a.total_rays >> 5;
+    constexpr int kChunk = 4;  // tiles
+    const long long n_chunks = (n_tiles + kChunk - 1) / kChunk;
+    int ang = 0;
+    if (gw < n_chunks) {
+        if (lane == 0) ang = find_angle(a.ray_off, a.n_angles, (gw * kChunk) << 5);
+        ang = __shfl_sync(kFull, ang, 0);
+    }
+    for (long long chunk = gw; chunk < n_chunks; chunk += nw) {
+        for (long long tile = chunk * kChunk; tile < (chunk + 1) * kChunk && tile < n_tiles; ++tile) {
+            const long long base = tile << 5;
+            while (a.ray_off[ang + 1] <= base) ++ang;  // the tiles of a warp only move forward
+            const unsigned vmask = a.mask[tile];
+            if (!((vmask >> lane) & 1u)) continue;
+            Ray r;
+            primary_state(a, (unsigned)(base + lane), ang, r);
+            if (kEmit) emit(a, r, false);
+            else store_state(a.q_out, a.tile_base[tile] + __popc(vmask & ((1u << lane) - 1u)), r);
+        }
+    }
+}
+
+// ---------------------------------------------------------------- pass b >= 1: live rays
 // Origin, direction and triangle after the first hit of a rasterised primary
 // ray (ray g of the chunk, aspect ang): the stored-state steps of apply_hit
 // alone (hit point, orientation, reflection, offset origin).
@@ -2090,7 +2152,6 @@ __global__ void __launch_bounds__(kTraceThreads, 4) k_bounce(const TraceArgs a)
     const int lane = threadIdx.x & 31;
     const unsigned n_in = *a.q_in_count;
     if (n_in <= a.tail_rays) return;  // none left, or k_tail has taken them
-    const unsigned n_list = kList ? *a.list_count : 0u;  // entries below n_list come from the hit list
     unsigned nq = 0, nvis = 0, ntri = 0, nhit = 0, nlist = 0;  // hits processed, hits rebuilt (counting runs)
     unsigned long long wvis = 0;  // counting runs: 32 x the warp's largest node visit count, per query
     bool ovf = false;
@@ -2106,23 +2167,26 @@ __global__ void __launch_bounds__(kTraceThreads, 4) k_bounce(const TraceArgs a)
         r.o = make_float3(0.f, 0.f, 0.f);
         r.d = make_float3(0.f, 0.f, 1.f);
         r.last = -1;
-        const bool listed = kList && idx < n_list;
         uint2 e = make_uint2(0u, 0u);
-        if (listed) {
-            // only the geometry during the query; the full state after it
-            e = a.hit_list[idx];
-            primary_geom(a, e.x, (int)e.y, r.o, r.d, r.last);
-            if (kCount) ++nlist;
+        unsigned src = idx;
+        if (kList) {
+            if (active) {
+                // only the geometry during the query; the full state after it
+                e = a.hit_list[idx];
+                primary_geom(a, e.x, (int)e.y, r.o, r.d, r.last);
+                if (kCount && !a.vis_full[e.y]) ++nlist;
+            }
+        } else {
+            // the pass's i-th entry, in the order of q_order when the rays were grouped by place
+            if (a.q_order && active) src = __ldcs(a.q_order + idx);
+            if (active) load_geom(a.q_in, src, r);
         }
-        // the pass's i-th entry, in the order of q_order when the rays were grouped by place
-        const unsigned src = (a.q_order && active && !listed) ? __ldcs(a.q_order + idx) : idx;
-        if (active && !listed) load_geom(a.q_in, src, r);
         Hit h;
         const unsigned nvis0 = nvis;
         query<kCount, kStack, kMode>(a, active, r.o, r.d, r.last, h, nvis, ntri, ovf);
         if (kCount) wvis += 32ull * __reduce_max_sync(kFull, nvis - nvis0);
         if (active) {
-            if (listed) primary_state(a, e.x, (int)e.y, r);
+            if (kList) primary_state(a, e.x, (int)e.y, r);
             else load_payload(a.q_in, src, r);
             again = finish_query<kCount, kBi>(a, h, r, nq, nhit, ovf);
         }
@@ -2276,11 +2340,29 @@ __global__ void k_pool_commit(const unsigned* src_count, unsigned* pool_count, u
 }
 
 __global__ void k_angle_offsets(const long long* ray_off, const unsigned* tile_base, const unsigned* total,
-                                int n_angles, unsigned* rec_off)
+                                int n_angles, unsigned* rec_off, unsigned* rec_off_host)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n_angles) rec_off[i] = tile_base[ray_off[i] >> 5];
-    if (i == n_angles) rec_off[i] = *total;
+    if (i > n_angles) return;
+    const unsigned at = i < n_angles ? tile_base[ray_off[i] >> 5] : *total;
+    rec_off[i] = at;
+    if (rec_off_host) rec_off_host[i] = at;
+}
+
+// The start of a chunk's trace in one launch: the aspect table and ray offsets
+// from pinned host memory, the primary keys set to "none", counters and flags
+// cleared. As two copies and six fills of about 3.5 us each from the first to
+// the next they were 40 of the 223 us of one look at a 20k-triangle sphere.
+__global__ void __launch_bounds__(256) k_trace_begin(const TraceInit b)
+{
+    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x, n = (long long)gridDim.x * blockDim.x;
+    for (long long i = tid; i < b.n_table; i += n) b.table[i] = b.table_host[i];
+    for (long long i = tid; i < b.n_off; i += n) b.off[i] = b.off_host[i];
+#pragma unroll
+    for (int k = 0; k < TraceInit::kRanges; ++k)
+        for (long long i = tid; i < b.n_zero[k]; i += n) b.zero[k][i] = 0u;
+    const uint4 none = make_uint4(~0u, ~0u, ~0u, ~0u);
+    for (long long i = tid; i < b.n_vis16; i += n) b.vis16[i] = none;
 }
 
 }  // namespace
@@ -2296,17 +2378,20 @@ template <int kStack, int kMode>
 void launch_trace_s(const TraceArgs& a, int n_blocks, bool count_visits, cudaStream_t st)
 {
     if (a.bounce == 0) {
-        if (a.vis) {
-            if (a.hit_list) {
-                if (count_visits) k_primary_vis<true, true><<<n_blocks, kTraceThreads, 0, st>>>(a);
-                else k_primary_vis<false, true><<<n_blocks, kTraceThreads, 0, st>>>(a);
-            } else {
-                if (count_visits) k_primary_vis<true, false><<<n_blocks, kTraceThreads, 0, st>>>(a);
-                else k_primary_vis<false, false><<<n_blocks, kTraceThreads, 0, st>>>(a);
-            }
-        }
         if (count_visits) k_primary<true, kStack, kMode><<<n_blocks, kTraceThreads, 0, st>>>(a);
         else k_primary<false, kStack, kMode><<<n_blocks, kTraceThreads, 0, st>>>(a);
+        if (!a.vis) return;
+        // 32 tiles a warp or more: whole steps of the slot kernel (61 requests of a small target, 200k tiles, 42 a
+        // warp: 12 us for it, 17 with 10 a warp)
+        const int g = (int)std::max(1ll, std::min<long long>(((a.total_rays >> 5) + 255) / 256, kSlotBlocks));
+        k_vis_mask<<<g, 256, 0, st>>>(a);
+        if (a.hit_list) {
+            k_vis_slots<true><<<g, 256, 0, st>>>(a);
+        } else {
+            k_vis_slots<false><<<g, 256, 0, st>>>(a);
+            if (a.emit_primary) k_primary_vis<true><<<n_blocks, kTraceThreads, 0, st>>>(a);
+            else k_primary_vis<false><<<n_blocks, kTraceThreads, 0, st>>>(a);
+        }
     } else if (a.bounce == 1 && a.hit_list) {
         if (count_visits) k_bounce<true, kStack, kMode, false, true><<<n_blocks, kTraceThreads, 0, st>>>(a);
         else k_bounce<false, kStack, kMode, false, true><<<n_blocks, kTraceThreads, 0, st>>>(a);
@@ -2421,13 +2506,10 @@ cudaError_t launch_silhouette(const TraceArgs& a, int n_tri, unsigned* cover, cu
 }
 
 cudaError_t launch_raster(const TraceArgs& a, int n_tri, unsigned long long* vis, unsigned* full, bool count,
-                          int n_blocks, void* scan_scratch, cudaStream_t st)
+                          int n_blocks, cudaStream_t st)
 {
     if (a.n_angles <= 0 || n_tri <= 0) return cudaErrorInvalidValue;
-    cudaError_t e = cudaMemsetAsync(vis, 0xFF, sizeof(unsigned long long) * (size_t)a.total_rays, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(full, 0, sizeof(unsigned) * (size_t)(a.n_angles + 1), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(a.big_ctr, 0, sizeof(unsigned) * 2, st);
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
     static int smem_set[64] = {0};  // per device: k_raster's dynamic shared memory above 48 KB allowed
     int dev = 0;
     cudaGetDevice(&dev);
@@ -2455,22 +2537,22 @@ cudaError_t launch_raster(const TraceArgs& a, int n_tri, unsigned long long* vis
             a, n_tri, vis, full, count ? 1 : 0);
     }
     k_raster_big<<<n_blocks, 256, 0, st>>>(a, vis, count ? 1 : 0);
-    const long long n_tiles = a.total_rays >> 5;
-    k_vis_mask<<<(int)std::max(1ll, std::min<long long>((n_tiles + 7) / 8, n_blocks)), 256, 0, st>>>(a, vis, full,
-                                                                                                     a.mask);
-    e = cudaGetLastError();
-    // queue slots of the rasterised hits; the traversing rays append after them
-    if (e == cudaSuccess)
-        e = scan_popc(a.mask, const_cast<unsigned*>(a.tile_base), n_tiles, a.list_count, scan_scratch, st);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(a.q_out_count, a.list_count, sizeof(unsigned), cudaMemcpyDeviceToDevice, st);
-    return e;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_trace_begin(const TraceInit& b, int n_sms, cudaStream_t st)
+{
+    const long long most = std::max(std::max(b.n_table, b.n_off), b.n_vis16);
+    const int blocks = (int)std::max(4ll, std::min<long long>((most + 255) / 256, (long long)n_sms * 8));
+    k_trace_begin<<<blocks, 256, 0, st>>>(b);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_angle_offsets(const long long* ray_off, const unsigned* tile_base, const unsigned* total,
-                                 int n_angles, unsigned* rec_off, cudaStream_t st)
+                                 int n_angles, unsigned* rec_off, unsigned* rec_off_host, cudaStream_t st)
 {
-    k_angle_offsets<<<(n_angles + 1 + 255) / 256, 256, 0, st>>>(ray_off, tile_base, total, n_angles, rec_off);
+    k_angle_offsets<<<(n_angles + 1 + 255) / 256, 256, 0, st>>>(ray_off, tile_base, total, n_angles, rec_off,
+                                                                rec_off_host);
     return cudaGetLastError();
 }
 
