@@ -1141,7 +1141,9 @@ struct BatchPlan {
     PoArgs pa;
     // device buffers
     DevBuf angles, rayoff, pang, recoff, mask, tilebase, scan_scr, q0, q1, ctr64, ctr32, stats, rec, items, nitems,
-        valid, freq_t, kfreq, partial, cover, vis, visfull, hitlist, rbig, rbigctr, slotscr;
+        freq_t, kfreq, partial, cover, vis, visfull, hitlist, rbig, rbigctr, slotscr;
+    // stats: the counters, then each chunk's record count; the batch's last step copies them here (pinned)
+    unsigned long long* stats_host = nullptr;
     cudaStream_t cap = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -1155,9 +1157,10 @@ void free_plan(BatchPlan* p)
     if (p->cap) cudaStreamDestroy(p->cap);
     DevBuf* all[] = {&p->angles, &p->rayoff, &p->pang,   &p->recoff, &p->mask,   &p->tilebase, &p->scan_scr,
                      &p->q0,     &p->q1,     &p->ctr64,  &p->ctr32,  &p->stats,  &p->rec,      &p->items,
-                     &p->nitems, &p->valid,  &p->freq_t, &p->kfreq,  &p->partial, &p->cover,
+                     &p->nitems, &p->freq_t, &p->kfreq,  &p->partial, &p->cover,
                      &p->vis,    &p->visfull, &p->hitlist, &p->rbig, &p->rbigctr, &p->slotscr};
     for (DevBuf* b : all) b->release();
+    if (p->stats_host) cudaFreeHost(p->stats_host);
     delete p;
 }
 
@@ -1268,7 +1271,7 @@ cudaError_t enqueue_plan(const sbr_ctx* c, BatchPlan& P, cudaStream_t st)
         PoAngle* pang = P.pang.as<PoAngle>() + a0;
         if (e == cudaSuccess)
             e = launch_po_items(P.recoff.as<unsigned>(), pang, na, P.pa.n_pol, P.tune.po_item, P.items.as<PoItem>(),
-                                P.nitems.as<int>(), P.valid.as<long long>() + k, st);
+                                P.nitems.as<int>(), P.stats.as<long long>() + kStatCount + k, st);
         if (e == cudaSuccess && P.items_bound[k] > 0) {
             PoArgs pa = P.pa;
             pa.rec = P.rec.as<Record>();
@@ -1285,6 +1288,9 @@ cudaError_t enqueue_plan(const sbr_ctx* c, BatchPlan& P, cudaStream_t st)
             e = launch_po_final(P.partial.as<double>(), P.items.as<PoItem>(), pang, na, P.max_nf, P.kfreq.as<double>(),
                                 P.pa.n_pol, P.E, P.R, st);
     }
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(P.stats_host, P.stats.p, sizeof(unsigned long long) * (kStatCount + P.cut.size() - 1),
+                            cudaMemcpyDeviceToHost, st);
     return e;
 }
 
@@ -1365,11 +1371,12 @@ int build_plan(sbr_ctx* c, BatchPlan& P)
     CK(P.q1.ensure(sizeof(RayState) * (size_t)max_rays), "alloc ray queue");
     CK(P.ctr64.ensure(sizeof(unsigned long long) * 2 * (kMaxBounces + 2)), "alloc counters");
     CK(P.ctr32.ensure(sizeof(unsigned) * 2 * (kMaxBounces + 2) + 64), "alloc counters");
-    CK(P.stats.ensure(sizeof(unsigned long long) * kStatCount), "alloc stats");
+    const size_t b_stats = sizeof(unsigned long long) * (kStatCount + nc);
+    CK(P.stats.ensure(b_stats), "alloc stats");
+    CK(cudaMallocHost((void**)&P.stats_host, b_stats), "alloc stats copy");
     CK(P.rec.ensure(sizeof(Record) * (size_t)std::max(max_rec, 1ll)), "alloc records");
     CK(P.items.ensure(sizeof(PoItem) * (size_t)std::max(max_items, 1ll)), "alloc items");
     CK(P.nitems.ensure(sizeof(int)), "alloc item count");
-    CK(P.valid.ensure(sizeof(long long) * nc), "alloc valid counts");
     CK(P.partial.ensure(sizeof(double) * (size_t)std::max(max_part, 1ll)), "alloc partials");
     CK(P.freq_t.ensure(sizeof(float4) * P.freq.size()), "alloc freq");
     CK(P.kfreq.ensure(sizeof(double) * P.freq.size()), "alloc freq");
@@ -1957,14 +1964,11 @@ int sbr_sync(sbr_ctx* c, sbr_trace_stats* stats)
     CK(cudaSetDevice(c->device), "cudaSetDevice");
     BatchPlan& P = *c->plan;
     const size_t nc = P.cut.size() - 1;
-    unsigned long long hs[kStatCount];
-    std::vector<long long> hv(nc);
     CK(cudaStreamSynchronize(c->stream), "batch sync");
-    CK(cudaMemcpy(hs, P.stats.p, sizeof(hs), cudaMemcpyDeviceToHost), "copy stats");
-    CK(cudaMemcpy(hv.data(), P.valid.p, sizeof(long long) * nc, cudaMemcpyDeviceToHost), "copy valid counts");
     c->plan_pending = false;
+    const unsigned long long* hs = P.stats_host;
     long long valid = 0;
-    for (long long v : hv) valid += v;
+    for (size_t k = 0; k < nc; ++k) valid += (long long)hs[kStatCount + k];
     if (stats) {
         memset(stats, 0, sizeof(*stats));
         stats->n_angles = (int64_t)P.req.size();

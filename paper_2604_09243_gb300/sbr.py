@@ -87,6 +87,9 @@ class Request(C.Structure):
                 ("freq_offset", C.c_int64), ("n_freq", C.c_int32), ("reserved", C.c_int32)]
 
 
+_REQUEST = np.dtype([(n, "f8" if t is C.c_double else ("i8" if t is C.c_int64 else "i4")) for n, t in Request._fields_])
+
+
 class RayGrid(C.Structure):
     _fields_ = [("nu", C.c_int64), ("nv", C.c_int64), ("lu", C.c_double), ("lv", C.c_double),
                 ("spacing", C.c_double), ("eps", C.c_double),
@@ -471,13 +474,17 @@ class Context:
 def _requests(requests):
     """(list of request dicts, sbr_request array, concatenated frequency array)."""
     reqs = list(requests)
-    freqs = np.ascontiguousarray(np.concatenate([np.atleast_1d(np.asarray(r["freqs"], np.float64)) for r in reqs]))
+    parts = [np.asarray(r["freqs"], np.float64) for r in reqs]
+    parts = [p if p.ndim else p.reshape(1) for p in parts]
+    freqs = np.ascontiguousarray(np.concatenate(parts))
+    # the fields column by column into the array's memory (61 requests: 90 us with a structure each)
     arr = (Request * len(reqs))()
-    off = 0
-    for k, r in enumerate(reqs):
-        nf = len(np.atleast_1d(r["freqs"]))
-        arr[k] = Request(float(r["az"]), float(r["el"]), float(r["spacing"]), off, nf, 0)
-        off += nf
+    view = np.frombuffer(arr, _REQUEST)
+    for name, key in (("az_deg", "az"), ("el_deg", "el"), ("ray_spacing_m", "spacing")):
+        view[name] = [float(r[key]) for r in reqs]
+    nf = np.array([len(p) for p in parts], np.int64)
+    view["n_freq"] = nf
+    view["freq_offset"] = np.cumsum(nf) - nf
     return reqs, arr, freqs
 
 
