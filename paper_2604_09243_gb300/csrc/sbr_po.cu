@@ -49,6 +49,22 @@ __device__ __forceinline__ void phase_cs(const PoArgs& a, float4 fq, double kd, 
     }
 }
 
+// 2 r of phase_cs's compensated form for two tubes at a frequency (x, -x and y
+// twice each), every operation the same rounding on both halves: with the
+// product negated, n - p = fma(rint(-p), -1, -p) and r = fma(n - p, -1, e).
+__device__ __forceinline__ float2 phase_arg2(float2 fx, float2 nx, float2 fy, float2 lh, float2 ll)
+{
+    const float2 m1 = make_float2(-1.f, -1.f);
+    const float2 np = __fmul2_rn(nx, lh);
+    float2 e = __ffma2_rn(fx, lh, np);
+    // (scalar additions: a packed product and the packed addition that takes it are contracted to one rounding)
+    const float2 u = __fmul2_rn(fx, ll), v = __fmul2_rn(fy, lh);
+    e = __fadd2_rn(e, make_float2(__fadd_rn(u.x, v.x), __fadd_rn(u.y, v.y)));
+    const float2 q = __ffma2_rn(make_float2(rintf(np.x), rintf(np.y)), m1, np);
+    const float2 r = __ffma2_rn(q, m1, e);
+    return __fadd2_rn(r, r);
+}
+
 // Sums of kN values over a warp, every sum in the order of the plain butterfly
 // (lane distance 16, 8, 4, 2, 1). As long as a lane holds several values it
 // keeps one half of them and sends its partner the other, so that kN values
@@ -86,11 +102,12 @@ __device__ __forceinline__ int warp_sum_index(int lane)
 // frequencies at a time when kPol = 2, two when kPol = 4, one barrier each
 // (the partial sums of consecutive reductions alternate between two buffers).
 // Each sum is formed in the same order whatever kPol, so the results do not
-// depend on it. Bound by instruction issue (~45 per tube and frequency in the
-// phase and its products): 9 aspects of 175k tubes, 201 frequencies, 4
-// polarisations in 472 us, 670 G tube-frequencies/s; 635 us with every sum
-// exchanged at every step of the butterfly and the other phase modes' code in
-// the loop.
+// depend on it. Bound by instruction issue (~40 per tube and frequency in the
+// phase, sine, cosine and products): 9 aspects of 175k tubes, 201 frequencies, 4
+// polarisations in 450 us, 703 G tube-frequencies/s; 472 us with one tube at a
+// time (two now share the packed FP32 instructions, and a cosine and a sine
+// their products), 635 us with every sum exchanged at every step of the
+// butterfly and the other phase modes' code in the loop.
 constexpr int kSums = 16;
 template <int kPoPer, int kPol, bool kComp>
 __global__ void __launch_bounds__(kPoThreads) k_po(const PoArgs a)
@@ -102,10 +119,11 @@ __global__ void __launch_bounds__(kPoThreads) k_po(const PoArgs a)
     int buf = 0;
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
         const PoItem I = a.items[item];
-        float cf[kPoPer][kPol];
-        float lh[kPoPer], ll[kPoPer];
+        float2 cf[kPoPer][kPol];  // (c, -c): factors of the cosine and sine
+        float2 lh[kPoPer / 2], ll[kPoPer / 2];
 #pragma unroll
         for (int k = 0; k < kPoPer; ++k) {
+            float xh = 0.f, xl = 0.f;
             const int idx = k * kPoThreads + tid;
             if (idx < I.count) {
                 const float4* p = reinterpret_cast<const float4*>(a.rec + I.first + idx);
@@ -117,37 +135,58 @@ __global__ void __launch_bounds__(kPoThreads) k_po(const PoArgs a)
                     const float vec = sel == 0 ? x.x : (sel == 1 ? x.y : (sel == 2 ? x.z : x.w));
                     float v = 0.f;
                     if (q < a.n_pol) v = a.scalar ? (sel < 2 ? y.x : 0.f) : vec;
-                    cf[k][q] = v;
+                    cf[k][q] = make_float2(v, -v);
                 }
-                lh[k] = y.y;
-                ll[k] = y.z;
+                xh = y.y;
+                xl = y.z;
             } else {
 #pragma unroll
-                for (int q = 0; q < kPol; ++q) cf[k][q] = 0.f;
-                lh[k] = 0.f;
-                ll[k] = 0.f;
+                for (int q = 0; q < kPol; ++q) cf[k][q] = make_float2(0.f, 0.f);
+            }
+            if (k & 1) {
+                lh[k / 2].y = xh;
+                ll[k / 2].y = xl;
+            } else {
+                lh[k / 2].x = xh;
+                ll[k / 2].x = xl;
             }
         }
         for (int f0 = 0; f0 < I.nf; f0 += kF, buf ^= 1) {
-            float acc[kSums];
+            float2 sum2[kSums / 2];  // (re, im)
 #pragma unroll
-            for (int v = 0; v < kSums; ++v) acc[v] = 0.f;
+            for (int v = 0; v < kSums / 2; ++v) sum2[v] = make_float2(0.f, 0.f);
 #pragma unroll
             for (int fj = 0; fj < kF; ++fj) {
                 if (f0 + fj >= I.nf) break;
                 const float4 fq = a.freq[I.f0 + f0 + fj];
                 const double kd = kComp ? 0.0 : a.kfreq[I.f0 + f0 + fj];
+                const float2 fx = make_float2(fq.x, fq.x), nx = make_float2(-fq.x, -fq.x), fy = make_float2(fq.y, fq.y);
 #pragma unroll
-                for (int k = 0; k < kPoPer; ++k) {
+                for (int k = 0; k < kPoPer; k += 2) {
+                    // (a tube past the item's end adds zeros)
                     if (k * kPoThreads + tid >= I.count) break;
-                    float c, s;
-                    phase_cs<kComp>(a, fq, kd, lh[k], ll[k], c, s);
+                    float2 e0, e1;  // (cos, sin)
+                    if (kComp) {
+                        const float2 t = phase_arg2(fx, nx, fy, lh[k / 2], ll[k / 2]);
+                        sincospif(t.x, &e0.y, &e0.x);
+                        sincospif(t.y, &e1.y, &e1.x);
+                    } else {
+                        phase_cs<kComp>(a, fq, kd, lh[k / 2].x, ll[k / 2].x, e0.x, e0.y);
+                        phase_cs<kComp>(a, fq, kd, lh[k / 2].y, ll[k / 2].y, e1.x, e1.y);
+                    }
 #pragma unroll
                     for (int q = 0; q < kPol; ++q) {
-                        acc[(fj * kPol + q) * 2] = fmaf(cf[k][q], c, acc[(fj * kPol + q) * 2]);
-                        acc[(fj * kPol + q) * 2 + 1] = fmaf(-cf[k][q], s, acc[(fj * kPol + q) * 2 + 1]);
+                        float2& v = sum2[fj * kPol + q];
+                        v = __ffma2_rn(cf[k][q], e0, v);
+                        v = __ffma2_rn(cf[k + 1][q], e1, v);
                     }
                 }
+            }
+            float acc[kSums];
+#pragma unroll
+            for (int v = 0; v < kSums / 2; ++v) {
+                acc[2 * v] = sum2[v].x;
+                acc[2 * v + 1] = sum2[v].y;
             }
             const float sum = warp_sums<kSums>(acc);
             if ((lane & 1) == 0) s_red[buf][w][warp_sum_index<kSums>(lane)] = sum;
