@@ -1234,13 +1234,6 @@ __device__ __forceinline__ void tri_cell_edges(const AngleDev& A, float ids, flo
     tri_cell_edges_p(pr, i0, i1, j0, j1, E);
 }
 
-__device__ __forceinline__ bool cell_inside(const CellEdges& E, int di, int dj)
-{
-    const float x = (float)di, y = (float)dj;
-    return fmaf(E.nx[0], x, fmaf(E.ny[0], y, E.c[0])) <= 0.f && fmaf(E.nx[1], x, fmaf(E.ny[1], y, E.c[1])) <= 0.f &&
-           fmaf(E.nx[2], x, fmaf(E.ny[2], y, E.c[2])) <= 0.f;
-}
-
 __global__ void __launch_bounds__(256) k_silhouette(const float4* __restrict__ tris, int n_tri,
                                                     const AngleDev* __restrict__ angles,
                                                     const long long* __restrict__ ray_off, int n_angles,
@@ -1400,7 +1393,7 @@ __device__ __forceinline__ void raster_cell(const RasterGrid& G, const TraceArgs
 //   g0 = (p0.x, p0.y, p0.z, du.x)   g1 = (du.y, du.z, dv.x, dv.y)   g2 = (dv.z, v0.x, v0.y, v0.z)
 //   r0 = (p.x, p.y, p.z, p2.x)      r1 = (p2.y, p2.z, nn.x, nn.y)   r2 = (nn.z, det, bd, bU)
 //   r3 = (bV, bT, n.x, n.y)         r4 = (n.z, dh, dl, rd)           [plane key K]
-//   e0 = (nx0, ny0, c0, nx1)        e1 = (ny1, c1, nx2, ny2)         e2 = (c2, 1 / w, tnear, ray_off)
+//   e0 = (nx0, ny0, c0, nx1)        e1 = (ny1, c1, nx2, ny2)         e2 = (c2, -, tnear, ray_off)
 //   m0 = (i0, j0, w, orig)          m1 = (aspect, triangle, nbu, tw)
 // tnear: below the smallest stored distance any cell of the range can give
 // this triangle (a cell whose ray already holds a closer hit is skipped).
@@ -1455,19 +1448,79 @@ __device__ __forceinline__ void append_big(const TraceArgs& a, unsigned* full, b
     }
 }
 
+// The cells of row y inside an item's moved edges: columns [lo, lo + cnt) of
+// w <= 65536, found on the values of a cell's pretest (nx x + g <= 0 is
+// x <= -g / nx) and widened by more than the quotient's error, so that no cell
+// the pretest passes is left out. Each triangle's box holds about three times
+// the cells of the triangle itself (29M and 9M for an aircraft aspect at
+// 10 GHz); testing them one by one left two lanes of three idle in the exact
+// test that follows: k_raster 8.2 ms for 37 such aspects, 4.7 with spans.
+__device__ __forceinline__ void row_span(const float* nx, const float* ny, const float* c, float y, int w, int& lo, int& cnt)
+{
+    float x0 = 0.f, x1 = (float)(w - 1);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const float g = fmaf(ny[k], y, c[k]), q = __fdividef(-g, nx[k]);
+        if (nx[k] >= 1e-20f) x1 = fminf(x1, q);
+        else if (nx[k] <= -1e-20f) x0 = fmaxf(x0, q);
+        else if (g > 1e-15f) x1 = -1.f;  // along the row (either zero): all of its cells or none
+    }
+    // (a quotient may be infinite or none: 0 <= lo <= w + 1, -1 <= the last column < w)
+    const float tol = fmaf((float)w, 1e-6f, 0.01f);
+    lo = __float2int_ru(fminf(x0, (float)(w + 1)) - tol);
+    lo = max(lo, 0);
+    cnt = max(min(__float2int_rd(fmaxf(x1, -1.f) + tol), w - 1) - lo + 1, 0);
+}
+
+// Calls cell(k, row, column) for the cells of the lanes' rows (row `row` of
+// triangle k < 32, columns [lo, lo + cnt)), 32 cells at a time, one per lane.
+// A warp's rows hold fewer than 65,536 cells before the last one. spans: the
+// warp's 32 entries; every lane calls it.
+template <class Cell>
+__device__ __forceinline__ void each_cell(uint2* spans, int k, int row, int lo, int cnt, Cell cell)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned le = 0xFFFFFFFFu >> (31 - lane);
+    int end = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(kFull, end, o);
+        if (lane >= o) end += y;
+    }
+    const int start = end - cnt, cells = __shfl_sync(kFull, end, 31);
+    const unsigned some = __ballot_sync(kFull, cnt > 0);
+    // the rows with cells, in order: first cell number | triangle, row | first column
+    if (cnt > 0) spans[__popc(some & (le >> 1))] = make_uint2(start | (k << 16), row | (lo << 16));
+    __syncwarp();
+    for (int cb = 0; cb < cells; cb += 32) {
+        // lane l's row: the last one that starts at cell cb + l or before
+        const unsigned at = (unsigned)(start - cb);
+        const unsigned starts = __reduce_or_sync(kFull, cnt > 0 && at < 32u ? 1u << at : 0u);
+        const int earlier = __popc(__ballot_sync(kFull, cnt > 0 && start < cb));
+        if (cb + lane < cells) {
+            const uint2 s = spans[earlier + __popc(starts & le) - 1];
+            cell((int)(s.x >> 16), (int)(s.y & 0xFFFFu), (int)(s.y >> 16) + cb + lane - (int)(s.x & 0xFFFFu));
+        }
+    }
+    __syncwarp();  // spans[] may be rewritten
+}
+
 // Items q = aspect * n_tri + triangle, one per lane in grid-stride order
 // (aspect-major: neighbouring lanes take neighbouring triangles of one
 // aspect). Each lane projects its triangle and, for a range of at most
 // kRasterFlat cells, writes the triangle's constants to shared memory; the
-// warp then walks the (triangle, cell) pairs of its 32 triangles, lane l taking
-// pairs l, l + 32, ..., so every lane works until the warp's cells run out. A
-// triangle with a larger range is appended to the list `big` (warp-aggregated)
-// for k_raster_big. Each cell passes the edge pretest before the triangle test.
+// warp then walks the rows of its 32 triangles, 32 at a time, a row per lane,
+// and the cells of these rows' spans, a cell per lane (each_cell), so every
+// lane works until the warp's cells run out. A triangle with a larger range is
+// appended to the list `big` (warp-aggregated) for k_raster_big. Bound by
+// instruction issue (66 %, 25.5 lanes; 17.5 lanes and 1.8 times the
+// instructions when every cell of a box was a lane's).
 __global__ void __launch_bounds__(256, 4) k_raster(const TraceArgs a, int n_tri, unsigned long long* vis, unsigned* full,
                                                    int count)
 {
     extern __shared__ RasterItem s_items[];
     __shared__ int s_off[kRasterWarps][33];
+    __shared__ uint2 s_span[kRasterWarps][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     RasterItem* my = s_items + warp * 32;
     int* off = s_off[warp];
@@ -1481,7 +1534,7 @@ __global__ void __launch_bounds__(256, 4) k_raster(const TraceArgs a, int n_tri,
     for (unsigned long long base = q0 - lane; base < n_items; base += stride) {
         bool want_big = false;
         int4 rng = make_int4(0, 0, 0, 0);
-        int nc = 0;
+        int nr = 0;  // rows of the lane's triangle
         if (base + lane < n_items) {
             const AngleDev& A = a.angles[ang];
             const float4* tp = a.tris + 3 * (size_t)t;
@@ -1533,20 +1586,20 @@ __global__ void __launch_bounds__(256, 4) k_raster(const TraceArgs a, int n_tri,
                         const float zm = fminf(z0, fminf(z1, z2));
                         const float slack = K.dh != 0.f ? 0.32f * B.w / fabsf(K.dh) : FLT_MAX;
                         const float tnear = zm - (1e-4f * fabsf(zm) + 1e-3f + slack);
-                        it.e2 = make_float4(c2, 1.f / (float)(i1 - i0 + 1), isfinite(tnear) ? tnear : -FLT_MAX,
+                        it.e2 = make_float4(c2, 0.f, isfinite(tnear) ? tnear : -FLT_MAX,
                                             __int_as_float((int)a.ray_off[ang]));
                         it.g0 = make_float4(G.p0.x, G.p0.y, G.p0.z, G.du.x);
                         it.g1 = make_float4(G.du.y, G.du.z, G.dv.x, G.dv.y);
                         it.m0 = make_int4(i0, j0, i1 - i0 + 1, __float_as_int(P.w));
                         it.m1 = make_int4(ang, t, G.nbu, G.tw);
-                        nc = (int)ncell;
+                        nr = j1 - j0 + 1;
                     }
                 }
             }
         }
         append_big(a, full, want_big, t, ang, rng.x, rng.y, rng.z, rng.w);
-        // inclusive scan of the cell counts: off[k] = first pair of lane k's triangle
-        int incl = nc;
+        // inclusive scan of the rows: off[k] = first row of lane k's triangle
+        int incl = nr;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int y = __shfl_up_sync(kFull, incl, o);
@@ -1557,56 +1610,57 @@ __global__ void __launch_bounds__(256, 4) k_raster(const TraceArgs a, int n_tri,
         __syncwarp();
         const int total = __shfl_sync(kFull, incl, 31);
         int k = 0;
-        for (int c = lane; c < total; c += 32) {
-            while (off[k + 1] <= c) ++k;
-            const RasterItem& it = my[k];
-            const int loc = c - off[k];
-            const int4 m0 = it.m0;
-            const float4 e0 = it.e0, e1 = it.e1, e2 = it.e2;
-            // (loc + 0.5) / w is at least 0.5 / w from an integer and loc, w <= 512: the FP32 product floors exactly
-            const int dj = __float2int_rz(((float)loc + 0.5f) * e2.y), di = loc - dj * m0.z;
-            {
-                const float x = (float)di, y = (float)dj;
-                if (!(fmaf(e0.x, x, fmaf(e0.y, y, e0.z)) <= 0.f && fmaf(e0.w, x, fmaf(e1.x, y, e1.y)) <= 0.f &&
-                      fmaf(e1.z, x, fmaf(e1.w, y, e2.x)) <= 0.f))
-                    continue;
+        for (int rb = 0; rb < total; rb += 32) {
+            int cnt = 0, lo = 0, row = 0;
+            if (rb + lane < total) {
+                while (off[k + 1] <= rb + lane) ++k;
+                const RasterItem& it = my[k];
+                const float4 e0 = it.e0, e1 = it.e1, e2 = it.e2;
+                const float nx[3] = {e0.x, e0.w, e1.z}, ny[3] = {e0.y, e1.x, e1.w}, c[3] = {e0.z, e1.y, e2.x};
+                row = rb + lane - off[k];
+                row_span(nx, ny, c, (float)row, it.m0.z, lo, cnt);
             }
-            const int i = m0.x + di, j = m0.y + dj;
-            const int4 m1 = it.m1;
-            const int tw = m1.w, sh = 5 - tw;  // tile of W = 2^tw by H = 2^sh rays
-            const long long pidx = (long long)__float_as_int(e2.w) + ((long long)((j >> sh) * m1.z + (i >> tw)) << 5) +
-                                   ((j & ((1 << sh) - 1)) << tw) + (i & ((1 << tw) - 1));
-            // the ray's closest hit so far (keys only decrease; a stale value is larger): nearer than any
-            // distance this triangle can give, the cell is decided
-            if (__uint_as_float((unsigned)(__ldcg(vis + pidx) >> 32)) < e2.z) continue;
-            ++ntri;
-            const float4 g0 = it.g0, g1 = it.g1, g2 = it.g2;
-            const float fi = (float)i, fj = (float)j;
-            const float3 o = make_float3(__fadd_rn(__fadd_rn(g0.x, __fmul_rn(fi, g0.w)), __fmul_rn(fj, g1.z)),
-                                         __fadd_rn(__fadd_rn(g0.y, __fmul_rn(fi, g1.x)), __fmul_rn(fj, g1.w)),
-                                         __fadd_rn(__fadd_rn(g0.z, __fmul_rn(fi, g1.y)), __fmul_rn(fj, g2.x)));
-            const float3 v0 = make_float3(g2.y, g2.z, g2.w);
-            const float3 sv = make_float3(__fsub_rn(o.x, v0.x), __fsub_rn(o.y, v0.y), __fsub_rn(o.z, v0.z));
-            const float4 r0 = it.r0, r1 = it.r1, r2 = it.r2, r3 = it.r3;
-            float tc, et;
-            const int f = filter_core(dot_s(sv, make_float3(r0.x, r0.y, r0.z)), dot_s(sv, make_float3(r0.w, r1.x, r1.y)),
-                                      dot_s(sv, make_float3(r1.z, r1.w, r2.x)), r2.y, r2.w, r3.x, r2.z, r3.y, tc, et);
-            if (f == 0) continue;
-            if (f >= 2) {
-                const AngleDev& A = a.angles[m1.x];
-                const int r = tri_refine(a.tris, a.tri_v12, m1.y, o, make_float3(A.dir[0], A.dir[1], A.dir[2]), f, tc);
-                if (count) count_open(a.stats, r);
-                if (!(r & 1)) continue;
-            }
-            const float4 r4 = it.r4;
-            PlaneKey K;
-            K.n = make_float3(r3.z, r3.w, r4.x);
-            K.dh = r4.y;
-            K.dl = r4.z;
-            K.rd = r4.w;
-            const float th = plane_key_t(K, v0, o, tc);
-            if (th >= 0.f && th <= FLT_MAX)
-                atomicMin(vis + pidx, ((unsigned long long)__float_as_uint(th) << 32) | (unsigned)m0.w);
+            each_cell(s_span[warp], k, row, lo, cnt, [&](int tri, int dj, int di) {
+                const RasterItem& it = my[tri];
+                const int4 m0 = it.m0;
+                const float4 e2 = it.e2;
+                const int i = m0.x + di, j = m0.y + dj;
+                const int4 m1 = it.m1;
+                const int tw = m1.w, sh = 5 - tw;  // tile of W = 2^tw by H = 2^sh rays
+                const long long pidx = (long long)__float_as_int(e2.w) + ((long long)((j >> sh) * m1.z + (i >> tw)) << 5) +
+                                       ((j & ((1 << sh) - 1)) << tw) + (i & ((1 << tw) - 1));
+                // the ray's closest hit so far (keys only decrease; a stale value is larger): nearer than any
+                // distance this triangle can give, the cell is decided
+                if (__uint_as_float((unsigned)(__ldcg(vis + pidx) >> 32)) < e2.z) return;
+                ++ntri;
+                const float4 g0 = it.g0, g1 = it.g1, g2 = it.g2;
+                const float fi = (float)i, fj = (float)j;
+                const float3 o = make_float3(__fadd_rn(__fadd_rn(g0.x, __fmul_rn(fi, g0.w)), __fmul_rn(fj, g1.z)),
+                                             __fadd_rn(__fadd_rn(g0.y, __fmul_rn(fi, g1.x)), __fmul_rn(fj, g1.w)),
+                                             __fadd_rn(__fadd_rn(g0.z, __fmul_rn(fi, g1.y)), __fmul_rn(fj, g2.x)));
+                const float3 v0 = make_float3(g2.y, g2.z, g2.w);
+                const float3 sv = make_float3(__fsub_rn(o.x, v0.x), __fsub_rn(o.y, v0.y), __fsub_rn(o.z, v0.z));
+                const float4 r0 = it.r0, r1 = it.r1, r2 = it.r2, r3 = it.r3;
+                float tc, et;
+                const int f = filter_core(dot_s(sv, make_float3(r0.x, r0.y, r0.z)), dot_s(sv, make_float3(r0.w, r1.x, r1.y)),
+                                          dot_s(sv, make_float3(r1.z, r1.w, r2.x)), r2.y, r2.w, r3.x, r2.z, r3.y, tc, et);
+                if (f == 0) return;
+                if (f >= 2) {
+                    const AngleDev& A = a.angles[m1.x];
+                    const int r = tri_refine(a.tris, a.tri_v12, m1.y, o, make_float3(A.dir[0], A.dir[1], A.dir[2]), f, tc);
+                    if (count) count_open(a.stats, r);
+                    if (!(r & 1)) return;
+                }
+                const float4 r4 = it.r4;
+                PlaneKey K;
+                K.n = make_float3(r3.z, r3.w, r4.x);
+                K.dh = r4.y;
+                K.dl = r4.z;
+                K.rd = r4.w;
+                const float th = plane_key_t(K, v0, o, tc);
+                if (th >= 0.f && th <= FLT_MAX)
+                    atomicMin(vis + pidx, ((unsigned long long)__float_as_uint(th) << 32) | (unsigned)m0.w);
+            });
         }
         __syncwarp();  // the next round rewrites my[] and off[]
         t += step_t;
@@ -1628,13 +1682,15 @@ __global__ void __launch_bounds__(256, 4) k_raster(const TraceArgs a, int n_tri,
 
 // The listed large triangles, warp w taking entries w, w + warps, ... (every
 // warp has hundreds of entries, so the few very large triangles average out),
-// their cells 32 at a time.
+// the cells of their rows' spans 32 at a time (0.16 ms for 37 aircraft aspects
+// at 10 GHz, 0.70 with every cell of the box a lane's).
 __global__ void __launch_bounds__(256, 3) k_raster_big(const TraceArgs a, unsigned long long* vis, int count)
 {
     const int lane = threadIdx.x & 31;
     const unsigned n_big = min(a.big_ctr[0], a.big_cap);
     const unsigned nw = (gridDim.x * blockDim.x) >> 5;
     unsigned long long ntri = 0;
+    __shared__ uint2 s_span[8][32];
     for (unsigned it = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < n_big; it += nw) {
         const int4 b = a.big[it];
         const int td = b.x, ad = b.y;
@@ -1651,21 +1707,13 @@ __global__ void __launch_bounds__(256, 3) k_raster_big(const TraceArgs a, unsign
         const PlaneKey K = plane_key(a.tri_nrm, td, G.d);
         CellEdges E;
         tri_cell_edges(A, cell_scale(A), P, B, C, i0, i1, j0, j1, E);
-        const int ncell = w * h;
-        // cell c = (c / w, c % w) from (j0, i0); steps of 32 cells: sj rows and si columns
-        const int sj = 32 / w, si = 32 - sj * w, l0 = lane / w;
-        int i = i0 + (lane - l0 * w), j = j0 + l0;
-        for (int cidx = lane; cidx < ncell; cidx += 32) {
-            if (cell_inside(E, i - i0, j - j0)) {
-                raster_cell(G, a, R, K, td, orig, i, j, vrow, count);
+        for (int rb = 0; rb < h; rb += 32) {
+            int lo = 0, cnt = 0;
+            if (rb + lane < h) row_span(E.nx, E.ny, E.c, (float)(rb + lane), w, lo, cnt);
+            each_cell(s_span[threadIdx.x >> 5], 0, rb + lane, lo, cnt, [&](int, int dj, int di) {
+                raster_cell(G, a, R, K, td, orig, i0 + di, j0 + dj, vrow, count);
                 ++ntri;
-            }
-            i += si;
-            j += sj;
-            if (i > i1) {
-                i -= w;
-                ++j;
-            }
+            });
         }
     }
     if (count) {
@@ -2520,10 +2568,10 @@ cudaError_t launch_raster(const TraceArgs& a, int n_tri, unsigned long long* vis
         smem_set[dev] = 1;
     }
     const long long per_aspect = a.total_rays / a.n_angles;
-    // Twice as many triangles as rays or more, down to half as many (primary pass of 40 aspects, sparse against
-    // k_raster, ms): 983k triangles at 0.14 rays per triangle 0.52 / 1.29, 0.57: 1.16 / 1.94, 1.29: 2.23 / 2.59;
-    // 97k triangles at 1.45: 0.31 / 0.36, 5.8: 1.15 / 0.87; 10k at 0.6: 0.067 / 0.069, 3.8: 0.132 / 0.120
-    if (per_aspect < 2ll * n_tri) {
+    // Fewer than three rays for two triangles (primary pass of 40 aspects, sparse against k_raster, ms): 983k
+    // triangles at 0.14 rays per triangle 0.48 / 1.33, 0.57: 1.06 / 1.70, 1.29: 1.99 / 2.19; 97k triangles at 0.71:
+    // 0.171 / 0.218, 1.45: 0.265 / 0.267, 5.8: 1.16 / 0.52; 10k at 0.6: 0.052 / 0.056, 1.36: 0.064 / 0.060
+    if (2 * per_aspect < 3ll * n_tri) {
         // as many aspects per triangle as leave every resident warp a few items
         const long long n_blk = ((long long)n_tri + 31) / 32;
         int aspects = kSparseAspects;
