@@ -146,8 +146,11 @@ cudaError_t bvh_build(const BvhBuild& b, cudaStream_t st);
 struct TraceArgs {
     const float4* nodes;          // binary nodes, or 4-wide nodes when wide = 1
     const float4* nodes2;         // binary nodes (visibility queries, whatever the traversal)
+    const float4* nodes4;         // 4-wide nodes (k_trapped)
     unsigned tail_rays;           // bounce pass: when at most this many rays are left, k_tail follows them to their
                                   // end (0: never); the pass kernel then returns
+    unsigned* hand_count;         // with tail_rays: k_tail hands the rays that go on after some bounces to q_out and
+                                  // counts them here, and k_trapped follows those (null: it follows all itself)
     int wide;
     int packet;                   // 1: warp-cooperative traversal of the binary tree
     int bistatic;                 // 1: some aspect of the chunk has a bistatic receiver (visibility tests)

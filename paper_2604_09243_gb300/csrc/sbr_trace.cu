@@ -2251,7 +2251,10 @@ __global__ void __launch_bounds__(kTraceThreads, 4) k_bounce(const TraceArgs a)
 // queue slot between them; the rays are spread over all warps, so few share one.
 // Up to one ray per resident thread (155,648): with more, the lanes whose rays
 // have ended are worth the compaction between passes. aircraft_deep_cavity
-// (3 GHz, 45 aspects, 100 bounces): 22.5 -> 11.9 ms.
+// (3 GHz, 45 aspects, 100 bounces): 22.5 -> 11.9 ms. Rays still there after
+// kHandAfter bounces are trapped: where many more may follow (a.hand_count) they
+// go to k_trapped.
+constexpr int kHandAfter = 10;
 template <bool kCount, int kStack, int kMode, bool kBi>
 __global__ void __launch_bounds__(kTraceThreads, 4) k_tail(const TraceArgs a)
 {
@@ -2271,6 +2274,7 @@ __global__ void __launch_bounds__(kTraceThreads, 4) k_tail(const TraceArgs a)
     r.d = make_float3(0.f, 0.f, 1.f);
     r.last = -1;
     if (active) load_geom(q, src, r);
+    int turn = 0;
     while (__any_sync(kFull, active)) {
         Hit h;
         const unsigned nvis0 = nvis;
@@ -2282,10 +2286,181 @@ __global__ void __launch_bounds__(kTraceThreads, 4) k_tail(const TraceArgs a)
             load_state(q, src, r);
             r.o = o, r.d = d, r.last = last;
             active = finish_query<kCount, kBi>(a, h, r, nq, nhit, ovf);
-            if (active) store_state(q, src, r);
         }
+        if (!kCount && a.hand_count && ++turn == kHandAfter) {
+            const unsigned left = __ballot_sync(kFull, active);
+            if (left) append(a.q_out, a.hand_count, left, r);
+            break;
+        }
+        if (active) store_state(q, src, r);
     }
     flush_stats<kCount>(a, nq, nvis, ntri, ovf, nhit, 0u, (threadIdx.x & 31) == 0 ? wvis : 0ull);
+}
+
+// Closest hits of 32 / kCoopLanes rays by a warp, kCoopLanes lanes each (o, d,
+// skip and the result the same in every lane of a ray; has: there is one). Up to
+// kCoopLanes / 4 4-wide nodes are taken from a stack at a time, a lane per
+// child, the nearest on top, and up to kCoopLanes triangles of the leaves
+// reached, a lane each, their loads in flight together: a ray's chain of
+// dependent fetches is as long as the tree is deep instead of one for every node
+// and triangle it meets. Every lane keeps its own candidates and the smallest
+// (t32, original triangle index) is taken at the end, so the hit is that of any
+// other order of visits. A nearly full stack is left to one node at a time;
+// false where the children did not fit all the same (the caller's to trace).
+constexpr int kCoopLanes = 32, kCoopStack = 128, kCoopWide = 40, kCoopTris = kCoopLanes + kCoopLanes * 16;
+struct CoopQueue {
+    int2 node[kCoopStack];  // node, its near distance
+    int tri[kCoopTris];
+};
+__device__ __forceinline__ bool closest_hit_coop(const TraceArgs& a, CoopQueue& q, bool has, float3 o, float3 d, int skip,
+                                                 Hit& h)
+{
+    const int lane = threadIdx.x & 31, at0 = lane & ~(kCoopLanes - 1), l = lane - at0, g = l >> 2, c = l & 3;
+    constexpr unsigned kRay = kCoopLanes == 32 ? kFull : (1u << (kCoopLanes & 31)) - 1u;
+    const unsigned lt = (1u << l) - 1u;
+    const float3 inv = make_float3(safe_rcp(d.x), safe_rcp(d.y), safe_rcp(d.z));
+    const float3 oi = make_float3(o.x * inv.x, o.y * inv.y, o.z * inv.z);
+    h.t = FLT_MAX;
+    h.k = -1;
+    h.orig = INT_MAX;
+    h.lo = FLT_MAX;
+    h.key = -1.f;
+    float tmax = FLT_MAX;
+    int sp = has ? 1 : 0, tp = 0;
+    bool fits = true;
+    if (l == 0) q.node[0] = make_int2(0, 0);
+    for (int it = 0; it < a.visit_limit && __any_sync(kFull, sp > 0 || tp > 0); ++it) {
+        __syncwarp();
+        const int nt = min(kCoopLanes, tp);
+        tp -= nt;
+        const int n = tp > 0 ? 0 : min(sp > kCoopWide ? 1 : kCoopLanes / 4, sp);
+        const int2 e = g < n ? q.node[sp - 1 - g] : make_int2(0, 0);
+        const int k = l < nt ? q.tri[tp + l] : skip;
+        sp -= n;
+        const bool open = g < n && __int_as_float(e.y) <= tmax * kBoxGrow;
+        const float* nd = reinterpret_cast<const float*>(a.nodes4 + (size_t)kNode4Float4 * e.x) + c;
+        const float4* tq = a.tris + 3 * (size_t)k;
+        float b[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        int ref = kEmptyRef;
+        float4 A = make_float4(0.f, 0.f, 0.f, 0.f), B = A, C = A;
+        if (open) {
+#pragma unroll
+            for (int u = 0; u < 6; ++u) b[u] = __ldg(nd + 4 * u);
+            ref = __float_as_int(__ldg(nd + 24));
+        }
+        if (k != skip) A = __ldg(tq), B = __ldg(tq + 1), C = __ldg(tq + 2);
+        const float x0 = fmaf(b[0], inv.x, -oi.x), x1 = fmaf(b[1], inv.x, -oi.x);
+        const float y0 = fmaf(b[2], inv.y, -oi.y), y1 = fmaf(b[3], inv.y, -oi.y);
+        const float z0 = fmaf(b[4], inv.z, -oi.z), z1 = fmaf(b[5], inv.z, -oi.z);
+        const float tn = fmaxf(fmaxf(fminf(x0, x1), fminf(y0, y1)), fmaxf(fminf(z0, z1), 0.f));
+        const float tf = fminf(fminf(fmaxf(x0, x1), fmaxf(y0, y1)), fminf(fmaxf(z0, z1), tmax));
+        const bool in = ref != kEmptyRef && tn <= tf * kBoxGrow;
+        if (k != skip) {
+            float tc = 0.f, et = FLT_MAX;
+            int f = tri_filter(A, B, C, o, d, tc, et);
+            if (f >= 2) {
+                f = tri_refine(a.tris, a.tri_v12, k, o, d, f + 2, tc) & 1;
+                et = FLT_MAX;
+            }
+            if (f) consider_hit(tri_refs(a), k, __float_as_int(A.w), tc, et, o, d, h);
+        }
+        if (__any_sync(kFull, k != skip)) {
+            float t = h.t;
+#pragma unroll
+            for (int u = kCoopLanes / 2; u > 0; u >>= 1) t = fminf(t, __shfl_xor_sync(kFull, t, u));
+            tmax = t;
+        }
+        // inner children: those of deeper entries below, the farther of a node's below the nearer
+        const unsigned mi = (__ballot_sync(kFull, in && ref >= 0) >> at0) & kRay;
+        int at = 4 * g + 4 < kCoopLanes ? __popc(mi >> (4 * g + 4)) : 0;
+#pragma unroll
+        for (int u = 1; u < 4; ++u) {
+            const float t = __shfl_xor_sync(kFull, tn, u);
+            at += ((mi >> (l ^ u)) & 1u) && (t > tn || (t == tn && (l ^ u) > l)) ? 1 : 0;
+        }
+        // (every lane goes on to the votes below, also of a ray that has run out of room)
+        const bool room = sp + __popc(mi) <= kCoopStack;
+        if (room && in && ref >= 0) q.node[sp + at] = make_int2(ref, __float_as_int(tn));
+        sp = room ? sp + __popc(mi) : 0;
+        tp = room ? tp : 0;
+        fits = fits && room;
+        const int first = leaf_first(ref), cnt = room && in && ref < 0 ? leaf_count(ref) : 0;
+        for (int u = 0; __any_sync(kFull, u < cnt); ++u) {
+            const unsigned m = (__ballot_sync(kFull, u < cnt) >> at0) & kRay;
+            if (u < cnt) q.tri[tp + __popc(m & lt)] = first + u;
+            tp += __popc(m);
+        }
+    }
+    if (sp > 0 || tp > 0) fits = false;  // out of iterations
+    key_closest(tri_refs(a), o, d, h);
+    // the smallest (t32, index) of the ray's lanes, and whose it is
+    float t = h.k >= 0 ? h.t : FLT_MAX;
+    int orig = h.k >= 0 ? h.orig : INT_MAX, k = h.k;
+#pragma unroll
+    for (int u = kCoopLanes / 2; u > 0; u >>= 1) {
+        const float ot = __shfl_xor_sync(kFull, t, u);
+        const int oo = __shfl_xor_sync(kFull, orig, u), ok = __shfl_xor_sync(kFull, k, u);
+        if (ok >= 0 && (k < 0 || ot < t || (ot == t && oo < orig))) {
+            t = ot;
+            orig = oo;
+            k = ok;
+        }
+    }
+    h.t = t;
+    h.orig = orig;
+    h.k = k;
+    __syncwarp();
+    return fits;
+}
+
+// The rays k_tail has handed over (a.q_out, *a.hand_count), each followed to its
+// end by kCoopLanes lanes: a bounce takes 18k cycles instead of the 30k of one
+// lane, and no warp has several of them by chance. Its own kernel, since the
+// queues' shared memory is L1 that the other traversals use (inside k_tail:
+// aircraft_1ghz_cut 1.5 % slower). aircraft_deep_cavity 11.8 -> 10.3 ms with 32
+// lanes a ray and rays handed over after 10 bounces (16 lanes 10.4, 8 lanes
+// 10.9; after 6 bounces 10.8, 14 10.5, 20 10.7).
+template <bool kBi>
+__global__ void __launch_bounds__(kTraceThreads, 2) k_trapped(const TraceArgs a)
+{
+    __shared__ CoopQueue s_queue[kTraceThreads / kCoopLanes];
+    const unsigned n_in = *a.q_in_count, n = *a.hand_count;
+    if (n_in == 0 || n_in > a.tail_rays || n == 0) return;  // k_tail has not had this pass
+    const int lane = threadIdx.x & 31, at0 = lane & ~(kCoopLanes - 1);
+    const unsigned warps = (gridDim.x * blockDim.x) >> 5, rays = warps * (32 / kCoopLanes);
+    const bool lead = lane == at0;
+    unsigned idx = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) + (unsigned)(lane / kCoopLanes) * warps;
+    unsigned nq = 0, unused = 0;
+    bool ovf = false, has = idx < n;
+    Ray r;
+    r.o = make_float3(0.f, 0.f, 0.f);
+    r.d = make_float3(0.f, 0.f, 1.f);
+    r.last = -1;
+    if (lead && has) load_state(a.q_out, idx, r);
+    while (__any_sync(kFull, has)) {
+        const float3 o = make_float3(__shfl_sync(kFull, r.o.x, at0), __shfl_sync(kFull, r.o.y, at0),
+                                     __shfl_sync(kFull, r.o.z, at0));
+        const float3 d = make_float3(__shfl_sync(kFull, r.d.x, at0), __shfl_sync(kFull, r.d.y, at0),
+                                     __shfl_sync(kFull, r.d.z, at0));
+        Hit h;
+        const bool fits =
+            closest_hit_coop(a, s_queue[threadIdx.x / kCoopLanes], has, o, d, __shfl_sync(kFull, r.last, at0), h);
+        bool again = false;
+        if (lead && has) {
+            if (!fits) {
+                closest_hit<false, 64>(a.nodes2, tri_refs(a), o, d, r.last, a.visit_limit, h, unused, unused, ovf);
+                key_closest(tri_refs(a), o, d, h);
+            }
+            again = finish_query<false, kBi>(a, h, r, nq, unused, ovf);
+        }
+        again = __shfl_sync(kFull, (int)again, at0) != 0;
+        if (has && !again) {
+            idx += rays;
+            has = idx < n;
+            if (lead && has) load_state(a.q_out, idx, r);
+        }
+    }
+    flush_stats<false>(a, nq, 0u, 0u, ovf);
 }
 
 // every ray of the queue writes its record (B_max = 1 without the escape check)
@@ -2496,6 +2671,10 @@ cudaError_t launch_trace(const TraceArgs& a, int n_blocks, bool count_visits, in
     if (a.bounce > 0 && a.tail_rays) {
         if (a.octant) launch_tail<3>(a, n_blocks, count_visits, st);
         else launch_tail<0>(a, n_blocks, count_visits, st);
+        if (a.hand_count) {
+            if (a.bistatic) k_trapped<true><<<n_blocks, kTraceThreads, 0, st>>>(a);
+            else k_trapped<false><<<n_blocks, kTraceThreads, 0, st>>>(a);
+        }
     }
     if (a.bistatic && a.bounce > 0) {
         // bounce passes of chunks with a bistatic aspect: per-lane traversal, 64-entry stack, visibility tests
