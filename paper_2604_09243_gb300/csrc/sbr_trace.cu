@@ -2297,26 +2297,23 @@ __global__ void __launch_bounds__(kTraceThreads, 4) k_tail(const TraceArgs a)
     flush_stats<kCount>(a, nq, nvis, ntri, ovf, nhit, 0u, (threadIdx.x & 31) == 0 ? wvis : 0ull);
 }
 
-// Closest hits of 32 / kCoopLanes rays by a warp, kCoopLanes lanes each (o, d,
-// skip and the result the same in every lane of a ray; has: there is one). Up to
-// kCoopLanes / 4 4-wide nodes are taken from a stack at a time, a lane per
-// child, the nearest on top, and up to kCoopLanes triangles of the leaves
-// reached, a lane each, their loads in flight together: a ray's chain of
-// dependent fetches is as long as the tree is deep instead of one for every node
-// and triangle it meets. Every lane keeps its own candidates and the smallest
-// (t32, original triangle index) is taken at the end, so the hit is that of any
-// other order of visits. A nearly full stack is left to one node at a time;
-// false where the children did not fit all the same (the caller's to trace).
-constexpr int kCoopLanes = 32, kCoopStack = 128, kCoopWide = 40, kCoopTris = kCoopLanes + kCoopLanes * 16;
+// Closest hit of one ray by a whole warp (o, d, skip and the result the same in
+// every lane). Up to eight 4-wide nodes are taken from a stack at a time, a lane
+// per child, the nearest on top, and up to 32 triangles of the leaves reached, a
+// lane each, their loads in flight together: a ray's chain of dependent fetches
+// is as long as the tree is deep instead of one for every node and triangle it
+// meets. Every lane keeps its own candidates and the smallest (t32, original
+// triangle index) is taken at the end, so the hit is that of any other order of
+// visits. A nearly full stack is left to one node at a time; false where the
+// children did not fit all the same (the caller's to trace).
+constexpr int kCoopStack = 128, kCoopWide = 40, kCoopTris = 32 + 8 * 4 * 16;
 struct CoopQueue {
     int2 node[kCoopStack];  // node, its near distance
     int tri[kCoopTris];
 };
-__device__ __forceinline__ bool closest_hit_coop(const TraceArgs& a, CoopQueue& q, bool has, float3 o, float3 d, int skip,
-                                                 Hit& h)
+__device__ __forceinline__ bool closest_hit_coop(const TraceArgs& a, CoopQueue& q, float3 o, float3 d, int skip, Hit& h)
 {
-    const int lane = threadIdx.x & 31, at0 = lane & ~(kCoopLanes - 1), l = lane - at0, g = l >> 2, c = l & 3;
-    constexpr unsigned kRay = kCoopLanes == 32 ? kFull : (1u << (kCoopLanes & 31)) - 1u;
+    const int l = threadIdx.x & 31, g = l >> 2, c = l & 3;
     const unsigned lt = (1u << l) - 1u;
     const float3 inv = make_float3(safe_rcp(d.x), safe_rcp(d.y), safe_rcp(d.z));
     const float3 oi = make_float3(o.x * inv.x, o.y * inv.y, o.z * inv.z);
@@ -2326,14 +2323,14 @@ __device__ __forceinline__ bool closest_hit_coop(const TraceArgs& a, CoopQueue& 
     h.lo = FLT_MAX;
     h.key = -1.f;
     float tmax = FLT_MAX;
-    int sp = has ? 1 : 0, tp = 0;
+    int sp = 1, tp = 0;
     bool fits = true;
     if (l == 0) q.node[0] = make_int2(0, 0);
-    for (int it = 0; it < a.visit_limit && __any_sync(kFull, sp > 0 || tp > 0); ++it) {
+    for (int it = 0; it < a.visit_limit && (sp > 0 || tp > 0); ++it) {
         __syncwarp();
-        const int nt = min(kCoopLanes, tp);
+        const int nt = min(32, tp);
         tp -= nt;
-        const int n = tp > 0 ? 0 : min(sp > kCoopWide ? 1 : kCoopLanes / 4, sp);
+        const int n = tp > 0 ? 0 : min(sp > kCoopWide ? 1 : 8, sp);
         const int2 e = g < n ? q.node[sp - 1 - g] : make_int2(0, 0);
         const int k = l < nt ? q.tri[tp + l] : skip;
         sp -= n;
@@ -2367,37 +2364,38 @@ __device__ __forceinline__ bool closest_hit_coop(const TraceArgs& a, CoopQueue& 
         if (__any_sync(kFull, k != skip)) {
             float t = h.t;
 #pragma unroll
-            for (int u = kCoopLanes / 2; u > 0; u >>= 1) t = fminf(t, __shfl_xor_sync(kFull, t, u));
+            for (int u = 16; u > 0; u >>= 1) t = fminf(t, __shfl_xor_sync(kFull, t, u));
             tmax = t;
         }
         // inner children: those of deeper entries below, the farther of a node's below the nearer
-        const unsigned mi = (__ballot_sync(kFull, in && ref >= 0) >> at0) & kRay;
-        int at = 4 * g + 4 < kCoopLanes ? __popc(mi >> (4 * g + 4)) : 0;
+        const unsigned mi = __ballot_sync(kFull, in && ref >= 0);
+        int at = g < 7 ? __popc(mi >> (4 * g + 4)) : 0;
 #pragma unroll
         for (int u = 1; u < 4; ++u) {
             const float t = __shfl_xor_sync(kFull, tn, u);
             at += ((mi >> (l ^ u)) & 1u) && (t > tn || (t == tn && (l ^ u) > l)) ? 1 : 0;
         }
-        // (every lane goes on to the votes below, also of a ray that has run out of room)
-        const bool room = sp + __popc(mi) <= kCoopStack;
-        if (room && in && ref >= 0) q.node[sp + at] = make_int2(ref, __float_as_int(tn));
-        sp = room ? sp + __popc(mi) : 0;
-        tp = room ? tp : 0;
-        fits = fits && room;
-        const int first = leaf_first(ref), cnt = room && in && ref < 0 ? leaf_count(ref) : 0;
-        for (int u = 0; __any_sync(kFull, u < cnt); ++u) {
-            const unsigned m = (__ballot_sync(kFull, u < cnt) >> at0) & kRay;
+        if (sp + __popc(mi) > kCoopStack) {
+            fits = false;
+            break;
+        }
+        if (in && ref >= 0) q.node[sp + at] = make_int2(ref, __float_as_int(tn));
+        sp += __popc(mi);
+        const int first = leaf_first(ref), cnt = in && ref < 0 ? leaf_count(ref) : 0;
+        for (int u = 0;; ++u) {
+            const unsigned m = __ballot_sync(kFull, u < cnt);
+            if (!m) break;
             if (u < cnt) q.tri[tp + __popc(m & lt)] = first + u;
             tp += __popc(m);
         }
     }
-    if (sp > 0 || tp > 0) fits = false;  // out of iterations
+    fits = fits && sp == 0 && tp == 0;  // (not out of iterations)
     key_closest(tri_refs(a), o, d, h);
     // the smallest (t32, index) of the ray's lanes, and whose it is
     float t = h.k >= 0 ? h.t : FLT_MAX;
     int orig = h.k >= 0 ? h.orig : INT_MAX, k = h.k;
 #pragma unroll
-    for (int u = kCoopLanes / 2; u > 0; u >>= 1) {
+    for (int u = 16; u > 0; u >>= 1) {
         const float ot = __shfl_xor_sync(kFull, t, u);
         const int oo = __shfl_xor_sync(kFull, orig, u), ok = __shfl_xor_sync(kFull, k, u);
         if (ok >= 0 && (k < 0 || ot < t || (ot == t && oo < orig))) {
@@ -2414,52 +2412,64 @@ __device__ __forceinline__ bool closest_hit_coop(const TraceArgs& a, CoopQueue& 
 }
 
 // The rays k_tail has handed over (a.q_out, *a.hand_count), each followed to its
-// end by kCoopLanes lanes: a bounce takes 18k cycles instead of the 30k of one
+// end by a warp: a bounce takes 18k cycles instead of the 30k of one
 // lane, and no warp has several of them by chance. Its own kernel, since the
 // queues' shared memory is L1 that the other traversals use (inside k_tail:
 // aircraft_1ghz_cut 1.5 % slower). aircraft_deep_cavity 11.8 -> 10.3 ms with 32
 // lanes a ray and rays handed over after 10 bounces (16 lanes 10.4, 8 lanes
-// 10.9; after 6 bounces 10.8, 14 10.5, 20 10.7).
+// 10.9; after 6 bounces 10.8, 14 10.5, 20 10.7). With more than two rays per
+// warp the GPU is busy with a lane each: 40,000 rays of a bistatic trace with
+// 67 bounces in 3.5 ms, 8.5 ms by whole warps.
+constexpr unsigned kTrappedPerWarp = 2;
 template <bool kBi>
 __global__ void __launch_bounds__(kTraceThreads, 2) k_trapped(const TraceArgs a)
 {
-    __shared__ CoopQueue s_queue[kTraceThreads / kCoopLanes];
+    __shared__ CoopQueue s_queue[kTraceThreads / 32];
     const unsigned n_in = *a.q_in_count, n = *a.hand_count;
     if (n_in == 0 || n_in > a.tail_rays || n == 0) return;  // k_tail has not had this pass
-    const int lane = threadIdx.x & 31, at0 = lane & ~(kCoopLanes - 1);
-    const unsigned warps = (gridDim.x * blockDim.x) >> 5, rays = warps * (32 / kCoopLanes);
-    const bool lead = lane == at0;
-    unsigned idx = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) + (unsigned)(lane / kCoopLanes) * warps;
+    const int lane = threadIdx.x & 31;
+    const unsigned warps = (gridDim.x * blockDim.x) >> 5, warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     unsigned nq = 0, unused = 0;
-    bool ovf = false, has = idx < n;
+    bool ovf = false;
     Ray r;
     r.o = make_float3(0.f, 0.f, 0.f);
     r.d = make_float3(0.f, 0.f, 1.f);
     r.last = -1;
-    if (lead && has) load_state(a.q_out, idx, r);
-    while (__any_sync(kFull, has)) {
-        const float3 o = make_float3(__shfl_sync(kFull, r.o.x, at0), __shfl_sync(kFull, r.o.y, at0),
-                                     __shfl_sync(kFull, r.o.z, at0));
-        const float3 d = make_float3(__shfl_sync(kFull, r.d.x, at0), __shfl_sync(kFull, r.d.y, at0),
-                                     __shfl_sync(kFull, r.d.z, at0));
-        Hit h;
-        const bool fits =
-            closest_hit_coop(a, s_queue[threadIdx.x / kCoopLanes], has, o, d, __shfl_sync(kFull, r.last, at0), h);
-        bool again = false;
-        if (lead && has) {
-            if (!fits) {
-                closest_hit<false, 64>(a.nodes2, tri_refs(a), o, d, r.last, a.visit_limit, h, unused, unused, ovf);
-                key_closest(tri_refs(a), o, d, h);
+    auto alone = [&](Hit& h) {
+        closest_hit<false, 64>(a.nodes2, tri_refs(a), r.o, r.d, r.last, a.visit_limit, h, unused, unused, ovf);
+        key_closest(tri_refs(a), r.o, r.d, h);
+    };
+    if (n > kTrappedPerWarp * warps) {
+        // a ray per lane, over the blocks that are resident at once
+        const unsigned w = warps / 2;
+        for (unsigned idx = warp + (unsigned)lane * w; warp < w && idx < n; idx += 32u * w) {
+            load_state(a.q_out, idx, r);
+            bool again = true;
+            while (again) {
+                Hit h;
+                alone(h);
+                again = finish_query<false, kBi>(a, h, r, nq, unused, ovf);
             }
-            again = finish_query<false, kBi>(a, h, r, nq, unused, ovf);
         }
-        again = __shfl_sync(kFull, (int)again, at0) != 0;
-        if (has && !again) {
-            idx += rays;
-            has = idx < n;
-            if (lead && has) load_state(a.q_out, idx, r);
+    } else {
+        for (unsigned idx = warp; idx < n; idx += warps) {
+            if (lane == 0) load_state(a.q_out, idx, r);
+            for (bool again = true; again;) {
+                r.o = make_float3(__shfl_sync(kFull, r.o.x, 0), __shfl_sync(kFull, r.o.y, 0), __shfl_sync(kFull, r.o.z, 0));
+                r.d = make_float3(__shfl_sync(kFull, r.d.x, 0), __shfl_sync(kFull, r.d.y, 0), __shfl_sync(kFull, r.d.z, 0));
+                r.last = __shfl_sync(kFull, r.last, 0);
+                Hit h;
+                const bool fits = closest_hit_coop(a, s_queue[threadIdx.x >> 5], r.o, r.d, r.last, h);
+                again = false;
+                if (lane == 0) {
+                    if (!fits) alone(h);
+                    again = finish_query<false, kBi>(a, h, r, nq, unused, ovf);
+                }
+                again = __shfl_sync(kFull, (int)again, 0) != 0;
+            }
         }
     }
+    __syncwarp();
     flush_stats<false>(a, nq, 0u, 0u, ovf);
 }
 
@@ -2672,8 +2682,9 @@ cudaError_t launch_trace(const TraceArgs& a, int n_blocks, bool count_visits, in
         if (a.octant) launch_tail<3>(a, n_blocks, count_visits, st);
         else launch_tail<0>(a, n_blocks, count_visits, st);
         if (a.hand_count) {
-            if (a.bistatic) k_trapped<true><<<n_blocks, kTraceThreads, 0, st>>>(a);
-            else k_trapped<false><<<n_blocks, kTraceThreads, 0, st>>>(a);
+            const int g = (n_blocks + 1) & ~1;  // half of them resident at a time
+            if (a.bistatic) k_trapped<true><<<g, kTraceThreads, 0, st>>>(a);
+            else k_trapped<false><<<g, kTraceThreads, 0, st>>>(a);
         }
     }
     if (a.bistatic && a.bounce > 0) {

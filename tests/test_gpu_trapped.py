@@ -51,3 +51,25 @@ def test_trapped_rays_equal_pass_by_pass(G, spacing, bounces, kw):
             assert np.array_equal(u, v)
         for k in ("ray", "coef", "L"):
             assert np.array_equal(r0[a][k], r1[a][k])
+
+
+def test_more_trapped_rays_than_warps_take(G):
+    """5 mm grids into the inlets: more trapped rays than two per warp (9,728), which a lane each follows."""
+    import sbr_inputs as S
+
+    xyz, tri = S.aircraft(seed=1, target_tris=20_000)
+    ang = np.array([[180.0, 0.0], [178.0, 0.0], [182.0, 0.0], [180.0, 2.0]])
+    res = []
+    with G.Context(0) as c:
+        c.load_mesh(xyz, tri)
+        for depth in (64, 128):
+            c.set_tuning(stack_depth=depth)
+            st = c.trace(ang, 0.005, max_bounces=40)
+            E, _ = c.po_integrate([1e9], "HH,VV")
+            res.append((st, E, c.get_records(0)))
+    (s0, E0, r0), (s1, E1, r1) = res
+    for k in ("rays_launched", "ray_bounces", "valid_rays", "stack_overflows"):
+        assert s0[k] == s1[k], k
+    assert np.array_equal(E0, E1)
+    for k in ("ray", "coef", "L"):
+        assert np.array_equal(r0[k], r1[k])
