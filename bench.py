@@ -428,7 +428,7 @@ def _tensor_roofline(points, members, seconds, width=512, depth=6, n_fourier=256
     pk, src = peaks()
     peak = pk.get("bf16_tflops", 1900.0)
     ach = flops / seconds / 1e12
-    return {"bound": "tensor", "kernel": "k_gemm_tn (tcgen05, BF16 in, FP32 accumulate) in sbr_surrogate_predict",
+    return {"bound": "tensor", "kernel": "k_gemm (tcgen05, BF16 in, FP32 accumulate) in sbr_surrogate_predict",
             "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak, "traffic": None,
             "peak_source": f"bf16 dense GEMM burst, {src}", "flop": flops}
 
@@ -663,7 +663,7 @@ def run_gemm(args, ws, rank, local, pg):
         e1.record(stream)
         torch.cuda.synchronize()
         if int(err.item()):
-            raise RuntimeError("k_gemm_tn: a bounded wait gave up")
+            raise RuntimeError("k_gemm: a bounded wait gave up")
         ms = e0.elapsed_time(e1) / args.steps
         tf = 2.0 * M * N * K / (ms * 1e-3) / 1e12
         # algorithmic bytes: both operands read once, the FP32 result written once
@@ -675,13 +675,13 @@ def run_gemm(args, ws, rank, local, pg):
     hbm = pk.get("hbm_gbs", 6800.0)
     ridge = peak * 1e12 / (hbm * 1e9)
     if top["flop_per_byte"] < ridge:
-        roof = {"bound": "hbm", "kernel": "k_gemm_tn (tcgen05)", "achieved": top["gbs"], "peak": hbm, "unit": "GB/s",
+        roof = {"bound": "hbm", "kernel": "k_gemm (tcgen05)", "achieved": top["gbs"], "peak": hbm, "unit": "GB/s",
                 "frac": top["gbs"] / hbm, "traffic": None,
                 "peak_source": f"HBM copy bandwidth, {src}",
                 "flop_per_byte": top["flop_per_byte"], "ridge_flop_per_byte": ridge,
                 "tensor_frac": top["frac"], "attainable_tflops": top["flop_per_byte"] * hbm / 1e3}
     else:
-        roof = {"bound": "tensor", "kernel": "k_gemm_tn (tcgen05)", "achieved": top["tflops"], "peak": peak,
+        roof = {"bound": "tensor", "kernel": "k_gemm (tcgen05)", "achieved": top["tflops"], "peak": peak,
                 "unit": "TFLOP/s", "frac": top["frac"], "traffic": None,
                 "peak_source": f"bf16 dense GEMM burst, {src}", "flop_per_byte": top["flop_per_byte"],
                 "ridge_flop_per_byte": ridge}
@@ -944,7 +944,7 @@ def run_sbr(args, case, ws, rank, local, pg):
             "valid_rays_per_step": stats[0]["valid_rays"],
             "roofline": roof,
             "probes": {"l2_read_gbs": l2_gbs, "fp32_fma_tflops": fp32_tflops, "sm_count": n_sm, "l2_bytes": l2_bytes},
-            "primary": {"kernel": "k_raster+k_raster_big+k_vis_mask+k_primary_vis (rasterised primary hits)" if raster
+            "primary": {"kernel": "k_raster+k_raster_big+k_vis_mask+k_vis_slots (rasterised primary hits)" if raster
                         else "k_primary (traversed)", "ms_per_step": primary_s * 1e3,
                         "transport_ms_per_step": pass_all_s * 1e3, "raster_tests": cnt["raster_tests"],
                         "raster_tests_per_s": cnt["raster_tests"] / primary_s if raster and primary_s > 0 else None},
