@@ -6,7 +6,7 @@
 // frequency, evaluates e^{-j k L} per tube, multiplies by the tube coefficients
 // and reduces with warp shuffles and a shared-memory tree in FP32. The item
 // partial is stored in FP64; a second kernel adds the partials of an aspect in
-// item order in FP64, applies -j k / (4 pi) and sigma = 4 pi |E|^2 (Sec. 4).
+// a fixed order in FP64, applies -j k / (4 pi) and sigma = 4 pi |E|^2 (Sec. 4).
 // The order of every addition is fixed, so results are bitwise reproducible
 // (the paper notes run-to-run scatter of its FP32 sums, Sec. 5.1).
 //
