@@ -799,11 +799,17 @@ int sbr_surrogate_create(sbr_surrogate** out, int device, void* cuda_stream, con
         }
         for (auto& v : hb) v = o.fourier_sigma * nd01(rng);
         s->steps.push_back(0);
-        cudaMemcpy(s->P.as<float>() + e * off, hp.data(), sizeof(float) * off, cudaMemcpyHostToDevice);
-        cudaMemcpy(s->Bf.as<float>() + (size_t)e * 4 * s->nh, hb.data(), sizeof(float) * hb.size(), cudaMemcpyHostToDevice);
-        rc = refresh_bf16(s, e);
+        // on the object's stream, which nothing else orders after the default one; a pageable source is consumed
+        // when the call returns
+        if (cudaMemcpyAsync(s->P.as<float>() + e * off, hp.data(), sizeof(float) * off, cudaMemcpyHostToDevice,
+                            s->stream) != cudaSuccess ||
+            cudaMemcpyAsync(s->Bf.as<float>() + (size_t)e * 4 * s->nh, hb.data(), sizeof(float) * hb.size(),
+                            cudaMemcpyHostToDevice, s->stream) != cudaSuccess)
+            rc = SBR_ERR_CUDA;
+        if (rc == SBR_OK) rc = refresh_bf16(s, e);
     }
-    if (rc == SBR_OK && (cudaMemset(s->Pm.p, 0, s->Pm.cap) != cudaSuccess || cudaMemset(s->Pv.p, 0, s->Pv.cap) != cudaSuccess ||
+    if (rc == SBR_OK && (cudaMemsetAsync(s->Pm.p, 0, s->Pm.cap, s->stream) != cudaSuccess ||
+                         cudaMemsetAsync(s->Pv.p, 0, s->Pv.cap, s->stream) != cudaSuccess ||
                          cudaMemsetAsync(s->gerr.p, 0, sizeof(int), s->stream) != cudaSuccess ||
                          cudaStreamSynchronize(s->stream) != cudaSuccess))
         rc = SBR_ERR_CUDA;
@@ -899,7 +905,8 @@ int sbr_surrogate_train(sbr_surrogate* s, const double* x, const double* y, int6
     std::vector<float> yt((size_t)n * kOut);
     for (size_t i = 0; i < yt.size(); ++i) yt[i] = (float)(y[i] / s->target_scale);
     cudaError_t ce = cudaMalloc(&y4, sizeof(float) * yt.size());
-    if (ce == cudaSuccess) ce = cudaMemcpy(y4, yt.data(), sizeof(float) * yt.size(), cudaMemcpyHostToDevice);
+    if (ce == cudaSuccess)
+        ce = cudaMemcpyAsync(y4, yt.data(), sizeof(float) * yt.size(), cudaMemcpyHostToDevice, s->stream);
     if (ce != cudaSuccess) {
         cudaFree(x4);
         SCK(ce, "upload targets");

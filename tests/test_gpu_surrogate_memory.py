@@ -1,0 +1,46 @@
+"""The surrogate's use of streams and memory: its uploads stay on its own stream,
+and its calls fit where one member's arrays fit."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def G():
+    from paper_2604_09243_gb300 import build
+
+    build.build()
+    import paper_2604_09243_gb300 as G
+
+    return G
+
+
+def _samples(n, seed):
+    rng = np.random.default_rng(seed)
+    x = np.stack([rng.uniform(0, 360, n), rng.uniform(-30, 30, n), np.exp(rng.uniform(np.log(1e9), np.log(12e9), n))], 1)
+    return x, rng.normal(0, 1, (n, 4))
+
+
+def test_creation_uses_its_own_stream_alone(G):
+    """Parameters, Fourier matrices and Adam moments reach the device on the object's (non-blocking) stream: with the
+    default stream busy for a second or so the object is ready before that has ended, and trains to the same bits."""
+    torch = pytest.importorskip("torch")
+    net = dict(n_members=2, width=128, depth=2, n_fourier=128, fourier_sigma=2.0, seed=5)
+    x, y = _samples(512, 1)
+    ref = G.Surrogate(0, **net)
+    ref.train(x, y, epochs=2, batch=256)
+    torch.zeros(1, device="cuda")
+    torch.cuda.synchronize()
+    busy = torch.cuda.Event()
+    torch.cuda._sleep(2_000_000_000)
+    busy.record()
+    s = G.Surrogate(0, **net)
+    early = not busy.query()
+    torch.cuda.synchronize()
+    s.train(x, y, epochs=2, batch=256)
+    assert early
+    for e in range(2):
+        assert np.array_equal(s.params(e), ref.params(e)) and np.array_equal(s.fourier(e), ref.fourier(e))
+    s.close()
+    ref.close()
