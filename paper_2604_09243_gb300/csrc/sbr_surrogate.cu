@@ -430,12 +430,13 @@ struct sbr_surrogate {
     Layout L;
     long long n_params = 0;  // per member (a multiple of 4)
     long long n_bf = 0;      // BF16 hidden weights per member
-    // all members, n_params / n_bf / 4 nh apart: parameters, Adam moments, gradients, Fourier matrices, BF16 weights
-    Buf P, Pm, Pv, G, Bf, Wbf;
+    // all members, n_params / n_bf / 4 nh apart: parameters, Adam moments, Fourier matrices, BF16 weights
+    Buf P, Pm, Pv, Bf, Wbf;
     std::vector<long long> steps;
     // Workspace of a group of g members on a batch of M rows, member-major: h0 [g][M][nf], h [layer][g][M][width]
-    // (h_{l+1} at l), z and dz [layer][g][M][width], outputs and targets [g][M][4]. Kept and grown as needed.
-    Buf h0, h, z, dz, y, dy, xb, yb, red;
+    // (h_{l+1} at l), z and dz [layer][g][M][width], outputs and targets [g][M][4], gradients [g][n_params]. Kept and
+    // grown as needed.
+    Buf h0, h, z, dz, y, dy, xb, yb, red, G;
     Buf loss, gerr;
     float target_scale = 1.f;
     bool trained = false;
@@ -474,28 +475,58 @@ cudaError_t ensure_ws(sbr_surrogate* s, int M, int g, bool train)
     if (e == cudaSuccess) e = s->dz.ensure(sizeof(__nv_bfloat16) * R * W * D);
     if (e == cudaSuccess) e = s->dy.ensure(sizeof(float) * R * kOut);
     if (e == cudaSuccess) e = s->yb.ensure(sizeof(float) * R * kOut);
+    if (e == cudaSuccess) e = s->G.ensure(sizeof(float) * (size_t)s->n_params * g);
     const size_t parts = (size_t)((M + kRedRows - 1) / kRedRows) * g;
     if (e == cudaSuccess) e = s->red.ensure(sizeof(float) * parts * std::max<size_t>(kOut * (W + 1), D * W));
     return e;
 }
 
+void release_ws(sbr_surrogate* s)
+{
+    for (Buf* b : {&s->h0, &s->h, &s->z, &s->dz, &s->y, &s->dy, &s->xb, &s->yb, &s->red, &s->G}) b->release();
+}
+
+// an array of the call at hand; where the GPU is full the workspace kept from earlier calls makes room
+template <class T>
+cudaError_t call_alloc(sbr_surrogate* s, T** p, size_t count)
+{
+    cudaError_t e = cudaMalloc((void**)p, sizeof(T) * count);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        release_ws(s);
+        e = cudaMalloc((void**)p, sizeof(T) * count);
+    }
+    if (e != cudaSuccess) *p = nullptr;
+    return e;
+}
+
 // Members worked on at once: all of them while their workspace (200 MB per
 // member at 8192 rows of the default network) stays within kGroupBytes and can
-// be had, else fewer, down to one. A step of four members of 8192 rows takes
-// 0.75 ms of device time together, 3.1 ms one member at a time.
-constexpr size_t kGroupBytes = (size_t)8 << 30;
-int choose_group(sbr_surrogate* s, int M, int* g_out)
+// be had beside the group's permutations (at most kGroupPerm) and losses, else
+// fewer, down to one; the call's other arrays are there already. A step of four
+// members of 8192 rows takes 0.75 ms of device time together, 3.1 ms one member
+// at a time.
+constexpr size_t kGroupBytes = (size_t)8 << 30, kGroupPerm = (size_t)1 << 30;
+int choose_group(sbr_surrogate* s, int M, long long n, int epochs, int* g_out, int** dperm, double** dloss)
 {
     const size_t row = (size_t)s->opt.depth * s->opt.width * 8 + (size_t)s->opt.n_fourier * 2 + 128;
-    int g = (int)std::min<size_t>((size_t)s->opt.n_members, std::max<size_t>(1, kGroupBytes / (row * (size_t)M)));
-    cudaError_t e = ensure_ws(s, M, g, true);
-    while (e == cudaErrorMemoryAllocation && g > 1) {
+    size_t most = std::min<size_t>((size_t)s->opt.n_members, kGroupBytes / (row * (size_t)M));
+    most = std::min(most, kGroupPerm / (sizeof(int) * (size_t)n));
+    int g = (int)std::max<size_t>(1, most);
+    for (bool last = false;;) {
+        cudaError_t e = ensure_ws(s, M, g, true);
+        if (e == cudaSuccess) e = cudaMalloc((void**)dperm, sizeof(int) * (size_t)n * g);
+        if (e == cudaSuccess) e = cudaMalloc((void**)dloss, sizeof(double) * (size_t)epochs * g);
+        if (e == cudaSuccess) break;
         cudaGetLastError();
-        g = (g + 1) / 2;
-        for (Buf* b : {&s->h0, &s->h, &s->z, &s->dz, &s->y, &s->dy, &s->xb, &s->yb, &s->red}) b->release();
-        e = ensure_ws(s, M, g, true);
+        cudaFree(*dperm);
+        *dperm = nullptr;
+        *dloss = nullptr;
+        release_ws(s);
+        if (e != cudaErrorMemoryAllocation || last) SCK(e, "alloc training workspace");
+        if (g == 1) last = true;  // once more, without what earlier calls had left
+        else g = (g + 1) / 2;
     }
-    SCK(e, "alloc training workspace");
     *g_out = g;
     return SBR_OK;
 }
@@ -655,14 +686,18 @@ int check_gemm_err(sbr_surrogate* s)
 int upload_inputs(sbr_surrogate* s, const double* x, int64_t n, float** x4)
 {
     double* raw = nullptr;
-    SCK(cudaMalloc(&raw, sizeof(double) * 3 * (size_t)n), "alloc inputs");
-    SCK(cudaMalloc(x4, sizeof(float) * kIn * (size_t)n), "alloc inputs");
-    cudaError_t e = cudaMemcpyAsync(raw, x, sizeof(double) * 3 * (size_t)n, cudaMemcpyHostToDevice, s->stream);
+    cudaError_t e = call_alloc(s, x4, kIn * (size_t)n);
+    if (e == cudaSuccess) e = call_alloc(s, &raw, 3 * (size_t)n);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(raw, x, sizeof(double) * 3 * (size_t)n, cudaMemcpyHostToDevice, s->stream);
     if (e == cudaSuccess) {
         k_encode<<<blocks(n, 256), 256, 0, s->stream>>>(raw, (int)n, *x4);
         e = cudaStreamSynchronize(s->stream);
     }
     cudaFree(raw);
+    if (e != cudaSuccess) {
+        cudaFree(*x4);
+        *x4 = nullptr;
+    }
     SCK(e, "encode inputs");
     return SBR_OK;
 }
@@ -781,7 +816,7 @@ int sbr_surrogate_create(sbr_surrogate** out, int device, void* cuda_stream, con
     const size_t ne = (size_t)o.n_members;
     int rc = SBR_OK;
     if (s->P.ensure(sizeof(float) * off * ne) != cudaSuccess || s->Pm.ensure(sizeof(float) * off * ne) != cudaSuccess ||
-        s->Pv.ensure(sizeof(float) * off * ne) != cudaSuccess || s->G.ensure(sizeof(float) * off * ne) != cudaSuccess ||
+        s->Pv.ensure(sizeof(float) * off * ne) != cudaSuccess ||
         s->Bf.ensure(sizeof(float) * 4 * s->nh * ne) != cudaSuccess ||
         s->Wbf.ensure(sizeof(__nv_bfloat16) * offbf * ne) != cudaSuccess ||
         s->loss.ensure(sizeof(double)) != cudaSuccess || s->gerr.ensure(sizeof(int)) != cudaSuccess)
@@ -826,9 +861,8 @@ void sbr_surrogate_destroy(sbr_surrogate* s)
     if (!s) return;
     cudaSetDevice(s->device);
     cudaStreamSynchronize(s->stream);
-    for (Buf* b : {&s->P, &s->Pm, &s->Pv, &s->G, &s->Bf, &s->Wbf, &s->h0, &s->h, &s->z, &s->dz, &s->y, &s->dy, &s->xb,
-                   &s->yb, &s->red, &s->loss, &s->gerr})
-        b->release();
+    release_ws(s);
+    for (Buf* b : {&s->P, &s->Pm, &s->Pv, &s->Bf, &s->Wbf, &s->loss, &s->gerr}) b->release();
     if (s->own_stream) cudaStreamDestroy(s->stream);
     delete s;
 }
@@ -864,10 +898,19 @@ int sbr_surrogate_grads(sbr_surrogate* s, int member, const double* x, const dou
 {
     if (!s || !x || !y || n < 128 || n % 128 || member < 0 || member >= s->opt.n_members) return SBR_ERR_ARG;
     SCK(cudaSetDevice(s->device), "cudaSetDevice");
-    SCK(ensure_ws(s, (int)n, 1, true), "alloc training workspace");
     float* x4 = nullptr;
     int rc = upload_inputs(s, x, n, &x4);
     if (rc != SBR_OK) return rc;
+    cudaError_t ce = ensure_ws(s, (int)n, 1, true);
+    if (ce == cudaErrorMemoryAllocation) {  // once more, without what earlier calls had left
+        cudaGetLastError();
+        release_ws(s);
+        ce = ensure_ws(s, (int)n, 1, true);
+    }
+    if (ce != cudaSuccess) {
+        cudaFree(x4);
+        SCK(ce, "alloc training workspace");
+    }
     std::vector<float> yt((size_t)n * kOut);
     for (size_t i = 0; i < yt.size(); ++i) yt[i] = (float)(y[i] / s->target_scale);
     cudaMemcpyAsync(s->yb.p, yt.data(), sizeof(float) * yt.size(), cudaMemcpyHostToDevice, s->stream);
@@ -892,37 +935,40 @@ int sbr_surrogate_train(sbr_surrogate* s, const double* x, const double* y, int6
     if (n > (1ll << 31) - 1) return SBR_ERR_ARG;
     SCK(cudaSetDevice(s->device), "cudaSetDevice");
     const int M = (int)std::min<long long>(batch, (n / 128) * 128);
+    // the call's own arrays first, then the workspace of as many members at once as fit beside them: inputs, targets,
+    // and per member of the group one permutation per epoch and the per-epoch squared-error sums
+    float *x4 = nullptr, *y4 = nullptr;
+    int* dperm = nullptr;
+    double* dloss = nullptr;
     int group = 1;
-    int rc = choose_group(s, M, &group);
+    int rc = upload_inputs(s, x, n, &x4);
     if (rc != SBR_OK) return rc;
+    cudaError_t ce = call_alloc(s, &y4, (size_t)n * kOut);
+    if (ce != cudaSuccess) {
+        cudaFree(x4);
+        SCK(ce, "alloc targets");
+    }
+    rc = choose_group(s, M, n, epochs, &group, &dperm, &dloss);
+    if (rc != SBR_OK) {
+        cudaFree(x4);
+        cudaFree(y4);
+        return rc;
+    }
     // target scale: RMS of the targets
     double ss = 0.0;
     for (int64_t i = 0; i < n * kOut; ++i) ss += y[i] * y[i];
     s->target_scale = (float)std::max(sqrt(ss / (double)(n * kOut)), 1e-30);
-    float *x4 = nullptr, *y4 = nullptr;
-    rc = upload_inputs(s, x, n, &x4);
-    if (rc != SBR_OK) return rc;
     std::vector<float> yt((size_t)n * kOut);
     for (size_t i = 0; i < yt.size(); ++i) yt[i] = (float)(y[i] / s->target_scale);
-    cudaError_t ce = cudaMalloc(&y4, sizeof(float) * yt.size());
-    if (ce == cudaSuccess)
-        ce = cudaMemcpyAsync(y4, yt.data(), sizeof(float) * yt.size(), cudaMemcpyHostToDevice, s->stream);
-    if (ce != cudaSuccess) {
-        cudaFree(x4);
-        SCK(ce, "upload targets");
-    }
-    const long long steps_per_epoch = n / M;
-    // per member of the group one permutation per epoch and the per-epoch squared-error sums, on the device
-    int* dperm = nullptr;
-    double* dloss = nullptr;
-    ce = cudaMalloc(&dperm, sizeof(int) * (size_t)n * group);
-    if (ce == cudaSuccess) ce = cudaMalloc(&dloss, sizeof(double) * (size_t)epochs * group);
+    ce = cudaMemcpyAsync(y4, yt.data(), sizeof(float) * yt.size(), cudaMemcpyHostToDevice, s->stream);
     if (ce != cudaSuccess) {
         cudaFree(x4);
         cudaFree(y4);
         cudaFree(dperm);
-        SCK(ce, "alloc permutation");
+        cudaFree(dloss);
+        SCK(ce, "upload targets");
     }
+    const long long steps_per_epoch = n / M;
     std::vector<int> perm((size_t)n * group);
     std::vector<double> hloss((size_t)epochs * group);
     cudaMemsetAsync(s->gerr.p, 0, sizeof(int), s->stream);

@@ -44,3 +44,33 @@ def test_creation_uses_its_own_stream_alone(G):
         assert np.array_equal(s.params(e), ref.params(e)) and np.array_equal(s.fourier(e), ref.fourier(e))
     s.close()
     ref.close()
+
+
+def _fill(torch, leave):
+    """Tensors that take the GPU's free memory but for `leave` bytes."""
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free, _ = torch.cuda.mem_get_info()
+    return torch.empty(free - leave, dtype=torch.uint8, device="cuda")
+
+
+def test_training_fits_where_the_whole_ensemble_does_not(G):
+    """With 300 MB free the workspace of all four members (282 MB) fits only without the call's own arrays (48 MB while
+    the inputs are read, 96 MB in all): fewer members train together, to the same bits."""
+    torch = pytest.importorskip("torch")
+    net = dict(n_members=4, width=512, depth=2, n_fourier=128, fourier_sigma=2.0, seed=7)
+    x, y = _samples(2_000_000, 2)
+    ref = G.Surrogate(0, **net)
+    ref.train(x, y, epochs=1, batch=8192)
+    want = [ref.params(e) for e in range(4)]
+    ref.close()
+    s = G.Surrogate(0, **net)
+    hold = _fill(torch, 300 << 20)
+    try:
+        s.train(x, y, epochs=1, batch=8192)
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    for e in range(4):
+        assert np.array_equal(s.params(e), want[e])
+    s.close()
