@@ -1053,23 +1053,35 @@ int sbr_surrogate_predict(sbr_surrogate* s, const double* x, int64_t n, double* 
     SCK(cudaSetDevice(s->device), "cudaSetDevice");
     // all members at once, batches of about 512 MB of activations: 65536 rows of the default ensemble. Smaller ones
     // would stay in L2 but pay a pipeline fill and a last wave per launch (64 MB: 12.2, 256 MB: 8.9, 512 MB: 8.1,
-    // 1 GB: 7.9 ms for 300k points)
+    // 1 GB: 7.9 ms for 300k points). The Fourier features of a batch take no more than that either, and where the
+    // workspace does not fit beside the call's own arrays the batches are halved (a point's result depends on no
+    // other's).
     const int g = s->opt.n_members;
-    const long long fit = (512ll << 20) / (4ll * s->opt.width * g) / 128 * 128;
-    const int M = (int)std::min<int64_t>(std::max<long long>(1024, fit), ((n + 127) / 128) * 128);
-    SCK(ensure_ws(s, M, g, false), "alloc prediction workspace");
+    const long long wide = std::max(4ll * s->opt.width, 2ll * s->opt.n_fourier) * g;
+    const long long fit = (512ll << 20) / wide / 128 * 128;
+    int M = (int)std::min<int64_t>(std::max<long long>(1024, fit), ((n + 127) / 128) * 128);
     int rc = SBR_OK;
     float* x4 = nullptr;
     rc = upload_inputs(s, x, n, &x4);
     if (rc != SBR_OK) return rc;
     double* dmean = nullptr;
     float* dspread = nullptr;
-    cudaError_t ce = cudaMalloc(&dmean, sizeof(double) * kOut * (size_t)n);
-    if (ce == cudaSuccess) ce = cudaMalloc(&dspread, sizeof(float) * (size_t)n);
+    cudaError_t ce = call_alloc(s, &dmean, kOut * (size_t)n);
+    if (ce == cudaSuccess) ce = call_alloc(s, &dspread, (size_t)n);
+    for (bool last = false; ce == cudaSuccess;) {
+        ce = ensure_ws(s, M, g, false);
+        if (ce != cudaErrorMemoryAllocation || last) break;
+        cudaGetLastError();
+        release_ws(s);
+        if (M == 128) last = true;  // once more, without what earlier calls had left
+        else M = std::max(128, M / 2 / 128 * 128);
+        ce = cudaSuccess;
+    }
     if (ce != cudaSuccess) {
         cudaFree(x4);
         cudaFree(dmean);
-        SCK(ce, "alloc outputs");
+        cudaFree(dspread);
+        SCK(ce, "alloc outputs and workspace");
     }
     cudaMemsetAsync(s->gerr.p, 0, sizeof(int), s->stream);
     for (int64_t b0 = 0; b0 < n && rc == SBR_OK; b0 += M) {

@@ -74,3 +74,26 @@ def test_training_fits_where_the_whole_ensemble_does_not(G):
     for e in range(4):
         assert np.array_equal(s.params(e), want[e])
     s.close()
+
+
+@pytest.mark.parametrize("net,n,leave", [(dict(n_members=4, width=512, depth=2, n_fourier=128), 2_000_000, 300 << 20),
+                                         (dict(n_members=4, width=128, depth=1, n_fourier=8192), 300_000, 1200 << 20)])
+def test_prediction_fits_where_its_usual_batches_do_not(G, net, n, leave):
+    """A batch of 65,536 points of the wide network (0.6 GB of activations) does not fit into what is free, nor would
+    one sized by a narrow network's activations alone (17 GB of Fourier features): smaller ones give the same bits."""
+    torch = pytest.importorskip("torch")
+    x, y = _samples(n, 3)
+    s = G.Surrogate(0, fourier_sigma=2.0, seed=8, **net)
+    s.train(x[:256], y[:256], epochs=1, batch=256)
+    want = s.predict(x)
+    s.close()
+    s = G.Surrogate(0, fourier_sigma=2.0, seed=8, **net)
+    s.train(x[:256], y[:256], epochs=1, batch=256)
+    hold = _fill(torch, leave)
+    try:
+        got = s.predict(x)
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
+    s.close()
