@@ -406,8 +406,8 @@ int build_bvh(sbr_ctx* c, const sbr_bvh_opts* opt, const float* xyz, const int32
     CK(cudaStreamSynchronize(c->stream), "bvh build sync");
     if (herr[0]) {
         c->has_mesh = false;
-        if (herr[0] & 8) return fail(c, SBR_ERR_TIMEOUT, "sbr_build_bvh: a bounded device wait gave up");
         if (herr[0] & 4) return fail(c, SBR_ERR_CUDA, "sbr_build_bvh: the clustering did not converge");
+        if (herr[0] & 8) return fail(c, SBR_ERR_TIMEOUT, "sbr_build_bvh: a bounded device wait gave up");
         return fail(c, SBR_ERR_ARG, (herr[0] & 1) ? "sbr_build_bvh: triangle index out of range"
                                                   : "sbr_build_bvh: a vertex coordinate is not finite");
     }

@@ -933,7 +933,8 @@ __global__ void __launch_bounds__(kSmallThreads) k_collapse4_small(const float4*
 // index check on the host beside the build; the clustering 1.07 ms, bound by the
 // dependent steps of a round). Both run as one cooperative launch whose blocks (all resident) meet at a barrier between the steps; data written
 // by other blocks is read past L1. Every wait is bounded: a block that gives up
-// sets bit 8 of the error flag and leaves, and so do the others in turn.
+// sets bit 8 of the error flag and leaves, and the others' waits end when they
+// see a bit that leaves no tree behind.
 constexpr int kCoopThreads = 512;
 constexpr unsigned kCoopSpin = 1u << 22;
 
@@ -954,6 +955,10 @@ struct GridBarrier {
             while (*(volatile unsigned*)count < passed) {
                 if (++i > kCoopSpin) {
                     atomicOr(err, 8);
+                    bad = 1;
+                    break;
+                }
+                if ((i & 63u) == 0u && (*(volatile int*)err & kErrTree)) {
                     bad = 1;
                     break;
                 }
@@ -1008,11 +1013,11 @@ __device__ __forceinline__ void block_sum2(unsigned& a, unsigned& b, unsigned (*
 
 // The last rounds, of at most kSoloMax clusters, by one block in shared memory
 // (half of all rounds: the clusters shrink by a sixth each). Two clusters per
-// thread; false if the clustering does not converge.
+// thread; sets bit 4 of the error flag if the clustering does not converge.
 constexpr int kSoloMax = 2 * kCoopThreads;
 constexpr size_t kSoloSmem = kSoloMax * (2 * sizeof(float4) + 4 * sizeof(int));
 static_assert(kSoloSmem >= 2 * sizeof(float4) * (kCoopThreads + 128), "a tile and its halo fit too");
-__device__ bool ploc_solo(const PlocCoop& b, Clusters c, int m, int round)
+__device__ void ploc_solo(const PlocCoop& b, Clusters c, int m, int round)
 {
     constexpr int T = kCoopThreads;
     extern __shared__ float4 s_dyn[];
@@ -1035,7 +1040,7 @@ __device__ bool ploc_solo(const PlocCoop& b, Clusters c, int m, int round)
     for (; m > 1; ++round) {
         if (round >= (1 << 16)) {  // every round merges at least one pair
             if (tid == 0) atomicOr(b.err, 4);
-            return false;
+            return;
         }
         for (int i = tid; i < m; i += T) {
             const float4 l = lo[i], h = hi[i];
@@ -1102,7 +1107,6 @@ __device__ bool ploc_solo(const PlocCoop& b, Clusters c, int m, int round)
         m = (int)at;
         __syncthreads();
     }
-    return true;
 }
 
 // The PLOC rounds over tiles of kCoopThreads clusters, each block a contiguous
@@ -1206,8 +1210,9 @@ __global__ void __launch_bounds__(kCoopThreads) k_ploc_coop(const PlocCoop b)
         m = (int)total;
         cur ^= 1;
     }
-    if (blockIdx.x == 0 && !ploc_solo(b, b.cl[cur], m, round)) return;
+    if (blockIdx.x == 0) ploc_solo(b, b.cl[cur], m, round);
     if (!bar.wait()) return;
+    if (__ldcg(b.err) & kErrTree) return;  // block 0's clusters did not converge: every block sees it here
     // first positions of every node and triangle
     const int nx = 2 * n - 1;
     int pj = 0;

@@ -68,3 +68,25 @@ def test_refused_meshes_leave_the_context_usable(G):
             c.load_mesh(xyz, tri)
             st = c.trace([[170.0, 4.0]], 0.05, max_bounces=3)
             assert st["ray_bounces"] == ref["ray_bounces"] and st["valid_rays"] == ref["valid_rays"]
+
+
+@pytest.mark.parametrize("ties", [True, False])
+def test_clustering_that_ends_in_its_last_rounds_says_so(G, ties):
+    """66,000 coincident triangles pair up once a round, so the limit of 65,536 rounds falls into the last ones, which
+    one block runs while the others wait for it; 100 groups further apart than FP32 box areas reach stop pairing up
+    there. Both are reported as the clustering's failure, not as a wait that gave up, and the next mesh loads."""
+    if ties:
+        x = np.array([[0, 0, 0], [1, 0, 0], [0, 1, 0]], np.float32)
+        t = np.tile([[0, 1, 2]], (66_000, 1)).astype(np.int32)
+    else:
+        rng = np.random.default_rng(3)
+        at = np.repeat(np.arange(100) * 3e20, 200)[:, None, None] + rng.uniform(0, 1e17, (20_000, 1, 3))
+        x = (at + rng.uniform(0, 2e16, (20_000, 3, 3))).astype(np.float32).reshape(-1, 3)
+        t = np.arange(60_000, dtype=np.int32).reshape(-1, 3)
+    xyz, tri = _mesh(20_000)
+    with G.Context(0) as c:
+        with pytest.raises(G.SbrError) as e:
+            c.load_mesh(x, t)
+        assert e.value.code == -2 and "did not converge" in str(e.value)
+        c.load_mesh(xyz, tri)
+        assert c.trace([[170.0, 4.0]], 0.05, max_bounces=3)["valid_rays"] > 0
