@@ -341,8 +341,8 @@ typedef struct {
                             runs the FP32 test for each grid ray of its widened projected box and a 64-bit
                             atomic minimum of (t, original index) keeps the closest hit, so the hits are
                             those of the traversal; an aspect with a triangle spanning more than 2^24 grid
-                            cells, or with more than 65535 rays in a row or column, traverses instead. The
-                            silhouette mask is then not used. Default 1 */
+                            cells, with stacks of large triangles, or with more than 65535 rays in a row or
+                            column, traverses instead. The silhouette mask is then not used. Default 1 */
 } sbr_tuning;
 int sbr_get_tuning(const sbr_ctx* ctx, sbr_tuning* out);
 /* SBR_ERR_ARG for a value outside the ranges above. */

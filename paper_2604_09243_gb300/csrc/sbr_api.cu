@@ -654,7 +654,7 @@ int plan_chunks(sbr_ctx* c, TraceRun& R, std::vector<int64_t>& cut, long long* t
     if (c->tune.silhouette) CK(c->cover.ensure(sizeof(unsigned) * (size_t)(max_tiles + max_angles)), "alloc cover");
     if (c->tune.raster) {
         CK(c->vis.ensure(sizeof(unsigned long long) * (size_t)max_chunk), "alloc raster keys");
-        CK(c->visfull.ensure(sizeof(unsigned) * (size_t)(max_angles + 1)), "alloc raster flags");
+        CK(c->visfull.ensure(sizeof(unsigned) * vis_full_words(max_angles)), "alloc raster flags");
         CK(c->hitlist.ensure(sizeof(uint2) * (size_t)max_chunk), "alloc raster hit list");
         c->rbig_cap = raster_big_cap(max_chunk);
         CK(c->rbig.ensure(sizeof(int4) * (size_t)c->rbig_cap), "alloc raster triangle list");
@@ -765,7 +765,7 @@ TraceInit trace_init(unsigned long long* stats, const DevBuf& ctr64, const DevBu
     zero(ctr32.p, sizeof(unsigned) * 2 * (kMaxBounces + 2) + 64);
     if (stats) zero(stats, sizeof(unsigned long long) * kStatCount);
     if (raster) {
-        zero(visfull.p, sizeof(unsigned) * (size_t)(na + 1));
+        zero(visfull.p, sizeof(unsigned) * vis_full_words(na));
         zero(rbigctr.p, sizeof(unsigned) * 2);
         b.vis16 = vis.as<uint4>();
         b.n_vis16 = rays / 2;
@@ -1367,7 +1367,7 @@ int build_plan(sbr_ctx* c, BatchPlan& P)
     if (P.tune.silhouette) CK(P.cover.ensure(sizeof(unsigned) * (size_t)(max_tiles + max_angles)), "alloc cover");
     if (P.tune.raster) {
         CK(P.vis.ensure(sizeof(unsigned long long) * (size_t)max_rays), "alloc raster keys");
-        CK(P.visfull.ensure(sizeof(unsigned) * (size_t)(max_angles + 1)), "alloc raster flags");
+        CK(P.visfull.ensure(sizeof(unsigned) * vis_full_words(max_angles)), "alloc raster flags");
         CK(P.hitlist.ensure(sizeof(uint2) * (size_t)max_rays), "alloc raster hit list");
         P.big_cap = (unsigned)raster_big_cap(max_rays);
         CK(P.rbig.ensure(sizeof(int4) * (size_t)P.big_cap), "alloc raster triangle list");

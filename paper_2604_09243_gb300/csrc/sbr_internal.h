@@ -191,7 +191,8 @@ struct TraceArgs {
     const unsigned long long* vis; // optional (primary pass) [total_rays] closest-hit keys: rasterised, or of
                                    // the flagged aspects traversed
     const unsigned* vis_full;     // with vis: [n_angles + 1] 1 = the aspect's primary rays traverse the tree;
-                                  // [n_angles]: 1 if any aspect does
+                                  // [n_angles]: 1 if any aspect does; then the rasterisation's [n_angles] sums of
+                                  // the cells of each aspect's largest triangles (vis_full_words in all)
     unsigned* slot_scr;           // with vis: kSlotWords of scratch
     unsigned* rec_off;            // with vis: [n_angles + 1] first record of each aspect in the chunk, and the total
     unsigned* rec_off_host;       // the same in pinned host memory (may be null)
@@ -205,6 +206,7 @@ struct TraceArgs {
                                   // (ray, aspect) of each hit here instead of storing its state, and
                                   // bounce pass 1 rebuilds the state from the list
 };
+constexpr size_t vis_full_words(long long n_angles) { return 2 * (size_t)n_angles + 1; }
 int trace_blocks_per_sm();
 // rays that k_tail can take in a launch of n_blocks blocks
 unsigned trace_tail_rays(int n_blocks);
@@ -236,7 +238,8 @@ cudaError_t launch_silhouette(const TraceArgs& a, int n_tri, unsigned* cover, cu
 // (FP32 t bits << 32 | original triangle index) over the triangles whose FP32
 // test accepts primary ray g, or stays ~0 for none; full[aspect] = 1 and
 // full[n_angles] = 1 when a triangle covers more than kRasterMaxCells cells of
-// that aspect or does not fit the list (its rays then traverse the tree in the
+// that aspect or does not fit the list, or when its triangles above 2^14 cells
+// cover more than 20 box cells per ray (its rays then traverse the tree in the
 // primary pass, which writes their keys). vis, full and a.big_ctr must have been
 // cleared (launch_trace_begin). The primary pass sets a.mask to the valid bits
 // of the keys, a.tile_base to their exclusive scan, *a.q_out_count to their

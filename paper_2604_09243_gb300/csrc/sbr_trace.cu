@@ -1409,15 +1409,33 @@ constexpr size_t kRasterSmem = sizeof(RasterItem) * 32 * kRasterWarps;
 // Appends the large triangles of the warp's lanes (want; cell ranges i0..i1,
 // j0..j1 of aspect ang) to the list of k_raster_big, cut into bands of rows of
 // about kRasterBand cells: a warp of k_raster_big takes a band at a time, so a
-// plate of millions of cells is shared by all of them (an aspect with a triangle
-// above 2^14 cells used to traverse all its rays: 4.0 of 41 ms for 23 aircraft
+// plate of millions of cells is shared by all of them (traversing all rays of
+// an aspect for its triangles above 2^14 cells: 4.0 of 41 ms for 23 aircraft
 // aspects at 7 to 12 GHz). The aspects of entries that find the list full
-// traverse. Every lane of the warp calls it.
-constexpr int kRasterBand = 4096;
+// traverse, and so do those whose triangles above kRasterBanded cells cover
+// more than 20 box cells per ray: every layer is a test of every ray, while the
+// traversal stops at the first (4 aspects of 3000 x 3000 rays on stacked
+// plates of two triangles, B = 2, banded against traversed: 1 plate 1.5 / 4.1 ms,
+// 10: 4.0 / 4.4, 30: 9.0 / 4.7, 300: 73 / 8.2). Every lane of the warp calls it.
+constexpr int kRasterBand = 4096, kRasterBanded = 1 << 14;
 __device__ __forceinline__ void append_big(const TraceArgs& a, unsigned* full, bool want, int t, int ang, int i0, int i1,
                                            int j0, int j1)
 {
     if (!__any_sync(kFull, want)) return;
+    if (want) {
+        const unsigned cells = (unsigned)((i1 - i0 + 1) * (j1 - j0 + 1));
+        if (cells > kRasterBanded) {
+            // the aspect's sum of such triangles' cells, in units of 1024 (its last value, and so whether the aspect
+            // traverses, does not depend on the order; left alone above the limit, so that it cannot wrap)
+            unsigned* sum = full + a.n_angles + 1 + ang;
+            const unsigned most = (unsigned)(20 * (a.ray_off[ang + 1] - a.ray_off[ang]) >> 10), n = (cells + 1023u) >> 10;
+            if (__ldcg(sum) > most || atomicAdd(sum, n) + n > most) {
+                want = false;
+                atomicOr(full + ang, 1u);
+                atomicOr(full + a.n_angles, 1u);  // some aspect of the chunk traverses
+            }
+        }
+    }
     const int lane = threadIdx.x & 31;
     const int rows = want ? max(1, kRasterBand / (i1 - i0 + 1)) : 1;
     const unsigned n = want ? (unsigned)((j1 - j0 + rows) / rows) : 0u;  // bands
@@ -1694,6 +1712,7 @@ __global__ void __launch_bounds__(256, 3) k_raster_big(const TraceArgs a, unsign
     for (unsigned it = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < n_big; it += nw) {
         const int4 b = a.big[it];
         const int td = b.x, ad = b.y;
+        if (a.vis_full[ad]) continue;  // traverses
         const int i0 = b.z & 0xFFFF, j0 = (unsigned)b.z >> 16, w = (b.w & 0xFFFF) + 1, h = ((unsigned)b.w >> 16) + 1;
         const int i1 = i0 + w - 1, j1 = j0 + h - 1;
         const AngleDev& A = a.angles[ad];
