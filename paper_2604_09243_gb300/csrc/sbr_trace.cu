@@ -1386,6 +1386,22 @@ __device__ __forceinline__ void raster_cell(const RasterGrid& G, const TraceArgs
     }
 }
 
+// Below the smallest stored distance that a ray of the grid (origin p0,
+// direction d) can have on a triangle: the distances along d of the vertices
+// from the grid plane (the ray origins lie in it to within micrometres); the
+// stored distance of any hit is at least their minimum less the key's plane
+// slack (0.08 bUV / |d.n|, as in key_of), 1e-4 of it and 1 mm.
+__device__ __forceinline__ float raster_tnear(float4 P, float4 B, float4 C, float3 p0, float3 d, const PlaneKey& K)
+{
+    const float3 q0 = make_float3(P.x - p0.x, P.y - p0.y, P.z - p0.z);
+    const float z0 = dot_s(q0, d), z1 = z0 + dot_s(make_float3(B.x, B.y, B.z), d),
+                z2 = z0 + dot_s(make_float3(C.x, C.y, C.z), d);
+    const float zm = fminf(z0, fminf(z1, z2));
+    const float slack = K.dh != 0.f ? 0.32f * B.w / fabsf(K.dh) : FLT_MAX;
+    const float tnear = zm - (1e-4f * fabsf(zm) + 1e-3f + slack);
+    return isfinite(tnear) ? tnear : -FLT_MAX;
+}
+
 // A triangle of the flattened rasterisation and everything its cells need,
 // one per lane in shared memory as 13 16-byte words (a stride of 52 words: the
 // 16-byte accesses of 8 lanes to different triangles fall in distinct banks,
@@ -1418,10 +1434,9 @@ constexpr size_t kRasterSmem = sizeof(RasterItem) * 32 * kRasterWarps;
 // plates of two triangles, B = 2, banded against traversed: 1 plate 1.5 / 4.1 ms,
 // 10: 4.0 / 4.4, 30: 9.0 / 4.7, 300: 73 / 8.2). Every lane of the warp calls it.
 constexpr int kRasterBand = 4096, kRasterBanded = 1 << 14;
-__device__ __forceinline__ void append_big(const TraceArgs& a, unsigned* full, bool want, int t, int ang, int i0, int i1,
-                                           int j0, int j1)
+__device__ __noinline__ void append_some(const TraceArgs& a, unsigned* full, bool want, int t, int ang, int i0, int i1,
+                                         int j0, int j1)
 {
-    if (!__any_sync(kFull, want)) return;
     if (want) {
         const unsigned cells = (unsigned)((i1 - i0 + 1) * (j1 - j0 + 1));
         if (cells > kRasterBanded) {
@@ -1464,6 +1479,13 @@ __device__ __forceinline__ void append_big(const TraceArgs& a, unsigned* full, b
         atomicOr(full + ang, 1u);
         atomicOr(full + a.n_angles, 1u);  // some aspect of the chunk traverses
     }
+}
+
+// (the warps with any, out of line)
+__device__ __forceinline__ void append_big(const TraceArgs& a, unsigned* full, bool want, int t, int ang, int i0, int i1,
+                                           int j0, int j1)
+{
+    if (__any_sync(kFull, want)) append_some(a, full, want, t, ang, i0, i1, j0, j1);
 }
 
 // The cells of row y inside an item's moved edges: columns [lo, lo + cnt) of
@@ -1595,16 +1617,7 @@ __global__ void __launch_bounds__(256, 4) k_raster(const TraceArgs a, int n_tri,
                         it.r3.z = K.n.x;
                         it.r3.w = K.n.y;
                         it.r4 = make_float4(K.n.z, K.dh, K.dl, K.rd);
-                        // distances along d of the vertices from the grid plane (the ray origins lie in it to
-                        // within micrometres); the stored distance of any hit on the triangle is at least their
-                        // minimum less the key's plane slack (0.08 bUV / |d.n|, as in key_of), 1e-4 of it and 1 mm
-                        const float3 q0 = make_float3(P.x - G.p0.x, P.y - G.p0.y, P.z - G.p0.z);
-                        const float z0 = dot_s(q0, G.d), z1 = z0 + dot_s(make_float3(B.x, B.y, B.z), G.d),
-                                    z2 = z0 + dot_s(make_float3(C.x, C.y, C.z), G.d);
-                        const float zm = fminf(z0, fminf(z1, z2));
-                        const float slack = K.dh != 0.f ? 0.32f * B.w / fabsf(K.dh) : FLT_MAX;
-                        const float tnear = zm - (1e-4f * fabsf(zm) + 1e-3f + slack);
-                        it.e2 = make_float4(c2, 0.f, isfinite(tnear) ? tnear : -FLT_MAX,
+                        it.e2 = make_float4(c2, 0.f, raster_tnear(P, B, C, G.p0, G.d, K),
                                             __int_as_float((int)a.ray_off[ang]));
                         it.g0 = make_float4(G.p0.x, G.p0.y, G.p0.z, G.du.x);
                         it.g1 = make_float4(G.du.y, G.du.z, G.dv.x, G.dv.y);
@@ -1698,10 +1711,123 @@ __global__ void __launch_bounds__(256, 4) k_raster(const TraceArgs a, int n_tri,
     }
 }
 
+// One (triangle, cell) pair: the traversal's test of primary ray (i, j) against triangle t, a hit's key kept. A ray
+// whose hit so far is nearer than tnear (raster_tnear; kNear) needs none; returns the tests made.
+template <bool kNear = false>
+__device__ __forceinline__ unsigned sparse_pair(const TraceArgs& a, unsigned long long* vis, int t, int ang, int ij,
+                                                int count, float tnear = 0.f)
+{
+    const AngleDev& A = a.angles[ang];
+    const int i = ij & 0xFFFF, j = (int)((unsigned)ij >> 16);
+    auto at = [&]() {
+        const int tw = A.tw_log2, sh = 5 - tw;
+        return a.ray_off[ang] + ((long long)((j >> sh) * A.nbu + (i >> tw)) << 5) + ((j & ((1 << sh) - 1)) << tw) +
+               (i & ((1 << tw) - 1));
+    };
+    if (kNear && __uint_as_float((unsigned)(__ldcg(vis + at()) >> 32)) < tnear) return 0u;
+    const float3 o = primary_origin(A, i, j), d = make_float3(A.dir[0], A.dir[1], A.dir[2]);
+    const float4* tp = a.tris + 3 * (size_t)t;
+    const float4 P = __ldg(tp), B = __ldg(tp + 1), C = __ldg(tp + 2);
+    float tc, et;
+    const int f = tri_filter(P, B, C, o, d, tc, et);
+    if (f == 0) return 1u;
+    if (f >= 2) {
+        const int r = tri_refine(a.tris, a.tri_v12, t, o, d, f + 2, tc);
+        if (count) count_open(a.stats, r);
+        if (!(r & 1)) return 1u;
+    }
+    const PlaneKey K = plane_key(a.tri_nrm, t, d);
+    const float th = plane_key_t(K, make_float3(P.x, P.y, P.z), o, tc);
+    if (th >= 0.f && th <= FLT_MAX)
+        atomicMin(vis + at(), ((unsigned long long)__float_as_uint(th) << 32) | (unsigned)__float_as_int(P.w));
+    return 1u;
+}
+
+// The cells of up to 32 triangles of a sparse grid, lane l's triangle t of
+// aspect ang (t < 0: none): their edges in shared memory, their rows' spans a
+// row per lane, the spans' cells a cell per lane. Returns the lane's tests.
+__host__ __device__ __forceinline__ unsigned sparse_list_cap(const TraceArgs& a)
+{
+    const long long n = a.total_rays * (long long)(sizeof(RayState) / sizeof(int2));
+    return (unsigned)(n < (1ll << 30) ? n : 1ll << 30);
+}
+struct __align__(16) SparseItem {
+    float4 e0, e1;  // the edges of RasterItem
+    float c2, tnear;
+    int w, ij, t, ang;
+    int pad[2];
+};
+__device__ __forceinline__ unsigned sparse_walk(const TraceArgs& a, unsigned long long* vis, int t, int ang, int count)
+{
+    __shared__ SparseItem s_items[kRasterWarps][32];
+    __shared__ int s_off[kRasterWarps][33];
+    __shared__ uint2 s_span[kRasterWarps][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    SparseItem* my = s_items[warp];
+    int* off = s_off[warp];
+    int nr = 0;
+    if (t >= 0) {
+        const AngleDev& A = a.angles[ang];
+        const float4* tp = a.tris + 3 * (size_t)t;
+        int i0, i1, j0, j1;
+        TriProj pr;
+        const float4 P = __ldg(tp), B = __ldg(tp + 1), C = __ldg(tp + 2);
+        tri_project(A, cell_scale(A), P, B, C, pr);
+        if (tri_cells_p(A, pr, i0, i1, j0, j1)) {
+            const float3 d = make_float3(A.dir[0], A.dir[1], A.dir[2]);
+            const PlaneKey K = plane_key(a.tri_nrm, t, d);
+            CellEdges E;
+            tri_cell_edges_p(pr, i0, i1, j0, j1, E);
+            SparseItem& it = my[lane];
+            it.e0 = make_float4(E.nx[0], E.ny[0], E.c[0], E.nx[1]);
+            it.e1 = make_float4(E.ny[1], E.c[1], E.nx[2], E.ny[2]);
+            it.c2 = E.c[2];
+            it.tnear = raster_tnear(P, B, C, make_float3(A.p0[0], A.p0[1], A.p0[2]), d, K);
+            it.w = i1 - i0 + 1;
+            it.ij = i0 | (j0 << 16);
+            it.t = t;
+            it.ang = ang;
+            nr = j1 - j0 + 1;
+        }
+    }
+    int incl = nr;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += y;
+    }
+    off[lane + 1] = incl;
+    if (lane == 0) off[0] = 0;
+    __syncwarp();
+    const int total = __shfl_sync(kFull, incl, 31);
+    unsigned n = 0;
+    int k = 0;
+    for (int rb = 0; rb < total; rb += 32) {
+        int cnt = 0, lo = 0, row = 0;
+        if (rb + lane < total) {
+            while (off[k + 1] <= rb + lane) ++k;
+            const SparseItem& it = my[k];
+            const float4 e0 = it.e0, e1 = it.e1;
+            const float nx[3] = {e0.x, e0.w, e1.z}, ny[3] = {e0.y, e1.x, e1.w}, c[3] = {e0.z, e1.y, it.c2};
+            row = rb + lane - off[k];
+            row_span(nx, ny, c, (float)row, it.w, lo, cnt);
+        }
+        each_cell(s_span[warp], k, row, lo, cnt, [&](int tri, int dj, int di) {
+            const SparseItem& it = my[tri];
+            n += sparse_pair<true>(a, vis, it.t, it.ang, it.ij + (di | (dj << 16)), count, it.tnear);
+        });
+    }
+    __syncwarp();  // my[] and off[] may be rewritten
+    return n;
+}
+
 // The listed large triangles, warp w taking entries w, w + warps, ... (every
 // warp has hundreds of entries, so the few very large triangles average out),
 // the cells of their rows' spans 32 at a time (0.16 ms for 37 aircraft aspects
-// at 10 GHz, 0.70 with every cell of the box a lane's).
+// at 10 GHz, 0.70 with every cell of the box a lane's). kSparse: then the
+// middling triangles that k_raster_sparse has listed (a.q_out), 32 a warp or as
+// many as keep every warp busy.
+template <bool kSparse>
 __global__ void __launch_bounds__(256, 3) k_raster_big(const TraceArgs a, unsigned long long* vis, int count)
 {
     const int lane = threadIdx.x & 31;
@@ -1735,6 +1861,14 @@ __global__ void __launch_bounds__(256, 3) k_raster_big(const TraceArgs a, unsign
             });
         }
     }
+    if (kSparse) {
+        const unsigned n = min(a.big_ctr[1], sparse_list_cap(a)), per = min(32u, (n + nw - 1) / nw);
+        const int2* list = reinterpret_cast<const int2*>(a.q_out);
+        for (unsigned it = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per; it < n; it += nw * per) {
+            const int2 e = (unsigned)lane < per && it + lane < n ? list[it + lane] : make_int2(-1, 0);
+            ntri += sparse_walk(a, vis, e.x, e.y, count);
+        }
+    }
     if (count) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) ntri += __shfl_xor_sync(kFull, ntri, o);
@@ -1746,17 +1880,23 @@ __global__ void __launch_bounds__(256, 3) k_raster_big(const TraceArgs a, unsign
 }
 
 // ---------------------------------------------------------------- rasterisation of sparse grids
-// Where an aspect has fewer grid rays than twice the triangles (the aircraft at
-// 1 GHz: 0.14 rays per triangle), most triangles cover no cell and the others
-// one or a few: the set-up of k_raster for a warp walk costs more than the
-// tests. Here a lane keeps one triangle and projects it for up to 16 aspects in
+// Where a chunk's aspects have fewer than three grid rays (padding included, on
+// the mean) for two triangles (the aircraft at 1 GHz: 0.14 rays per triangle),
+// most triangles cover no cell and the others one or a few: the set-up of
+// k_raster for a warp walk costs more than the tests. Here a lane keeps one triangle and projects it for up to 16 aspects in
 // turn (the triangle is read once for all of them, an aspect in three broadcast
 // loads); the (triangle, cell) pairs of triangles of at most kSparseCells cells
 // collect in a queue of the warp, and 32 of them at a time take the traversal's
-// triangle test. Larger triangles go to the list of k_raster_big. Bound by
+// triangle test. Triangles of at most kSparseFlat cells are listed in queue 0,
+// idle until the first states are written, and k_raster_big walks the rows'
+// spans of 32 of them at a time (those that find no room are queued cell by
+// cell); larger ones go to its list of large triangles. 6 aspects of 800 x 800
+// rays over sheets whose triangles span 5 x 5 cells, beside a fine sphere, B = 2:
+// 4, 16 and 64 sheets in 1.3, 2.1 and 5.3 ms, with a warp each for triangles of
+// more than 16 cells 2.0, 5.8 and 15.5 (the list full from 8 sheets on). Bound by
 // instruction issue: ~235 instructions per 32 (triangle, aspect) items at 1 GHz
 // against ~820 of k_raster, 354 M items in 3.2 against 10.0 ms.
-constexpr int kSparseCells = 16, kSparseAspects = 16;
+constexpr int kSparseCells = 16, kSparseFlat = 256, kSparseAspects = 16;
 
 // The aspect's fields that the projection reads
 struct AspectView {
@@ -1798,30 +1938,18 @@ __device__ __forceinline__ bool sparse_cells(const AspectView& A, const float* x
     return i0 <= i1 && j0 <= j1;
 }
 
-// one (triangle, cell) pair: the traversal's test of primary ray (i, j) against triangle t, a hit's key kept
-__device__ __forceinline__ void sparse_pair(const TraceArgs& a, unsigned long long* vis, int t, int ang, int ij, int count)
+// Lists triangle t of aspect ang for the lanes of m (every lane of the warp calls it, those of m learn whether there
+// was room). Out of line, so that it does not burden the projection.
+__device__ __noinline__ bool sparse_list(const TraceArgs& a, unsigned m, int t, int ang)
 {
-    const AngleDev& A = a.angles[ang];
-    const int i = ij & 0xFFFF, j = (int)((unsigned)ij >> 16);
-    const float3 o = primary_origin(A, i, j), d = make_float3(A.dir[0], A.dir[1], A.dir[2]);
-    const float4* tp = a.tris + 3 * (size_t)t;
-    const float4 P = __ldg(tp), B = __ldg(tp + 1), C = __ldg(tp + 2);
-    float tc, et;
-    const int f = tri_filter(P, B, C, o, d, tc, et);
-    if (f == 0) return;
-    if (f >= 2) {
-        const int r = tri_refine(a.tris, a.tri_v12, t, o, d, f + 2, tc);
-        if (count) count_open(a.stats, r);
-        if (!(r & 1)) return;
-    }
-    const PlaneKey K = plane_key(a.tri_nrm, t, d);
-    const float th = plane_key_t(K, make_float3(P.x, P.y, P.z), o, tc);
-    if (th >= 0.f && th <= FLT_MAX) {
-        const int tw = A.tw_log2, sh = 5 - tw;
-        const long long pidx = a.ray_off[ang] + ((long long)((j >> sh) * A.nbu + (i >> tw)) << 5) +
-                               ((j & ((1 << sh) - 1)) << tw) + (i & ((1 << tw) - 1));
-        atomicMin(vis + pidx, ((unsigned long long)__float_as_uint(th) << 32) | (unsigned)__float_as_int(P.w));
-    }
+    const int lane = threadIdx.x & 31;
+    const unsigned cap = sparse_list_cap(a);
+    unsigned slot = cap;  // (a full list is left alone, so that its counter cannot wrap)
+    if (lane == 0 && __ldcg(a.big_ctr + 1) < cap) slot = atomicAdd(a.big_ctr + 1, (unsigned)__popc(m));
+    slot = __shfl_sync(kFull, slot, 0) + __popc(m & ((1u << lane) - 1u));
+    if (!((m >> lane) & 1u) || slot >= cap) return false;
+    reinterpret_cast<int2*>(a.q_out)[slot] = make_int2(t, ang);
+    return true;
 }
 
 __global__ void __launch_bounds__(256, 3) k_raster_sparse(const TraceArgs a, int n_tri, int aspects, unsigned long long* vis,
@@ -1857,7 +1985,7 @@ __global__ void __launch_bounds__(256, 3) k_raster_sparse(const TraceArgs a, int
                     if (nc > kRasterMaxCells || __float_as_int(A.a.w) > 65535 || __float_as_int(A.b.w) > 65535) {
                         atomicOr(full + ang, 1u);
                         atomicOr(full + a.n_angles, 1u);  // some aspect of the chunk traverses
-                    } else if (nc > kSparseCells) {
+                    } else if (nc > kSparseFlat) {
                         want_big = true;
                     } else {
                         n_cell = (int)nc;
@@ -1865,9 +1993,16 @@ __global__ void __launch_bounds__(256, 3) k_raster_sparse(const TraceArgs a, int
                 }
             }
             append_big(a, full, want_big, t, ang, i0, i1, j0, j1);
+            unsigned mc = __ballot_sync(kFull, n_cell > 0);
+            if (!mc) continue;
+            const unsigned ml = __ballot_sync(kFull, n_cell > kSparseCells);
+            if (ml) {
+                if (sparse_list(a, ml, t, ang)) n_cell = 0;
+                mc = __ballot_sync(kFull, n_cell > 0);
+            }
             // the triangle's cells row by row, one of each lane's at a time
             int ci = i0, cj = j0;
-            for (unsigned mc = __ballot_sync(kFull, n_cell > 0); mc; mc = __ballot_sync(kFull, n_cell > 0)) {
+            for (; mc; mc = __ballot_sync(kFull, n_cell > 0)) {
                 if (n_cell > 0) {
                     const int at = n_wait + __popc(mc & ((1u << lane) - 1u));
                     qt[at] = t;
@@ -2788,12 +2923,13 @@ cudaError_t launch_raster(const TraceArgs& a, int n_tri, unsigned long long* vis
         while (aspects > 1 && items() < 8ll * n_blocks) aspects /= 2;
         k_raster_sparse<<<(int)std::min<long long>((items() + kRasterWarps - 1) / kRasterWarps, n_blocks),
                           32 * kRasterWarps, 0, st>>>(a, n_tri, aspects, vis, full, count ? 1 : 0);
+        k_raster_big<true><<<n_blocks, 256, 0, st>>>(a, vis, count ? 1 : 0);
     } else {
         const long long need = ((long long)a.n_angles * n_tri + 255) / 256;
         k_raster<<<(int)std::max(1ll, std::min<long long>(need, n_blocks)), 32 * kRasterWarps, kRasterSmem, st>>>(
             a, n_tri, vis, full, count ? 1 : 0);
+        k_raster_big<false><<<n_blocks, 256, 0, st>>>(a, vis, count ? 1 : 0);
     }
-    k_raster_big<<<n_blocks, 256, 0, st>>>(a, vis, count ? 1 : 0);
     return cudaGetLastError();
 }
 

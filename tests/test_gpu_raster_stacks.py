@@ -52,3 +52,23 @@ def test_stacks_of_large_triangles(G, n, rays, ang, traversed):
     xyz, tri = _stack(n)
     sr, _ = _both(G, xyz, tri, np.array(ang, float), 1.0 / rays)
     assert (sr["node_visits"] > 0) == traversed
+
+
+def _join(*meshes):
+    off = np.cumsum([0] + [len(x) for x, _ in meshes])
+    return np.concatenate([x for x, _ in meshes]), np.concatenate([t + o for (_, t), o in zip(meshes, off)]).astype(np.int32)
+
+
+# 140,000 triangles of 81 to 100 box cells, more than the list of large ones has room for (65,536 entries), which do
+# not go there; beside them a plate of 400 cells, which does; boxes of 16 to 25 cells and of 225 to 289, on both sides
+# of the two limits (16 and 256); more of some 300 cells than the list holds, whose aspects traverse
+@pytest.mark.parametrize("n,rays,side,plate,traversed", [(70_000, 9, 1.0, 0, False), (70_000, 20, 0.45, 1, False),
+                                                         (20_000, 4, 1.0, 0, False), (3000, 11, 1.0, 0, False),
+                                                         (3000, 15, 1.0, 0, False), (40_000, 17, 1.0, 0, True)])
+def test_stacks_under_sparse_grids(G, n, rays, side, plate, traversed):
+    mesh = _stack(n, side, gap=2.0 ** -13)
+    if plate:
+        x, t = _stack(1, 1.0)
+        mesh = _join(mesh, (x + np.array([0, 0, 9.0], np.float32), t), (x - np.array([0, 0, 1.0], np.float32), t))
+    sr, _ = _both(G, *mesh, np.array([[0.0, 90.0], [3.0, 88.0], [90.0, 90.0]]), 1.0 / rays)
+    assert (sr["node_visits"] > 0) == traversed
