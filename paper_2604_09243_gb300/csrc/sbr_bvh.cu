@@ -927,12 +927,12 @@ __global__ void __launch_bounds__(kSmallThreads) k_collapse4_small(const float4*
 
 // ---------------------------------------------------------------- builds in one launch
 // The clustering takes some 85 rounds for a million triangles and the 4-wide
-// collapse one step per level, each a few microseconds of work: six launches per
-// round and a host read every four made the rounds 2.9 of the 7.1 ms that loading
-// the 983k-triangle aircraft and a first look at it took (3.4 ms now, with the
-// index check on the host beside the build; the clustering 1.07 ms, bound by the
-// dependent steps of a round). Both run as one cooperative launch whose blocks (all resident) meet at a barrier between the steps; data written
-// by other blocks is read past L1. Every wait is bounded: a block that gives up
+// collapse one step per level, each a few microseconds of work. Both run as one
+// cooperative launch whose blocks (all resident) meet at a barrier between the
+// steps: 1.07 ms for the clustering of the 983k-triangle aircraft, bound by the
+// dependent steps of a round (2.9 ms with six launches per round and a host read
+// every four). Loading it and a first look at it take 3.4 ms with the index check
+// on the host beside the build. Data written by other blocks is read past L1. Every wait is bounded: a block that gives up
 // sets bit 8 of the error flag and leaves, and the others' waits end when they
 // see a bit that leaves no tree behind.
 constexpr int kCoopThreads = 512;

@@ -27,12 +27,13 @@
 // What bounds it: the GELU epilogues cost ~36 instructions per output, twice
 // the MMAs' time at K = 512, and one epilogue warp per scheduler left them
 // latency-bound (issue 30 %). Four per scheduler where only BF16 is stored
-// (prediction: issue 72 %, 4 x 65536 x 512 x 512 in 188 us = 730 TFLOP/s, 111 us
-// per member alone before), two where FP32 staging rows take the shared memory.
-// Training's products are bound by their activations: 43 us per layer of 4
-// members x 8192 rows (134 MB moved, 3.1 TB/s) forward and 44 backward, 122 us
-// for all 24 weight gradients (51 GFLOP, 420 TFLOP/s, 2.3 tiles per SM), against
-// 23 us per member and layer and 46 us per weight gradient one by one.
+// (prediction: issue 72 %, 4 x 65536 x 512 x 512 in 188 us = 730 TFLOP/s; a
+// member alone with one epilogue warp per scheduler 111 us), two where FP32
+// staging rows take the shared memory. Training's forward and backward products
+// are bound by their activations: 43 us per layer of 4 members x 8192 rows (134
+// MB moved, 3.1 TB/s) forward and 44 backward. All 24 weight gradients take 122
+// us (94.5 GFLOP, 775 TFLOP/s, 2.3 tiles per SM). One by one: 23 us per member
+// and layer, 46 us per weight gradient.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>

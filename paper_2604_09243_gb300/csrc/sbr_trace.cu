@@ -913,7 +913,8 @@ __device__ __forceinline__ void tile_ij(const AngleDev& A, int p, int& i, int& j
 // ends at the first certain hit (whether one exists depends on no order). Out of
 // line, so that its registers do not burden the bounce kernel, which asks it at
 // one place (33 bistatic aspects of a 250k-triangle aircraft at 3 GHz: with the
-// first hits listed instead of stored, 6.82 -> 6.51 ms per trace and PO sum).
+// first hits listed instead of stored, 6.51 ms per trace and PO sum; 6.82 with a
+// closest-hit query and stored states).
 __device__ __noinline__ bool any_hit(const TraceArgs& a, float3 o, float3 d, int skip, bool& overflow)
 {
     constexpr int kStack = 64;
@@ -2405,9 +2406,13 @@ __global__ void __launch_bounds__(kTraceThreads, 4) k_bounce(const TraceArgs a)
 // queue slot between them; the rays are spread over all warps, so few share one.
 // Up to one ray per resident thread (155,648): with more, the lanes whose rays
 // have ended are worth the compaction between passes. aircraft_deep_cavity
-// (3 GHz, 45 aspects, 100 bounces): 22.5 -> 11.9 ms. Rays still there after
+// (3 GHz, 45 aspects, 100 bounces): 11.9 ms, 22.5 pass by pass. Rays still there after
 // kHandAfter bounces are trapped: where many more may follow (a.hand_count) they
-// go to k_trapped.
+// go to k_trapped. Handed over after 6, 10, 14, 20 bounces: the 983k-triangle
+// aircraft at 3 GHz, 100 bounces 10.4, 10.0, 10.1, 10.2 ms; 250k triangles 6.8,
+// 6.8, 6.9, 7.0; 60k at 6 GHz, 60 bounces 4.37, 4.40, 4.45, 4.50; 983k at 1.5
+// GHz, 40 bounces, no escape rule 5.92, 6.02, 6.08, 6.23 (after 4: 11.7, 8.0,
+// 4.8, 6.0; never: 11.4, 7.8, 4.7, 6.4).
 constexpr int kHandAfter = 10;
 template <bool kCount, int kStack, int kMode, bool kBi>
 __global__ void __launch_bounds__(kTraceThreads, 4) k_tail(const TraceArgs a)
@@ -2457,9 +2462,18 @@ __global__ void __launch_bounds__(kTraceThreads, 4) k_tail(const TraceArgs a)
 // lane each, their loads in flight together: a ray's chain of dependent fetches
 // is as long as the tree is deep instead of one for every node and triangle it
 // meets. Every lane keeps its own candidates and the smallest (t32, original
-// triangle index) is taken at the end, so the hit is that of any other order of
-// visits. A nearly full stack is left to one node at a time; false where the
-// children did not fit all the same (the caller's to trace).
+// triangle index) of the lanes' closest is taken at the end, while a single
+// lane (consider_hit) drops a candidate whose distance interval lies beyond
+// another's and compares stored distances only where the intervals overlap. The
+// two agree where the interval's half-width (at least 28 u |S| / |d.n|, S from
+// vertex 0 to the origin) covers the plane slack u L / |d.n| by which a stored
+// distance may differ: unless the origin is within about L / 28 of vertex 0.
+// There the two candidates would have to lie within that slack of each other,
+// far inside the edge band. A nearly full stack is left to
+// one node at a time; false where the children did not fit all the same (the
+// caller's to trace). That takes more than 21 levels one below the other, each
+// with four children that the ray enters, on top of some 60 boxes that wait: a
+// balanced tree of that depth has 4^21 nodes, and no test reaches it.
 constexpr int kCoopStack = 128, kCoopWide = 40, kCoopTris = 32 + 8 * 4 * 16;
 struct CoopQueue {
     int2 node[kCoopStack];  // node, its near distance
@@ -2569,11 +2583,10 @@ __device__ __forceinline__ bool closest_hit_coop(const TraceArgs& a, CoopQueue& 
 // end by a warp: a bounce takes 18k cycles instead of the 30k of one
 // lane, and no warp has several of them by chance. Its own kernel, since the
 // queues' shared memory is L1 that the other traversals use (inside k_tail:
-// aircraft_1ghz_cut 1.5 % slower). aircraft_deep_cavity 11.8 -> 10.3 ms with 32
-// lanes a ray and rays handed over after 10 bounces (16 lanes 10.4, 8 lanes
-// 10.9; after 6 bounces 10.8, 14 10.5, 20 10.7). With more than two rays per
-// warp the GPU is busy with a lane each: 40,000 rays of a bistatic trace with
-// 67 bounces in 3.5 ms, 8.5 ms by whole warps.
+// aircraft_1ghz_cut 1.5 % slower). aircraft_deep_cavity in 10.3 ms with 32
+// lanes a ray (16 lanes 10.4, 8 lanes 10.9, 11.8 left to k_tail). With more than
+// two rays per warp the GPU is busy with a lane each: 40,000 rays of a bistatic
+// trace with 67 bounces in 3.5 ms, 8.5 ms by whole warps.
 constexpr unsigned kTrappedPerWarp = 2;
 template <bool kBi>
 __global__ void __launch_bounds__(kTraceThreads, 2) k_trapped(const TraceArgs a)
