@@ -509,11 +509,20 @@ cudaError_t launch_gemm_bn(const GemmProblem& P, int sms, int dev, int* err, cud
     // 256 columns (three quarters of the operand reads per output) where half the tiles still make an even last
     // wave and the epilogue stores BF16 only: 300k x 4 members' prediction 6.85 against 8.3 ms with 128 columns. With
     // FP32 pre-activations stored or read the epilogue's memory traffic sets the time and smaller tiles balance
-    // better: 43 against 48 us per forward layer of 4 x 8192 rows. 64 columns where 128 would leave SMs idle.
+    // better: 43 against 48 us per forward layer of 4 x 8192 rows.
     if constexpr (kMode == kEpiGelu)
         if (P.N % 256 == 0 && P.n2 % 256 == 0 && tiles >= 4ll * sms)
             return launch_gemm<256, kMnA, kMnB, kMode>(P, sms, dev, err, st);
-    if (tiles >= sms) return launch_gemm<128, kMnA, kMnB, kMode>(P, sms, dev, err, st);
+    // A wave of tiles of 64, 128 and 256 columns takes times like 344, 408 and 536 (22, 26.6 and 34.6 us at K = 4096),
+    // so what counts is how many waves there are: 64 columns pay where they are one wave (128 x 8192 x 4096: 25 us,
+    // 26.6 with 128), 128 where 64 would be two (512 x 4096 x 4096: 26.6, 43.9 with 64), and for the plain product,
+    // whose epilogue only stores, 256 where that saves more waves than it lengthens (2048 x 1280 x 8192: 59 us, 83
+    // with 128; 4096 x 4096 x 4096: 112, 143; 65536 x 512 x 512: 46, 49.5)
+    auto waves = [&](long long n) { return (n + sms - 1) / sms; };
+    if constexpr (kMode == kEpiF32 && !kMnA && !kMnB)
+        if (P.N % 256 == 0 && !P.n2 && 2 * tiles > sms && 536 * waves((tiles + 1) / 2) < 408 * waves(tiles))
+            return launch_gemm<256, kMnA, kMnB, kMode>(P, sms, dev, err, st);
+    if (2 * tiles > sms) return launch_gemm<128, kMnA, kMnB, kMode>(P, sms, dev, err, st);
     return launch_gemm<64, kMnA, kMnB, kMode>(P, sms, dev, err, st);
 }
 
