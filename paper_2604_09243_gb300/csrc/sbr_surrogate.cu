@@ -394,6 +394,8 @@ __global__ void k_ens_stats(const float* y, int n_members, long long stride, int
 
 inline unsigned blocks(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 
+constexpr size_t kKeepBytes = (size_t)64 << 20;
+
 struct Buf {
     void* p = nullptr;
     size_t cap = 0;
@@ -437,6 +439,10 @@ struct sbr_surrogate {
     // (h_{l+1} at l), z and dz [layer][g][M][width], outputs and targets [g][M][4], gradients [g][n_params]. Kept and
     // grown as needed.
     Buf h0, h, z, dz, y, dy, xb, yb, red, G;
+    // Arrays of a call: inputs as given and encoded, targets, permutations and losses, predictions. Kept up to
+    // kKeepBytes each: taken from the allocator and given back on every call they cost 0.1 to 0.2 ms whenever they
+    // were alone in a mapping of it.
+    Buf raw, x4, y4, perm, eloss, mean, spread;
     Buf loss, gerr;
     float target_scale = 1.f;
     bool trained = false;
@@ -487,18 +493,26 @@ void release_ws(sbr_surrogate* s)
 }
 
 // an array of the call at hand; where the GPU is full the workspace kept from earlier calls makes room
-template <class T>
-cudaError_t call_alloc(sbr_surrogate* s, T** p, size_t count)
+cudaError_t call_alloc(sbr_surrogate* s, Buf& b, size_t bytes)
 {
-    cudaError_t e = cudaMalloc((void**)p, sizeof(T) * count);
+    cudaError_t e = b.ensure(bytes);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
         release_ws(s);
-        e = cudaMalloc((void**)p, sizeof(T) * count);
+        e = b.ensure(bytes);
     }
-    if (e != cudaSuccess) *p = nullptr;
     return e;
 }
+
+// gives back at the end of a call what is too large to keep
+struct CallArrays {
+    sbr_surrogate* s;
+    ~CallArrays()
+    {
+        for (Buf* b : {&s->raw, &s->x4, &s->y4, &s->perm, &s->eloss, &s->mean, &s->spread})
+            if (b->cap > kKeepBytes) b->release();
+    }
+};
 
 // Members worked on at once: all of them while their workspace (200 MB per
 // member at 8192 rows of the default network) stays within kGroupBytes and can
@@ -507,7 +521,7 @@ cudaError_t call_alloc(sbr_surrogate* s, T** p, size_t count)
 // members of 8192 rows takes 0.75 ms of device time together, 3.1 ms one member
 // at a time.
 constexpr size_t kGroupBytes = (size_t)8 << 30, kGroupPerm = (size_t)1 << 30;
-int choose_group(sbr_surrogate* s, int M, long long n, int epochs, int* g_out, int** dperm, double** dloss)
+int choose_group(sbr_surrogate* s, int M, long long n, int epochs, int* g_out)
 {
     const size_t row = (size_t)s->opt.depth * s->opt.width * 8 + (size_t)s->opt.n_fourier * 2 + 128;
     size_t most = std::min<size_t>((size_t)s->opt.n_members, kGroupBytes / (row * (size_t)M));
@@ -515,14 +529,12 @@ int choose_group(sbr_surrogate* s, int M, long long n, int epochs, int* g_out, i
     int g = (int)std::max<size_t>(1, most);
     for (bool last = false;;) {
         cudaError_t e = ensure_ws(s, M, g, true);
-        if (e == cudaSuccess) e = cudaMalloc((void**)dperm, sizeof(int) * (size_t)n * g);
-        if (e == cudaSuccess) e = cudaMalloc((void**)dloss, sizeof(double) * (size_t)epochs * g);
+        if (e == cudaSuccess) e = s->perm.ensure(sizeof(int) * (size_t)n * g);
+        if (e == cudaSuccess) e = s->eloss.ensure(sizeof(double) * (size_t)epochs * g);
         if (e == cudaSuccess) break;
         cudaGetLastError();
-        cudaFree(*dperm);
-        *dperm = nullptr;
-        *dloss = nullptr;
         release_ws(s);
+        for (Buf* b : {&s->perm, &s->eloss, &s->raw, &s->mean, &s->spread}) b->release();
         if (e != cudaErrorMemoryAllocation || last) SCK(e, "alloc training workspace");
         if (g == 1) last = true;  // once more, without what earlier calls had left
         else g = (g + 1) / 2;
@@ -683,22 +695,15 @@ int check_gemm_err(sbr_surrogate* s)
     return SBR_OK;
 }
 
-int upload_inputs(sbr_surrogate* s, const double* x, int64_t n, float** x4)
+// the n inputs at x, encoded into s->x4
+int upload_inputs(sbr_surrogate* s, const double* x, int64_t n)
 {
-    double* raw = nullptr;
-    cudaError_t e = call_alloc(s, x4, kIn * (size_t)n);
-    if (e == cudaSuccess) e = call_alloc(s, &raw, 3 * (size_t)n);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(raw, x, sizeof(double) * 3 * (size_t)n, cudaMemcpyHostToDevice, s->stream);
-    if (e == cudaSuccess) {
-        k_encode<<<blocks(n, 256), 256, 0, s->stream>>>(raw, (int)n, *x4);
-        e = cudaStreamSynchronize(s->stream);
-    }
-    cudaFree(raw);
-    if (e != cudaSuccess) {
-        cudaFree(*x4);
-        *x4 = nullptr;
-    }
-    SCK(e, "encode inputs");
+    SCK(call_alloc(s, s->x4, sizeof(float) * kIn * (size_t)n), "alloc inputs");
+    SCK(call_alloc(s, s->raw, sizeof(double) * 3 * (size_t)n), "alloc inputs");
+    SCK(cudaMemcpyAsync(s->raw.p, x, sizeof(double) * 3 * (size_t)n, cudaMemcpyHostToDevice, s->stream), "copy inputs");
+    k_encode<<<blocks(n, 256), 256, 0, s->stream>>>(s->raw.as<double>(), (int)n, s->x4.as<float>());
+    SCK(cudaStreamSynchronize(s->stream), "encode inputs");
+    if (s->raw.cap > kKeepBytes) s->raw.release();
     return SBR_OK;
 }
 
@@ -862,7 +867,9 @@ void sbr_surrogate_destroy(sbr_surrogate* s)
     cudaSetDevice(s->device);
     cudaStreamSynchronize(s->stream);
     release_ws(s);
-    for (Buf* b : {&s->P, &s->Pm, &s->Pv, &s->Bf, &s->Wbf, &s->loss, &s->gerr}) b->release();
+    for (Buf* b : {&s->P, &s->Pm, &s->Pv, &s->Bf, &s->Wbf, &s->loss, &s->gerr, &s->raw, &s->x4, &s->y4, &s->perm, &s->eloss,
+                   &s->mean, &s->spread})
+        b->release();
     if (s->own_stream) cudaStreamDestroy(s->stream);
     delete s;
 }
@@ -898,28 +905,25 @@ int sbr_surrogate_grads(sbr_surrogate* s, int member, const double* x, const dou
 {
     if (!s || !x || !y || n < 128 || n % 128 || member < 0 || member >= s->opt.n_members) return SBR_ERR_ARG;
     SCK(cudaSetDevice(s->device), "cudaSetDevice");
-    float* x4 = nullptr;
-    int rc = upload_inputs(s, x, n, &x4);
+    CallArrays arrays{s};
+    int rc = upload_inputs(s, x, n);
     if (rc != SBR_OK) return rc;
     cudaError_t ce = ensure_ws(s, (int)n, 1, true);
     if (ce == cudaErrorMemoryAllocation) {  // once more, without what earlier calls had left
         cudaGetLastError();
         release_ws(s);
+        for (Buf* b : {&s->raw, &s->y4, &s->perm, &s->eloss, &s->mean, &s->spread}) b->release();
         ce = ensure_ws(s, (int)n, 1, true);
     }
-    if (ce != cudaSuccess) {
-        cudaFree(x4);
-        SCK(ce, "alloc training workspace");
-    }
+    SCK(ce, "alloc training workspace");
     std::vector<float> yt((size_t)n * kOut);
     for (size_t i = 0; i < yt.size(); ++i) yt[i] = (float)(y[i] / s->target_scale);
     cudaMemcpyAsync(s->yb.p, yt.data(), sizeof(float) * yt.size(), cudaMemcpyHostToDevice, s->stream);
     cudaMemsetAsync(s->gerr.p, 0, sizeof(int), s->stream);
     cudaMemsetAsync(s->loss.p, 0, sizeof(double), s->stream);
-    rc = forward(s, member, 1, (int)n, x4, 0, s->y.as<float>(), true);
+    rc = forward(s, member, 1, (int)n, s->x4.as<float>(), 0, s->y.as<float>(), true);
     if (rc == SBR_OK) rc = backward(s, member, 1, (int)n, s->loss.as<double>(), 0);
     if (rc == SBR_OK) rc = check_gemm_err(s);
-    cudaFree(x4);
     if (rc != SBR_OK) return rc;
     double hl = 0.0;
     SCK(cudaMemcpy(&hl, s->loss.p, sizeof(double), cudaMemcpyDeviceToHost), "copy loss");
@@ -937,37 +941,23 @@ int sbr_surrogate_train(sbr_surrogate* s, const double* x, const double* y, int6
     const int M = (int)std::min<long long>(batch, (n / 128) * 128);
     // the call's own arrays first, then the workspace of as many members at once as fit beside them: inputs, targets,
     // and per member of the group one permutation per epoch and the per-epoch squared-error sums
-    float *x4 = nullptr, *y4 = nullptr;
-    int* dperm = nullptr;
-    double* dloss = nullptr;
     int group = 1;
-    int rc = upload_inputs(s, x, n, &x4);
+    CallArrays arrays{s};
+    int rc = upload_inputs(s, x, n);
     if (rc != SBR_OK) return rc;
-    cudaError_t ce = call_alloc(s, &y4, (size_t)n * kOut);
-    if (ce != cudaSuccess) {
-        cudaFree(x4);
-        SCK(ce, "alloc targets");
-    }
-    rc = choose_group(s, M, n, epochs, &group, &dperm, &dloss);
-    if (rc != SBR_OK) {
-        cudaFree(x4);
-        cudaFree(y4);
-        return rc;
-    }
+    SCK(call_alloc(s, s->y4, sizeof(float) * kOut * (size_t)n), "alloc targets");
+    rc = choose_group(s, M, n, epochs, &group);
+    if (rc != SBR_OK) return rc;
+    float *x4 = s->x4.as<float>(), *y4 = s->y4.as<float>();
+    int* dperm = s->perm.as<int>();
+    double* dloss = s->eloss.as<double>();
     // target scale: RMS of the targets
     double ss = 0.0;
     for (int64_t i = 0; i < n * kOut; ++i) ss += y[i] * y[i];
     s->target_scale = (float)std::max(sqrt(ss / (double)(n * kOut)), 1e-30);
     std::vector<float> yt((size_t)n * kOut);
     for (size_t i = 0; i < yt.size(); ++i) yt[i] = (float)(y[i] / s->target_scale);
-    ce = cudaMemcpyAsync(y4, yt.data(), sizeof(float) * yt.size(), cudaMemcpyHostToDevice, s->stream);
-    if (ce != cudaSuccess) {
-        cudaFree(x4);
-        cudaFree(y4);
-        cudaFree(dperm);
-        cudaFree(dloss);
-        SCK(ce, "upload targets");
-    }
+    SCK(cudaMemcpyAsync(y4, yt.data(), sizeof(float) * yt.size(), cudaMemcpyHostToDevice, s->stream), "upload targets");
     const long long steps_per_epoch = n / M;
     std::vector<int> perm((size_t)n * group);
     std::vector<double> hloss((size_t)epochs * group);
@@ -1037,11 +1027,7 @@ int sbr_surrogate_train(sbr_surrogate* s, const double* x, const double* y, int6
                     loss_per_epoch[(size_t)(e0 + e) * epochs + ep] =
                         (float)(hloss[(size_t)e * epochs + ep] / ((double)M * kOut * (double)steps_per_epoch));
     }
-    cudaFree(dperm);
-    cudaFree(dloss);
     if (rc == SBR_OK) rc = check_gemm_err(s);
-    cudaFree(x4);
-    cudaFree(y4);
     if (rc == SBR_OK) s->trained = true;
     return rc;
 }
@@ -1060,29 +1046,24 @@ int sbr_surrogate_predict(sbr_surrogate* s, const double* x, int64_t n, double* 
     const long long wide = std::max(4ll * s->opt.width, 2ll * s->opt.n_fourier) * g;
     const long long fit = (512ll << 20) / wide / 128 * 128;
     int M = (int)std::min<int64_t>(std::max<long long>(1024, fit), ((n + 127) / 128) * 128);
-    int rc = SBR_OK;
-    float* x4 = nullptr;
-    rc = upload_inputs(s, x, n, &x4);
+    CallArrays arrays{s};
+    int rc = upload_inputs(s, x, n);
     if (rc != SBR_OK) return rc;
-    double* dmean = nullptr;
-    float* dspread = nullptr;
-    cudaError_t ce = call_alloc(s, &dmean, kOut * (size_t)n);
-    if (ce == cudaSuccess) ce = call_alloc(s, &dspread, (size_t)n);
-    for (bool last = false; ce == cudaSuccess;) {
-        ce = ensure_ws(s, M, g, false);
-        if (ce != cudaErrorMemoryAllocation || last) break;
+    SCK(call_alloc(s, s->mean, sizeof(double) * kOut * (size_t)n), "alloc outputs");
+    SCK(call_alloc(s, s->spread, sizeof(float) * (size_t)n), "alloc outputs");
+    for (bool last = false;;) {
+        const cudaError_t e = ensure_ws(s, M, g, false);
+        if (e == cudaSuccess) break;
         cudaGetLastError();
         release_ws(s);
+        for (Buf* b : {&s->raw, &s->y4, &s->perm, &s->eloss}) b->release();
+        if (e != cudaErrorMemoryAllocation || last) SCK(e, "alloc prediction workspace");
         if (M == 128) last = true;  // once more, without what earlier calls had left
         else M = std::max(128, M / 2 / 128 * 128);
-        ce = cudaSuccess;
     }
-    if (ce != cudaSuccess) {
-        cudaFree(x4);
-        cudaFree(dmean);
-        cudaFree(dspread);
-        SCK(ce, "alloc outputs and workspace");
-    }
+    const float* x4 = s->x4.as<float>();
+    double* dmean = s->mean.as<double>();
+    float* dspread = s->spread.as<float>();
     cudaMemsetAsync(s->gerr.p, 0, sizeof(int), s->stream);
     for (int64_t b0 = 0; b0 < n && rc == SBR_OK; b0 += M) {
         const int cnt = (int)std::min<int64_t>(M, n - b0);
@@ -1107,9 +1088,6 @@ int sbr_surrogate_predict(sbr_surrogate* s, const double* x, int64_t n, double* 
         rc = cudaMemcpy(spread_db, dspread, sizeof(float) * (size_t)n, cudaMemcpyDeviceToHost) == cudaSuccess
                  ? SBR_OK
                  : SBR_ERR_CUDA;
-    cudaFree(x4);
-    cudaFree(dmean);
-    cudaFree(dspread);
     return rc;
 }
 

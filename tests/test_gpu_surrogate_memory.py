@@ -97,3 +97,30 @@ def test_prediction_fits_where_its_usual_batches_do_not(G, net, n, leave):
         torch.cuda.empty_cache()
     assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
     s.close()
+
+
+def test_arrays_kept_between_calls_hold_nothing_over(G):
+    """Calls of every kind and of falling and rising sizes on one object, some of them with arrays of more than the 64 MB
+    that are kept, give the bits of the same training on an object that makes no other calls."""
+    net = dict(n_members=2, width=128, depth=1, n_fourier=128, fourier_sigma=2.0, seed=11)
+    x, y = _samples(40_000, 4)
+    big = np.tile(x, (75, 1))  # 3,000,000 points: 72 MB of inputs, 96 MB of predictions
+    a, b = G.Surrogate(0, **net), G.Surrogate(0, **net)
+    a.train(x, y, epochs=1, batch=1024)
+    all_big = a.predict(big)
+    a.grads(x[:256], y[:256])
+    a.train(x[:5000], y[:5000], epochs=3, batch=512)
+    small = a.predict(x[:700])
+    a.train(x, y, epochs=2, batch=2048)
+    b.train(x, y, epochs=1, batch=1024)
+    one = b.predict(x)
+    b.train(x[:5000], y[:5000], epochs=3, batch=512)
+    two = b.predict(x[:700])
+    b.train(x, y, epochs=2, batch=2048)
+    for k in range(2):
+        assert np.array_equal(all_big[k], np.concatenate([one[k]] * 75))
+        assert np.array_equal(small[k], two[k])
+    for e in range(2):
+        assert np.array_equal(a.params(e), b.params(e))
+    a.close()
+    b.close()
