@@ -27,19 +27,20 @@ namespace {
 constexpr int kPoThreads = 256;
 constexpr int kWarps = kPoThreads / 32;
 
-// kComp: the compensated phase alone (the default), without the other modes' branches and slow paths
-template <bool kComp>
-__device__ __forceinline__ void phase_cs(const PoArgs& a, float4 fq, double kd, float lh, float ll, float& c,
-                                         float& s)
+// kPhase: PoArgs::phase_mode, a kernel each: in one kernel the modes pay for each other's registers and slow paths (500
+// frequencies of 12 aircraft aspects, VV, FP32 phase: 0.83 ms, 1.41 where the FP64 phase shares the kernel; four
+// polarisations at 64 frequencies, FP64 phase: 3.8 and 4.1 ms)
+template <int kPhase>
+__device__ __forceinline__ void phase_cs(float4 fq, double kd, float lh, float ll, float& c, float& s)
 {
-    if (kComp || a.phase_mode == 0) {
+    if (kPhase == 0) {
         const float p = __fmul_rn(fq.x, lh);
         float e = __fmaf_rn(fq.x, lh, -p);
         e = __fadd_rn(e, __fadd_rn(__fmul_rn(fq.x, ll), __fmul_rn(fq.y, lh)));
         const float n = rintf(p);
         const float r = __fadd_rn(__fsub_rn(p, n), e);
         sincospif(2.f * r, &s, &c);
-    } else if (a.phase_mode == 1) {
+    } else if (kPhase == 1) {
         sincosf(fq.z * lh, &s, &c);
     } else {
         double sd, cd;
@@ -109,7 +110,7 @@ __device__ __forceinline__ int warp_sum_index(int lane)
 // their products), 635 us with every sum exchanged at every step of the
 // butterfly and the other phase modes' code in the loop.
 constexpr int kSums = 16;
-template <int kPoPer, int kPol, bool kComp>
+template <int kPoPer, int kPol, int kPhase>
 __global__ void __launch_bounds__(kPoThreads) k_po(const PoArgs a)
 {
     constexpr int kF = kSums / (2 * kPol);  // frequencies per block reduction
@@ -159,20 +160,20 @@ __global__ void __launch_bounds__(kPoThreads) k_po(const PoArgs a)
             for (int fj = 0; fj < kF; ++fj) {
                 if (f0 + fj >= I.nf) break;
                 const float4 fq = a.freq[I.f0 + f0 + fj];
-                const double kd = kComp ? 0.0 : a.kfreq[I.f0 + f0 + fj];
+                const double kd = kPhase != 2 ? 0.0 : a.kfreq[I.f0 + f0 + fj];
                 const float2 fx = make_float2(fq.x, fq.x), nx = make_float2(-fq.x, -fq.x), fy = make_float2(fq.y, fq.y);
 #pragma unroll
                 for (int k = 0; k < kPoPer; k += 2) {
                     // (a tube past the item's end adds zeros)
                     if (k * kPoThreads + tid >= I.count) break;
                     float2 e0, e1;  // (cos, sin)
-                    if (kComp) {
+                    if constexpr (kPhase == 0) {
                         const float2 t = phase_arg2(fx, nx, fy, lh[k / 2], ll[k / 2]);
                         sincospif(t.x, &e0.y, &e0.x);
                         sincospif(t.y, &e1.y, &e1.x);
                     } else {
-                        phase_cs<kComp>(a, fq, kd, lh[k / 2].x, ll[k / 2].x, e0.x, e0.y);
-                        phase_cs<kComp>(a, fq, kd, lh[k / 2].y, ll[k / 2].y, e1.x, e1.y);
+                        phase_cs<kPhase>(fq, kd, lh[k / 2].x, ll[k / 2].x, e0.x, e0.y);
+                        phase_cs<kPhase>(fq, kd, lh[k / 2].y, ll[k / 2].y, e1.x, e1.y);
                     }
 #pragma unroll
                     for (int q = 0; q < kPol; ++q) {
@@ -236,7 +237,7 @@ __device__ __forceinline__ bool po_wait(uint64_t* bar, unsigned parity)
     return false;
 }
 
-template <int kPol, bool kComp>
+template <int kPol, int kPhase>
 __global__ void __launch_bounds__(kPoThreads) k_po_bulk(const PoArgs a)
 {
     constexpr int kF = 4 / kPol;
@@ -321,9 +322,9 @@ __global__ void __launch_bounds__(kPoThreads) k_po_bulk(const PoArgs a)
             for (int fj = 0; fj < kF; ++fj) {
                 if (fj >= I.nf) break;
                 const float4 fq = a.freq[I.f0 + fj];
-                const double kd = kComp ? 0.0 : a.kfreq[I.f0 + fj];
+                const double kd = kPhase != 2 ? 0.0 : a.kfreq[I.f0 + fj];
                 float c, sn;
-                phase_cs<kComp>(a, fq, kd, y.y, y.z, c, sn);
+                phase_cs<kPhase>(fq, kd, y.y, y.z, c, sn);
 #pragma unroll
                 for (int q = 0; q < kPol; ++q) {
                     acc[(fj * kPol + q) * 2] = fmaf(cf[q], c, acc[(fj * kPol + q) * 2]);
@@ -491,7 +492,7 @@ __global__ void __launch_bounds__(kSlices* kOutB) k_po_final(const double* parti
 
 namespace {
 
-template <bool kComp>
+template <int kPhase>
 cudaError_t launch_po_mode(const PoArgs& a, cudaStream_t st, int n_blocks)
 {
     const int grid = n_blocks > 0 ? n_blocks : a.n_items;
@@ -504,23 +505,23 @@ cudaError_t launch_po_mode(const PoArgs& a, cudaStream_t st, int n_blocks)
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e == cudaSuccess)
-            e = two ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_po_bulk<2, kComp>, kPoThreads, 0)
-                    : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_po_bulk<4, kComp>, kPoThreads, 0);
+            e = two ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_po_bulk<2, kPhase>, kPoThreads, 0)
+                    : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_po_bulk<4, kPhase>, kPoThreads, 0);
         if (e != cudaSuccess) return e;
         const int g = (int)std::min<long long>(a.n_items, (long long)sms * std::max(occ, 1));
-        if (two) k_po_bulk<2, kComp><<<g, kPoThreads, 0, st>>>(a);
-        else k_po_bulk<4, kComp><<<g, kPoThreads, 0, st>>>(a);
+        if (two) k_po_bulk<2, kPhase><<<g, kPoThreads, 0, st>>>(a);
+        else k_po_bulk<4, kPhase><<<g, kPoThreads, 0, st>>>(a);
         return cudaGetLastError();
     }
     if (per == 2) {
-        if (two) k_po<2, 2, kComp><<<grid, kPoThreads, 0, st>>>(a);
-        else k_po<2, 4, kComp><<<grid, kPoThreads, 0, st>>>(a);
+        if (two) k_po<2, 2, kPhase><<<grid, kPoThreads, 0, st>>>(a);
+        else k_po<2, 4, kPhase><<<grid, kPoThreads, 0, st>>>(a);
     } else if (per == 8) {
-        if (two) k_po<8, 2, kComp><<<grid, kPoThreads, 0, st>>>(a);
-        else k_po<8, 4, kComp><<<grid, kPoThreads, 0, st>>>(a);
+        if (two) k_po<8, 2, kPhase><<<grid, kPoThreads, 0, st>>>(a);
+        else k_po<8, 4, kPhase><<<grid, kPoThreads, 0, st>>>(a);
     } else if (per == 4) {
-        if (two) k_po<4, 2, kComp><<<grid, kPoThreads, 0, st>>>(a);
-        else k_po<4, 4, kComp><<<grid, kPoThreads, 0, st>>>(a);
+        if (two) k_po<4, 2, kPhase><<<grid, kPoThreads, 0, st>>>(a);
+        else k_po<4, 4, kPhase><<<grid, kPoThreads, 0, st>>>(a);
     } else {
         return cudaErrorInvalidValue;
     }
@@ -531,7 +532,8 @@ cudaError_t launch_po_mode(const PoArgs& a, cudaStream_t st, int n_blocks)
 
 cudaError_t launch_po(const PoArgs& a, cudaStream_t st, int n_blocks)
 {
-    return a.phase_mode == 0 ? launch_po_mode<true>(a, st, n_blocks) : launch_po_mode<false>(a, st, n_blocks);
+    if (a.phase_mode == 0) return launch_po_mode<0>(a, st, n_blocks);
+    return a.phase_mode == 1 ? launch_po_mode<1>(a, st, n_blocks) : launch_po_mode<2>(a, st, n_blocks);
 }
 
 namespace {
