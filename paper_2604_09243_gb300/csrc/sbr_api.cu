@@ -298,6 +298,7 @@ AngleDev to_dev(const sbr_ray_grid& g, long long ray_off, int tw, const double* 
     d.r_nu = d.nu;
     d.r_nv = d.nv;
     d.r_ids = d.ids;
+    d.r_m0 = 0.01f + (fabsf(d.p0[0]) + fabsf(d.p0[1]) + fabsf(d.p0[2])) * d.ids * 0x1p-22f;
     return d;
 }
 

@@ -54,14 +54,15 @@ struct __align__(16) AngleDev {  // 256 bytes
     float rxdir[3];                     // -rxr in FP32 (= dir monostatic): the path term of the receiver
     float ids;                          // 1 / sqrt(dA) in FP32: grid cells per metre (rasterisation)
     float pad2[3];
-    // what the projection of a triangle onto a sparse grid reads, in three 16-byte words
+    // what the projection of a triangle onto a sparse grid reads, in three 16-byte words, and the margin
     float r_p0[3];
     int r_nu;
     float r_hs[3];                      // hhat ids
     int r_nv;
     float r_vs[3];                      // vhat ids
     float r_ids;
-    float pad3[4];
+    float r_m0;                         // margin of a projected range in cells: 0.01 + 2^-22 |p0|_1 / spacing
+    float pad3[3];
 };
 static_assert(sizeof(AngleDev) == 256, "AngleDev layout");
 

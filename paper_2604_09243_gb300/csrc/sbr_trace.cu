@@ -1127,7 +1127,11 @@ __device__ __forceinline__ void query(const TraceArgs& a, bool active, float3 o,
 // only hit a triangle whose projection contains (u, v); the FP32 ray origin,
 // the intersection slack (2^-12 of the determinant) and the FP32 projection
 // below all stay within the margin of 0.01 cell + 2^-10 of the triangle's
-// projected extent + 2^-18 of its distance from P0 (in cells). One thread
+// projected extent + 2^-18 of its distance from P0 + 2^-22 of |P0|_1 (in cells).
+// The last covers the roundings that grow with the coordinates, not with the
+// target: u |v_k| of a vertex v0 + e and 2 u |o_k| of a ray origin per component,
+// 3 u |P0|_1 along an axis beyond what the distance covers (a target of 10 m at
+// 10 km from the origin on an 8 mm grid: 0.4 cells). One thread
 // projects one triangle for one aspect and ORs its cells into the tile words.
 // A triangle whose widened box spans more than 2^16 cells sets the aspect's
 // "all rays" flag (word total_tiles + aspect) instead.
@@ -1139,7 +1143,7 @@ __device__ __forceinline__ float cell_scale(const AngleDev& A) { return A.ids; }
 // The triangle's vertices projected onto the aspect's grid (in cells from P0),
 // their ranges and their largest distance from P0 (in cells)
 struct TriProj {
-    float u[3], v[3], umin, umax, vmin, vmax, mag;
+    float u[3], v[3], umin, umax, vmin, vmax, mag, m0;  // m0: AngleDev::r_m0
 };
 
 __device__ __forceinline__ void tri_project(const AngleDev& A, float ids, float4 a, float4 b, float4 c, TriProj& pr)
@@ -1151,6 +1155,7 @@ __device__ __forceinline__ void tri_project(const AngleDev& A, float ids, float4
     pr.vmin = FLT_MAX;
     pr.vmax = -FLT_MAX;
     pr.mag = 0.f;
+    pr.m0 = A.r_m0;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         const float dx = px[k] - A.p0[0], dy = py[k] - A.p0[1], dz = pz[k] - A.p0[2];
@@ -1170,7 +1175,7 @@ __device__ __forceinline__ bool tri_cells_p(const AngleDev& A, const TriProj& pr
 {
     const float umin = pr.umin, umax = pr.umax, vmin = pr.vmin, vmax = pr.vmax;
     if (!(umin <= umax) || !(vmin <= vmax)) return false;  // NaN vertices: no ray can hit it
-    const float m = 0.01f + (umax - umin + vmax - vmin) * (1.f / 1024.f) + pr.mag * (1.f / 262144.f);
+    const float m = pr.m0 + (umax - umin + vmax - vmin) * (1.f / 1024.f) + pr.mag * (1.f / 262144.f);
     const float fi0 = ceilf(umin - m), fi1 = floorf(umax + m), fj0 = ceilf(vmin - m), fj1 = floorf(vmax + m);
     if (fi1 < 0.f || fj1 < 0.f || fi0 > (float)(A.nu - 1) || fj0 > (float)(A.nv - 1)) return false;
     i0 = max(0, (int)fi0);
@@ -1210,7 +1215,7 @@ __device__ __forceinline__ void tri_cell_edges_p(const TriProj& pr, int i0, int 
         v[k] = pr.v[k] - (float)j0;
     }
     const float m =
-        0.01f + (pr.umax - pr.umin + pr.vmax - pr.vmin) * (1.f / 1024.f) + pr.mag * (1.f / 262144.f) + 0.002f;
+        pr.m0 + (pr.umax - pr.umin + pr.vmax - pr.vmin) * (1.f / 1024.f) + pr.mag * (1.f / 262144.f) + 0.002f;
     const float a2 = (u[1] - u[0]) * (v[2] - v[0]) - (v[1] - v[0]) * (u[2] - u[0]);
     const float sg = a2 > 0.f ? 1.f : -1.f;
     const bool flat = !(fabsf(a2) > 1e-2f);
@@ -1389,7 +1394,8 @@ __device__ __forceinline__ void raster_cell(const RasterGrid& G, const TraceArgs
 
 // Below the smallest stored distance that a ray of the grid (origin p0,
 // direction d) can have on a triangle: the distances along d of the vertices
-// from the grid plane (the ray origins lie in it to within micrometres); the
+// from the grid plane (the ray origins lie in it to within micrometres and a few
+// roundings of the coordinates, 2^-21 |p0|_1 with those of the vertices); the
 // stored distance of any hit is at least their minimum less the key's plane
 // slack (0.08 bUV / |d.n|, as in key_of), 1e-4 of it and 1 mm.
 __device__ __forceinline__ float raster_tnear(float4 P, float4 B, float4 C, float3 p0, float3 d, const PlaneKey& K)
@@ -1399,7 +1405,8 @@ __device__ __forceinline__ float raster_tnear(float4 P, float4 B, float4 C, floa
                 z2 = z0 + dot_s(make_float3(C.x, C.y, C.z), d);
     const float zm = fminf(z0, fminf(z1, z2));
     const float slack = K.dh != 0.f ? 0.32f * B.w / fabsf(K.dh) : FLT_MAX;
-    const float tnear = zm - (1e-4f * fabsf(zm) + 1e-3f + slack);
+    const float at = (fabsf(p0.x) + fabsf(p0.y) + fabsf(p0.z)) * 0x1p-21f;
+    const float tnear = zm - (1e-4f * fabsf(zm) + 1e-3f + at + slack);
     return isfinite(tnear) ? tnear : -FLT_MAX;
 }
 
@@ -1902,13 +1909,14 @@ constexpr int kSparseCells = 16, kSparseFlat = 256, kSparseAspects = 16;
 // The aspect's fields that the projection reads
 struct AspectView {
     float4 a, b, c;  // (p0, nu), (hs, nv), (vs, ids)
+    float m0;
 };
 __device__ __forceinline__ AspectView aspect_view(const AngleDev* p)
 {
     static_assert(offsetof(AngleDev, r_p0) % 16 == 0 && offsetof(AngleDev, r_ids) == offsetof(AngleDev, r_p0) + 44,
                   "AspectView reads three 16-byte words");
     const float4* w = reinterpret_cast<const float4*>(p->r_p0);
-    return AspectView{__ldg(w), __ldg(w + 1), __ldg(w + 2)};
+    return AspectView{__ldg(w), __ldg(w + 1), __ldg(w + 2), __ldg(&p->r_m0)};
 }
 
 // The cell range of a triangle (vertices x, y, z; size L = max(|e1|_1, |e2|_1)):
@@ -1931,7 +1939,7 @@ __device__ __forceinline__ bool sparse_cells(const AspectView& A, const float* x
     }
     const float umin = fminf(fminf(uv[0].x, uv[1].x), uv[2].x), umax = fmaxf(fmaxf(uv[0].x, uv[1].x), uv[2].x);
     const float vmin = fminf(fminf(uv[0].y, uv[1].y), uv[2].y), vmax = fmaxf(fmaxf(uv[0].y, uv[1].y), uv[2].y);
-    const float m = 0.01f + (umax - umin + vmax - vmin) * (1.f / 1024.f) + mag * (1.f / 262144.f);
+    const float m = A.m0 + (umax - umin + vmax - vmin) * (1.f / 1024.f) + mag * (1.f / 262144.f);
     i0 = max(0, __float2int_ru(umin - m));
     i1 = min(__float_as_int(A.a.w) - 1, __float2int_rd(umax + m));
     j0 = max(0, __float2int_ru(vmin - m));
