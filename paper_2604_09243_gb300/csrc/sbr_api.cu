@@ -96,7 +96,7 @@ struct sbr_ctx {
     DevBuf angles, rayoff, mask, tilebase, scan_scr, recoff, q0, q1, ctr64, ctr32, stats, rec, cover;
     DevBuf hit_tri, hit_t, hit_nb;
     DevBuf tripos, vis, visfull;  // position of each original triangle; raster keys and per-aspect flags
-    DevBuf rbig, rbigctr;         // large triangles of a rasterised chunk and their two counters
+    DevBuf rbig, rbigctr;         // large triangles of a rasterised chunk and its counters
     DevBuf slotscr;               // scratch of the primary pass's masks and slots
     unsigned long long* stats_host = nullptr;  // pinned copy of stats
     long long rbig_cap = 0;
@@ -659,7 +659,7 @@ int plan_chunks(sbr_ctx* c, TraceRun& R, std::vector<int64_t>& cut, long long* t
         CK(c->hitlist.ensure(sizeof(uint2) * (size_t)max_chunk), "alloc raster hit list");
         c->rbig_cap = raster_big_cap(max_chunk);
         CK(c->rbig.ensure(sizeof(int4) * (size_t)c->rbig_cap), "alloc raster triangle list");
-        CK(c->rbigctr.ensure(sizeof(unsigned) * 2), "alloc raster triangle counters");
+        CK(c->rbigctr.ensure(sizeof(unsigned) * 4), "alloc raster triangle counters");
         CK(c->slotscr.ensure(sizeof(unsigned) * kSlotWords), "alloc slot scratch");
     }
     CK(c->tilebase.ensure(sizeof(unsigned) * (size_t)all_tiles), "alloc tile base");
@@ -769,7 +769,7 @@ TraceInit trace_init(unsigned long long* stats, const DevBuf& ctr64, const DevBu
     if (stats) zero(stats, sizeof(unsigned long long) * kStatCount);
     if (raster) {
         zero(visfull.p, sizeof(unsigned) * vis_full_words(na));
-        zero(rbigctr.p, sizeof(unsigned) * 2);
+        zero(rbigctr.p, sizeof(unsigned) * 4);
         b.vis16 = vis.as<uint4>();
         b.n_vis16 = rays / 2;
     }
@@ -1374,7 +1374,7 @@ int build_plan(sbr_ctx* c, BatchPlan& P)
         CK(P.hitlist.ensure(sizeof(uint2) * (size_t)max_rays), "alloc raster hit list");
         P.big_cap = (unsigned)raster_big_cap(max_rays);
         CK(P.rbig.ensure(sizeof(int4) * (size_t)P.big_cap), "alloc raster triangle list");
-        CK(P.rbigctr.ensure(sizeof(unsigned) * 2), "alloc raster triangle counters");
+        CK(P.rbigctr.ensure(sizeof(unsigned) * 4), "alloc raster triangle counters");
         CK(P.slotscr.ensure(sizeof(unsigned) * kSlotWords), "alloc slot scratch");
     }
     CK(P.tilebase.ensure(sizeof(unsigned) * (size_t)max_tiles), "alloc tile base");

@@ -201,8 +201,8 @@ struct TraceArgs {
     const int* tri_pos;           // with vis: [n_tri] position in tris of each original triangle index
     int4* big;                    // with vis: triangles of more than 512 (sparse grids: 256) cells, (triangle, aspect, i0 | j0 << 16,
                                   // (i1 - i0) | (j1 - j0) << 16), tested by warps after the per-thread pass
-    unsigned* big_ctr;            // with vis: [2] entries appended to big, and to the list of middling triangles of a
-                                  // sparse grid, (triangle, aspect) at q_out, which holds no rays yet
+    unsigned* big_ctr;            // with vis: [4] entries appended to big, and to the list of middling triangles of a
+                                  // sparse grid, (triangle, aspect) at q_out, which holds no rays yet; work taken (sparse)
     unsigned big_cap;             // with vis: capacity of big (an aspect whose entry does not fit traverses)
     uint2* hit_list;              // optional (with vis, a bounce pass follows): the primary pass lists
                                   // (ray, aspect) of each hit here instead of storing its state, and

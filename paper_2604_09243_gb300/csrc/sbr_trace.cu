@@ -1442,9 +1442,10 @@ constexpr size_t kRasterSmem = sizeof(RasterItem) * 32 * kRasterWarps;
 // plates of two triangles, B = 2, banded against traversed: 1 plate 1.5 / 4.1 ms,
 // 10: 4.0 / 4.4, 30: 9.0 / 4.7, 300: 73 / 8.2). Every lane of the warp calls it.
 constexpr int kRasterBand = 4096, kRasterBanded = 1 << 14;
-__device__ __noinline__ void append_some(const TraceArgs& a, unsigned* full, bool want, int t, int ang, int i0, int i1,
-                                         int j0, int j1)
+__device__ __forceinline__ void append_big(const TraceArgs& a, unsigned* full, bool want, int t, int ang, int i0, int i1,
+                                           int j0, int j1)
 {
+    if (!__any_sync(kFull, want)) return;
     if (want) {
         const unsigned cells = (unsigned)((i1 - i0 + 1) * (j1 - j0 + 1));
         if (cells > kRasterBanded) {
@@ -1489,11 +1490,12 @@ __device__ __noinline__ void append_some(const TraceArgs& a, unsigned* full, boo
     }
 }
 
-// (the warps with any, out of line)
-__device__ __forceinline__ void append_big(const TraceArgs& a, unsigned* full, bool want, int t, int ang, int i0, int i1,
-                                           int j0, int j1)
+// the same out of line, for warps with any (k_raster_sparse, whose projection it would burden; inline a band takes 37 ns
+// of a lane, out of line 91)
+__device__ __noinline__ void append_some(const TraceArgs& a, unsigned* full, bool want, int t, int ang, int i0, int i1,
+                                         int j0, int j1)
 {
-    if (__any_sync(kFull, want)) append_some(a, full, want, t, ang, i0, i1, j0, j1);
+    append_big(a, full, want, t, ang, i0, i1, j0, j1);
 }
 
 // The cells of row y inside an item's moved edges: columns [lo, lo + cnt) of
@@ -1765,11 +1767,11 @@ struct __align__(16) SparseItem {
     int w, ij, t, ang;
     int pad[2];
 };
-__device__ __forceinline__ unsigned sparse_walk(const TraceArgs& a, unsigned long long* vis, int t, int ang, int count)
+__device__ __forceinline__ unsigned sparse_walk(const TraceArgs& a, unsigned long long* vis, int t, int ang, uint2* spans,
+                                                int count)
 {
     __shared__ SparseItem s_items[kRasterWarps][32];
     __shared__ int s_off[kRasterWarps][33];
-    __shared__ uint2 s_span[kRasterWarps][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     SparseItem* my = s_items[warp];
     int* off = s_off[warp];
@@ -1820,7 +1822,7 @@ __device__ __forceinline__ unsigned sparse_walk(const TraceArgs& a, unsigned lon
             row = rb + lane - off[k];
             row_span(nx, ny, c, (float)row, it.w, lo, cnt);
         }
-        each_cell(s_span[warp], k, row, lo, cnt, [&](int tri, int dj, int di) {
+        each_cell(spans, k, row, lo, cnt, [&](int tri, int dj, int di) {
             const SparseItem& it = my[tri];
             n += sparse_pair<true>(a, vis, it.t, it.ang, it.ij + (di | (dj << 16)), count, it.tnear);
         });
@@ -1829,53 +1831,73 @@ __device__ __forceinline__ unsigned sparse_walk(const TraceArgs& a, unsigned lon
     return n;
 }
 
+// One entry of the list of large triangles by a warp: the cells of its rows'
+// spans 32 at a time, their tests added to the lane's ntri.
+__device__ __forceinline__ void raster_entry(const TraceArgs& a, unsigned long long* vis, int lane, unsigned it,
+                                             uint2* spans, int count, unsigned long long& ntri)
+{
+    const int4 b = a.big[it];
+    const int td = b.x, ad = b.y;
+    if (a.vis_full[ad]) return;  // traverses
+    const int i0 = b.z & 0xFFFF, j0 = (unsigned)b.z >> 16, w = (b.w & 0xFFFF) + 1, h = ((unsigned)b.w >> 16) + 1;
+    const int i1 = i0 + w - 1, j1 = j0 + h - 1;
+    const AngleDev& A = a.angles[ad];
+    const RasterGrid G = raster_grid(A);
+    const float4* tp = a.tris + 3 * (size_t)td;
+    const float4 P = __ldg(tp), B = __ldg(tp + 1), C = __ldg(tp + 2);
+    const RasterTri R = raster_tri(G, P, B, C, i0, i1, j0, j1);
+    if (!(R.bd >= 0.f)) return;  // warp-uniform
+    const unsigned orig = (unsigned)__float_as_int(P.w);
+    unsigned long long* vrow = vis + a.ray_off[ad];
+    const PlaneKey K = plane_key(a.tri_nrm, td, G.d);
+    CellEdges E;
+    tri_cell_edges(A, cell_scale(A), P, B, C, i0, i1, j0, j1, E);
+    for (int rb = 0; rb < h; rb += 32) {
+        int lo = 0, cnt = 0;
+        if (rb + lane < h) row_span(E.nx, E.ny, E.c, (float)(rb + lane), w, lo, cnt);
+        each_cell(spans, 0, rb + lane, lo, cnt, [&](int, int dj, int di) {
+            raster_cell(G, a, R, K, td, orig, i0 + di, j0 + dj, vrow, count);
+            ++ntri;
+        });
+    }
+}
+
 // The listed large triangles, warp w taking entries w, w + warps, ... (every
-// warp has hundreds of entries, so the few very large triangles average out),
-// the cells of their rows' spans 32 at a time (0.16 ms for 37 aircraft aspects
-// at 10 GHz, 0.70 with every cell of the box a lane's). kSparse: then the
-// middling triangles that k_raster_sparse has listed (a.q_out), 32 a warp or as
-// many as keep every warp busy.
+// warp has hundreds of entries, so the few very large triangles average out;
+// 0.16 ms for 37 aircraft aspects at 10 GHz, 0.70 with every cell of the box a
+// lane's). kSparse: and then the middling triangles that k_raster_sparse has
+// listed (a.q_out), 32 at a time or as many as keep every warp busy; mostly there
+// are none of either, so the grid is what stays resident (launch and return in
+// 1.9 us, 4.3 with the dense grid's) and the warps take the work by a counter.
 template <bool kSparse>
 __global__ void __launch_bounds__(256, 3) k_raster_big(const TraceArgs a, unsigned long long* vis, int count)
 {
+    __shared__ uint2 s_span[8][32];
     const int lane = threadIdx.x & 31;
+    uint2* spans = s_span[threadIdx.x >> 5];
     const unsigned n_big = min(a.big_ctr[0], a.big_cap);
     const unsigned nw = (gridDim.x * blockDim.x) >> 5;
     unsigned long long ntri = 0;
-    __shared__ uint2 s_span[8][32];
-    for (unsigned it = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < n_big; it += nw) {
-        const int4 b = a.big[it];
-        const int td = b.x, ad = b.y;
-        if (a.vis_full[ad]) continue;  // traverses
-        const int i0 = b.z & 0xFFFF, j0 = (unsigned)b.z >> 16, w = (b.w & 0xFFFF) + 1, h = ((unsigned)b.w >> 16) + 1;
-        const int i1 = i0 + w - 1, j1 = j0 + h - 1;
-        const AngleDev& A = a.angles[ad];
-        const RasterGrid G = raster_grid(A);
-        const float4* tp = a.tris + 3 * (size_t)td;
-        const float4 P = __ldg(tp), B = __ldg(tp + 1), C = __ldg(tp + 2);
-        const RasterTri R = raster_tri(G, P, B, C, i0, i1, j0, j1);
-        if (!(R.bd >= 0.f)) continue;  // warp-uniform
-        const unsigned orig = (unsigned)__float_as_int(P.w);
-        unsigned long long* vrow = vis + a.ray_off[ad];
-        const PlaneKey K = plane_key(a.tri_nrm, td, G.d);
-        CellEdges E;
-        tri_cell_edges(A, cell_scale(A), P, B, C, i0, i1, j0, j1, E);
-        for (int rb = 0; rb < h; rb += 32) {
-            int lo = 0, cnt = 0;
-            if (rb + lane < h) row_span(E.nx, E.ny, E.c, (float)(rb + lane), w, lo, cnt);
-            each_cell(s_span[threadIdx.x >> 5], 0, rb + lane, lo, cnt, [&](int, int dj, int di) {
-                raster_cell(G, a, R, K, td, orig, i0 + di, j0 + dj, vrow, count);
-                ++ntri;
-            });
-        }
-    }
     if (kSparse) {
-        const unsigned n = min(a.big_ctr[1], sparse_list_cap(a)), per = min(32u, (n + nw - 1) / nw);
+        const unsigned n = min(a.big_ctr[1], sparse_list_cap(a)), per = max(1u, min(32u, (n + nw - 1) / nw));
+        const unsigned work = n_big + (n + per - 1) / per;
         const int2* list = reinterpret_cast<const int2*>(a.q_out);
-        for (unsigned it = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per; it < n; it += nw * per) {
-            const int2 e = (unsigned)lane < per && it + lane < n ? list[it + lane] : make_int2(-1, 0);
-            ntri += sparse_walk(a, vis, e.x, e.y, count);
+        while (work > 0) {
+            unsigned it = 0;
+            if (lane == 0) it = atomicAdd(a.big_ctr + 2, 1u);
+            it = __shfl_sync(kFull, it, 0);
+            if (it >= work) break;
+            if (it < n_big) {
+                raster_entry(a, vis, lane, it, spans, count, ntri);
+            } else {
+                it = (it - n_big) * per;
+                const int2 e = (unsigned)lane < per && it + lane < n ? list[it + lane] : make_int2(-1, 0);
+                ntri += sparse_walk(a, vis, e.x, e.y, spans, count);
+            }
         }
+    } else {
+        for (unsigned it = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < n_big; it += nw)
+            raster_entry(a, vis, lane, it, spans, count, ntri);
     }
     if (count) {
 #pragma unroll
@@ -1900,7 +1922,7 @@ __global__ void __launch_bounds__(256, 3) k_raster_big(const TraceArgs a, unsign
 // spans of 32 of them at a time (those that find no room are queued cell by
 // cell); larger ones go to its list of large triangles. 6 aspects of 800 x 800
 // rays over sheets whose triangles span 5 x 5 cells, beside a fine sphere, B = 2:
-// 4, 16 and 64 sheets in 1.3, 2.1 and 5.3 ms, with a warp each for triangles of
+// 4, 16 and 64 sheets in 1.3, 2.1 and 5.0 ms, with a warp each for triangles of
 // more than 16 cells 2.0, 5.8 and 15.5 (the list full from 8 sheets on). Bound by
 // instruction issue: ~235 instructions per 32 (triangle, aspect) items at 1 GHz
 // against ~820 of k_raster, 354 M items in 3.2 against 10.0 ms.
@@ -2001,7 +2023,7 @@ __global__ void __launch_bounds__(256, 3) k_raster_sparse(const TraceArgs a, int
                     }
                 }
             }
-            append_big(a, full, want_big, t, ang, i0, i1, j0, j1);
+            if (__any_sync(kFull, want_big)) append_some(a, full, want_big, t, ang, i0, i1, j0, j1);
             unsigned mc = __ballot_sync(kFull, n_cell > 0);
             if (!mc) continue;
             const unsigned ml = __ballot_sync(kFull, n_cell > kSparseCells);
@@ -2944,7 +2966,7 @@ cudaError_t launch_raster(const TraceArgs& a, int n_tri, unsigned long long* vis
         while (aspects > 1 && items() < 8ll * n_blocks) aspects /= 2;
         k_raster_sparse<<<(int)std::min<long long>((items() + kRasterWarps - 1) / kRasterWarps, n_blocks),
                           32 * kRasterWarps, 0, st>>>(a, n_tri, aspects, vis, full, count ? 1 : 0);
-        k_raster_big<true><<<n_blocks, 256, 0, st>>>(a, vis, count ? 1 : 0);
+        k_raster_big<true><<<std::max(1, n_blocks * 3 / 16), 256, 0, st>>>(a, vis, count ? 1 : 0);
     } else {
         const long long need = ((long long)a.n_angles * n_tri + 255) / 256;
         k_raster<<<(int)std::max(1ll, std::min<long long>(need, n_blocks)), 32 * kRasterWarps, kRasterSmem, st>>>(
